@@ -381,6 +381,9 @@ struct cse_ctx {
     uint8_t* bt_d2;         // drop bits at the second analysis
     uint32_t* bt_d2s;       // the same over sorted code triples, 3 bits an entry (packed form)
     bool bt_packed;         // the simulation kernel runs the packed per-trial form
+    uint8_t* bt_score;      // score of each final count, the largest of them bt_top: the packed form's
+    int32_t bt_top;         //   final plane holds scores (strictly rising with the count)
+    uint32_t* bt_dmin;      // least final S per (counted treatment - control) score difference (float bits)
     float4* bt_f4;          // final-analysis P(theta_self > theta_0) of the three treatments per sorted code triple
     float4* bk_q;           // basket design: (1 - P(theta_i > t_i | x)) per count state (see sim_basket.cu)
     uint32_t* keys;         // per-CTA statistic keys for order-statistic selection
@@ -406,6 +409,14 @@ struct cse_ctx {
     double prof_ms[KID_COUNT];
     int64_t prof_n[KID_COUNT];
 };
+
+// The packed four-arm form keeps its count table in two planes (see k_axis_counts):
+// both interim segments' counts in one byte, and the final count's score.
+inline bool cse_count_nibbles(const cse_ctx* c)
+{
+    return c->D.stat == CSE_STAT_BAYES4 && c->bt_tables && c->bt_packed && !c->bt_direct;
+}
+
 
 // bracket a kernel launch with profiler events (no-ops unless enabled)
 void cse_prof_begin(cse_ctx* c, int kid, cudaStream_t s);

@@ -430,27 +430,6 @@ __device__ __forceinline__ float design_stat_packed(const Looks& L, const Packed
     return use == 0u ? INFINITY : 1.0f - pm;
 }
 
-// A streaming load of the count table that does not allocate in L1 (each count
-// byte is read once per tile): L1 then keeps more final-table lines (refined
-// sample 25.45 -> 25.25 ms).
-__device__ __forceinline__ uint2 ld_stream2(const uint8_t* p)
-{
-    uint2 v;
-    asm("ld.global.nc.L1::no_allocate.v2.u32 {%0, %1}, [%2];" : "=r"(v.x), "=r"(v.y) : "l"(p));
-    return v;
-}
-
-// Byte transpose of four words: out[j] byte a = in[a] byte j.
-__device__ __forceinline__ void transpose4(const uint32_t in[4], uint32_t out[4])
-{
-    const uint32_t t0 = __byte_perm(in[0], in[1], 0x5140u), t1 = __byte_perm(in[2], in[3], 0x5140u);
-    const uint32_t t2 = __byte_perm(in[0], in[1], 0x7362u), t3 = __byte_perm(in[2], in[3], 0x7362u);
-    out[0] = __byte_perm(t0, t1, 0x5410u);
-    out[1] = __byte_perm(t0, t1, 0x7632u);
-    out[2] = __byte_perm(t2, t3, 0x5410u);
-    out[3] = __byte_perm(t2, t3, 0x7632u);
-}
-
 __device__ __forceinline__ int warp_sum_i(int v)
 {
 #pragma unroll
@@ -502,15 +481,6 @@ __device__ void find_kth(const uint32_t* hist, int nb, int ks, int* s_scan, int*
     __syncthreads();
 }
 
-// PACKED (with TABLES): the per-trial statistic by design_stat_packed, with
-// 512 threads and 2 CTAs per SM (the second-look table takes 61 KB of shared
-// memory per CTA; 64 registers a thread); otherwise 256 threads and 5 CTAs.
-template <bool PACKED>
-constexpr int b4_threads()
-{
-    return PACKED ? 512 : BT;
-}
-
 // Shared memory of the packed form: tri[v] = c (c + 1) / 2 and tri[256 + v] =
 // c (c + 1) (c + 2) / 6 for c = v >> 1 (final-look codes with their use bit),
 // tri[512 + u], tri[768 + u] the same for c = u >> 2 (second-look codes with the
@@ -536,49 +506,557 @@ __device__ __forceinline__ void packed_tables(int tid, int nth, int* tri, uint32
     }
 }
 
-template <bool TABLES, bool SELECT, bool PACKED>
-__global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 5)
-    k_sim_bayes4(TileArgs T, Looks L, float drop, const uint8_t* __restrict__ cnt, int32_t NA, int32_t k_stride,
-                 int32_t K_tiles, const uint8_t* __restrict__ D1g, const uint8_t* __restrict__ D2,
-                 const float4* __restrict__ F4, float lambda_up, SimOut o, uint32_t* __restrict__ keys,
-                 int32_t* __restrict__ counter, int32_t* __restrict__ err, const PackedConst Q,
-                 const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
+// ---------------------------------------------------------------------------
+// The tabulated simulation: only the trials that can decide anything are
+// evaluated.
+//
+// A tile's outputs depend on the trials with S < lambda (R, Xrej, score) and on
+// the k_i smallest S (k_i / K_i <= alpha: about two in a hundred), yet the drop
+// decisions and the final-table gather cost ~140 thread instructions a trial.
+// A lower bound on S from the final counts alone settles the rest.  With a
+// strictly rising score u of the final counts and D = max over the counted
+// treatments of u(count) - u(control's count),
+//   D < d  =>  S >= sigma(d) := min over the final-table entries of an active
+//                               treatment with score difference at most d - 1,
+// for any drop pattern, since every counted treatment's 1 - P is such an entry
+// (k_table_dmin).  A pass at difference d therefore evaluates the candidates
+// D >= d only: exact for R when lambda <= sigma(d), and for the order statistic
+// when the k_i-th smallest S among the candidates is at most sigma(d) (checked;
+// otherwise the pass is repeated at a lower d, down to every trial).
+//
+// The score is the angular transform asin(sqrt(.)), scaled to 0 .. 98: with raw
+// counts one difference means a smaller S for counts near 0 or n than in the
+// middle, and sigma(d) has to cover the worst (refined platten, d chosen with
+// hindsight: 21 % of the trials are candidates by raw counts, 14 % by score, 10 %
+// by the exact two-argument bound; 2.3 % are needed).
+//
+// The test D >= d runs on packed bytes, four trials a word: bit 7 of byte
+// u_i + (0x80 - d - u_0), no carry crossing a byte for the d allowed: 1.5
+// instructions a trial.  Each warp queues its candidates in shared memory and
+// evaluates them 32 at a time.  A tile starts with its first kSample trials, all
+// evaluated, and raises d after them and after 1, 2, 4, ... steps as far as the
+// keys found so far allow with a margin that shrinks to zero towards the end.
+// Keys go to the CTA's own stretch of global memory (4 % of the trials) and into
+// 256 bins of 1/16 octave; the order statistic is ranked within its bin.
+//
+// What bounds it: issue slots at the latency of the candidates' scattered reads
+// (47 % issue, 52 % ALU pipe, 62 warp instructions per 32 trials of which the
+// candidates take four fifths).  262,144 refined tiles x 65,536 trials:
+// 103 -> 40 ms; the 16^4 grid at K = 2^14: 5.6 -> 2.2 ms.  Measured on the way:
+// evaluating every candidate by raw counts with a margin fixed by the sample 65
+// ms, with d raised along the pass 51 ms; final-table loads that skip L1 lost
+// 10 %.
+//
+// Tiles: a group of NT / G threads per tile (named barriers), G tiles a block;
+// G = 1 only when there are too few tiles to give every group one.
+// ---------------------------------------------------------------------------
+constexpr double kScoreTop = 98.0;   // largest score (differences then span -29 .. 30 without carries)
+constexpr int kSample = 512;     // first trials of a tile, all evaluated to place d
+constexpr int kAllK = 1024;      // up to this K every trial is evaluated
+constexpr int kQueue = 288;      // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
+constexpr int kList = 256;       // keys of the selected bin ranked in shared memory
+
+// Bin of a key (S >= 0 as bits) in a group's 256-bin histogram: sixteen bins an
+// octave from 2^-16 up, the ends clamped.  Monotone in S.
+__device__ __forceinline__ int key_bin(uint32_t key)
 {
-    static_assert(TABLES || !PACKED, "the packed form reads the tables");
-    constexpr int NTH = b4_threads<PACKED>();
-    constexpr int NW = NTH / 32;
-    __shared__ uint32_t hist[2048];
+    return min(max((int)(key >> 19) - (int)(0x37800000u >> 19), 0), 255);
+}
+
+// dmin[D + u(n3)] (float bits, preset to +inf) = the least S an active treatment
+// with final score difference D to the control can give, over every state of the
+// final table.
+__global__ void __launch_bounds__(256) k_table_dmin(const float4* __restrict__ F4, Looks L,
+                                                    const uint8_t* __restrict__ score, uint32_t* __restrict__ dmin)
+{
+    __shared__ uint32_t m[2 * CSE_MAX_NMAX + 1];
+    __shared__ int u[CSE_MAX_NMAX + 1];
+    for (int j = threadIdx.x; j <= 2 * CSE_MAX_NMAX; j += blockDim.x) m[j] = 0x7F800000u;
+    for (int j = threadIdx.x; j <= L.n3; j += blockDim.x) u[j] = score[j];
+    __syncthreads();
+    const int top = u[L.n3];
+    const int64_t tot = (int64_t)(L.n3 + 1) * L.NT;
+    for (int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; s < tot; s += (int64_t)gridDim.x * blockDim.x) {
+        int t[3];
+        decode_triple((int)(s % L.NT), &t[0], &t[1], &t[2]);
+        const int c = (int)(s / L.NT);
+        const float4 q = __ldg(F4 + s);
+        const float p[3] = {q.x, q.y, q.z};
+#pragma unroll
+        for (int k = 0; k < 3; ++k)   // 0 <= P <= 1 (a0 <= Z term by term), so S's bits order as integers
+            if (t[k] >= L.S2) atomicMin(&m[u[t[k] - L.S2] - u[c] + top], __float_as_uint(1.0f - fmaxf(-1.0f, p[k])));
+    }
+    __syncthreads();
+    for (int j = threadIdx.x; j <= 2 * top; j += blockDim.x)
+        if (m[j] != 0x7F800000u) atomicMin(&dmin[j], m[j]);
+}
+
+template <int TT, int G>
+__device__ __forceinline__ void tile_sync(int g)
+{
+    // the TT threads of group g: named barrier 1 + g (barrier 0 is __syncthreads)
+    if (G == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(TT) : "memory");
+}
+
+// One warp: the bin of counts[0..256) holding the ks-th unit (from bin 0 up), -1
+// if the total is below ks, and the sum before it; ZERO clears the bins.
+template <bool ZERO>
+__device__ __forceinline__ int warp_pick256(uint32_t* counts, int ks, int lane, int* before)
+{
+    uint32_t h[8];
+    int local = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        h[j] = counts[lane * 8 + j];
+        local += (int)h[j];
+    }
+    if (ZERO)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) counts[lane * 8 + j] = 0u;
+    int incl = local;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, incl >= ks);
+    if (who == 0u) return -1;
+    const int src = __ffs(who) - 1;
+    int b = 0, cum = incl - local;
+#pragma unroll
+    for (int j = 0; j < 7; ++j)
+        if (b == j && cum + (int)h[j] < ks) {
+            cum += (int)h[j];
+            b = j + 1;
+        }
+    *before = __shfl_sync(0xffffffffu, cum, src);
+    return __shfl_sync(0xffffffffu, lane * 8 + b, src);
+}
+
+// Threads and blocks per SM: the packed form's shared-memory tables (57.6 KB)
+// and queues leave room for two blocks of 512; the byte form reads its tables
+// from global memory.
+template <bool PACKED>
+constexpr int b4_threads()
+{
+    return PACKED ? 512 : BT;
+}
+
+template <bool PACKED, int G>
+constexpr int b4_group()
+{
+    return b4_threads<PACKED>() / G;
+}
+
+template <bool SELECT, bool PACKED, int G, typename Off>
+__global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
+    k_sim_bayes4(TileArgs T, Looks L, const uint8_t* __restrict__ cnt, int32_t NA, int32_t k_stride, int32_t K_tiles,
+                 const uint8_t* __restrict__ D1g, const uint8_t* __restrict__ D2, const float4* __restrict__ F4,
+                 const uint8_t* __restrict__ score, const uint32_t* __restrict__ dmin, int32_t top, int32_t dlo,
+                 int32_t nd, float lambda_up, bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg, int32_t* __restrict__ counter, int32_t* __restrict__ err,
+                 const PackedConst Q, const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
+{
+    constexpr int NT = b4_threads<PACKED>();
+    constexpr int TT = b4_group<PACKED, G>();
+    constexpr int NW = TT / 32;
     __shared__ int s_tri[PACKED ? 1024 : 1];
     __shared__ uint32_t s_perm[PACKED ? 16 : 1];
+    __shared__ uint8_t s_inv[PACKED ? 128 : 1];   // final count of each score
+    __shared__ uint32_t s_raw[2 * CSE_MAX_NMAX + 1];
+    __shared__ float s_sig[2 * CSE_MAX_NMAX + 2];   // sigma(dlo + e), e < nd; +inf at e = 0 (every trial)
+    __shared__ int s_sbin[2 * CSE_MAX_NMAX + 2];    // its bin (256 at e = 0)
+    __shared__ int s_tile[G], s_next[G], s_pick[G], s_before[G], s_nlist[G], s_nk[G][NW];
+    __shared__ uint32_t s_res[G];
+    __shared__ int s_red[G][5][NW];
+    __shared__ unsigned long long s_min[G];   // order key of the least lambda_i of the group's tiles
+    // first-analysis drop table (two entries a byte) and, at d1_bytes (a multiple
+    // of 16), the sorted second-analysis table; then the warps' queues, the keys
+    // and the digit histograms
+    extern __shared__ __align__(16) uint8_t smem[];
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int g = tid / TT, lt = tid - g * TT, warp = lt >> 5;   // group, thread and warp in the group
+    const uint32_t* D2s = reinterpret_cast<const uint32_t*>(smem + d1_bytes);
+    uint32_t* const hists = reinterpret_cast<uint32_t*>(smem + d1_bytes + d2s_bytes);
+    uint32_t* const hist = hists + g * 256;
+    uint32_t* const list = hists + G * 256 + (SELECT ? g * kList : 0);
+    uint16_t* const queue = reinterpret_cast<uint16_t*>(hists + G * 256 + (SELECT ? G * kList : 0)) + (tid >> 5) * kQueue;
+    // each warp appends its keys to its own stretch of key_seg words
+    uint32_t* const kgrp = keys + (int64_t)(blockIdx.x * G + g) * NW * key_seg;
+    uint32_t* const kbuf = kgrp + (int64_t)warp * key_seg;
+    const unsigned below = (1u << lane) - 1u;
+
+    if (PACKED) {
+        const int m = L.n1 + 1, n1t = m * m * m * m;
+        for (int b = tid; 2 * b < n1t; b += NT)
+            smem[b] = (uint8_t)((D1g[2 * b] & 7) | ((2 * b + 1 < n1t ? D1g[2 * b + 1] & 7 : 0) << 4));
+        packed_tables(tid, NT, s_tri, s_perm);
+        // d2s_bytes: a multiple of 16, within the global table's allocation
+        for (int b = tid; b < d2s_bytes / 16; b += NT)
+            reinterpret_cast<uint4*>(smem + d1_bytes)[b] = __ldg(reinterpret_cast<const uint4*>(D2sg) + b);
+    }
+    if (PACKED)
+        for (int x = tid; x <= L.n3; x += NT) s_inv[score[x]] = (uint8_t)x;   // the scores are distinct
+    for (int j = tid; j <= 2 * top; j += NT) s_raw[j] = dmin[j];
+    for (int b = tid; b < G * 256; b += NT) hists[b] = 0u;
+    if (tid < G) s_min[tid] = ~0ull;
+    __syncthreads();
+    for (int e = tid; e < nd; e += NT) {
+        uint32_t v = 0x7F800000u;   // difference values below d = dlo + e
+        if (e > 0)
+            for (int j = 0; j < dlo + e + top; ++j) v = min(v, s_raw[j]);
+        s_sig[e] = __uint_as_float(v);
+        s_sbin[e] = e > 0 ? key_bin(v) : 256;
+    }
+    __syncthreads();
+    int e_lam = nd - 1;   // the highest d that is exact for the rejections
+    if (want_R) {
+        e_lam = 0;
+        for (int e = nd - 1; e > 0; --e)
+            if (s_sig[e] >= lambda_up) {
+                e_lam = e;
+                break;
+            }
+    }
+
+    if (lt == 0) s_next[g] = atomicAdd(counter, 1);
+    for (;;) {
+        if (lt == 0) {
+            s_tile[g] = s_next[g];
+            s_nlist[g] = 0;
+        }
+        tile_sync<TT, G>(g);
+        const int64_t i = s_tile[g];
+        if (i >= T.n_tiles) break;
+        if (lt == 0) s_next[g] = atomicAdd(counter, 1);   // the next tile, fetched while this one runs
+        const int K = T.K[i];
+        bool bad = (K < 1) || (K > K_tiles);
+        int v[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            v[a] = T.center_idx[i * 4 + a];
+            bad |= (v[a] < 0) || (v[a] >= T.n_axis[a]);
+        }
+        const uint32_t mask = T.null_mask[i] & 7u;   // counted treatments (none: S = +inf throughout)
+        const int Kc = (bad || mask == 0u) ? 0 : K;
+        // offsets of each arm's row of final scores; its interim rows lie whole
+        // planes before it
+        Off row[4];
+        const Off plane = (Off)NA * (Off)k_stride;
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+            row[a] = (PACKED ? 1 : 2) * plane + (Off)(T.axis_off[a] + (bad ? 0 : v[a])) * (Off)k_stride;
+        const int ks = (SELECT && !bad) ? o.ksel[i] : 0;
+        int r_acc = 0, xs[4] = {0, 0, 0, 0};
+        // a first pass starts with the sample (every trial) and moves d up as its
+        // keys allow; a repeated pass runs at one d
+        bool adapt = SELECT && ks >= 1 && Kc > kAllK;
+        int e = (SELECT && ks >= 1) ? 0 : e_lam;   // e = 0: every trial
+        double lam_i = -INFINITY;
+        for (int tries = 1;; ++tries) {
+            float sigma = s_sig[e];
+            int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
+            uint32_t a02 = 0u, a13 = 0u, waves = 0u;
+            // step -1 of a first pass: the sample, spread over the warps; then sixteen
+            // consecutive trials per thread and step from k0 on.  Bit 8 j + q of a
+            // thread's candidate word is trial 4 q + j.
+            constexpr int SW = kSample / NW;   // sample trials of a warp, a multiple of 16
+            const int k0 = adapt ? kSample : 0;
+            int st = adapt ? -1 : 0;
+            for (;; ++st) {
+                if (st >= 0 && k0 + st * (TT * 16) >= Kc) break;   // group-uniform
+                // first trial of the warp at the start of the queue's block of 64 steps
+                const int kb = st < 0 ? warp * SW : k0 + (st & ~63) * (TT * 16) + warp * 512;
+                const int stq = st < 0 ? 0 : st & 63;
+                const int kw = kb + stq * (TT * 16) + lane * 16;
+                const int kend = st < 0 ? (warp + 1) * SW : Kc;
+                uint32_t m = 0u;
+                if (kw < kend) {
+                    if (e == 0) {
+                        m = 0x0F0F0F0Fu;
+                    } else {
+                        const uint32_t zc = 0x80808080u - (uint32_t)(dlo + e) * 0x01010101u;
+                        const uint4 c = *reinterpret_cast<const uint4*>(cnt + (Off)(row[0] + (Off)kw));
+                        const uint32_t z[4] = {zc - c.x, zc - c.y, zc - c.z, zc - c.w};
+                        uint32_t t[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                        for (int a = 1; a < 4; ++a)
+                            if ((mask >> (a - 1)) & 1u) {
+                                const uint4 x = *reinterpret_cast<const uint4*>(cnt + (Off)(row[a] + (Off)kw));
+                                t[0] |= x.x + z[0];
+                                t[1] |= x.y + z[1];
+                                t[2] |= x.z + z[2];
+                                t[3] |= x.w + z[3];
+                            }
+                        m = ((t[0] >> 7) & 0x01010101u) | ((t[1] >> 6) & 0x02020202u) | ((t[2] >> 5) & 0x04040404u) |
+                            ((t[3] >> 4) & 0x08080808u);
+                    }
+                    if (kw + 16 > kend) {   // trials at or past K
+                        uint32_t in = 0u;
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int nb = min(max(kend - kw - 4 * q, 0), 4);
+                            in |= (nb == 4 ? 0x01010101u : (((1u << (8 * nb)) - 1u) & 0x01010101u)) << q;
+                        }
+                        m &= in;
+                    }
+                }
+                const int nm = __popc(m);
+                int incl = nm;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += y;
+                }
+                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                const bool flush = (st & 63) == 63 || k0 + (st + 1) * (TT * 16) >= Kc;
+                const int ent = (stq << 10) | (lane << 5);   // entry: step (6 bits), lane, bit
+                int done = 0;   // candidates of this step queued so far
+                do {
+                    // the lanes whose candidates fit the queue (a prefix of those left)
+                    const bool mine = incl - nm >= done && incl - done <= kQueue - qn;
+                    const unsigned who = __ballot_sync(0xffffffffu, mine);
+                    const int upto = __shfl_sync(0xffffffffu, incl, 31 - __clz(who));
+                    if (mine) {
+                        uint16_t* at = queue + qn + (incl - nm - done);
+                        while (m) {
+                            const int b = __ffs(m) - 1;
+                            m &= m - 1u;
+                            *at++ = (uint16_t)(ent | b);
+                        }
+                    }
+                    qn += upto - done;
+                    done = upto;
+                    __syncwarp();
+                    while (qn >= 32 || (flush && done == total && qn > 0)) {
+                        const int n = min(qn, 32);
+                        qn -= n;
+                        const int ev = queue[qn + (lane < n ? lane : 0)];
+                        const Off k = (Off)(kb + (ev >> 10) * (TT * 16) + ((ev & 0x3E0) >> 1) + ((ev & 7) << 2) +
+                                            ((ev >> 3) & 3));
+                        float S;
+                        uint32_t P2 = 0u;
+                        int xf[4];
+                        if constexpr (PACKED) {
+                            uint32_t E = 0u;
+#pragma unroll
+                            for (int a = 0; a < 4; ++a) {
+                                P2 |= (uint32_t)s_inv[__ldg(cnt + (Off)(row[a] + k))] << (8 * a);
+                                E |= (uint32_t)__ldg(cnt + (Off)(row[a] + k - plane)) << (8 * a);
+                            }
+                            const uint32_t P0 = (E >> 4) & 0x0F0F0F0Fu, P1 = P0 + (E & 0x0F0F0F0Fu);
+                            S = design_stat_packed(L, Q, smem, D2s, F4, s_tri, s_perm, P0, P1, P2, mask);
+                        } else {
+                            int xl[3][4];
+#pragma unroll
+                            for (int l = 0; l < 3; ++l)
+#pragma unroll
+                                for (int a = 0; a < 4; ++a) xl[l][a] = (int)__ldg(cnt + (Off)(row[a] + k - (Off)(2 - l) * plane));
+#pragma unroll
+                            for (int a = 0; a < 4; ++a) xf[a] = xl[2][a];
+                            const NodeConst C{};   // not read by the tabulated form
+                            S = design_stat<true>(L, D1g, D2, F4, C, 0.0f, xl, mask);
+                        }
+                        if (lane >= n) S = INFINITY;
+                        const uint32_t rej = (S < lambda_up) ? 1u : 0u;
+                        r_acc += (int)rej;
+                        if (PACKED) {
+                            a02 += (P2 & 0x00FF00FFu) * rej;
+                            a13 += __byte_perm(P2, 0u, 0x4341u) * rej;
+                            if ((++waves & 127u) == 0u) {   // 16-bit halves: 128 x 255 < 2^16
+                                xs[0] += (int)(a02 & 0xFFFFu);
+                                xs[2] += (int)(a02 >> 16);
+                                xs[1] += (int)(a13 & 0xFFFFu);
+                                xs[3] += (int)(a13 >> 16);
+                                a02 = a13 = 0u;
+                            }
+                        } else {
+#pragma unroll
+                            for (int a = 0; a < 4; ++a) xs[a] += (int)rej * xf[a];
+                        }
+                        if (SELECT) {
+                            const bool keep = S < sigma;
+                            const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                            if (ks >= 1) {
+                                if (keep) {
+                                    kbuf[wk + __popc(kept & below)] = __float_as_uint(S);
+                                    atomicAdd(&hist[key_bin(__float_as_uint(S))], 1u);
+                                }
+                                wk += __popc(kept);
+                            }
+                        }
+                        __syncwarp();   // the queue's entries read before the next round writes
+                    }
+                } while (done < total);
+                // after the sample and after 1, 2, 4, 8, ... steps of a first pass: d for
+                // the trials to come
+                if (SELECT && adapt && ((st + 1) & st) == 0) {
+                    tile_sync<TT, G>(g);
+                    if (warp == 0) {
+                        // the highest d such that the keys below sigma(d) so far, scaled to
+                        // all K trials and less 2.5 standard deviations, reach k_i
+                        const float seen = (float)min(k0 + (st + 1) * (TT * 16), Kc);
+                        const float f = ((float)Kc - seen) / seen, v = 2.5f * sqrtf(f * (1.0f + f));
+                        const float r = (v + sqrtf(v * v + 4.0f * (1.0f + f) * (float)ks)) / (2.0f * (1.0f + f));
+                        int before = 0;
+                        const int B = warp_pick256<false>(hist, (int)ceilf(r * r) + 1, lane, &before);
+                        int top = e;
+                        if (B >= 0)
+                            for (int j = lane; j <= e_lam; j += 32)
+                                if (s_sbin[j] > B) top = max(top, j);
+                        top = __reduce_max_sync(0xffffffffu, top);
+                        if (lane == 0) s_pick[g] = top;
+                    }
+                    tile_sync<TT, G>(g);
+                    e = s_pick[g];
+                    sigma = s_sig[e];
+                }
+            }
+            if (PACKED) {
+                xs[0] += (int)(a02 & 0xFFFFu);
+                xs[2] += (int)(a02 >> 16);
+                xs[1] += (int)(a13 & 0xFFFFu);
+                xs[3] += (int)(a13 >> 16);
+            }
+            if (!SELECT || ks < 1) break;
+            if (lane == 0) s_nk[g][warp] = wk;
+            tile_sync<TT, G>(g);
+            // the ks-th smallest key: its bin, then its rank among the bin's keys
+            int nk = 0;
+#pragma unroll
+            for (int w2 = 0; w2 < NW; ++w2) nk += s_nk[g][w2];
+            bool found = nk >= ks;
+            if (found) {
+                if (warp == 0) {
+                    int before = 0;
+                    const int b = warp_pick256<true>(hist, ks, lane, &before);
+                    if (lane == 0) {
+                        s_pick[g] = b;
+                        s_before[g] = before;
+                    }
+                }
+                tile_sync<TT, G>(g);
+                const int B = s_pick[g], kr = ks - s_before[g];
+                for (int k = lane; k < wk; k += 32) {   // each warp its own keys
+                    const uint32_t key = kbuf[k];
+                    if (key_bin(key) == B) {
+                        const int at = atomicAdd(&s_nlist[g], 1);
+                        if (at < kList) list[at] = key;
+                    }
+                }
+                tile_sync<TT, G>(g);
+                const int nl = s_nlist[g];
+                if (nl <= kList) {
+                    for (int j = lt; j < nl; j += TT) {
+                        const uint32_t key = list[j];
+                        int rank = 0;
+                        for (int q = 0; q < nl; ++q) {
+                            const uint32_t u = list[q];
+                            rank += (u < key || (u == key && q < j)) ? 1 : 0;
+                        }
+                        if (rank == kr - 1) s_res[g] = key;
+                    }
+                    tile_sync<TT, G>(g);
+                } else {   // radix select over the bin's keys: digits of 8, 8, 8 and 7 bits (S >= 0)
+                    uint32_t prefix = 0u, pmask = 0u;
+                    int kq = kr;
+                    for (int pass = 0; pass < 4; ++pass) {
+                        const int sh = pass < 3 ? 23 - 8 * pass : 0;
+                        const uint32_t dm = pass < 3 ? 0xFFu : 0x7Fu;
+                        for (int k = lane; k < wk; k += 32) {
+                            const uint32_t key = kbuf[k];
+                            if (key_bin(key) == B && (key & pmask) == prefix) atomicAdd(&hist[(key >> sh) & dm], 1u);
+                        }
+                        tile_sync<TT, G>(g);
+                        if (warp == 0) {
+                            int before = 0;
+                            const int digit = warp_pick256<true>(hist, kq, lane, &before);
+                            if (lane == 0) {
+                                s_pick[g] = digit;
+                                s_before[g] = before;
+                            }
+                        }
+                        tile_sync<TT, G>(g);
+                        prefix |= (uint32_t)s_pick[g] << sh;
+                        pmask |= dm << sh;
+                        kq -= s_before[g];
+                    }
+                    if (lt == 0) s_res[g] = prefix;
+                    tile_sync<TT, G>(g);
+                }
+                lam_i = (double)__uint_as_float(s_res[g]);
+                // exact unless it lies above the bound of the trials left out
+                found = lam_i <= (double)sigma;
+            } else {
+                for (int b = lt; b < 256; b += TT) hist[b] = 0u;
+                lam_i = INFINITY;   // with every trial evaluated, the k_i-th smallest S is +inf
+            }
+            if (found || e == 0) break;
+            // too few keys below sigma: the whole pass again at a lower d
+            e = tries < 4 ? max(e - 2 * tries, 0) : 0;
+            adapt = false;
+            r_acc = 0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) xs[a] = 0;
+            tile_sync<TT, G>(g);   // every thread has read the counts
+            if (lt == 0) s_nlist[g] = 0;
+            tile_sync<TT, G>(g);
+        }
+        r_acc = warp_sum_i(r_acc);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) xs[a] = warp_sum_i(xs[a]);
+        if (lane == 0) {
+            s_red[g][0][warp] = r_acc;
+            for (int a = 0; a < 4; ++a) s_red[g][1 + a][warp] = xs[a];
+        }
+        tile_sync<TT, G>(g);
+        if (lt == 0) {
+            if (bad) atomicOr(err, CSE_ERR_BAD_K);
+            int64_t Rt = 0, X[4] = {0, 0, 0, 0};
+            for (int w2 = 0; w2 < NW; ++w2) {
+                Rt += s_red[g][0][w2];
+                for (int a = 0; a < 4; ++a) X[a] += s_red[g][1 + a][w2];
+            }
+            if (o.R) o.R[i] = Rt;
+            if (o.cp_key)   // the tile's (K, R) in the Clopper-Pearson memo, as k_cp_mark would
+                o.cp_slot[i] = cp_memo_insert(((unsigned long long)(uint32_t)K << 32) | (uint32_t)Rt, o.cp_key,
+                                              o.cp_cap, o.cp_list, o.cp_nkeys);
+            for (int a = 0; a < 4; ++a) {
+                if (o.Xrej) o.Xrej[i * 4 + a] = X[a];
+                if (o.score) {
+                    const double sg = bad ? NAN : o.sig[T.axis_off[a] + v[a]];
+                    o.score[i * 4 + a] = (double)X[a] - (double)L.n3 * sg * (double)Rt;
+                }
+            }
+            if (SELECT && o.lam_tile) o.lam_tile[i] = lam_i;
+            if (SELECT) s_min[g] = min(s_min[g], order_key(lam_i));
+        }
+        tile_sync<TT, G>(g);
+    }
+    __syncthreads();   // every group done before the queue is reset
+    unsigned long long mine = ~0ull;
+    if (tid == 0)
+        for (int q = 0; q < G; ++q) mine = min(mine, s_min[q]);
+    queue_reset_min(counter, o.min_key, mine, SELECT ? o.min_out : nullptr);
+}
+
+// The direct form (plain path, CSE_OPT_BAYES_DIRECT, and designs whose tables
+// would not fit): the posterior evaluated for every trial, one tile per block.
+template <bool SELECT>
+__global__ void __launch_bounds__(BT, 5)
+    k_sim_bayes4_direct(TileArgs T, Looks L, float drop, const uint8_t* __restrict__ cnt, int32_t NA,
+                        int32_t k_stride, int32_t K_tiles, float lambda_up, SimOut o, uint32_t* __restrict__ keys,
+                        int32_t* __restrict__ counter, int32_t* __restrict__ err)
+{
+    constexpr int NTH = BT;
+    constexpr int NW = BWARP;
+    __shared__ uint32_t hist[2048];
     __shared__ int s_tile, s_scan[NW], s_res[2];
     __shared__ int s_red[5][NW];
     __shared__ unsigned long long s_min;   // order key of the least lambda_i of this CTA's tiles
     if (threadIdx.x == 0) s_min = ~0ull;
-    // first-analysis drop table (TABLES), then the packed form's second-analysis
-    // table at d1_bytes (a multiple of 16)
-    extern __shared__ __align__(16) uint8_t d1s[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    NodeConst C;
-    const uint8_t* D1 = D1g;
-    if (TABLES) {
-        const int m = L.n1 + 1, n1t = m * m * m * m;
-        if (PACKED) {   // two entries a byte
-            for (int b = tid; 2 * b < n1t; b += NTH)
-                d1s[b] = (uint8_t)((D1g[2 * b] & 7) | ((2 * b + 1 < n1t ? D1g[2 * b + 1] & 7 : 0) << 4));
-        } else {
-            for (int b = tid; b < n1t; b += NTH) d1s[b] = D1g[b];
-        }
-        D1 = d1s;
-    } else {
-        C = node_const();
-    }
-    const uint32_t* D2s = reinterpret_cast<const uint32_t*>(d1s + d1_bytes);
-    if (PACKED) {
-        packed_tables(tid, NTH, s_tri, s_perm);
-        // d2s_bytes: a multiple of 16, within the global table's allocation
-        for (int b = tid; b < d2s_bytes / 16; b += NTH)
-            reinterpret_cast<uint4*>(d1s + d1_bytes)[b] = __ldg(reinterpret_cast<const uint4*>(D2sg) + b);
-    }
+    const NodeConst C = node_const();
     uint32_t* kbuf = keys + (int64_t)blockIdx.x * k_stride;
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(counter, 1);
@@ -612,84 +1090,28 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 5)
                 for (int a = 0; a < 4; ++a)
                     w[l][a] = __ldg(reinterpret_cast<const uint32_t*>(cnt + (int64_t)row[l][a] * k_stride + k4));
         };
-        if constexpr (PACKED) {
-            // eight consecutive trials per thread and step (one 8-byte load per
-            // table row); the rejecting trials' final counts summed in 16-bit
-            // halves (arms 0 and 2, arms 1 and 3): at most 32 steps x 8 trials x
-            // 255 < 2^16 between flushes
-            for (int k8 = tid * 8; k8 < Kc;) {
-                uint32_t a02 = 0u, a13 = 0u;
-                for (int step = 0; step < 32 && k8 < Kc; ++step, k8 += NTH * 8) {
-                    uint32_t P[3][8], kq[8];
-                    {
-                        uint32_t wl[3][4], wh[3][4];
+        for (int k4 = tid * 4; k4 < Kc; k4 += NTH * 4) {
+            uint32_t w[3][4], kq[4];
+            load_rows(k4, w);
 #pragma unroll
-                        for (int l = 0; l < 3; ++l)
+            for (int j = 0; j < 4; ++j) {
+                float S = INFINITY;
+                if (k4 + j < Kc) {
+                    int xl[3][4];
 #pragma unroll
-                            for (int a = 0; a < 4; ++a) {
-                                const uint2 v2 =
-                                    ld_stream2(cnt + (int64_t)row[l][a] * k_stride + k8);
-                                wl[l][a] = v2.x;
-                                wh[l][a] = v2.y;
-                            }
+                    for (int l = 0; l < 3; ++l)
 #pragma unroll
-                        for (int l = 0; l < 3; ++l) {
-                            transpose4(wl[l], P[l]);
-                            transpose4(wh[l], P[l] + 4);
-                        }
-                    }
-                    auto sim8 = [&](auto full) {
+                        for (int a = 0; a < 4; ++a) xl[l][a] = (w[l][a] >> (8 * j)) & 0xFF;
+                    S = design_stat<false>(L, nullptr, nullptr, nullptr, C, drop, xl, mask);
+                    const int rej = (S < lambda_up) ? 1 : 0;
+                    r_acc += rej;
 #pragma unroll
-                        for (int j = 0; j < 8; ++j) {
-                            float S = INFINITY;
-                            if (decltype(full)::value || k8 + j < Kc) {
-                                S = design_stat_packed(L, Q, D1, D2s, F4, s_tri, s_perm, P[0][j], P[1][j], P[2][j],
-                                                       mask);
-                                const uint32_t rej = (S < lambda_up) ? 1u : 0u;
-                                r_acc += (int)rej;
-                                a02 += (P[2][j] & 0x00FF00FFu) * rej;
-                                a13 += __byte_perm(P[2][j], 0u, 0x4341u) * rej;
-                                if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
-                            }
-                            kq[j] = __float_as_uint(S);
-                        }
-                    };
-                    if (k8 + 8 <= Kc) sim8(std::true_type{});
-                    else sim8(std::false_type{});
-                    if (SELECT) {
-                        *reinterpret_cast<uint4*>(kbuf + k8) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
-                        *reinterpret_cast<uint4*>(kbuf + k8 + 4) = make_uint4(kq[4], kq[5], kq[6], kq[7]);
-                    }
+                    for (int a = 0; a < 4; ++a) xs[a] += rej * xl[2][a];   // integer multiply-add
+                    if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
                 }
-                xs[0] += (int)(a02 & 0xFFFFu);
-                xs[2] += (int)(a02 >> 16);
-                xs[1] += (int)(a13 & 0xFFFFu);
-                xs[3] += (int)(a13 >> 16);
+                kq[j] = __float_as_uint(S);
             }
-        } else {
-            for (int k4 = tid * 4; k4 < Kc; k4 += NTH * 4) {
-                uint32_t w[3][4], kq[4];
-                load_rows(k4, w);
-#pragma unroll
-                for (int j = 0; j < 4; ++j) {
-                    float S = INFINITY;
-                    if (k4 + j < Kc) {
-                        int xl[3][4];
-#pragma unroll
-                        for (int l = 0; l < 3; ++l)
-#pragma unroll
-                            for (int a = 0; a < 4; ++a) xl[l][a] = (w[l][a] >> (8 * j)) & 0xFF;
-                        S = design_stat<TABLES>(L, D1, D2, F4, C, drop, xl, mask);
-                        const int rej = (S < lambda_up) ? 1 : 0;
-                        r_acc += rej;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) xs[a] += rej * xl[2][a];   // integer multiply-add
-                        if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
-                    }
-                    kq[j] = __float_as_uint(S);
-                }
-                if (SELECT) *reinterpret_cast<uint4*>(kbuf + k4) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
-            }
+            if (SELECT) *reinterpret_cast<uint4*>(kbuf + k4) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
         }
         r_acc = warp_sum_i(r_acc);
 #pragma unroll
@@ -756,9 +1178,15 @@ template <bool TABLES>
 __global__ void k_emit_bayes4(TileArgs T, Looks L, float drop, const uint8_t* __restrict__ cnt, int32_t NA,
                               int32_t k_stride, int32_t K_tiles, const uint8_t* __restrict__ D1,
                               const uint8_t* __restrict__ D2, const float4* __restrict__ F4,
-                              const int64_t* __restrict__ off, float* __restrict__ S_out, int32_t* __restrict__ err)
+                              const int64_t* __restrict__ off, float* __restrict__ S_out, int32_t* __restrict__ err,
+                              bool nib, const uint8_t* __restrict__ score)
 {
-    const NodeConst C = node_const();
+    __shared__ uint8_t inv[128];
+    if (nib)
+        for (int x = threadIdx.x; x <= L.n3; x += blockDim.x) inv[score[x]] = (uint8_t)x;
+    __syncthreads();
+    NodeConst C;
+    if (!TABLES) C = node_const();
     for (int64_t i = blockIdx.x; i < T.n_tiles; i += gridDim.x) {
         const int K = T.K[i];
         bool bad = (K < 1) || (K > K_tiles);
@@ -774,9 +1202,17 @@ __global__ void k_emit_bayes4(TileArgs T, Looks L, float drop, const uint8_t* __
         const uint32_t mask = T.null_mask[i];
         for (int k = threadIdx.x; k < K; k += blockDim.x) {
             int xl[3][4];
-            for (int l = 0; l < 3; ++l)
-                for (int a = 0; a < 4; ++a)
-                    xl[l][a] = cnt[((int64_t)l * NA + T.axis_off[a] + v[a]) * k_stride + k];
+            for (int a = 0; a < 4; ++a) {
+                const uint8_t* p = cnt + (int64_t)(T.axis_off[a] + v[a]) * k_stride + k;
+                const int64_t plane = (int64_t)NA * k_stride;
+                if (nib) {   // the packed form's two planes
+                    xl[0][a] = p[0] >> 4;
+                    xl[1][a] = xl[0][a] + (p[0] & 15);
+                    xl[2][a] = inv[p[plane]];
+                } else {
+                    for (int l = 0; l < 3; ++l) xl[l][a] = p[l * plane];
+                }
+            }
             S_out[off[i] + k] = design_stat<TABLES>(L, D1, D2, F4, C, drop, xl, mask);
         }
     }
@@ -811,20 +1247,64 @@ int64_t b4_d2s_bytes(const Looks& L)
     return b4_round16(4 * (((int64_t)(L.n2 + 1) * b4_nt2(L) + 9) / 10));
 }
 
-// bytes of the first-analysis table in the kernel's shared memory: a byte an
-// entry, or two entries a byte in the packed form; padded to 16
-int64_t b4_d1_bytes(const Looks& L, bool packed)
+// bytes of the first-analysis table in the packed form's shared memory (two
+// entries a byte), padded to 16
+int64_t b4_d1_bytes(const Looks& L)
 {
     const int64_t n = (int64_t)(L.n1 + 1) * (L.n1 + 1) * (L.n1 + 1) * (L.n1 + 1);
-    return b4_round16(packed ? (n + 1) / 2 : n);
+    return b4_round16((n + 1) / 2);
 }
 
-template <bool TABLES, bool SEL, bool PACKED>
+// Selection keys: `rows` rows of `words` words.
+int b4_grow_keys(cse_ctx* c, int64_t rows, int64_t words)
+{
+    const size_t need = (size_t)rows * (size_t)words * sizeof(uint32_t);
+    if (need <= c->keys_cap) return CSE_OK;
+    cudaFree(c->keys);
+    c->keys = nullptr;
+    c->keys_cap = 0;
+    if (cudaMalloc(&c->keys, need) != cudaSuccess) {
+        cudaGetLastError();
+        return CSE_OOM;
+    }
+    c->keys_cap = need;
+    return CSE_OK;
+}
+
+template <typename Kern>
+int b4_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t blocks, int64_t* grid)
+{
+    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return CSE_UNSUPPORTED_DESIGN;
+    }
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
+    *grid = (int64_t)per_sm * c->num_sms;
+    if (*grid > blocks) *grid = blocks;
+    return CSE_OK;
+}
+
+// The range of differences d the byte test holds for scores 0 .. top without a
+// carry across bytes: 0 <= 128 - d - top and 128 - d + top <= 255 (d = dlo stands
+// for every trial).
+void b4_diff_range(int32_t top, int32_t* dlo, int32_t* nd)
+{
+    const int lo = top - 127 > -top ? top - 127 : -top;
+    const int hi = 128 - top < top + 1 ? 128 - top : top + 1;
+    *dlo = lo;
+    *nd = hi > lo ? hi - lo + 1 : 1;
+}
+
+template <bool SEL, bool PACKED, int G, typename Off>
 int launch_b4(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, double lambda,
               const SimOut& o, cudaStream_t s)
 {
-    auto kern = k_sim_bayes4<TABLES, SEL, PACKED>;
-    constexpr int NTH = b4_threads<PACKED>();
+    auto kern = k_sim_bayes4<SEL, PACKED, G, Off>;
+    constexpr int NT = b4_threads<PACKED>();
     const Looks L = make_looks(c->D);
     PackedConst Q{};
     if (PACKED) {
@@ -836,42 +1316,65 @@ int launch_b4(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32
         Q.off2 = s2 * 0x01010100u;
         Q.nt2 = b4_nt2(L);
     }
-    const int32_t d1_bytes = TABLES ? (int32_t)b4_d1_bytes(L, PACKED) : 0;
+    const int32_t d1_bytes = PACKED ? (int32_t)b4_d1_bytes(L) : 0;
     const int32_t d2s_bytes = PACKED ? (int32_t)b4_d2s_bytes(L) : 0;
-    const size_t smem = (size_t)d1_bytes + (size_t)d2s_bytes;
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return CSE_UNSUPPORTED_DESIGN;
-    }
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NTH, smem) != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        return CSE_CUDA_ERROR;
-    }
-    int64_t grid = (int64_t)per_sm * c->num_sms;
-    if (grid > T.n_tiles) grid = T.n_tiles;
-    if (SEL) {
-        const size_t need = (size_t)grid * (size_t)k_stride * sizeof(uint32_t);
-        if (need > c->keys_cap) {
-            cudaFree(c->keys);
-            c->keys = nullptr;
-            c->keys_cap = 0;
-            if (cudaMalloc(&c->keys, need) != cudaSuccess) {
-                cudaGetLastError();
-                return CSE_OOM;
-            }
-            c->keys_cap = need;
-        }
-    }
+    const size_t smem = (size_t)d1_bytes + (size_t)d2s_bytes + (size_t)G * 256 * 4 + (SEL ? (size_t)G * kList * 4 : 0) +
+                        (size_t)(NT / 32) * kQueue * 2;
+    int64_t grid = 0;
+    int st = b4_grid(c, kern, NT, smem, (T.n_tiles + G - 1) / G, &grid);
+    if (st != CSE_OK) return st;
+    // a warp's keys: its share of the sample and its 512 trials of every step
+    constexpr int TT = b4_group<PACKED, G>(), NW = TT / 32;
+    const int32_t key_seg = kSample / NW + (K_tiles + TT * 16 - 1) / (TT * 16) * 512;
+    if (SEL && (st = b4_grow_keys(c, grid * G, (int64_t)NW * key_seg)) != CSE_OK) return st;
+    int32_t dlo = 0, nd = 1;
+    b4_diff_range(c->bt_top, &dlo, &nd);
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
     cse_prof_begin(c, KID_SIM_BAYES4, s);
-    kern<<<(unsigned)grid, NTH, smem, s>>>(T, L, (float)c->D.drop, c->cnt, NA, k_stride, K_tiles, c->bt_d1, c->bt_d2,
-                                           c->bt_f4, lambda_float_up(lambda), o, c->keys, c->counter, c->err, Q,
-                                           c->bt_d2s, d1_bytes, d2s_bytes);
+    kern<<<(unsigned)grid, NT, smem, s>>>(T, L, c->cnt, NA, k_stride, K_tiles, c->bt_d1, c->bt_d2, c->bt_f4,
+                                          c->bt_score, c->bt_dmin, c->bt_top, dlo, nd, lambda_float_up(lambda),
+                                          o.R || o.Xrej || o.score || o.cp_key, o, c->keys, key_seg, c->counter, c->err,
+                                          Q, c->bt_d2s, d1_bytes, d2s_bytes);
     cse_prof_end(c, s);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+template <bool SEL>
+int launch_b4_direct(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, double lambda,
+                     const SimOut& o, cudaStream_t s)
+{
+    auto kern = k_sim_bayes4_direct<SEL>;
+    int64_t grid = 0;
+    int st = b4_grid(c, kern, BT, 0, T.n_tiles, &grid);
+    if (st != CSE_OK) return st;
+    if (SEL && (st = b4_grow_keys(c, grid, k_stride)) != CSE_OK) return st;
+    if (SEL && o.min_out) c->min_folded = true;
+    if (o.cp_key) c->cp_marked = true;
+    cse_prof_begin(c, KID_SIM_BAYES4, s);
+    kern<<<(unsigned)grid, BT, 0, s>>>(T, make_looks(c->D), (float)c->D.drop, c->cnt, NA, k_stride, K_tiles,
+                                       lambda_float_up(lambda), o, c->keys, c->counter, c->err);
+    cse_prof_end(c, s);
+    c->launches += 1;
+    return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+// Groups of a block: four tiles a block (two in the byte form) once every group
+// of the resident blocks has a tile, one tile a block below that.
+template <bool SEL, bool PACKED>
+int launch_b4_tables(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, double lambda,
+                     const SimOut& o, cudaStream_t s)
+{
+    constexpr int G = PACKED ? 4 : 2;
+    // 32-bit offsets into the count table while it is smaller than 4 GB
+    if ((uint64_t)(PACKED ? 2 : 3) * (uint64_t)NA * (uint64_t)k_stride > 0xFFFFFFFFull)
+        return launch_b4<SEL, PACKED, 1, uint64_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);
+    // (the groups' key rows are K words each: no more than one tile a block for
+    // the largest K, which keeps the keys of a launch below 1.3 GB)
+    if (T.n_tiles >= (int64_t)c->num_sms * 2 * G && K_tiles <= (1 << 17))
+        return launch_b4<SEL, PACKED, G, uint32_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);
+    return launch_b4<SEL, PACKED, 1, uint32_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);
 }
 
 }  // namespace
@@ -894,9 +1397,10 @@ int cse_bayes4_setup(cse_ctx* c, cudaStream_t s)
     k_table_d1<<<(unsigned)((n1 + 255) / 256), 256, 0, s>>>(c->bt_d1, L, drop);
     k_table_d2<<<(unsigned)((n2 + 255) / 256), 256, 0, s>>>(c->bt_d2, L, drop);
     // the packed per-trial form: every final-look code in seven bits, second-look
-    // codes in six, and both shared-memory tables within 96 KB (2 CTAs per SM)
+    // codes in six, both interim segments' counts in a nibble, and both
+    // shared-memory tables within 70 KB (2 CTAs per SM)
     const int64_t d2s = b4_d2s_bytes(L);
-    c->bt_packed = L.S3 <= 128 && L.S2 <= 64 && b4_d1_bytes(L, true) + d2s <= 96 * 1024;
+    c->bt_packed = L.S3 <= 128 && L.S2 <= 64 && L.n1 <= 15 && L.n2 - L.n1 <= 15 && b4_d1_bytes(L) + d2s <= 70 * 1024;
     if (c->bt_packed) {
         if (cudaMalloc(&c->bt_d2s, (size_t)d2s) != cudaSuccess) {
             cudaGetLastError();
@@ -911,8 +1415,33 @@ int cse_bayes4_setup(cse_ctx* c, cudaStream_t s)
         c->launches += 1;
     }
     k_table_f4<<<(unsigned)((n3 + 255) / 256), 256, 0, s>>>(c->bt_f4, L);
+    // scores of the final counts: in the packed form the angular transform (near
+    // constant variance, so one difference cuts at about the same S for every
+    // control count) scaled to 0 .. kScoreTop where that keeps them distinct; the
+    // counts themselves otherwise
+    std::vector<uint8_t> score((size_t)L.n3 + 1);
+    const double lo = asin(sqrt(1.0 / (L.n3 + 2.0))), hi = asin(sqrt((L.n3 + 1.0) / (L.n3 + 2.0)));
+    bool distinct = c->bt_packed;
+    for (int x = 0; x <= L.n3; ++x) {
+        score[x] = (uint8_t)lround(kScoreTop * (asin(sqrt((x + 1.0) / (L.n3 + 2.0))) - lo) / (hi - lo));
+        distinct &= x == 0 || score[x] > score[x - 1];
+    }
+    if (!distinct)
+        for (int x = 0; x <= L.n3; ++x) score[x] = (uint8_t)x;
+    c->bt_top = score[L.n3];
+    std::vector<uint32_t> none((size_t)(2 * c->bt_top + 1), 0x7F800000u);
+    if (cudaMalloc(&c->bt_dmin, none.size() * 4) != cudaSuccess || cudaMalloc(&c->bt_score, score.size()) != cudaSuccess) {
+        cudaGetLastError();
+        return CSE_OOM;
+    }
+    if (cudaMemcpyAsync(c->bt_dmin, none.data(), none.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(c->bt_score, score.data(), score.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
+    k_table_dmin<<<(unsigned)(4 * c->num_sms), 256, 0, s>>>(c->bt_f4, L, c->bt_score, c->bt_dmin);
     cse_prof_end(c, s);
-    c->launches += 3;
+    c->launches += 4;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
@@ -923,10 +1452,12 @@ int cse_launch_emit_bayes4(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_
     const Looks L = make_looks(c->D);
     if (c->bt_tables && !c->bt_direct)
         k_emit_bayes4<true><<<(unsigned)grid, 256, 0, s>>>(T, L, (float)c->D.drop, c->cnt, NA, k_stride, K_tiles,
-                                                           c->bt_d1, c->bt_d2, c->bt_f4, off, S_out, c->err);
+                                                           c->bt_d1, c->bt_d2, c->bt_f4, off, S_out, c->err,
+                                                           cse_count_nibbles(c), c->bt_score);
     else
         k_emit_bayes4<false><<<(unsigned)grid, 256, 0, s>>>(T, L, (float)c->D.drop, c->cnt, NA, k_stride, K_tiles,
-                                                            c->bt_d1, c->bt_d2, c->bt_f4, off, S_out, c->err);
+                                                            c->bt_d1, c->bt_d2, c->bt_f4, off, S_out, c->err,
+                                                           cse_count_nibbles(c), c->bt_score);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
@@ -937,11 +1468,11 @@ int cse_launch_sim_bayes4(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_s
     const bool sel = (o.lam_tile != nullptr && o.ksel != nullptr);
     if (c->bt_tables && !c->bt_direct) {
         if (c->bt_packed)
-            return sel ? launch_b4<true, true, true>(c, T, NA, k_stride, K_tiles, lambda, o, s)
-                       : launch_b4<true, false, true>(c, T, NA, k_stride, K_tiles, lambda, o, s);
-        return sel ? launch_b4<true, true, false>(c, T, NA, k_stride, K_tiles, lambda, o, s)
-                   : launch_b4<true, false, false>(c, T, NA, k_stride, K_tiles, lambda, o, s);
+            return sel ? launch_b4_tables<true, true>(c, T, NA, k_stride, K_tiles, lambda, o, s)
+                       : launch_b4_tables<false, true>(c, T, NA, k_stride, K_tiles, lambda, o, s);
+        return sel ? launch_b4_tables<true, false>(c, T, NA, k_stride, K_tiles, lambda, o, s)
+                   : launch_b4_tables<false, false>(c, T, NA, k_stride, K_tiles, lambda, o, s);
     }
-    return sel ? launch_b4<false, true, false>(c, T, NA, k_stride, K_tiles, lambda, o, s)
-               : launch_b4<false, false, false>(c, T, NA, k_stride, K_tiles, lambda, o, s);
+    return sel ? launch_b4_direct<true>(c, T, NA, k_stride, K_tiles, lambda, o, s)
+               : launch_b4_direct<false>(c, T, NA, k_stride, K_tiles, lambda, o, s);
 }

@@ -132,12 +132,17 @@ __global__ void k_thresholds(uint32_t* __restrict__ thr, double* __restrict__ si
 // run's first value, then a forward scan: ~0.4 uniforms pass per axis step on
 // the 256-value grids) instead of a binary search per value.  A threshold
 // below the previous one (unsorted axis values) restarts with a binary search.
+//
+// nib (the packed four-arm form): two planes instead of three, plane 0 the two
+// interim segments' counts in the two halves of a byte (first segment << 4 |
+// second segment; both at most 15), plane 1 the score of the final cumulative
+// count.
 constexpr int KB = 32;
 __global__ void __launch_bounds__(256) k_axis_counts(uint8_t* __restrict__ cnt, const uint32_t* __restrict__ U,
                                                      const uint32_t* __restrict__ thr, TileArgs T,
                                                      int32_t NA, int32_t K_max_ctx, int32_t K_tiles,
                                                      int32_t k_stride, int32_t n_looks, int4 looks,
-                                                     int32_t n_max)
+                                                     int32_t n_max, bool nib, const uint8_t* __restrict__ score)
 {
     pdl_entry();
     __shared__ uint32_t rows[KB * (CSE_MAX_NMAX + 1)];
@@ -150,6 +155,9 @@ __global__ void __launch_bounds__(256) k_axis_counts(uint8_t* __restrict__ cnt, 
         const int row = i / n_max;
         rows[row * stride + (i - row * n_max)] = src[i];
     }
+    __shared__ uint8_t s_score[CSE_MAX_NMAX + 1];
+    if (nib)
+        for (int i = threadIdx.x; i <= n_max; i += blockDim.x) s_score[i] = score[i];
     __syncthreads();
     const int kk = threadIdx.x & (KB - 1);
     const int nw = blockDim.x / KB, w = threadIdx.x / KB;
@@ -186,6 +194,13 @@ __global__ void __launch_bounds__(256) k_axis_counts(uint8_t* __restrict__ cnt, 
         const bool back = t < tp;
         tp = t;
         j0 = advance(r, len0, j0, t, back);
+        if (nib) {
+            j1 = advance(r1, len1, j1, t, back);
+            j2 = advance(r2, len2, j2, t, back);
+            out[0] = (uint8_t)((j0 << 4) | j1);
+            out[look_stride] = s_score[j0 + j1 + j2];
+            continue;
+        }
         out[0] = (uint8_t)j0;
         if (n_looks > 1) {
             j1 = advance(r1, len1, j1, t, back);
@@ -372,11 +387,15 @@ int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, 
 {
     dim3 grid((K_tiles + KB - 1) / KB, T.d);
     int4 lk = make_int4(c->D.look_n[0], c->D.look_n[1], c->D.look_n[2], 0);
+    const bool nib = cse_count_nibbles(c);
     cse_prof_begin(c, KID_AXIS_COUNTS, s);
     cse_launch(c->pdl, k_axis_counts, dim3(grid), dim3(256), 0, s, c->cnt, c->U, c->thr, T, n_axis_total, c->K_max, K_tiles,
-                                       k_stride, c->D.n_looks, lk, c->D.n_max);
-    cse_launch(c->pdl, k_axis_box, dim3(n_axis_total), dim3(256), 0, s, c->cnt, n_axis_total, k_stride, K_tiles, c->D.n_looks - 1, c->bb);
+                                       k_stride, c->D.n_looks, lk, c->D.n_max, nib, c->bt_score);
+    c->launches += 1;
+    if (!cse_posterior_design(c->D.stat)) {   // the z-test cell kernel reads the boxes
+        cse_launch(c->pdl, k_axis_box, dim3(n_axis_total), dim3(256), 0, s, c->cnt, n_axis_total, k_stride, K_tiles, c->D.n_looks - 1, c->bb);
+        c->launches += 1;
+    }
     cse_prof_end(c, s);
-    c->launches += 2;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
