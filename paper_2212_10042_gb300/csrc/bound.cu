@@ -766,256 +766,310 @@ CSE_HD double cp_upper(int64_t R, int64_t N, double delta)
     return cp_finish_fp64(R, N, delta, u);
 }
 
-// Search interval of the cooperative FP32 stage: lo = 0 and hi = 1 or 14 standard
-// deviations above the mean of Beta(R+1, N-R) (a log-concave law, so F(hi) is
-// below e^-13 there).
-CSE_HD void cp_interval(int64_t R, int64_t N, float* lo, float* hi)
-{
-    const float a = (float)R + 1.0f, b = (float)(N - R), s = a + b;
-    const float mean = a / s;
-    const float sd = sqrtf(a * b / (s * s * (s + 1.0f)));
-    *lo = 0.0f;
-    *hi = fminf(1.0f, mean + 14.0f * sd + 4.0f / s);
-}
-
-// Point j of one round of the cooperative search: 32 interior points split
-// (lo, hi) into 33 equal parts.
-CSE_HD void cp_round_points(float lo, float hi, int j, float* uj)
-{
-    *uj = lo + (hi - lo) * ((float)(j + 1) / 33.0f);
-}
-
 // ---------------------------------------------------------------------------
-// Warp-wide FP64 evaluation of the Clopper-Pearson equation.  On this part an
-// FP64 warp instruction costs the same pipe time however many lanes it has
-// active, so the per-key FP64 work is spread over the 32 lanes:
+// Clopper-Pearson by groups of L lanes, one key a group.
+//
+// An FP64 warp instruction takes the same pipe time (64 cycles) however many of
+// its lanes are active, so a key's FP64 work is spread over the lanes of a group
+// and a warp solves 32 / L keys with one instruction stream:
 //  * the continued fraction as a composition of linear fractional maps, i.e. a
-//    product of 2x2 matrices (associative): each lane multiplies 8 consecutive
-//    levels, a 5-step shuffle tree forms the ordered product, and the product
-//    of the first 16 lanes gives, for free, the convergent at half the depth,
+//    product of 2x2 matrices (associative): each lane multiplies its consecutive
+//    levels, a shuffle tree forms the ordered product, and the product of the
+//    first half of the lanes gives, for free, the convergent at half the depth,
 //    which is the convergence test;
-//  * the small-R binomial sum as a warp prefix product of term ratios.
-// Every lane returns the same value.
+//  * the two log1p of the prefactor, its three Stirling terms and the logarithm of
+//    the fraction one a lane;
+//  * the small-R binomial sum as an ordered product of (product, sum) pairs.
+// The density over the tail, which the Halley step needs, follows from the
+// fraction alone: pdf / tail = 1 / (h u (1 - u)).
+// A key starts at the two-term Cornish-Fisher point of Beta(R + 1, N - R), takes
+// FP32 Halley steps of the same evaluation to ~1e-5 standard deviations, then one
+// FP64 Halley step (error of the order of the step cubed).  Levels needed for
+// N <= 65536 at delta = 0.01, 0.005: at most 28 for 1e-6, 110 for 1e-15; a pass
+// holds 32 in FP32 and 96 in FP64 (two to a step of the contracted fraction).
 // ---------------------------------------------------------------------------
+template <typename T>
 struct Mat2 {
-    double m00, m01, m10, m11;
+    T m00, m01, m10, m11;
 };
 
-__device__ __forceinline__ Mat2 mat2_mul(const Mat2& A, const Mat2& B)
+template <typename T>
+__device__ __forceinline__ Mat2<T> mat2_mul(const Mat2<T>& A, const Mat2<T>& B)
 {
     return {fma(A.m00, B.m00, A.m01 * B.m10), fma(A.m00, B.m01, A.m01 * B.m11),
             fma(A.m10, B.m00, A.m11 * B.m10), fma(A.m10, B.m01, A.m11 * B.m11)};
 }
 
-__device__ __forceinline__ int exp_field(double x)
+// x 2^k (x normal or zero, the result too): an integer addition to the exponent
+// field instead of an FP64 multiplication.
+__device__ __forceinline__ double scale_exp(double x, int k)
 {
-    return (__double2hiint(x) >> 20) & 0x7ff;
+    const int hi = __double2hiint(x);
+    return (hi & 0x7FFFFFFF) ? __hiloint2double(hi + (k << 20), __double2loint(x)) : 0.0;
 }
 
 // Scales by the power of two that brings the largest entry into [1, 2): exact,
-// and the convergents are ratios of entries, so they are unchanged.
-__device__ __forceinline__ Mat2 mat2_norm(Mat2 A)
+// and the convergents are ratios of entries, so they are unchanged.  Entries below
+// 2^-900 of the largest become zero.  (FP32 entries stay in range without it.)
+__device__ __forceinline__ void mat2_norm(Mat2<double>& A)
 {
-    int e = max(max(exp_field(A.m00), exp_field(A.m01)), max(exp_field(A.m10), exp_field(A.m11)));
-    e = min(max(e, 1), 2045);
-    const double sc = __hiloint2double((2046 - e) << 20, 0);
+    auto ex = [](double x) { return (__double2hiint(x) >> 20) & 0x7ff; };
+    const int e0 = ex(A.m00), e1 = ex(A.m01), e2 = ex(A.m10), e3 = ex(A.m11);
+    const int e = max(max(e0, e1), max(e2, e3)), k = 1023 - e;
+    A.m00 = e0 > e - 900 ? scale_exp(A.m00, k) : 0.0;
+    A.m01 = e1 > e - 900 ? scale_exp(A.m01, k) : 0.0;
+    A.m10 = e2 > e - 900 ? scale_exp(A.m10, k) : 0.0;
+    A.m11 = e3 > e - 900 ? scale_exp(A.m11, k) : 0.0;
+}
+
+__device__ __forceinline__ void mat2_norm(Mat2<float>& A)
+{
+    const float m = fmaxf(fmaxf(A.m00, A.m01), fmaxf(A.m10, A.m11));   // entries are not negative
+    const int e = min(max((__float_as_int(m) >> 23) & 0xff, 1), 253);
+    const float sc = __int_as_float((254 - e) << 23);
     A.m00 *= sc;
     A.m01 *= sc;
     A.m10 *= sc;
     A.m11 *= sc;
-    return A;
 }
 
-__device__ __forceinline__ Mat2 mat2_shfl_down(const Mat2& A, int s)
+// Right-multiplies C by the map t -> p / (q + k t), [[0, p], [k, q]].
+template <typename T>
+__device__ __forceinline__ void cf_step(Mat2<T>& C, T p, T q, T k)
 {
-    return {__shfl_down_sync(0xffffffffu, A.m00, s), __shfl_down_sync(0xffffffffu, A.m01, s),
-            __shfl_down_sync(0xffffffffu, A.m10, s), __shfl_down_sync(0xffffffffu, A.m11, s)};
-}
-
-__device__ __forceinline__ Mat2 mat2_bcast(const Mat2& A, int src)
-{
-    return {__shfl_sync(0xffffffffu, A.m00, src), __shfl_sync(0xffffffffu, A.m01, src),
-            __shfl_sync(0xffffffffu, A.m10, src), __shfl_sync(0xffffffffu, A.m11, src)};
-}
-
-// Right-multiplies C by the map t -> d / (1 + t), d = p / q, as the matrix
-// [[0, p], [q, q]] (a common factor q does not change the map).
-__device__ __forceinline__ void cf_level(Mat2& C, double p, double q)
-{
-    const double c00 = C.m00, c10 = C.m10;
-    C.m00 = C.m01 * q;
+    const T c00 = C.m00, c10 = C.m10;
+    C.m00 = C.m01 * k;
     C.m01 = fma(c00, p, C.m01 * q);
-    C.m10 = C.m11 * q;
+    C.m10 = C.m11 * k;
     C.m11 = fma(c10, p, C.m11 * q);
 }
 
-// The fraction 1/(1 + d1/(1 + d2/(1 + ...))) of I_x(a, b) (same d_j as beta_cf),
-// as the composition of the maps t -> 1/(1 + t) (level 0) and t -> d_j/(1 + t)
-// applied to t = 0: with Q = N_0 N_1 ... N_n, the n-level convergent is
-// Q01 / Q11, a ratio of two entries of one column, and rescaling Q by a power
-// of two leaves it exact.  Lane chunk g holds levels 8g .. 8g+7, so level 0
-// is multiplied first, in sequence, where the leading partial fractions
-// cancel (d_{2m+1} near -1 for x near the mean).  For integer b the fraction
-// ends at d_{2b} = 0; the levels past it are left out.
-__device__ double beta_cf_warp(double a, double b, double x, int lane)
+template <typename T, int L>
+__device__ __forceinline__ Mat2<T> mat2_down(const Mat2<T>& A, int s, unsigned mask)
 {
-    constexpr int PAIRS = 4;   // levels (d_{2m}, d_{2m+1}) per lane per pass
-    Mat2 P = {1.0, 0.0, 0.0, 1.0};
-    double f = 0.0;
-    for (int pass = 0; pass < 16; ++pass) {   // 256 levels a pass
-        Mat2 C = {1.0, 0.0, 0.0, 1.0};
-        const double g = (double)(pass * 32 + lane);
+    return {__shfl_down_sync(mask, A.m00, s, L), __shfl_down_sync(mask, A.m01, s, L),
+            __shfl_down_sync(mask, A.m10, s, L), __shfl_down_sync(mask, A.m11, s, L)};
+}
+
+template <typename T, int L>
+__device__ __forceinline__ Mat2<T> mat2_first(const Mat2<T>& A, unsigned mask)
+{
+    return {__shfl_sync(mask, A.m00, 0, L), __shfl_sync(mask, A.m01, 0, L), __shfl_sync(mask, A.m10, 0, L),
+            __shfl_sync(mask, A.m11, 0, L)};
+}
+
+// h with I_x(a, b) = x^a (1-x)^b / B(a, b) h, from lam = a - (a + b) x >= 0: the even
+// contraction of the fraction 1/(1 + d1/(1 + d2/(1 + ...))) of beta_cf, whose step
+// n is the map t -> alpha_n / (beta_n + t) with
+//   alpha_n = (a+n-1)(a+b+n-1) n (b-n) x^2 / (a+2n-1)^2      (alpha_0 = 1),
+//   beta_n  = (a+2n)(1 + d_{2n} + d_{2n+1})
+//           = n + n(b-n)x/(a+2n-1) + (a+n)(lam + 1 + n(2-x))/(a+2n+1):
+// all terms positive for n < b, so nothing cancels (d_{2n+1} is near -1), and
+// for integer b the fraction ends at n = b; the steps past it are left out.  h is
+// the composition of the maps applied to t = 0: with Q the product of their
+// matrices, Q01 / Q11.  In FP64 a step is multiplied through by (a+2n-1)^2
+// (a+2n+1) instead of divided (a common factor does not change the map); in FP32
+// it is scaled by a + 2n, which keeps the entries in range.  The convergents close
+// in geometrically, so a half-depth difference of 1e-9 (FP32: 1e-3) leaves the
+// full depth at rounding; one pass does at the usual delta, more are needed as u
+// nears the mean.
+template <typename T, int L>
+__device__ T beta_cf_group(T a, T b, T x, T lam, int l, unsigned mask)
+{
+    constexpr bool F64 = sizeof(T) == 8;
+    constexpr int STEPS = (F64 ? 48 : 16) / L;   // per lane and pass
+    const T s = a + b;
+    Mat2<T> P = {(T)1, (T)0, (T)0, (T)1};
+    T f = (T)0;
+    for (int pass = 0; pass < 40; ++pass) {
+        Mat2<T> C = {(T)1, (T)0, (T)0, (T)1};
+        const T g = (T)((pass * L + l) * STEPS);
 #pragma unroll
-        for (int i = 0; i < PAIRS; ++i) {
-            const double m = fma((double)PAIRS, g, (double)i);
-            if (m < b) {
-                const double a2m = fma(2.0, m, a);
-                if (m > 0.0)   // d_{2m} = m(b-m) x / ((a+2m-1)(a+2m))
-                    cf_level(C, (m * (b - m)) * x, (a2m - 1.0) * a2m);
-                else           // level 0: t -> 1/(1 + t)
-                    C = {0.0, 1.0, 1.0, 1.0};
-                const double am = a + m;   // d_{2m+1} = -(a+m)(a+b+m) x / ((a+2m)(a+2m+1))
-                cf_level(C, -(am * (am + b)) * x, a2m * (a2m + 1.0));
+        for (int i = 0; i < STEPS; ++i) {
+            const T n = g + (T)i;
+            if (n < b) {
+                const T an = a + n, dm = an + (n - (T)1), dp = an + (n + (T)1);
+                const T w = n * (b - n) * x, c = fma(n, (T)2 - x, lam + (T)1);
+                const T num = n > (T)0 ? (an - (T)1) * (s + (n - (T)1)) * (w * x) : (T)1;
+                if (F64) {
+                    const T d2 = dm * dm;
+                    // n = 0: alpha = 1, so the factor is dp alone
+                    if (n > (T)0) cf_step(C, num * dp, fma(d2, fma(an, c, n * dp), w * dm * dp), d2 * dp);
+                    else cf_step(C, dp, an * c, dp);
+                } else {
+                    const float im = fdiv_fast(1.0f, (float)dm), ip = fdiv_fast(1.0f, (float)dp);
+                    const float k = fdiv_fast(1.0f, (float)(an + n));   // 1 / (a + 2n)
+                    const float pv = n > (T)0 ? (float)num * im * im * k : k;
+                    cf_step<T>(C, (T)pv, (T)(((float)n + (float)w * im + (float)(an * c) * ip) * k), (T)k);
+                }
             }
+            // a step grows FP64 entries by at most 2^85, shrinks FP32 ones by at most 2^-20
+            if (F64 ? (i % 6) == 5 : (i % 4) == 3) mat2_norm(C);
         }
-        C = mat2_norm(C);
-        Mat2 half = C;
+        mat2_norm(C);
+        Mat2<T> half = C;
 #pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {   // lane 0 ends with lanes 0..2sh-1
-            C = mat2_norm(mat2_mul(C, mat2_shfl_down(C, sh)));
-            if (sh == 8) half = C;
+        for (int sh = 1; sh < L; sh <<= 1) {   // lane 0 ends with lanes 0..2sh-1
+            half = C;
+            C = mat2_mul(C, mat2_down<T, L>(C, sh, mask));
+            mat2_norm(C);
         }
-        const Mat2 Pm = mat2_mul(P, mat2_bcast(half, 0));
-        P = mat2_norm(mat2_mul(P, mat2_bcast(C, 0)));
-        const double f_mid = Pm.m01 / Pm.m11;
+        // lane 0 forms both convergents; the group takes its decision
+        const Mat2<T> Ph = mat2_mul(P, half);
+        P = mat2_mul(P, C);
+        mat2_norm(P);
+        P = mat2_first<T, L>(P, mask);
+        const T f_mid = __shfl_sync(mask, Ph.m01 / Ph.m11, 0, L);
         f = P.m01 / P.m11;
-        if (fabs(f - f_mid) <= 1e-14 * fabs(f)) break;
+        if (!(fabs(f - f_mid) > (T)(F64 ? 1e-9 : 1e-3) * fabs(f))) break;
     }
     return f;
 }
 
-// The logarithms and Stirling remainders of log_bpre, one per lane: lane k
-// evaluates term k (the same function of the same argument as the serial
-// form, so the values agree bit for bit) and every lane receives all of them.
-//   0 log u, 1 log1p(-u), 2 log1p(e/a), 3 log1p(-e/b), 4 log(ab/(a+b)),
-//   5 log(a+b), 6 log1p(a/b), 7 log1p(b/a), 8 log b, 9..11 stirling_rem(a, b, a+b)
-constexpr int N_PREFIX_TERMS = 12;
-__device__ void prefix_terms_warp(double a, double b, double u, int lane, double* T)
+template <typename T, int L>
+__device__ __forceinline__ T group_sum(T v, unsigned mask)
 {
-    const double e = fma(u, a + b, -a);
-    double num = 1.0, den = 1.0;
-    int kind = 0;   // 0 log(num/den), 1 log1p(num/den), 2 Stirling remainder of den, 3 none
-    switch (lane) {
-    case 0: num = u; break;
-    case 1: num = -u; kind = 1; break;
-    case 2: num = e; den = a; kind = 1; break;
-    case 3: num = -e; den = b; kind = 1; break;
-    case 4: num = a * b; den = a + b; break;
-    case 5: num = a + b; break;
-    case 6: num = a; den = b; kind = 1; break;
-    case 7: num = b; den = a; kind = 1; break;
-    case 8: num = b; break;
-    case 9: den = a; kind = 2; break;
-    case 10: den = b; kind = 2; break;
-    case 11: den = a + b; kind = 2; break;
-    default: kind = 3;
-    }
-    const double q = num / den;
-    double v = 0.0;
-    if (kind == 0) {
-        v = log(q);
-    } else if (kind == 1) {
-        v = log1p(q);
-    } else if (kind == 2) {   // stirling_rem with r = 1/z
-        const double r2 = q * q;
-        v = q * (1.0 / 12.0 - r2 * (1.0 / 360.0 - r2 * (1.0 / 1260.0 - r2 * (1.0 / 1680.0 - r2 / 1188.0))));
-    }
 #pragma unroll
-    for (int k = 0; k < N_PREFIX_TERMS; ++k) T[k] = __shfl_sync(0xffffffffu, v, k);
+    for (int sh = L / 2; sh > 0; sh >>= 1) v += __shfl_xor_sync(mask, v, sh, L);
+    return v;
 }
 
-// log_bpre from the lane-evaluated terms (same formulas, same operation order).
-__device__ double log_bpre_terms(double a, double b, const double* T)
-{
-    const double L2PI = 1.8378770664093454836;
-    if (a >= 10.0 && b >= 10.0) return a * T[2] + b * T[3] + 0.5 * T[4] - 0.5 * L2PI - (T[9] + T[10] - T[11]);
-    if (b >= 10.0) return a * T[0] + b * T[1] - lgamma_small_int(a) + a * T[5] + (b - 0.5) * T[6] - a + T[11] - T[10];
-    if (a >= 10.0) return a * T[0] + b * T[1] - lgamma_small_int(b) + b * T[5] + (a - 0.5) * T[7] - b + T[11] - T[9];
-    return a * T[0] + b * T[1] - lgamma_small_int(a) - lgamma_small_int(b) + lgamma_small_int(a + b);
-}
+__device__ __forceinline__ double g_log(double x) { return log(x); }
+__device__ __forceinline__ float g_log(float x) { return logf(x); }
+__device__ __forceinline__ double g_log1p(double x) { return log1p(x); }
+__device__ __forceinline__ float g_log1p(float x) { return log1pf(x); }
+__device__ __forceinline__ double g_stirling(double z) { return stirling_rem(z); }
+__device__ __forceinline__ float g_stirling(float z) { return stirling_rem_f(z); }
 
-__device__ double log_binom_cdf_warp(double a, double b, double u, double* lpdf, int lane)
+// Log of the tail the solve works on and *r = density at u over that tail, for a, b >= 10
+// (a = R + 1, b = N - R): upper (u above the mean) P(Binom <= R) = I_{1-u}(b, a), else its
+// complement I_u(a, b).
+template <typename T, int L>
+__device__ T log_tail_cf(T a, T b, T u, bool upper, T* r, int l, unsigned mask)
 {
-    double T[N_PREFIX_TERMS];
-    prefix_terms_warp(a, b, u, lane, T);
-    const double lp = log_bpre_terms(a, b, T);
-    *lpdf = lp - T[0] - T[1];
-    if (u >= (a + 1.0) / (a + b + 2.0)) return lp + log(beta_cf_warp(b, a, 1.0 - u, lane)) - T[8];
-    return log1p(-exp(lp) * beta_cf_warp(a, b, u, lane) / a);
-}
-
-// Small R: the terms t_j = prod_{i<=j} r_i, r_i = (N-i+1) w / i, by a warp
-// prefix product; their sum by a butterfly (bitwise equal in every lane).
-__device__ double log_binom_cdf_small_warp(int64_t R, int64_t N, double u, double* lpdf, int lane)
-{
-    const double l1u = log1p(-u);
-    const double w = u / (1.0 - u);
-    double carry = 1.0, sum = 0.0, tR = 1.0;
-    for (int64_t j0 = 1; j0 <= R; j0 += 32) {
-        const int64_t j = j0 + lane;
-        double t = (j <= R) ? (double)(N - j + 1) * w / (double)j : 1.0;
+    const T s = a + b, e = fma(u, s, -a);   // u (a + b) - a
+    const T cf = upper ? beta_cf_group<T, L>(b, a, (T)1 - u, e, l, mask) : beta_cf_group<T, L>(a, b, u, -e, l, mask);
+    *r = (T)1 / (cf * u * ((T)1 - u));
+    T v = (T)0;
 #pragma unroll
-        for (int sh = 1; sh < 32; sh <<= 1) {
-            const double o = __shfl_up_sync(0xffffffffu, t, sh);
-            if (lane >= sh) t *= o;
+    for (int t = 0; t < 6; t += L) {   // term t + l on lane l
+        const int k = t + l;
+        if (k < 2) {
+            const T z = k ? b : a;
+            v += z * g_log1p((k ? -e : e) / z);
+        } else if (k < 5) {
+            const T st = g_stirling(k == 2 ? a : k == 3 ? b : s);
+            v += k == 4 ? st : -st;
+        } else if (k == 5) {   // log(sqrt(a b / (a + b)) cf)
+            v += (T)0.5 * g_log(cf * cf * (a * b / s));
         }
-        t *= carry;
-        double ts = (j <= R) ? t : 0.0;
-#pragma unroll
-        for (int sh = 16; sh > 0; sh >>= 1) ts += __shfl_xor_sync(0xffffffffu, ts, sh);
-        sum += ts;
-        const int64_t last = R - j0;   // lane holding j = R, when in this pass
-        if (last < 32) tR = __shfl_sync(0xffffffffu, t, (int)last);
-        carry = __shfl_sync(0xffffffffu, t, 31);
     }
-    sum += 1.0;
-    const double base = (double)N * l1u;
-    const double lg = log(lane == 0 ? (double)(N - R) * tR : sum);   // two logarithms, two lanes
-    *lpdf = __shfl_sync(0xffffffffu, lg, 0) + base - l1u;
-    return base + __shfl_sync(0xffffffffu, lg, 1);
+    return group_sum<T, L>(v, mask) - (T)0.91893853320467274178;   // log(2 pi) / 2
 }
 
-// cp_finish_fp64 with the warp-wide evaluation (all lanes call it together).
-__device__ double cp_finish_warp(int64_t R, int64_t N, double delta, double u, int lane)
+// The same for R < CP_SMALL_R, each lane taking a stretch of the terms: upper
+//   log P(Binom(N, u) <= R) = N log(1-u) + log sum_{j<=R} C(N,j) w^j, w = u / (1-u),
+// else (delta > 0.9, u well below the mean)
+//   log P(Binom(N, u) > R) = log t_{R+1} + log(1 + sum of the next terms over t_{R+1}),
+// whose terms fall fast: kTailTerms of them reach below rounding.
+constexpr int kTailTerms = 96;
+
+template <typename T, int L>
+__device__ T log_tail_sum(int R, T N, T u, bool upper, T* r, int l, unsigned mask)
+{
+    const T w = u / ((T)1 - u);
+    const int R1 = upper ? R : R + 1;
+    const int per = (R1 + L - 1) / L, j0 = l * per + 1, j1 = min(R1, (l + 1) * per);
+    T p = (T)1, sum = (T)0;   // product and sum of the partial products of the stretch
+    for (int j = j0; j <= j1; ++j) {
+        p *= (N - (T)(j - 1)) * w / (T)j;
+        sum += p;
+    }
+    auto chain = [&](T& p0, T& s0) {   // the ordered composition over the lanes, in every lane
+#pragma unroll
+        for (int sh = 1; sh < L; sh <<= 1) {
+            const T p2 = __shfl_down_sync(mask, p0, sh, L), s2 = __shfl_down_sync(mask, s0, sh, L);
+            s0 = fma(p0, s2, s0);
+            p0 *= p2;
+        }
+        p0 = __shfl_sync(mask, p0, 0, L);
+        s0 = __shfl_sync(mask, s0, 0, L) + (T)1;
+    };
+    chain(p, sum);
+    if (upper) {
+        *r = (N - (T)R) * p / (sum * ((T)1 - u));
+        return fma(N, g_log1p(-u), g_log(sum));
+    }
+    T q = (T)1, tail = (T)0;
+    for (int i = 0; i < kTailTerms / L; ++i) {
+        const T j = (T)(R + 2 + l * (kTailTerms / L) + i);
+        q *= (N - (j - (T)1)) * w / j;   // zero from j = N + 1 on
+        tail += q;
+    }
+    chain(q, tail);
+    *r = (T)(R + 1) / (u * tail);
+    return fma(N, g_log1p(-u), g_log(p * tail));
+}
+
+// One Halley step on phi(u) = log tail - target from f = phi(u): phi' = -r (upper)
+// or r, phi'' = phi' ((a-1)/u - (b-1)/(1-u)) - r^2; kept inside the bracket (lo,
+// hi), which the sign of f narrows.  The second-order term in FP32: it enters
+// times f.
+template <typename T>
+__device__ __forceinline__ T cp_halley(T u, T f, T r, T a, T b, bool upper, T* lo, T* hi)
+{
+    const T p1 = upper ? -r : r;
+    const float uf = (float)u, pf = (float)p1;
+    const float p2 = pf * (((float)a - 1.0f) / uf - ((float)b - 1.0f) / (1.0f - uf)) - pf * pf;
+    const T den = (T)2 * p1 * p1 - f * (T)p2;
+    if ((f > (T)0) == upper) *lo = u;
+    else *hi = u;
+    const T un = u - (T)2 * f * p1 / den;
+    return (un >= *lo && un <= *hi) ? un : (T)0.5 * (*lo + *hi);
+}
+
+// u with P(Binom(N, u) <= R) = delta, 0 < R < N, all lanes of a group together; comp =
+// 1 - delta from the caller, who may know it to more digits; z is the normal
+// quantile of comp.
+template <int L>
+__device__ double cp_upper_group(int64_t R, int64_t N, double delta, double comp, float z, int l, unsigned mask)
 {
     const double a = (double)R + 1.0, b = (double)(N - R);
-    const double ld = log(delta);
-    const bool small = R < CP_SMALL_R && N - R > CP_SMALL_R;
+    const bool small = R < CP_SMALL_R && (N - R > CP_SMALL_R || delta > 0.9);
+    if (!small && (a < 10.0 || b < 10.0)) return cp_upper(R, N, delta);   // few trials: every lane alike
+    const bool upper = delta <= (small ? 0.9 : 0.5);
+    const double target = log(upper ? delta : comp);
+    const float af = (float)a, bf = (float)b, sf = af + bf;
+    const float mean = af / sf, sd = sqrtf(af * bf / (sf * sf * (sf + 1.0f)));
+    const float skew = 2.0f * (bf - af) * sqrtf(sf + 1.0f) / ((sf + 2.0f) * sqrtf(af * bf));
+    float u = mean + sd * (z + skew * (z * z - 1.0f) * (1.0f / 6.0f));
+    u = fminf(fmaxf(u, 0.02f * mean), 0.5f * (mean + 1.0f));
+    float lof = 0.0f, hif = 1.0f;
+    for (int it = 0; it < 12; ++it) {
+        float r;
+        const float lt = small ? log_tail_sum<float, L>((int)R, (float)N, u, upper, &r, l, mask)
+                               : log_tail_cf<float, L>(af, bf, u, upper, &r, l, mask);
+        const float un = cp_halley<float>(u, lt - (float)target, r, af, bf, upper, &lof, &hif);
+        const float step = __shfl_sync(mask, fabsf(un - u), 0, L);   // one decision for the group
+        u = __shfl_sync(mask, un, 0, L);
+        if (!(__shfl_sync(mask, r, 0, L) > 0.0f)) break;
+        if (!(step > 1e-3f * fminf(sd, fminf(u, 1.0f - u)))) break;   // the next one would be ~1e-9 of it
+    }
+    double ud = (u > 0.0f && u < 1.0f) ? (double)u : (double)mean;   // a poor start costs FP64 steps
     double lo = 0.0, hi = 1.0;
     for (int it = 0; it < 60; ++it) {
-        double lpdf;
-        double lF = small ? log_binom_cdf_small_warp(R, N, u, &lpdf, lane)
-                          : log_binom_cdf_warp(a, b, u, &lpdf, lane);
-        lF = __shfl_sync(0xffffffffu, lF, 0);   // keep the control flow warp-uniform
-        lpdf = __shfl_sync(0xffffffffu, lpdf, 0);
-        const double f = lF - ld;
-        if (f == 0.0) break;
-        const double r = exp(lpdf - lF);
-        const double p1 = -r;
-        const double p2 = -r * ((a - 1.0) / u - (b - 1.0) / (1.0 - u)) - r * r;
-        const double den = 2.0 * p1 * p1 - f * p2;
-        const double du = (den != 0.0) ? -2.0 * f * p1 / den : -f / p1;
-        if (fabs(du) <= 4e-16 * u) break;
-        if (f > 0.0) lo = u; else hi = u;
-        double un = u + du;
-        if (!(un > lo && un < hi)) un = 0.5 * (lo + hi);
-        const double step = fabs(un - u);
-        u = un;
-        if (step <= 3e-6 * fmin(u, 1.0 - u) || hi - lo <= 4e-16 * hi) break;
+        double r;
+        const double lt = small ? log_tail_sum<double, L>((int)R, (double)N, ud, upper, &r, l, mask)
+                                : log_tail_cf<double, L>(a, b, ud, upper, &r, l, mask);
+        const double un = cp_halley<double>(ud, lt - target, r, a, b, upper, &lo, &hi);
+        const double step = __shfl_sync(mask, fabs(un - ud), 0, L);
+        ud = __shfl_sync(mask, un, 0, L);
+        // far on the wrong side of the mean the fraction loses its sign: the serial solve
+        if (!(__shfl_sync(mask, r, 0, L) > 0.0)) return cp_upper(R, N, delta);
+        if (!(step > 2e-5 * fmin((double)sd, fmin(ud, 1.0 - ud))) || hi - lo <= 4e-16 * hi) break;
     }
-    return u;
+    return ud;
 }
-
 
 // Device-side argument checks of tile i: a tile must meet some null hypothesis
 // (null_mask != 0) and have half-widths h >= 0 (h = 0: a point); false and the
@@ -1118,77 +1172,54 @@ __global__ void k_cp_mark(int64_t n_tiles, const int64_t* __restrict__ R, const 
     slot[i] = cp_memo_insert(key, keys, cap, list, n_keys);
 }
 
-// Distinct (K, R) keys 0 .. n_warp-1 take one warp each (the latency of one
-// key is the solve's critical path when keys are few): 4 rounds of 32 FP32
-// evaluations (one per lane) narrow the root to ~1e-6 relative, then the warp
-// finishes it in FP64.  Key w goes to block w % warp_blocks, so keys spread
-// over the SMs before they share one.  Keys beyond n_warp (many distinct keys:
-// throughput matters) take one thread each in the remaining blocks, which run
-// beside the warp blocks.  (16 warps a block with one key each took the
-// two-arm 256^2 solve from 66 to 56 us, but at 128 registers a block then
-// fills an SM, the thread blocks wait for the warp blocks, and the 2^18 batch
-// and the basket lost 0.45 and 0.52 ms.)
-constexpr int CP_WARPS_PER_BLOCK = 4;
-constexpr int CP_KEYS_PER_WARP = 2;
+// The distinct (K, R) keys, a group of 8 lanes each: key t goes to group t / W of
+// warp t % W (W warps in the grid), so keys spread over the warps before they
+// share one.  Beyond kCpManyKeys the FP64 pipe is full and the total work counts:
+// 2 lanes a key do less of it (fewer tree steps, more of the serial levels).
+// Bound by the latency of one warp's chain of FP64 instructions until every
+// sub-partition has a few warps.  Against a warp for each of the first 1,216 keys
+// (bracketing by FP32 rounds, 256 levels) and a thread for each further key: one
+// arm, 64 keys 37 -> 28 us; 1,500 distinct keys 212 -> 29; 6,036 keys 353 -> 64;
+// two-arm batch 350 -> 60; basket 16^4 274 -> 110.
+constexpr int kCpThreads = 128;
+constexpr int kCpBlocksPerSM = 3;
+constexpr int kCpManyKeys = 40000;
 
-__global__ void __launch_bounds__(32 * CP_WARPS_PER_BLOCK) k_cp_solve(unsigned long long* __restrict__ keys,
-                                                  const uint32_t* __restrict__ list,
-                                                  const int32_t* __restrict__ n_keys, double delta0,
-                                                  double delta1, double* __restrict__ u0s, int warp_blocks)
+template <int L>
+__device__ __forceinline__ void cp_solve_keys(unsigned long long* __restrict__ keys, const uint32_t* __restrict__ list,
+                                              int n, double delta0, double delta1, float z0,
+                                              double* __restrict__ u0s)
 {
-    pdl_entry();
-    const int n = *n_keys;
-    const int n_warp = min(n, warp_blocks * CP_WARPS_PER_BLOCK * CP_KEYS_PER_WARP);
-    if ((int)blockIdx.x < warp_blocks) {
-        const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-        for (int w = blockIdx.x + warp_blocks * wib; w < n_warp; w += warp_blocks * CP_WARPS_PER_BLOCK) {
-            const uint32_t h = list[w];
-            const unsigned long long key = keys[h];
-            const int64_t R = (int64_t)(uint32_t)key, N = (int64_t)((key >> 32) & 0x7FFFFFFFull);
-            const double delta = (key >> 63) ? delta1 : delta0;
-            if (R >= N || R <= 0) {
-                if (lane == 0) {
-                    u0s[h] = R >= N ? 1.0 : -expm1(log(delta) / (double)N);
-                    keys[h] = kEmptyKey;   // the table is empty again for the next call
-                }
-                continue;
-            }
-            const float ldf = logf((float)delta);
-            float lo, hi;
-            cp_interval(R, N, &lo, &hi);
-            for (int round = 0; round < 4; ++round) {
-                float uj;
-                cp_round_points(lo, hi, lane, &uj);
-                const float f = cp_f32(R, N, uj, ldf, nullptr);
-                const unsigned below = __ballot_sync(0xffffffffu, !(f > 0.0f));   // root at or left of uj
-                if (below == 0u) {
-                    lo = __shfl_sync(0xffffffffu, uj, 31);
-                } else {
-                    const int jf = __ffs(below) - 1;
-                    const float uj_hi = __shfl_sync(0xffffffffu, uj, jf);
-                    const float uj_lo = __shfl_sync(0xffffffffu, uj, jf > 0 ? jf - 1 : 0);
-                    hi = uj_hi;
-                    if (jf > 0) lo = uj_lo;
-                }
-            }
-            // The FP64 stage is safeguarded on [0, 1]: an FP32 bracket that missed
-            // the FP64 root only costs it extra steps.
-            const double u = cp_finish_warp(R, N, delta, 0.5 * ((double)lo + (double)hi), lane);
-            if (lane == 0) {
-                u0s[h] = u;
-                keys[h] = kEmptyKey;
-            }
-        }
-        return;
-    }
-    const int stride = (gridDim.x - warp_blocks) * blockDim.x;
-    for (int t = n_warp + (blockIdx.x - warp_blocks) * blockDim.x + threadIdx.x; t < n; t += stride) {
+    const int lane = threadIdx.x & 31, l = lane & (L - 1), g = lane / L;
+    const unsigned mask = (L == 32 ? 0xffffffffu : ((1u << L) - 1u) << (g * L));
+    const int W = gridDim.x * (kCpThreads / 32);
+    for (int t = g * W + (threadIdx.x >> 5) * gridDim.x + blockIdx.x; t < n; t += W * (32 / L)) {
         const uint32_t h = list[t];
         const unsigned long long key = keys[h];
         const int64_t R = (int64_t)(uint32_t)key, N = (int64_t)((key >> 32) & 0x7FFFFFFFull);
-        u0s[h] = cp_upper(R, N, (key >> 63) ? delta1 : delta0);
-        keys[h] = kEmptyKey;
+        const bool tag = (key >> 63) != 0;   // the lower bound's solve at delta1 = 1 - delta0
+        const double delta = tag ? delta1 : delta0, comp = tag ? delta0 : delta1;
+        double u;
+        if (R >= N) u = 1.0;
+        else if (R <= 0) u = -expm1((tag ? log1p(-comp) : log(delta)) / (double)N);
+        else u = cp_upper_group<L>(R, N, delta, comp, tag ? -z0 : z0, l, mask);
+        __syncwarp(mask);
+        if (l == 0) {
+            u0s[h] = u;
+            keys[h] = kEmptyKey;   // the table is empty again for the next call
+        }
     }
+}
+
+__global__ void __launch_bounds__(kCpThreads, kCpBlocksPerSM) k_cp_solve(unsigned long long* __restrict__ keys,
+                                                         const uint32_t* __restrict__ list,
+                                                         const int32_t* __restrict__ n_keys, double delta0,
+                                                         double delta1, float z0, double* __restrict__ u0s)
+{
+    pdl_entry();
+    const int n = *n_keys;
+    if (n <= kCpManyKeys) cp_solve_keys<8>(keys, list, n, delta0, delta1, z0, u0s);
+    else cp_solve_keys<2>(keys, list, n, delta0, delta1, z0, u0s);
 }
 
 // Upper: u0 = Clopper-Pearson upper bound of R / K, bound = optimised tile
@@ -1228,7 +1259,7 @@ __global__ void __launch_bounds__(128) k_bounds(TileArgs T, int32_t n_max, const
         if (2 * Ri > Ki) {
             const double ap = PLAIN ? cp_upper_plain(Ki - Ri, Ki, delta)
                                     : memo ? u0s[slot[i]] : cp_upper(Ki - Ri, Ki, delta);
-            l = 1.0 - ap;
+            l = Ri == Ki ? exp(log(delta) / (double)Ki) : 1.0 - ap;   // l^K = delta when every trial rejects
             la = log(ap);
         } else if (Ri <= 0) {
             l = 0.0;
@@ -1323,6 +1354,18 @@ __global__ void k_backward(int64_t n, int32_t d, const double* __restrict__ g, c
 
 }  // namespace
 
+// z with Phi(z) = p (0 < p < 1), to ~1e-7: the start of the Clopper-Pearson solves.
+double normal_quantile(double p)
+{
+    double lo = -40.0, hi = 40.0;
+    for (int it = 0; it < 60; ++it) {
+        const double mid = 0.5 * (lo + hi);
+        if (0.5 * erfc(-mid * 0.70710678118654752440) < p) lo = mid;
+        else hi = mid;
+    }
+    return 0.5 * (lo + hi);
+}
+
 template <int D>
 void launch_bounds_d(cse_ctx* c, unsigned blocks, const TileArgs& T, const int64_t* R, double delta, bool lower,
                      double* u0, double* bound, double* qstar, const int32_t* slot, const double* geom,
@@ -1376,11 +1419,11 @@ int cse_launch_bounds(cse_ctx* c, const TileArgs& T, const int64_t* R, double de
                        (uint32_t)c->cp_cap, c->cp_slot, c->cp_list, c->cp_nkeys, lower);
             c->launches += 1;
         }
-        const int64_t warp_keys = (int64_t)c->num_sms * CP_WARPS_PER_BLOCK * CP_KEYS_PER_WARP;
-        constexpr int cp_threads = 32 * CP_WARPS_PER_BLOCK;
-        const int64_t thread_blocks = std::max<int64_t>(0, (T.n_tiles - warp_keys + cp_threads - 1) / cp_threads);
-        cse_launch(c->pdl, k_cp_solve, dim3((unsigned)(c->num_sms + thread_blocks)), dim3(cp_threads), 0,
-                   s, c->cp_key, c->cp_list, c->cp_nkeys, delta, 1.0 - delta, c->cp_val, c->num_sms);
+        // a group of 8 lanes per key at most, spread over the SMs
+        const int64_t full = (int64_t)c->num_sms * kCpBlocksPerSM;
+        const int64_t blocks_cp = std::min<int64_t>(full, (T.n_tiles + kCpThreads / 32 - 1) / (kCpThreads / 32));
+        cse_launch(c->pdl, k_cp_solve, dim3((unsigned)blocks_cp), dim3(kCpThreads), 0, s, c->cp_key, c->cp_list,
+                   c->cp_nkeys, delta, 1.0 - delta, (float)normal_quantile(1.0 - delta), c->cp_val);
         cse_prof_end(c, s);
         c->launches += 1;
         slot = c->cp_slot;
