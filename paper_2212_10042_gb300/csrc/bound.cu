@@ -30,14 +30,11 @@ constexpr int BISECT_F32 = 4;        // FP32 bisection steps on [0, SMAX] before
 constexpr int SECANT_F32 = 16;       // cap on FP32 secant (Illinois) steps
 constexpr float SECANT_TOL = 1e-5f;  // FP32 stage ends when the bracket is this narrow ...
 constexpr float SECANT_STEP = 5e-6f; // ... or when a secant step is this short
+constexpr int kSplitWarps = 3;      // warps a sub-partition up to which the signs are split (split_signs)
 constexpr int POLISH_IT = 80;   // cap on FP64 safeguarded-Newton steps
 
 struct ArmGeom {
     double th, h, n, sp0, d1p, d1m;   // d1p/d1m = sp(th +/- h) - sp(th)
-};
-
-struct ArmGeomF {
-    float th, h, n, sig0, sp0, d1p, d1m;
 };
 
 CSE_HD __forceinline__ double softplus(double x) { return fmax(x, 0.0) + log1p(exp(-fabs(x))); }
@@ -52,62 +49,11 @@ CSE_HD __forceinline__ void arm_init(ArmGeom& g, double th, double h, double n)
     g.d1m = softplus(th - h) - g.sp0;
 }
 
-CSE_HD __forceinline__ void arm_init_f(ArmGeomF& f, const ArmGeom& g)
-{
-    f.th = (float)g.th;
-    f.h = (float)g.h;
-    f.n = (float)g.n;
-    f.sig0 = (float)(1.0 / (1.0 + exp(-g.th)));
-    f.sp0 = (float)g.sp0;
-    f.d1p = (float)g.d1p;
-    f.d1m = (float)g.d1m;
-}
-
 // ---------------------------------------------------------------------------
 // Per-arm terms.  phi_a(q, v) = n [sp(th + q v) - sp(th)] / q - n [sp(th + v) - sp(th)];
 // Phi(q) = sum_a max over v = +-h_a of phi_a; derivatives follow the maximising
 // branch (on a tie, the one with the larger first derivative: right derivatives).
 // ---------------------------------------------------------------------------
-
-// FP32: the difference sp(th + x) - sp(th) = log1p(sigmoid(th) expm1(x)) for small
-// |x| (no cancellation), directly otherwise.
-template <int D>
-CSE_HD void tilt_phi_f(const ArmGeomF* G, float q, float* Phi, float* dPhi)
-{
-    constexpr int d = D;
-    float P = 0.f, dP = 0.f;
-    const float iq = 1.0f / q;
-#pragma unroll
-    for (int a = 0; a < d; ++a) {
-        float best = -INFINITY, bestd = 0.f;
-#pragma unroll
-        for (int sg = 0; sg < 2; ++sg) {
-            const float v = sg ? -G[a].h : G[a].h;
-            const float x = q * v;
-            const float y = G[a].th + x;
-            const float e = expf(-fabsf(y));
-            const float l1e = log1pf(e);
-            const float r = e / (1.0f + e);
-            float Dd;
-            if (fabsf(x) < 0.5f) Dd = log1pf(G[a].sig0 * expm1f(x));
-            else Dd = fmaxf(y, 0.0f) + l1e - G[a].sp0;
-            const float phi = G[a].n * (Dd * iq - (sg ? G[a].d1m : G[a].d1p));
-            // x sigmoid(y) - D without cancellation at large |x|
-            float hq;
-            if (fabsf(x) < 0.5f) hq = x * ((y >= 0.f) ? 1.0f - r : r) - Dd;
-            else hq = (y >= 0.f) ? (G[a].sp0 - G[a].th) - x * r - l1e : x * r - l1e + G[a].sp0;
-            const float dphi = G[a].n * hq * iq * iq;
-            if (phi > best || (phi == best && dphi > bestd)) {
-                best = phi;
-                bestd = dphi;
-            }
-        }
-        P += best;
-        dP += bestd;
-    }
-    *Phi = P;
-    *dPhi = dP;
-}
 
 // FP64 value and first two q-derivatives along the maximising branches.
 template <int D>
@@ -193,21 +139,9 @@ CSE_HD double obj_ds(const ArmGeom* G, int kind, double lc, double s, double* d2
     return q * g1;
 }
 
-template <int D>
-CSE_HD float obj_ds_f(const ArmGeomF* G, int kind, float lc, float s)
-{
-    const float q = expf(s);
-    float P, dP;
-    tilt_phi_f<D>(G, q, &P, &dP);
-    if (kind == 0) return q * (lc / (q * q) + dP);
-    const float qm = q - 1.0f;
-    // sign of -dM/dq: -(log alpha - Phi) ... expressed without dividing by (q-1)^2
-    return -(-(lc - P) - q * qm * dP);
-}
-
 // Coordinates in which the FP32 secant interpolates G'(s) linearly.  With Phi
 // linear in q (its first-order form for small q h), kind 0 has dG/dq = G'(s)/q
-// affine in 1/q^2, and kind 1 has the sign function of obj_ds_f affine in
+// affine in 1/q^2, and kind 1 has the sign function of LaneTilt::ds32 affine in
 // (q - 1)^2: so y = G'(s) e^{-s} against t = e^{-2s} for kind 0, and y = that
 // function against t = (e^s - 1)^2 for kind 1.  The secant then converges in a
 // few steps.
@@ -229,22 +163,196 @@ CSE_HD __forceinline__ float secant_s(int kind, float t)
     return kind == 0 ? -0.5f * logf(t) : log1pf(sqrtf(t));
 }
 
+// Quotient for the FP32 search stages, which need ~1e-6: the device uses the
+// two-instruction approximate division (2 ulp).
+CSE_HD __forceinline__ float fdiv_fast(float x, float y)
+{
+#ifdef __CUDA_ARCH__
+    return __fdividef(x, y);
+#else
+    return x / y;
+#endif
+}
+
+// ---------------------------------------------------------------------------
+// A tile's objective by a group of lanes.  An FP64 warp instruction takes the
+// same pipe time (64 cycles) with any number of active lanes, and one thread a
+// tile left the pipe half idle on the 256^2 grid (1.7 warps a sub-partition) and
+// a 64-tile call waiting for one warp's chain of ~1,000 of them.  The arms' terms
+// are independent, so each lane takes one arm (D lanes a tile) or, SPLIT, one arm
+// and one sign of v (2 D lanes); shuffles form the maximum over the signs and the
+// sum over the arms, and every lane of the group follows the same search.
+// ---------------------------------------------------------------------------
+template <int D, bool SPLIT>
+struct LaneTilt {
+    static constexpr int NL = SPLIT ? 2 * D : D;   // lanes a tile
+    static constexpr int NS = SPLIT ? 1 : 2;       // signs a lane
+    double th, h, n, sp0;
+    double d1[NS];     // sp(th + v) - sp(th) of the lane's signs (v = +h, then -h)
+    float thf, hf, nf, sig0, sp0f, d1f[NS];
+    int sg;            // first sign of the lane
+    unsigned mask;     // the group's lanes
+
+    __device__ __forceinline__ double v(int k) const { return (sg + k) ? -h : h; }
+
+    __device__ __forceinline__ void init_f32()
+    {
+        thf = (float)th;
+        hf = (float)h;
+        nf = (float)n;
+        sig0 = fdiv_fast(1.0f, 1.0f + expf(-thf));
+        sp0f = (float)sp0;
+#pragma unroll
+        for (int k = 0; k < NS; ++k) d1f[k] = (float)d1[k];
+    }
+
+    __device__ __forceinline__ void init(double theta, double half, double n_max)
+    {
+        th = theta;
+        h = half;
+        n = n_max;
+        sp0 = softplus(th);
+#pragma unroll
+        for (int k = 0; k < NS; ++k) d1[k] = softplus(th + v(k)) - sp0;
+        init_f32();
+    }
+
+    // the other sign's value when the signs are split
+    template <typename T>
+    __device__ __forceinline__ T other(T x) const
+    {
+        return __shfl_xor_sync(mask, x, 1, NL);
+    }
+
+    template <typename T>
+    __device__ __forceinline__ T arms_sum(T x) const
+    {
+#pragma unroll
+        for (int o = NL / 2; o >= (SPLIT ? 2 : 1); o >>= 1) x += __shfl_xor_sync(mask, x, o, NL);
+        return x;
+    }
+
+    // FP32 Phi and its q-derivative.  The difference sp(th + x) - sp(th) =
+    // log1p(sigmoid(th) expm1(x)) for small |x| (no cancellation), directly otherwise.
+    __device__ __forceinline__ void phi32(float q, float* Phi, float* dPhi) const
+    {
+        const float iq = fdiv_fast(1.0f, q);
+        float p[2], dp[2];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const float x = q * ((sg + k) ? -hf : hf);
+            const float y = thf + x;
+            const float e = expf(-fabsf(y));
+            const float l1e = log1pf(e);
+            const float r = fdiv_fast(e, 1.0f + e);
+            float Dd, hq;   // hq = x sigmoid(y) - Dd without cancellation at large |x|
+            if (fabsf(x) < 0.5f) {
+                Dd = log1pf(sig0 * expm1f(x));
+                hq = x * ((y >= 0.f) ? 1.0f - r : r) - Dd;
+            } else {
+                Dd = fmaxf(y, 0.0f) + l1e - sp0f;
+                hq = (y >= 0.f) ? (sp0f - thf) - x * r - l1e : x * r - l1e + sp0f;
+            }
+            p[k] = nf * (Dd * iq - d1f[k]);
+            dp[k] = nf * hq * iq * iq;
+        }
+        if (SPLIT) {   // in the order +h, -h on both lanes
+            const float po = other(p[0]), dpo = other(dp[0]);
+            p[1] = sg ? p[0] : po;
+            dp[1] = sg ? dp[0] : dpo;
+            p[0] = sg ? po : p[0];
+            dp[0] = sg ? dpo : dp[0];
+        }
+        const bool second = p[1] > p[0] || (p[1] == p[0] && dp[1] > dp[0]);
+        *Phi = arms_sum(second ? p[1] : p[0]);
+        *dPhi = arms_sum(second ? dp[1] : dp[0]);
+    }
+
+    // sign function of the search in FP32: q dg/dq (kind 0), or minus dM/dq without
+    // its division by (q - 1)^2 (kind 1)
+    __device__ __forceinline__ float ds32(int kind, float lc, float s) const
+    {
+        const float q = expf(s);
+        float P, dP;
+        phi32(q, &P, &dP);
+        return kind == 0 ? fdiv_fast(lc, q) + q * dP : (lc - P) + q * (q - 1.0f) * dP;
+    }
+
+    // FP64 dG/ds, d2G/ds2, value and the first-order distance in s to the nearest
+    // crossing of an arm's two branches (see tilt_phi and obj_ds)
+    __device__ double ds64(int kind, double lc, double s, double* d2, double* val, double* kdist) const
+    {
+        const double q = exp(s), iq = 1.0 / q;
+        double p[2], dp[2], d2p[2];
+#pragma unroll
+        for (int k = 0; k < NS; ++k) {
+            const double vk = v(k), qv = q * vk, x = th + qv;
+            const double e = exp(-fabs(x));
+            const double l1e = log1p(e);
+            const double sp = fmax(x, 0.0) + l1e - sp0;
+            const double r = e / (1.0 + e);   // sigmoid(-|x|)
+            const double hq = (x >= 0.0) ? (sp0 - th) - qv * r - l1e : qv * r - l1e + sp0;
+            p[k] = n * (sp * iq - d1[k]);
+            dp[k] = n * hq * iq * iq;
+            d2p[k] = n * iq * (vk * vk * r * (1.0 - r) - 2.0 * hq * iq * iq);
+        }
+        if (SPLIT) {
+            const double po = other(p[0]), dpo = other(dp[0]), d2po = other(d2p[0]);
+            p[1] = sg ? p[0] : po;
+            dp[1] = sg ? dp[0] : dpo;
+            d2p[1] = sg ? d2p[0] : d2po;
+            p[0] = sg ? po : p[0];
+            dp[0] = sg ? dpo : dp[0];
+            d2p[0] = sg ? d2po : d2p[0];
+        }
+        const bool second = p[1] > p[0] || (p[1] == p[0] && dp[1] > dp[0]);
+        const double P = arms_sum(second ? p[1] : p[0]);
+        const double dP = arms_sum(second ? dp[1] : dp[0]);
+        const double d2P = arms_sum(second ? d2p[1] : d2p[0]);
+        if (kdist) {   // FP32: it is compared with a step of 1e-5
+            float kd = fdiv_fast((float)fabs(p[0] - p[1]), fmaxf((float)fabs(dp[0] - dp[1]), 1e-30f));
+#pragma unroll
+            for (int o = NL / 2; o >= (SPLIT ? 2 : 1); o >>= 1) kd = fminf(kd, __shfl_xor_sync(mask, kd, o, NL));
+            *kdist = (double)(kd * (float)iq);
+        }
+        double g1, g2, w;
+        if (kind == 0) {
+            w = (1.0 - iq) * lc + P;
+            g1 = lc * iq * iq + dP;
+            g2 = -2.0 * lc * iq * iq * iq + d2P;
+        } else {
+            const double iqm = 1.0 / (q - 1.0), t = q * iqm, B = lc - P;
+            w = -(t * B);
+            g1 = B * iqm * iqm + t * dP;
+            g2 = -(2.0 * iqm * iqm * (B * iqm + dP) - t * d2P);
+        }
+        if (val) *val = w;
+        if (d2) *d2 = q * g1 + q * q * g2;
+        return q * g1;
+    }
+
+    // lim_{q->inf} Phi(q) = sum_a max(n h_a - n d1p, -n d1m)
+    __device__ double phi_inf() const
+    {
+        double m = (sg == 0) ? h - d1[0] : -d1[0];
+        if (SPLIT) m = fmax(m, other(m));
+        else m = fmax(m, -d1[NS - 1]);
+        return arms_sum(n * m);
+    }
+};
+
 // Minimiser of the quasi-convex G over s in [0, SMAX].  FP32 stage: the sign of
 // G' at s = 0, a few bisection steps, then a bracketing secant (Illinois: the
 // stale end's value is halved when the same end moves twice running) in the
 // coordinates of secant_point, down to ~1e-5 in s.  FP64 stage: safeguarded
 // Newton from the secant's last point refines it (bisection fallback).
 // Returns s*, *val = G(s*).
-template <int D>
-CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
+template <int D, bool SPLIT>
+__device__ double q_search(const LaneTilt<D, SPLIT>& G, int kind, double lc, double* val)
 {
-    constexpr int d = D;
-    ArmGeomF Gf[D];
-#pragma unroll
-    for (int a = 0; a < d; ++a) arm_init_f(Gf[a], G[a]);
     float flo = 0.0f, fhi = (float)SMAX, sx = NAN;
     const float lcf = (float)lc;
-    const float f0 = obj_ds_f<D>(Gf, kind, lcf, 0.0f);
+    const float f0 = G.ds32(kind, lcf, 0.0f);
     const bool at_one = !(f0 < 0.0f);
     if (at_one) {
         // G' not negative at q = 1: the boundary case below decides (FP64)
@@ -253,7 +361,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
         float fa = f0, fb = NAN;
         for (int it = 0; it < BISECT_F32; ++it) {
             const float mid = 0.5f * (flo + fhi);
-            const float fm = obj_ds_f<D>(Gf, kind, lcf, mid);
+            const float fm = G.ds32(kind, lcf, mid);
             if (fm < 0.0f) { flo = mid; fa = fm; } else { fhi = mid; fb = fm; }
         }
         float ta, ya, tb, yb;
@@ -276,7 +384,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
                     xn = xs;
                 }
             }
-            const float fx = obj_ds_f<D>(Gf, kind, lcf, xn);
+            const float fx = G.ds32(kind, lcf, xn);
             float tx, yx;
             secant_point(kind, xn, fx, &tx, &yx);
             sx = xn;
@@ -298,7 +406,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
     // Tilt-Bound the value at q = 1 is 0 exactly (U = 1).
     if (kind == 0 && at_one) {
         double v0;
-        if (!(obj_ds<D>(G, kind, lc, 0.0, nullptr, &v0) < 0.0)) {
+        if (!(G.ds64(kind, lc, 0.0, nullptr, &v0, nullptr) < 0.0)) {
             *val = v0;
             return 0.0;
         }
@@ -311,7 +419,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
         // one FP64 evaluation: at a smooth optimum a Newton step from the FP32
         // estimate and the second-order Taylor value are exact to O(step^3)
         double d2, v, kd;
-        const double g1 = obj_ds<D>(G, kind, lc, s, &d2, &v, &kd);
+        const double g1 = G.ds64(kind, lc, s, &d2, &v, &kd);
         if (d2 > 0.0) {
             const double step = g1 / d2;
             if (fabs(step) <= 4e-5 && kd > 16.0 * fabs(step) + 1e-6 && s - step > 0.0 && s - step < SMAX) {
@@ -326,7 +434,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
         const double flo_m = fmax(0.0, (double)flo - 1e-2), fhi_m = fmin(SMAX, (double)fhi + 1e-2);
         for (int it = 0; it < 6; ++it) {
             double d2, v;
-            const double g1 = obj_ds<D>(G, kind, lc, s, &d2, &v);
+            const double g1 = G.ds64(kind, lc, s, &d2, &v, nullptr);
             if (g1 == 0.0) {
                 *val = v;
                 return s;
@@ -345,19 +453,19 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
     // robust path (kinks of the piecewise-smooth objective, or an FP32 bracket
     // spoilt by rounding): verified bracket, safeguarded Newton with bisection
     double lo = fmax(0.0, (double)flo - 1e-3), hi = fmin(SMAX, (double)fhi + 1e-3);
-    if (lo > 0.0 && !(obj_ds<D>(G, kind, lc, lo, nullptr, nullptr) < 0.0)) lo = 0.0;
+    if (lo > 0.0 && !(G.ds64(kind, lc, lo, nullptr, nullptr, nullptr) < 0.0)) lo = 0.0;
     if (kind == 0 && lo == 0.0 && !at_one) {   // the boundary test above, for a spoilt bracket
         double v0;
-        if (!(obj_ds<D>(G, kind, lc, 0.0, nullptr, &v0) < 0.0)) {
+        if (!(G.ds64(kind, lc, 0.0, nullptr, &v0, nullptr) < 0.0)) {
             *val = v0;
             return 0.0;
         }
     }
-    if (hi < SMAX && obj_ds<D>(G, kind, lc, hi, nullptr, nullptr) < 0.0) hi = SMAX;
+    if (hi < SMAX && G.ds64(kind, lc, hi, nullptr, nullptr, nullptr) < 0.0) hi = SMAX;
     s = fmin(fmax((double)sx, lo), hi);
     for (int it = 0; it < POLISH_IT; ++it) {
         double d2;
-        const double g1 = obj_ds<D>(G, kind, lc, s, &d2, nullptr);
+        const double g1 = G.ds64(kind, lc, s, &d2, nullptr, nullptr);
         if (g1 == 0.0) break;
         // a Newton step below 1e-11 at a smooth point: the value is then exact to
         // ~d2 1e-22, well past FP64 (at a kink g1 does not shrink and bisection runs on)
@@ -375,7 +483,7 @@ CSE_HD double q_search(const ArmGeom* G, int kind, double lc, double* val)
         }
         s = sn;
     }
-    obj_ds<D>(G, kind, lc, s, nullptr, val);
+    G.ds64(kind, lc, s, nullptr, val, nullptr);
     return s;
 }
 
@@ -398,8 +506,33 @@ CSE_HD double q_search_plain(const ArmGeom* G, int kind, double lc, double* val)
 // log inf_q max_v U(theta0, v, q, a) from log a (a = 1 - l keeps its digits as
 // log1p(-l)); *qstar the minimiser.  q = 1 gives U = 1 exactly, so the result
 // is at most 0.
-template <int D, bool PLAIN = false>
-CSE_HD double tilt_bound_log_la(const ArmGeom* G, double la, double* qstar)
+// Template parameters: the objective (an arm array, plain form, or a LaneTilt).
+template <int D>
+CSE_HD double search_any(const ArmGeom* G, int kind, double lc, double* val)
+{
+    return q_search_plain<D>(G, kind, lc, val);
+}
+
+template <int D, bool SPLIT>
+__device__ double search_any(const LaneTilt<D, SPLIT>& G, int kind, double lc, double* val)
+{
+    return q_search(G, kind, lc, val);
+}
+
+template <int D>
+CSE_HD double phi_inf_any(const ArmGeom* G)
+{
+    return tilt_phi_inf<D>(G);
+}
+
+template <int D, bool SPLIT>
+__device__ double phi_inf_any(const LaneTilt<D, SPLIT>& G)
+{
+    return G.phi_inf();
+}
+
+template <int D, typename Obj>
+__device__ double tilt_bound_log_la(const Obj& G, double la, double* qstar)
 {
     if (la >= 0.0) {
         *qstar = 1.0;
@@ -410,9 +543,9 @@ CSE_HD double tilt_bound_log_la(const ArmGeom* G, double la, double* qstar)
         return -INFINITY;
     }
     double val;
-    const double s = PLAIN ? q_search_plain<D>(G, 0, la, &val) : q_search<D>(G, 0, la, &val);
+    const double s = search_any<D>(G, 0, la, &val);
     if (s > SMAX - 1e-6) {
-        const double vinf = la + tilt_phi_inf<D>(G);
+        const double vinf = la + phi_inf_any<D>(G);
         if (vinf <= val) {
             *qstar = INFINITY;
             return vinf;
@@ -427,8 +560,8 @@ CSE_HD double tilt_bound_log_la(const ArmGeom* G, double la, double* qstar)
 }
 
 // inf_q max_v U(theta0, v, q, a); returns log bound, *qstar.
-template <int D, bool PLAIN = false>
-CSE_HD double tilt_bound_log(const ArmGeom* G, double a, double* qstar)
+template <int D, typename Obj>
+__device__ double tilt_bound_log(const Obj& G, double a, double* qstar)
 {
     if (a >= 1.0) {
         *qstar = 1.0;
@@ -438,19 +571,19 @@ CSE_HD double tilt_bound_log(const ArmGeom* G, double a, double* qstar)
         *qstar = INFINITY;
         return -INFINITY;
     }
-    return tilt_bound_log_la<D, PLAIN>(G, log(a), qstar);
+    return tilt_bound_log_la<D>(G, log(a), qstar);
 }
 
 // sup_q min_v U^-1(theta0, v, q, alpha); returns log alpha', *qstar.
-template <int D, bool PLAIN = false>
-CSE_HD double alpha_prime_log(const ArmGeom* G, double alpha, double* qstar)
+template <int D, typename Obj>
+__device__ double alpha_prime_log(const Obj& G, double alpha, double* qstar)
 {
     const double lal = log(alpha);
     double val;
-    const double s = PLAIN ? q_search_plain<D>(G, 1, lal, &val) : q_search<D>(G, 1, lal, &val);
+    const double s = search_any<D>(G, 1, lal, &val);
     val = -val;
     if (s > SMAX - 1e-6) {
-        const double vinf = lal - tilt_phi_inf<D>(G);
+        const double vinf = lal - phi_inf_any<D>(G);
         if (vinf >= val) {
             *qstar = INFINITY;
             return vinf;
@@ -576,17 +709,6 @@ CSE_HD double beta_cf(double a, double b, double x)
         }
     }
     return Am1 / Bm1;
-}
-
-// Quotient for the FP32 search stage, which needs ~1e-6: the device uses the
-// two-instruction approximate division (2 ulp).
-CSE_HD __forceinline__ float fdiv_fast(float x, float y)
-{
-#ifdef __CUDA_ARCH__
-    return __fdividef(x, y);
-#else
-    return x / y;
-#endif
 }
 
 // FP32 modified Lentz evaluation of the same fraction (start of the solve).
@@ -1028,6 +1150,13 @@ __device__ __forceinline__ T cp_halley(T u, T f, T r, T a, T b, bool upper, T* l
     return (un >= *lo && un <= *hi) ? un : (T)0.5 * (*lo + *hi);
 }
 
+// The serial solve, called (rarely) rather than inlined: its registers would halve
+// the warps of the group solve.
+__device__ __noinline__ double cp_upper_serial(int64_t R, int64_t N, double delta)
+{
+    return cp_upper(R, N, delta);
+}
+
 // u with P(Binom(N, u) <= R) = delta, 0 < R < N, all lanes of a group together; comp =
 // 1 - delta from the caller, who may know it to more digits; z is the normal
 // quantile of comp.
@@ -1036,7 +1165,7 @@ __device__ double cp_upper_group(int64_t R, int64_t N, double delta, double comp
 {
     const double a = (double)R + 1.0, b = (double)(N - R);
     const bool small = R < CP_SMALL_R && (N - R > CP_SMALL_R || delta > 0.9);
-    if (!small && (a < 10.0 || b < 10.0)) return cp_upper(R, N, delta);   // few trials: every lane alike
+    if (!small && (a < 10.0 || b < 10.0)) return cp_upper_serial(R, N, delta);   // few trials: every lane alike
     const bool upper = delta <= (small ? 0.9 : 0.5);
     const double target = log(upper ? delta : comp);
     const float af = (float)a, bf = (float)b, sf = af + bf;
@@ -1065,7 +1194,7 @@ __device__ double cp_upper_group(int64_t R, int64_t N, double delta, double comp
         const double step = __shfl_sync(mask, fabs(un - ud), 0, L);
         ud = __shfl_sync(mask, un, 0, L);
         // far on the wrong side of the mean the fraction loses its sign: the serial solve
-        if (!(__shfl_sync(mask, r, 0, L) > 0.0)) return cp_upper(R, N, delta);
+        if (!(__shfl_sync(mask, r, 0, L) > 0.0)) return cp_upper_serial(R, N, delta);
         if (!(step > 2e-5 * fmin((double)sd, fmin(ud, 1.0 - ud))) || hi - lo <= 4e-16 * hi) break;
     }
     return ud;
@@ -1102,38 +1231,52 @@ __device__ bool load_tile(const TileArgs& T, int64_t i, double n_max, ArmGeom* G
     return true;
 }
 
-// The per-arm softplus terms of a tile (sp(th), sp(th + h) - sp(th),
-// sp(th - h) - sp(th)), 3 doubles per arm, as k_alpha_prime computed them:
-// k_bounds of the same step reads them instead of recomputing (same values).
-template <int D>
-__device__ void store_geom(const ArmGeom* G, int64_t i, double* __restrict__ geom)
+// The same by the group of lanes l = 0 .. NL-1, each its own arm (and sign); the
+// checks hold for the whole tile.  geom: each tile's softplus terms (sp(th),
+// sp(th + h) - sp(th), sp(th - h) - sp(th), 3 doubles an arm), written by
+// k_alpha_prime (store) and read by k_bounds of the same step (load), which takes
+// the same values instead of recomputing them.
+template <int D, bool SPLIT>
+__device__ bool load_lane(const TileArgs& T, int64_t i, int l, double n_max, LaneTilt<D, SPLIT>& G, int32_t* err,
+                          const double* __restrict__ geom_in, double* __restrict__ geom_out)
 {
+    constexpr int NL = LaneTilt<D, SPLIT>::NL;
+    const int a = SPLIT ? l >> 1 : l;
+    G.sg = SPLIT ? l & 1 : 0;
+    G.mask = (NL == 32 ? 0xffffffffu : ((1u << NL) - 1u) << ((threadIdx.x & 31) & ~(NL - 1)));
+    const double h = T.halfwidth[i * D + a];
+    const int v = T.center_idx[i * D + a];
+    int na = T.n_axis[0];
+    const double* axis = T.axis[0];
 #pragma unroll
-    for (int a = 0; a < D; ++a) {
-        geom[(i * D + a) * 3 + 0] = G[a].sp0;
-        geom[(i * D + a) * 3 + 1] = G[a].d1p;
-        geom[(i * D + a) * 3 + 2] = G[a].d1m;
-    }
-}
-
-template <int D>
-__device__ bool load_tile_geom(const TileArgs& T, int64_t i, double n_max, ArmGeom* G, int32_t* err,
-                               const double* __restrict__ geom)
-{
-    if (!tile_args_ok<D>(T, i, err)) return false;
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        const int v = T.center_idx[i * D + a];
-        if (v < 0 || v >= T.n_axis[a]) {
-            atomicOr(err, CSE_ERR_BAD_K);
-            return false;
+    for (int b = 1; b < D; ++b)   // by selection: no runtime index into the argument
+        if (a == b) {
+            na = T.n_axis[b];
+            axis = T.axis[b];
         }
-        G[a].th = T.axis[a][v];
-        G[a].h = T.halfwidth[i * D + a];
-        G[a].n = n_max;
-        G[a].sp0 = geom[(i * D + a) * 3 + 0];
-        G[a].d1p = geom[(i * D + a) * 3 + 1];
-        G[a].d1m = geom[(i * D + a) * 3 + 2];
+    const bool ok = T.null_mask[i] != 0u && h >= 0.0 && v >= 0 && v < na;   // false for a NaN half-width too
+    if (!__all_sync(G.mask, ok)) {
+        if (l == 0) atomicOr(err, CSE_ERR_BAD_K);
+        return false;
+    }
+    const double th = axis[v];
+    if (geom_in) {
+        const double* g = geom_in + (i * D + a) * 3;
+        G.th = th;
+        G.h = h;
+        G.n = n_max;
+        G.sp0 = g[0];
+        G.d1[0] = g[1 + G.sg];
+        if (!SPLIT) G.d1[SPLIT ? 0 : 1] = g[2];
+        G.init_f32();
+    } else {
+        G.init(th, h, n_max);
+    }
+    if (geom_out) {
+        double* g = geom_out + (i * D + a) * 3;
+        if (G.sg == 0) g[0] = G.sp0;
+        g[1 + G.sg] = G.d1[0];
+        if (!SPLIT) g[2] = G.d1[SPLIT ? 0 : 1];
     }
     return true;
 }
@@ -1229,85 +1372,123 @@ __global__ void __launch_bounds__(kCpThreads, kCpBlocksPerSM) k_cp_solve(unsigne
 // 1 - delta and log(1 - l) = log1p(-l); for R > K/2 (l near 1) 1 - l is the
 // upper solve for the K - R failures at delta (binomial symmetry), taken
 // directly so that its digits are not lost to the subtraction.
-template <int D, bool PLAIN, bool LOWER>
-__global__ void __launch_bounds__(128) k_bounds(TileArgs T, int32_t n_max, const int64_t* __restrict__ R,
-                                                double delta, double* __restrict__ u0,
-                                                double* __restrict__ bound, double* __restrict__ qstar,
-                                                int32_t* __restrict__ err, const int32_t* __restrict__ slot,
-                                                const double* __restrict__ u0s, const double* __restrict__ geom,
-                                                int32_t* __restrict__ nkeys_reset)
+template <int D, bool LOWER, typename Obj, typename Cp>
+__device__ __forceinline__ void bound_of(const Obj& G, int64_t Ri, int64_t Ki, double delta, Cp cp, double* u_out,
+                                         double* b_out, double* q_out)
 {
-    pdl_entry();
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= T.n_tiles) return;
-    // k_cp_solve has read the key count (it ran before this kernel): zero it for the next call
-    if (i == 0 && nkeys_reset) *nkeys_reset = 0;
-    ArmGeom G[D];
-    const bool ok = geom ? load_tile_geom<D>(T, i, (double)n_max, G, err, geom)
-                         : load_tile<D>(T, i, (double)n_max, G, err);
-    if (!ok) {
-        if (u0) u0[i] = NAN;
-        if (bound) bound[i] = NAN;
-        if (qstar) qstar[i] = NAN;
-        return;
-    }
-    double q;
     if (LOWER) {
-        const int64_t Ri = R[i], Ki = T.K[i];
-        const bool memo = !PLAIN && slot && slot[i] >= 0;
         double l, la;
         if (2 * Ri > Ki) {
-            const double ap = PLAIN ? cp_upper_plain(Ki - Ri, Ki, delta)
-                                    : memo ? u0s[slot[i]] : cp_upper(Ki - Ri, Ki, delta);
+            const double ap = cp(Ki - Ri, delta);
             l = Ri == Ki ? exp(log(delta) / (double)Ki) : 1.0 - ap;   // l^K = delta when every trial rejects
             la = log(ap);
         } else if (Ri <= 0) {
             l = 0.0;
             la = 0.0;
         } else {
-            l = PLAIN ? cp_upper_plain(Ri - 1, Ki, 1.0 - delta)
-                      : memo ? u0s[slot[i]] : cp_upper(Ri - 1, Ki, 1.0 - delta);
+            l = cp(Ri - 1, 1.0 - delta);
             la = log1p(-l);
         }
-        const double lb = tilt_bound_log_la<D, PLAIN>(G, la, &q);
-        if (u0) u0[i] = l;
-        if (bound) bound[i] = (lb >= 0.0) ? 0.0 : -expm1(lb);
-        if (qstar) qstar[i] = q;
+        const double lb = tilt_bound_log_la<D>(G, la, q_out);
+        *u_out = l;
+        *b_out = (lb >= 0.0) ? 0.0 : -expm1(lb);
         return;
     }
-    double u;
-    if (PLAIN) u = cp_upper_plain(R[i], T.K[i], delta);
-    else if (slot && slot[i] >= 0) u = u0s[slot[i]];
-    else u = cp_upper(R[i], T.K[i], delta);
-    const double lb = tilt_bound_log<D, PLAIN>(G, u, &q);
+    const double u = cp(Ri, delta);
+    *u_out = u;
+    *b_out = exp(tilt_bound_log<D>(G, u, q_out));
+}
+
+// Plain form: one thread a tile, FP64 throughout, its own Clopper-Pearson solve.
+template <int D, bool LOWER>
+__global__ void __launch_bounds__(128) k_bounds_plain(TileArgs T, int32_t n_max, const int64_t* __restrict__ R,
+                                                      double delta, double* __restrict__ u0,
+                                                      double* __restrict__ bound, double* __restrict__ qstar,
+                                                      int32_t* __restrict__ err)
+{
+    pdl_entry();
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= T.n_tiles) return;
+    ArmGeom G[D];
+    double u = NAN, b = NAN, q = NAN;
+    if (load_tile<D>(T, i, (double)n_max, G, err)) {
+        const int64_t Ki = T.K[i];
+        bound_of<D, LOWER>((const ArmGeom*)G, R[i], Ki, delta,
+                           [&](int64_t r, double dl) { return cp_upper_plain(r, Ki, dl); }, &u, &b, &q);
+    }
     if (u0) u0[i] = u;
-    if (bound) bound[i] = exp(lb);
+    if (bound) bound[i] = b;
     if (qstar) qstar[i] = q;
 }
 
-template <int D, bool PLAIN>
-__global__ void __launch_bounds__(128) k_alpha_prime(TileArgs T, int32_t n_max, double alpha,
-                                                     double* __restrict__ aprime, int32_t* __restrict__ ksel,
-                                                     int32_t* __restrict__ err, double* __restrict__ geom)
+// A group of NL lanes a tile (see LaneTilt).  slot: each tile's entry of the
+// Clopper-Pearson memo, whose values are u0s (every key it needs is there: the
+// table holds at least two slots a tile).
+template <int D, bool SPLIT, bool LOWER>
+__global__ void __launch_bounds__(64) k_bounds(TileArgs T, int32_t n_max, const int64_t* __restrict__ R, double delta,
+                                               double* __restrict__ u0, double* __restrict__ bound,
+                                               double* __restrict__ qstar, int32_t* __restrict__ err,
+                                               const int32_t* __restrict__ slot, const double* __restrict__ u0s,
+                                               const double* __restrict__ geom, int32_t* __restrict__ nkeys_reset)
+{
+    pdl_entry();
+    constexpr int NL = LaneTilt<D, SPLIT>::NL;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = t / NL;
+    const int l = (int)(t % NL);
+    if (i >= T.n_tiles) return;
+    // k_cp_solve has read the key count (it ran before this kernel): zero it for the next call
+    if (t == 0 && nkeys_reset) *nkeys_reset = 0;
+    LaneTilt<D, SPLIT> G;
+    double u = NAN, b = NAN, q = NAN;
+    if (load_lane(T, i, l, (double)n_max, G, err, geom, nullptr)) {
+        const int64_t Ki = T.K[i];
+        const int32_t sl = slot ? slot[i] : -1;
+        bound_of<D, LOWER>(G, R[i], Ki, delta,
+                           [&](int64_t, double) { return sl >= 0 ? u0s[sl] : NAN; }, &u, &b, &q);
+    }
+    if (l != 0) return;
+    if (u0) u0[i] = u;
+    if (bound) bound[i] = b;
+    if (qstar) qstar[i] = q;
+}
+
+__device__ __forceinline__ void store_alpha(double ap, int32_t K, int64_t i, double* __restrict__ aprime,
+                                            int32_t* __restrict__ ksel)
+{
+    if (aprime) aprime[i] = ap;
+    double kf = floor(((double)K + 1.0) * ap);
+    if (kf > (double)K) kf = (double)K;
+    if (ksel) ksel[i] = ap == ap ? (int32_t)kf : 0;
+}
+
+template <int D>
+__global__ void __launch_bounds__(128) k_alpha_prime_plain(TileArgs T, int32_t n_max, double alpha,
+                                                           double* __restrict__ aprime, int32_t* __restrict__ ksel,
+                                                           int32_t* __restrict__ err)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= T.n_tiles) return;
     ArmGeom G[D];
-    if (!load_tile<D>(T, i, (double)n_max, G, err)) {
-        if (aprime) aprime[i] = NAN;
-        if (ksel) ksel[i] = 0;
-        return;
-    }
-    if (geom) store_geom<D>(G, i, geom);
-    double q;
-    const double ap = exp(alpha_prime_log<D, PLAIN>(G, alpha, &q));
-    if (aprime) aprime[i] = ap;
-    const int32_t K = T.K[i];
-    double kf = floor(((double)K + 1.0) * ap);
-    if (kf > (double)K) kf = (double)K;
-    if (ksel) ksel[i] = (int32_t)kf;
+    double q, ap = NAN;
+    if (load_tile<D>(T, i, (double)n_max, G, err)) ap = exp(alpha_prime_log<D>((const ArmGeom*)G, alpha, &q));
+    store_alpha(ap, T.K[i], i, aprime, ksel);
 }
 
+template <int D, bool SPLIT>
+__global__ void __launch_bounds__(64) k_alpha_prime(TileArgs T, int32_t n_max, double alpha,
+                                                    double* __restrict__ aprime, int32_t* __restrict__ ksel,
+                                                    int32_t* __restrict__ err, double* __restrict__ geom)
+{
+    constexpr int NL = LaneTilt<D, SPLIT>::NL;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, i = t / NL;
+    const int l = (int)(t % NL);
+    if (i >= T.n_tiles) return;
+    LaneTilt<D, SPLIT> G;
+    double q, ap = NAN;
+    if (load_lane(T, i, l, (double)n_max, G, err, (const double*)nullptr, geom))
+        ap = exp(alpha_prime_log<D>(G, alpha, &q));
+    if (l == 0) store_alpha(ap, T.K[i], i, aprime, ksel);
+}
 
 // min over v[0..n): each block folds its stretch on integer keys (ALU, not the
 // FP64 pipe), one atomicMin per block into *key (set to all ones before the
@@ -1366,42 +1547,72 @@ double normal_quantile(double p)
     return 0.5 * (lo + hi);
 }
 
-template <int D>
-void launch_bounds_d(cse_ctx* c, unsigned blocks, const TileArgs& T, const int64_t* R, double delta, bool lower,
-                     double* u0, double* bound, double* qstar, const int32_t* slot, const double* geom,
-                     cudaStream_t s)
+// Lanes a tile: two per arm while the tiles give every sub-partition at most
+// kSplitWarps warps (what counts is the latency of one tile's chain), one per arm
+// beyond (the FP64 pipe is full and the signs' common work is done once).  alpha' /
+// bound, against one thread a tile: one arm, 64 tiles 31 / 38 -> 21 / 17 us; two
+// arms, 1,891 tiles, band 67 + 58 -> 26 + 21; four arms, 6,036 tiles 183 -> 58
+// (bound); two arms, 32,896 tiles 75 / 62 -> 68 / 48 (92 / 72 with the signs split);
+// 2^18 tiles 557 / 411 -> 538 / 341; four arms, 59,992 tiles 261 / 219 -> 257 / 171.
+inline bool split_signs(const cse_ctx* c, const TileArgs& T)
 {
-    const int nm = c->D.n_max;
-    if (c->plain) {
-        if (lower)
-            cse_launch(c->pdl, k_bounds<D, true, true>, dim3(blocks), dim3(128), 0, s, T, nm, R, delta, u0, bound, qstar, c->err, nullptr, nullptr,
-                                                           nullptr, nullptr);
-        else
-            cse_launch(c->pdl, k_bounds<D, true, false>, dim3(blocks), dim3(128), 0, s, T, nm, R, delta, u0, bound, qstar, c->err, nullptr,
-                                                            nullptr, nullptr, nullptr);
-    } else {
-        // one thread a tile, 64-thread blocks: the tiles spread over more SMs
-        // than in blocks of 128 (two-arm 256^2: 66 -> 62 us, refined sample
-        // 272 -> 243 us)
-        int32_t* nk = slot ? c->cp_nkeys : nullptr;
-        const unsigned b64 = (unsigned)((T.n_tiles + 63) / 64);
-        if (lower)
-            cse_launch(c->pdl, k_bounds<D, false, true>, dim3(b64), dim3(64), 0, s, T, nm, R, delta, u0, bound, qstar, c->err, slot,
-                                                            c->cp_val, geom, nk);
-        else
-            cse_launch(c->pdl, k_bounds<D, false, false>, dim3(b64), dim3(64), 0, s, T, nm, R, delta, u0, bound, qstar, c->err, slot,
-                                                             c->cp_val, geom, nk);
-    }
+    return T.n_tiles * 2 * T.d <= (int64_t)c->num_sms * 4 * 32 * kSplitWarps;
+}
+
+template <int D, bool SPLIT>
+void launch_bounds_s(cse_ctx* c, const TileArgs& T, const int64_t* R, double delta, bool lower, double* u0,
+                     double* bound, double* qstar, const int32_t* slot, const double* geom, cudaStream_t s)
+{
+    constexpr int NL = LaneTilt<D, SPLIT>::NL;
+    const unsigned blocks = (unsigned)((T.n_tiles * NL + 63) / 64);
+    int32_t* nk = slot ? c->cp_nkeys : nullptr;
+    if (lower)
+        cse_launch(c->pdl, k_bounds<D, SPLIT, true>, dim3(blocks), dim3(64), 0, s, T, c->D.n_max, R, delta, u0, bound,
+                   qstar, c->err, slot, c->cp_val, geom, nk);
+    else
+        cse_launch(c->pdl, k_bounds<D, SPLIT, false>, dim3(blocks), dim3(64), 0, s, T, c->D.n_max, R, delta, u0, bound,
+                   qstar, c->err, slot, c->cp_val, geom, nk);
 }
 
 template <int D>
-void launch_alpha_d(cse_ctx* c, unsigned blocks, const TileArgs& T, double alpha, double* ap, int32_t* ksel,
-                    double* geom, cudaStream_t s)
+void launch_bounds_d(cse_ctx* c, const TileArgs& T, const int64_t* R, double delta, bool lower, double* u0,
+                     double* bound, double* qstar, const int32_t* slot, const double* geom, cudaStream_t s)
+{
+    if (c->plain) {
+        const unsigned blocks = (unsigned)((T.n_tiles + 127) / 128);
+        if (lower)
+            cse_launch(c->pdl, k_bounds_plain<D, true>, dim3(blocks), dim3(128), 0, s, T, c->D.n_max, R, delta, u0,
+                       bound, qstar, c->err);
+        else
+            cse_launch(c->pdl, k_bounds_plain<D, false>, dim3(blocks), dim3(128), 0, s, T, c->D.n_max, R, delta, u0,
+                       bound, qstar, c->err);
+    } else if (split_signs(c, T)) {
+        launch_bounds_s<D, true>(c, T, R, delta, lower, u0, bound, qstar, slot, geom, s);
+    } else {
+        launch_bounds_s<D, false>(c, T, R, delta, lower, u0, bound, qstar, slot, geom, s);
+    }
+}
+
+template <int D, bool SPLIT>
+void launch_alpha_s(cse_ctx* c, const TileArgs& T, double alpha, double* ap, int32_t* ksel, double* geom,
+                    cudaStream_t s)
+{
+    constexpr int NL = LaneTilt<D, SPLIT>::NL;
+    k_alpha_prime<D, SPLIT><<<(unsigned)((T.n_tiles * NL + 63) / 64), 64, 0, s>>>(T, c->D.n_max, alpha, ap, ksel,
+                                                                                c->err, geom);
+}
+
+template <int D>
+void launch_alpha_d(cse_ctx* c, const TileArgs& T, double alpha, double* ap, int32_t* ksel, double* geom,
+                    cudaStream_t s)
 {
     if (c->plain)
-        k_alpha_prime<D, true><<<blocks, 128, 0, s>>>(T, c->D.n_max, alpha, ap, ksel, c->err, nullptr);
+        k_alpha_prime_plain<D><<<(unsigned)((T.n_tiles + 127) / 128), 128, 0, s>>>(T, c->D.n_max, alpha, ap, ksel,
+                                                                                 c->err);
+    else if (split_signs(c, T))
+        launch_alpha_s<D, true>(c, T, alpha, ap, ksel, geom, s);
     else
-        k_alpha_prime<D, false><<<blocks, 128, 0, s>>>(T, c->D.n_max, alpha, ap, ksel, c->err, geom);
+        launch_alpha_s<D, false>(c, T, alpha, ap, ksel, geom, s);
 }
 
 int cse_launch_bounds(cse_ctx* c, const TileArgs& T, const int64_t* R, double delta, bool lower, double* u0,
@@ -1430,9 +1641,9 @@ int cse_launch_bounds(cse_ctx* c, const TileArgs& T, const int64_t* R, double de
     }
     cse_prof_begin(c, KID_BOUNDS, s);
     switch (T.d) {
-    case 1: launch_bounds_d<1>(c, blocks, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
-    case 2: launch_bounds_d<2>(c, blocks, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
-    case 4: launch_bounds_d<4>(c, blocks, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
+    case 1: launch_bounds_d<1>(c, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
+    case 2: launch_bounds_d<2>(c, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
+    case 4: launch_bounds_d<4>(c, T, R, delta, lower, u0, bound, qstar, slot, geom, s); break;
     default: return CSE_UNSUPPORTED_DESIGN;
     }
     cse_prof_end(c, s);
@@ -1447,26 +1658,29 @@ int cse_launch_bounds(cse_ctx* c, const TileArgs& T, const int64_t* R, double de
 // carveout only when idle.  Asking for the largest carveout lets both run.
 int cse_bound_set_attrs()
 {
-    const int pref = cudaSharedmemCarveoutMaxShared;
-    cudaError_t e = cudaSuccess;
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<1, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<2, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<4, false>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<1, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<2, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
-    if (e == cudaSuccess) e = cudaFuncSetAttribute(k_alpha_prime<4, true>, cudaFuncAttributePreferredSharedMemoryCarveout, pref);
+    auto most = [](auto kern) {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+    };
+    cudaError_t e = most(k_alpha_prime<1, false>);
+    if (e == cudaSuccess) e = most(k_alpha_prime<1, true>);
+    if (e == cudaSuccess) e = most(k_alpha_prime<2, false>);
+    if (e == cudaSuccess) e = most(k_alpha_prime<2, true>);
+    if (e == cudaSuccess) e = most(k_alpha_prime<4, false>);
+    if (e == cudaSuccess) e = most(k_alpha_prime<4, true>);
+    if (e == cudaSuccess) e = most(k_alpha_prime_plain<1>);
+    if (e == cudaSuccess) e = most(k_alpha_prime_plain<2>);
+    if (e == cudaSuccess) e = most(k_alpha_prime_plain<4>);
     return e == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
 int cse_launch_alpha_prime(cse_ctx* c, const TileArgs& T, double alpha, double* aprime_out,
                            int32_t* ksel, cudaStream_t s, double* geom)
 {
-    const unsigned blocks = (unsigned)((T.n_tiles + 127) / 128);
     cse_prof_begin(c, KID_ALPHA_PRIME, s);
     switch (T.d) {
-    case 1: launch_alpha_d<1>(c, blocks, T, alpha, aprime_out, ksel, geom, s); break;
-    case 2: launch_alpha_d<2>(c, blocks, T, alpha, aprime_out, ksel, geom, s); break;
-    case 4: launch_alpha_d<4>(c, blocks, T, alpha, aprime_out, ksel, geom, s); break;
+    case 1: launch_alpha_d<1>(c, T, alpha, aprime_out, ksel, geom, s); break;
+    case 2: launch_alpha_d<2>(c, T, alpha, aprime_out, ksel, geom, s); break;
+    case 4: launch_alpha_d<4>(c, T, alpha, aprime_out, ksel, geom, s); break;
     default: return CSE_UNSUPPORTED_DESIGN;
     }
     cse_prof_end(c, s);
