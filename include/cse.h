@@ -97,10 +97,9 @@ typedef struct {
     int32_t K_max;              /* host: max_i K_i (<= the context's K_max) */
 } cse_tiles;
 
-/* Context: copies the design, generates the CRN uniforms for sims
- * 0..K_max-1 (Philox4x32-10, key = seed), sorts them within each
- * (sim, arm, analysis segment), and builds the statistic tables.  Owns all
- * scratch.  Synchronises `stream` before returning.
+/* Context: copies the design, takes `seed` as the key of the CRN uniforms of sims
+ * 0..K_max-1 (Philox4x32-10; every simulating call draws the ones it needs) and
+ * builds the statistic tables.  Owns all scratch.  Synchronises `stream` before returning.
  * Errors: INVALID_ARG (null out, K_max < 1 or > 1<<20), UNSUPPORTED_DESIGN,
  * OOM, CUDA_ERROR. */
 int cse_create(cse_ctx** out, const cse_design* design, uint64_t seed, int32_t K_max,
@@ -263,11 +262,10 @@ int cse_statistics(cse_ctx* ctx, const cse_tiles* tiles, const int64_t* offsets,
                    cse_stream_t stream);
 
 /* Sets the key of the context's CRN uniforms to `seed` (a new batch of
- * simulations; same layout and sorting as cse_create).  No kernel runs here:
- * the next call that simulates regenerates the uniforms (and the randomised
- * test's words) on its own stream before its success counts, after it has
- * started its tile-only work (alpha', on the context's second stream), so the
- * two overlap.  `stream` is not used.  Errors: INVALID_ARG (NULL ctx). */
+ * simulations).  No kernel runs here: the calls that simulate draw the uniforms
+ * (and the randomised test's words) of the key in their count-table kernel, on
+ * their own stream, while their tile-only work (alpha') runs on the context's
+ * second stream.  `stream` is not used.  Errors: INVALID_ARG (NULL ctx). */
 int cse_reseed(cse_ctx* ctx, uint64_t seed, cse_stream_t stream);
 
 /* Autotuner: times the fused simulation pass of `tiles` (at `lambda`, with the
@@ -293,8 +291,8 @@ int cse_autotune(cse_ctx* ctx, const cse_tiles* tiles, double lambda, double alp
 enum { CSE_OPT_BAYES_DIRECT = 1, CSE_OPT_PLAIN = 2, CSE_OPT_SIM_THREADS = 3, CSE_OPT_CELLS_BOX = 4,
        CSE_OPT_PDL = 5, CSE_OPT_SIM_TILES = 7 };
 /* CSE_OPT_PLAIN: 1 selects the plain comparison path with the same results:
- * success counts by one binary search per (tile, sim, arm) in the sorted
- * uniforms (no axis count table), the bound pass entirely in FP64 (bisection
+ * success counts by one binary search per (tile, sim, arm) in sorted
+ * uniforms, which the first such call of a key generates (no axis count table), the bound pass entirely in FP64 (bisection
  * over q, Newton for Clopper-Pearson, no FP32 stage), and for BAYES4 and BERRY4
  * the direct per-trial posterior.  0 (default) is the chosen path.
  * CSE_OPT_SIM_THREADS (z-test designs): 64, 128, 256 or 512 fixes the block size

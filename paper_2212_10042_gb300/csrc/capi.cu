@@ -149,26 +149,38 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
     return CSE_OK;
 }
 
-// Uniforms of a new key if pending, success thresholds of every axis
-// coordinate, then the axis count tables.
-int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s)
+// Success thresholds of every axis coordinate, then the axis count tables (which
+// draw the context's uniforms themselves).  The plain z-test simulation searches
+// sorted uniforms per (tile, sim) instead: they are generated on its first call
+// after a new key; what else it runs may ask for the counts as well.
+int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = false)
 {
-    bool thr_done = false;   // a new key's uniforms kernel writes the thresholds as well
-    if (c->u_stale) {
-        CSE_TRY(cse_launch_uniforms(c, s, &P.T, P.NA, &thr_done));
-        c->u_stale = false;
+    CSE_TRY(cse_launch_thresholds(c, P.T, P.NA, s));
+    if (c->plain && !cse_posterior_design(c->D.stat)) {
+        if (!c->U) {
+            const size_t ub = sizeof(uint32_t) * (size_t)c->D.d * (size_t)c->K_max * (size_t)c->D.n_max;
+            if (cudaMalloc(&c->U, ub) != cudaSuccess) {
+                cudaGetLastError();
+                c->U = nullptr;
+                return CSE_OOM;
+            }
+        }
+        if (c->u_stale) {
+            CSE_TRY(cse_launch_uniforms(c, s));
+            c->u_stale = false;
+        }
+        if (!counts) return CSE_OK;
     }
-    if (!thr_done) CSE_TRY(cse_launch_thresholds(c, P.T, P.NA, s));
-    // the plain z-test path searches the sorted uniforms per (tile, sim) instead
-    if (!(c->plain && !cse_posterior_design(c->D.stat)))
-        CSE_TRY(cse_launch_axis_counts(c, P.T, P.NA, P.K_tiles, P.k_stride, s));
+    CSE_TRY(cse_launch_axis_counts(c, P.T, P.NA, P.K_tiles, P.k_stride, s));
+    // the z-test cell kernel reads each axis value's least and greatest count
+    if (!cse_posterior_design(c->D.stat)) CSE_TRY(cse_launch_axis_box(c, P.NA, P.K_tiles, P.k_stride, s));
     return CSE_OK;
 }
 
-int prepare(cse_ctx* c, const cse_tiles* t, cudaStream_t s, Prepared* P, bool geom = true)
+int prepare(cse_ctx* c, const cse_tiles* t, cudaStream_t s, Prepared* P, bool geom = true, bool counts = false)
 {
     CSE_TRY(prepare_args(c, t, P, geom));
-    return launch_tables(c, *P, s);
+    return launch_tables(c, *P, s, counts);
 }
 
 // alpha' (and the order-statistic index of each tile) on the side stream, in
@@ -176,13 +188,13 @@ int prepare(cse_ctx* c, const cse_tiles* t, cudaStream_t s, Prepared* P, bool ge
 // stream waits for it before the simulation pass reads ksel.  Capturable into a
 // CUDA graph (event fork/join).
 int tables_and_alpha_prime(cse_ctx* c, const Prepared& P, double alpha, double* aprime_out, cudaStream_t s,
-                           double* geom = nullptr)
+                           double* geom = nullptr, bool counts = false)
 {
     CUDA_TRY(cudaEventRecord(c->ev_fork, s));
     CUDA_TRY(cudaStreamWaitEvent(c->side, c->ev_fork, 0));
     CSE_TRY(cse_launch_alpha_prime(c, P.T, alpha, aprime_out, c->ksel, c->side, geom));
     CUDA_TRY(cudaEventRecord(c->ev_join, c->side));
-    CSE_TRY(launch_tables(c, P, s));
+    CSE_TRY(launch_tables(c, P, s, counts));
     CUDA_TRY(cudaStreamWaitEvent(s, c->ev_join, 0));
     return CSE_OK;
 }
@@ -229,7 +241,7 @@ int cse_reseed(cse_ctx* c, uint64_t seed, cse_stream_t stream)
     (void)stream;
     if (!c) return CSE_INVALID_ARG;
     c->seed = seed;
-    c->u_stale = true;   // regenerated by the next simulating call (launch_tables)
+    c->u_stale = true;   // the next simulating call draws from the new key
     return CSE_OK;
 }
 
@@ -467,8 +479,6 @@ int cse_create(cse_ctx** out, const cse_design* design, uint64_t seed, int32_t K
     cudaStream_t s = (cudaStream_t)stream;
     int st = CSE_OK;
     do {
-        const size_t ub = sizeof(uint32_t) * (size_t)ds.d * (size_t)K_max * (size_t)n_max;
-        if (cudaMalloc(&c->U, ub) != cudaSuccess) { st = CSE_OOM; break; }
         if (cudaMalloc(&c->tb, sizeof(uint32_t) * (size_t)K_max) != cudaSuccess) { st = CSE_OOM; break; }
         if (ds.stat == CSE_STAT_ONE_ARM_Z) {
             c->n_cells = n_max + 1;
@@ -508,8 +518,7 @@ int cse_create(cse_ctx** out, const cse_design* design, uint64_t seed, int32_t K
             break;
         }
         c->min_ticket = reinterpret_cast<unsigned int*>(c->min_key + 1);
-        st = cse_launch_uniforms(c, s);
-        if (st != CSE_OK) break;
+        c->u_stale = true;
         st = cse_launch_tables(c, s);
         if (st != CSE_OK) break;
         if (cudaDeviceGetAttribute(&c->num_sms, cudaDevAttrMultiProcessorCount, c->device) != cudaSuccess) {
@@ -712,7 +721,7 @@ int cse_validate_rand(cse_ctx* c, const cse_tiles* t, double lambda, uint32_t c_
     if (c && cse_posterior_design(c->D.stat)) return CSE_UNSUPPORTED_DESIGN;
     cudaStream_t s = (cudaStream_t)stream;
     Prepared P;
-    CSE_TRY(prepare(c, t, s, &P));
+    CSE_TRY(prepare(c, t, s, &P, true, true));
     int64_t* R = R_out ? R_out : c->R;
     SimOut o = {c->sig, R, Xrej_out, score_out, nullptr, nullptr};
     CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, lambda, c_thr, o, nullptr, s));
@@ -729,7 +738,7 @@ int cse_calibrate_rand(cse_ctx* c, const cse_tiles* t, double alpha, double* alp
     cudaStream_t s = (cudaStream_t)stream;
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
-    CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s));
+    CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s, nullptr, true));
     SimOut o = {c->sig, nullptr, nullptr, nullptr, lambda_tile_out, c->ksel};
     CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, INFINITY, 0u, o, c_tile_out, s));
     // (lambda*, c*) through the device scalars lam_dev and lam_dev + 1 (its low 4 bytes)
@@ -800,9 +809,7 @@ int cse_statistics(cse_ctx* c, const cse_tiles* t, const int64_t* offsets, float
     if (!offsets || !S_out) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     Prepared P;
-    CSE_TRY(prepare(c, t, s, &P));
-    if (c->plain && !cse_posterior_design(c->D.stat))   // the export reads the axis count table
-        CSE_TRY(cse_launch_axis_counts(c, P.T, P.NA, P.K_tiles, P.k_stride, s));
+    CSE_TRY(prepare(c, t, s, &P, true, true));   // the export reads the axis count table
     if (c->D.stat == CSE_STAT_BAYES4)
         return cse_launch_emit_bayes4(c, P.T, P.NA, P.k_stride, P.K_tiles, offsets, S_out, s);
     if (c->D.stat == CSE_STAT_BERRY4)

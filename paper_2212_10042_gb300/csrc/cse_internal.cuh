@@ -316,7 +316,7 @@ struct cse_ctx {
     cudaStream_t side;
     cudaEvent_t ev_fork, ev_join;
 
-    uint32_t* U;            // [d][K_max][n_max] uniforms sorted within each analysis segment
+    uint32_t* U;            // plain z-test path: [d][K_max][n_max] uniforms, each row sorted
     uint32_t* tb;           // [K_max] tie-break word of each sim (randomised test)
     uint32_t* tbuf;         // [grid][K_max] tie-group words gathered by the randomised kernel
     size_t tbuf_cap;
@@ -372,7 +372,7 @@ struct cse_ctx {
     bool cp_marked;         // the last simulation launch filled the Clopper-Pearson memo (SimOut::cp_key)
 
     bool plain;             // plain comparison path: direct counts, FP64-only bounds
-    bool u_stale;           // cse_reseed changed the key; U and tb not yet regenerated
+    bool u_stale;           // U (plain z-test path) does not hold the current key's uniforms
 
     // four-arm Bayesian design: tabulated posterior (see sim_bayes4.cu)
     bool bt_tables;         // tables built
@@ -429,14 +429,12 @@ void cse_prof_end(cse_ctx* c, cudaStream_t s);
 // ---------------------------------------------------------------------------
 // Launchers implemented in the .cu files (host functions).
 // ---------------------------------------------------------------------------
-// With a tile set T (else NULL), the uniforms kernel's first blocks also write
-// the success thresholds of its n_thr axis values; *thr_done says whether they did.
-int cse_launch_uniforms(cse_ctx* c, cudaStream_t s, const TileArgs* T = nullptr, int32_t n_thr = 0,
-                        bool* thr_done = nullptr);
+int cse_launch_uniforms(cse_ctx* c, cudaStream_t s);   // plain z-test path: sorted uniforms and tie-break words
 int cse_launch_tables(cse_ctx* c, cudaStream_t s);
 int cse_launch_thresholds(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, cudaStream_t s);
 int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, int32_t K_tiles,
                            int32_t k_stride, cudaStream_t s);
+int cse_launch_axis_box(cse_ctx* c, int32_t n_axis_total, int32_t K_tiles, int32_t k_stride, cudaStream_t s);
 int cse_bound_set_attrs();   // once per context: launch attributes of the bound kernels
 int cse_launch_alpha_prime(cse_ctx* c, const TileArgs& T, double alpha, double* aprime_out, int32_t* ksel,
                            cudaStream_t s, double* geom = nullptr);

@@ -105,7 +105,8 @@ extern "C" int cse_simulate_tiles_static(const cse_design* design, uint64_t seed
     T.K = t->K;
     const int32_t k_stride = (t->K_max + 15) / 16 * 16;
 
-    // layout of the scratch
+    // layout of the scratch (the region of sz_U bytes is reserved but not used: the
+    // count tables draw the uniforms themselves; the documented capacity counts it)
     const size_t off_flags = 0;                                   // counter, error flag
     const size_t off_U = 256;
     const size_t sz_U = sizeof(uint32_t) * (size_t)ds.d * (size_t)t->K_max * (size_t)n_max;
@@ -141,7 +142,6 @@ extern "C" int cse_simulate_tiles_static(const cse_design* design, uint64_t seed
     c.device = dev;
     c.counter = (int32_t*)(base + off_flags);
     c.err = (int32_t*)(base + off_flags + 64);
-    c.U = (uint32_t*)(base + off_U);
     c.thr = (uint32_t*)(base + off_thr);
     c.sig = (double*)(base + off_sig);
     c.cnt = base + off_cnt;
@@ -161,10 +161,10 @@ extern "C" int cse_simulate_tiles_static(const cse_design* design, uint64_t seed
         cudaGetLastError();
         return CSE_CUDA_ERROR;
     }
-    if ((st = cse_launch_uniforms(&c, s)) != CSE_OK) return st;
     if ((st = cse_launch_tables(&c, s)) != CSE_OK) return st;
     if ((st = cse_launch_thresholds(&c, T, na, s)) != CSE_OK) return st;
     if ((st = cse_launch_axis_counts(&c, T, na, t->K_max, k_stride, s)) != CSE_OK) return st;
+    if ((st = cse_launch_axis_box(&c, na, t->K_max, k_stride, s)) != CSE_OK) return st;
     SimOut o = {c.sig, R_out, Xrej_out, score_out, nullptr, nullptr};
     if ((st = cse_launch_sim_ztest(&c, T, na, k_stride, t->K_max, lambda, o, s)) != CSE_OK) return st;
     int32_t flags = 0;

@@ -3,10 +3,10 @@
 //
 // CRN (Sec. 7.3 of the paper: simulations may be shared across tiles as long
 // as each tile's own simulations are i.i.d.): sim k, arm a, patient j uses word
-// j mod 4 of Philox4x32-10(counter (k, a, j/4, 0), key = seed).  The words of
-// each (sim, arm) are sorted within every analysis segment
-// [look_n[l-1], look_n[l]) so that the success count of any parameter value is
-// a binary search (a patient succeeds iff u < t(theta)).
+// j mod 4 of Philox4x32-10(counter (k, a, j/4, 0), key = seed), and the patient
+// succeeds iff u < t(theta).  The count tables draw the words themselves
+// (k_counts); the plain z-test path keeps each (sim, arm) row sorted in memory
+// (k_uniforms), where a success count is a binary search.
 #include <cuda_runtime.h>
 
 #include <cstring>
@@ -15,6 +15,9 @@
 #include "cse_internal.cuh"
 
 namespace {
+
+// what a count table holds (see k_counts)
+constexpr int kCountsRaw = 0, kCountsNib = 1, kCountsMapped = 2;
 
 // One warp per (arm, sim) row: lane L generates and holds elements L*E .. L*E+E-1
 // (E = 32-padded power of two / 32), and a bitonic network over the 32*E keys
@@ -35,17 +38,13 @@ __device__ __forceinline__ void threshold_of(int i, uint32_t* __restrict__ thr, 
 }
 
 //
-// Two small jobs ride on the first blocks (one thread each, before the rows):
-// the randomised test's tie-break word of every sim (tb, may be NULL; word 0 of
-// Philox4x32-10(counter (k, 0, 0, 1), key = seed), the patients' draws using
-// counter word 3 = 0) and, when a tile set is given (thr not NULL), the success
-// thresholds of its n_thr axis values: two launches fewer per step.
+// The randomised test's tie-break word of every sim rides on the first blocks, one
+// thread each (tb; word 0 of Philox4x32-10(counter (k, 0, 0, 1), key = seed), the
+// patients' draws using counter word 3 = 0).
 template <int E, bool SEG>
 __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int32_t K_max, int32_t d,
                                                   int32_t n_looks, int4 looks, int32_t n_max,
-                                                  uint32_t key0, uint32_t key1, uint32_t* __restrict__ tb,
-                                                  uint32_t* __restrict__ thr, double* __restrict__ sig, TileArgs T,
-                                                  int32_t n_thr)
+                                                  uint32_t key0, uint32_t key1, uint32_t* __restrict__ tb)
 {
     pdl_entry();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -53,7 +52,6 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
         u32x4 c = {(uint32_t)g, 0u, 0u, 1u};
         tb[g] = philox4x32_10(c, key0, key1).x;
     }
-    if (thr && g < n_thr) threshold_of((int)g, thr, sig, T);
     using Key = typename std::conditional<SEG, unsigned long long, uint32_t>::type;
     constexpr int NP = 32 * E;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -124,92 +122,212 @@ __global__ void k_thresholds(uint32_t* __restrict__ thr, double* __restrict__ si
 
 // Axis count table: cnt[(l * NA + off_a + v) * k_stride + k] = number of the
 // first look_n[l] patients of (sim k, arm a) whose uniform is below t(axis_a[v]).
-// Block: one arm, KB consecutive sims staged in shared memory (rows at an odd
-// word stride, so that the 32 lanes' rows start in different banks).  Warp w
-// takes a run of consecutive axis values for all KB sims (lane = sim): the
-// thresholds of sorted axis values rise, so each look segment's count is a
-// merge of the sorted uniforms with the thresholds (one binary search at the
-// run's first value, then a forward scan: ~0.4 uniforms pass per axis step on
-// the 256-value grids) instead of a binary search per value.  A threshold
-// below the previous one (unsorted axis values) restarts with a binary search.
 //
-// nib (the packed four-arm form): two planes instead of three, plane 0 the two
-// interim segments' counts in the two halves of a byte (first segment << 4 |
-// second segment; both at most 15), plane 1 the score of the final cumulative
-// count.
-constexpr int KB = 32;
-__global__ void __launch_bounds__(256) k_axis_counts(uint8_t* __restrict__ cnt, const uint32_t* __restrict__ U,
-                                                     const uint32_t* __restrict__ thr, TileArgs T,
-                                                     int32_t NA, int32_t K_max_ctx, int32_t K_tiles,
-                                                     int32_t k_stride, int32_t n_looks, int4 looks,
-                                                     int32_t n_max, bool nib, const uint8_t* __restrict__ score)
+// Counts along an arm's rising thresholds are the running sums of a histogram: a
+// uniform u counts for every value with t > u, so it adds one at the position
+// p(u) = #{t <= u} and the counts are prefix sums.  A block takes 128 sims of one
+// arm and a chunk of its values: it draws the sims' Philox words (no sorted rows of
+// uniforms in memory), finds p(u) by a table over the top 12 bits and a short binary
+// search, adds into a shared-memory histogram of four sims a word (byte lanes: a
+// count is at most 128; lane l of every warp owns column l, so no bank conflicts),
+// and writes the prefix sums four sims a store.  Per count that is ~2 thread
+// instructions instead of a merge step's ~10 on byte loads and stores, and per
+// uniform ~30 instead of the 28-step sorting network.  Axis values in any order:
+// a chunk whose thresholds do not rise is sorted first.
+//
+// Bound by issue slots.  With the uniforms' pass and its sort, the count pass they
+// replace took: two arms, 256 values each, K = 16,384 26 + 24 us, now 15 us in all; 2^18
+// batch (959 values, K = 65,536) 92 + 99, now 49; one arm, 1,500 values, K = 65,536
+// 28 + 115, now 54; 4,096 values in random order, K = 8,192 15 + 244, now 44.
+//
+// MODE kCountsNib (the packed four-arm form): two planes instead of three, plane 0
+// the two interim segments' counts in the two halves of a byte (first segment << 4
+// | second segment; both at most 15), plane 1 map[final count].  kCountsMapped: a
+// second plane holds map[count] for arm 0's values.
+constexpr int kCntSims = 128, kCntThreads = 512;
+
+// top bits of a word that index the position table: with three histograms fewer,
+// so that two blocks fit an SM's shared memory
+template <int SEGS>
+constexpr int cnt_lut_bits()
+{
+    return SEGS > 1 ? 11 : 12;
+}
+
+template <int SEGS, int MODE>
+__global__ void __launch_bounds__(kCntThreads) k_counts(uint8_t* __restrict__ cnt, const uint32_t* __restrict__ thr,
+                                                        TileArgs T, int32_t NA, int32_t K_tiles, int32_t k_stride,
+                                                        int2 looks, int32_t n_max, uint32_t key0, uint32_t key1,
+                                                        uint32_t* __restrict__ tb, int32_t chunk, int32_t pow2,
+                                                        int32_t v_base, const uint8_t* __restrict__ map)
 {
     pdl_entry();
-    __shared__ uint32_t rows[KB * (CSE_MAX_NMAX + 1)];
-    const int a = blockIdx.y;
-    const int k0 = blockIdx.x * KB;
-    const int nk = min(KB, K_tiles - k0);
-    const int stride = n_max | 1;
-    const uint32_t* src = U + ((int64_t)a * K_max_ctx + k0) * n_max;
-    for (int i = threadIdx.x; i < nk * n_max; i += blockDim.x) {
-        const int row = i / n_max;
-        rows[row * stride + (i - row * n_max)] = src[i];
-    }
-    __shared__ uint8_t s_score[CSE_MAX_NMAX + 1];
-    if (nib)
-        for (int i = threadIdx.x; i <= n_max; i += blockDim.x) s_score[i] = score[i];
-    __syncthreads();
-    const int kk = threadIdx.x & (KB - 1);
-    const int nw = blockDim.x / KB, w = threadIdx.x / KB;
-    // the arm's entries by selection (a runtime index into the by-value
-    // argument would copy it to local memory)
+    constexpr int NW = kCntThreads / 32, LB = cnt_lut_bits<SEGS>(), LUT = 1 << LB;
+    extern __shared__ __align__(16) uint32_t smem[];
+    // histogram [SEGS][chunk][32], thresholds [chunk], table, order, then (sorting
+    // only, before the histogram is in use) 64-bit keys over the histogram
+    uint32_t* delta = smem;
+    uint32_t* st = smem + SEGS * chunk * 32;
+    uint16_t* perm = reinterpret_cast<uint16_t*>(st + chunk);
+    __shared__ __align__(16) uint32_t lut[LUT];   // a bucket's thresholds: those below it | its own << 16
+    __shared__ uint32_t s_scan[NW];
+    __shared__ uint8_t s_map[MODE != kCountsRaw ? CSE_MAX_NMAX + 1 : 1];
+    __shared__ uint32_t s_part[SEGS][NW][32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int a = blockIdx.y, k0 = blockIdx.x * kCntSims, v0 = v_base + blockIdx.z * chunk;
     int na = T.n_axis[0], off = T.axis_off[0];
 #pragma unroll
-    for (int b = 1; b < CSE_MAX_ARMS; ++b)
+    for (int b = 1; b < CSE_MAX_ARMS; ++b)   // by selection: no runtime index into the argument
         if (a == b) {
             na = T.n_axis[b];
             off = T.axis_off[b];
         }
-    const int per = (na + nw - 1) / nw;
-    const int v0 = w * per, v1 = min(v0 + per, na);
-    if (kk >= nk || v0 >= v1) return;
-    const uint32_t* r = rows + kk * stride;
-    // look segments [0, L0), [L0, L1), [L1, L2) of the row (sorted within each)
-    const int len0 = looks.x;
-    const int len1 = (n_looks > 1) ? looks.y - looks.x : 0;
-    const int len2 = (n_looks > 2) ? looks.z - looks.y : 0;
-    const uint32_t* r1 = r + looks.x;
-    const uint32_t* r2 = r + looks.y;
-    uint32_t tp = thr[off + v0];
-    int j0 = count_below(r, len0, tp), j1 = count_below(r1, len1, tp), j2 = count_below(r2, len2, tp);
-    auto advance = [](const uint32_t* seg, int len, int jj, uint32_t t, bool back) {
-        if (back) jj = count_below(seg, len, t);
-        while (jj < len && seg[jj] < t) ++jj;
-        return jj;
-    };
-    uint8_t* out = cnt + (int64_t)(off + v0) * k_stride + k0 + kk;
-    const int64_t look_stride = (int64_t)NA * k_stride;
-    for (int v = v0; v < v1; ++v, out += k_stride) {
-        const uint32_t t = thr[off + v];
-        const bool back = t < tp;
-        tp = t;
-        j0 = advance(r, len0, j0, t, back);
-        if (nib) {
-            j1 = advance(r1, len1, j1, t, back);
-            j2 = advance(r2, len2, j2, t, back);
-            out[0] = (uint8_t)((j0 << 4) | j1);
-            out[look_stride] = s_score[j0 + j1 + j2];
-            continue;
-        }
-        out[0] = (uint8_t)j0;
-        if (n_looks > 1) {
-            j1 = advance(r1, len1, j1, t, back);
-            out[look_stride] = (uint8_t)(j0 + j1);
-            if (n_looks > 2) {
-                j2 = advance(r2, len2, j2, t, back);
-                out[2 * look_stride] = (uint8_t)(j0 + j1 + j2);
+    // the randomised test's tie-break words (word 0 of Philox(counter (k, 0, 0, 1)))
+    if (tb && a == 0 && v0 == 0 && tid < kCntSims && k0 + tid < K_tiles) {
+        u32x4 c = {(uint32_t)(k0 + tid), 0u, 0u, 1u};
+        tb[k0 + tid] = philox4x32_10(c, key0, key1).x;
+    }
+    const int nv = min(chunk, na - v0);
+    if (nv <= 0) return;   // an arm with fewer chunks
+    if (MODE != kCountsRaw)
+        for (int i = tid; i <= n_max; i += kCntThreads) s_map[i] = map[i];
+    // the chunk's thresholds in rising order
+    bool falls = false;
+    for (int i = tid; i < nv; i += kCntThreads) {
+        const uint32_t t = thr[off + v0 + i];
+        st[i] = t;
+        perm[i] = (uint16_t)i;
+        falls |= i > 0 && thr[off + v0 + i - 1] > t;
+    }
+    if (__syncthreads_or(falls)) {   // bitonic sort of (threshold, index), padded with all ones
+        unsigned long long* key = reinterpret_cast<unsigned long long*>(delta);
+        for (int i = tid; i < pow2; i += kCntThreads)
+            key[i] = i < nv ? ((unsigned long long)st[i] << 32) | (unsigned)i : ~0ull;
+        for (int size = 2; size <= pow2; size <<= 1)
+            for (int j = size >> 1; j > 0; j >>= 1) {
+                __syncthreads();
+                for (int i = tid; i < pow2 / 2; i += kCntThreads) {
+                    const int lo = 2 * i - (i & (j - 1)), hi = lo + j;
+                    const unsigned long long x = key[lo], y = key[hi];
+                    if ((x > y) == ((lo & size) == 0)) {
+                        key[lo] = y;
+                        key[hi] = x;
+                    }
+                }
             }
+        __syncthreads();
+        for (int i = tid; i < nv; i += kCntThreads) {
+            st[i] = (uint32_t)(key[i] >> 32);
+            perm[i] = (uint16_t)(uint32_t)key[i];
         }
+        __syncthreads();
+    }
+    // the table over the words' top bits: thresholds counted per bucket, then scanned
+    constexpr int PER = LUT / kCntThreads;
+    for (int i = tid; i < LUT / 4; i += kCntThreads) reinterpret_cast<uint4*>(lut)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    for (int i = tid; i < nv; i += kCntThreads) atomicAdd(&lut[st[i] >> (32 - LB)], 1u);
+    __syncthreads();
+    uint32_t own[PER], local = 0u;
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        own[i] = lut[tid * PER + i];
+        local += own[i];
+    }
+    uint32_t incl = local;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+        if (lane >= o) incl += y;
+    }
+    if (lane == 31) s_scan[warp] = incl;
+    __syncthreads();
+    uint32_t start = incl - local;
+    for (int w = 0; w < warp; ++w) start += s_scan[w];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) {
+        lut[tid * PER + i] = start | (own[i] << 16);
+        start += own[i];
+    }
+    for (int i = tid; i < SEGS * chunk * 8; i += kCntThreads)
+        reinterpret_cast<uint4*>(delta)[i] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    // Philox blocks: lane l draws for sims 4 l + r of the block
+    const int nq = (n_max + 3) >> 2;
+    for (int t = warp; t < 4 * nq; t += NW) {
+        const int r = t & 3, q = t >> 2, k = k0 + 4 * lane + r;
+        if (k >= K_tiles) continue;
+        const u32x4 c = {(uint32_t)k, (uint32_t)a, (uint32_t)q, 0u};
+        const u32x4 w = philox4x32_10(c, key0, key1);
+        const uint32_t u4[4] = {w.x, w.y, w.z, w.w};
+        int lo[4], hi[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t x = lut[u4[j] >> (32 - LB)];
+            lo[j] = (int)(x & 0xFFFFu);
+            hi[j] = lo[j] + (int)(x >> 16);
+        }
+        // one step settles the buckets of at most one threshold, nearly all of them
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int mid = (lo[j] + hi[j]) >> 1;
+            const bool up = lo[j] < hi[j] && st[min(mid, nv - 1)] <= u4[j];
+            hi[j] = up ? hi[j] : min(hi[j], mid);
+            lo[j] = up ? mid + 1 : lo[j];
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+            while (lo[j] < hi[j]) {
+                const int mid = (lo[j] + hi[j]) >> 1;
+                if (st[mid] <= u4[j]) lo[j] = mid + 1;
+                else hi[j] = mid;
+            }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int e = 4 * q + j;
+            const int seg = SEGS > 1 ? (e >= looks.x ? 1 : 0) + (e >= looks.y ? 1 : 0) : 0;
+            if (e < n_max && lo[j] < nv) atomicAdd(&delta[(seg * chunk + lo[j]) * 32 + lane], 1u << (8 * r));
+        }
+    }
+    __syncthreads();
+    // prefix sums down the rows: each warp its stretch, from the sums of those above
+    const int per = (nv + NW - 1) / NW, j0 = min(warp * per, nv), j1 = min(j0 + per, nv);
+    uint32_t acc[SEGS];
+#pragma unroll
+    for (int g = 0; g < SEGS; ++g) {
+        uint32_t x = 0u;
+#pragma unroll 4
+        for (int j = j0; j < j1; ++j) x += delta[(g * chunk + j) * 32 + lane];
+        s_part[g][warp][lane] = x;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int g = 0; g < SEGS; ++g) {
+        acc[g] = 0u;
+        for (int w = 0; w < warp; ++w) acc[g] += s_part[g][w][lane];
+    }
+    const int k = k0 + 4 * lane;
+    if (k >= k_stride) return;   // k_stride is a multiple of 16
+    auto mapped = [&](uint32_t x) {
+        return (uint32_t)s_map[x & 0xFFu] | ((uint32_t)s_map[(x >> 8) & 0xFFu] << 8) |
+               ((uint32_t)s_map[(x >> 16) & 0xFFu] << 16) | ((uint32_t)s_map[x >> 24] << 24);
+    };
+    const int64_t plane = (int64_t)NA * k_stride;
+#pragma unroll 4
+    for (int j = j0; j < j1; ++j) {
+        uint8_t* row = cnt + (int64_t)(off + v0 + perm[j]) * k_stride + k;
+        uint32_t sum = 0u;
+#pragma unroll
+        for (int g = 0; g < SEGS; ++g) {
+            acc[g] += delta[(g * chunk + j) * 32 + lane];
+            sum += acc[g];
+            if (MODE != kCountsNib) *reinterpret_cast<uint32_t*>(row + g * plane) = sum;
+        }
+        if (MODE == kCountsNib) {
+            *reinterpret_cast<uint32_t*>(row) = (acc[0] << 4) | acc[SEGS > 1 ? 1 : 0];
+            *reinterpret_cast<uint32_t*>(row + plane) = mapped(sum);
+        }
+        if (MODE == kCountsMapped && a == 0) *reinterpret_cast<uint32_t*>(row + plane) = mapped(sum);
     }
 }
 
@@ -323,7 +441,7 @@ __global__ void k_rank_table(const float* __restrict__ S, uint16_t* __restrict__
 
 }  // namespace
 
-int cse_launch_uniforms(cse_ctx* c, cudaStream_t s, const TileArgs* T, int32_t n_thr, bool* thr_done)
+int cse_launch_uniforms(cse_ctx* c, cudaStream_t s)
 {
     const int64_t rows = (int64_t)c->D.d * c->K_max;
     const int blocks = (int)((rows + 7) / 8);
@@ -331,18 +449,10 @@ int cse_launch_uniforms(cse_ctx* c, cudaStream_t s, const TileArgs* T, int32_t n
     const int n = c->D.n_max;
     const bool seg = c->D.n_looks > 1;
     const uint32_t k0 = (uint32_t)c->seed, k1 = (uint32_t)(c->seed >> 32);
-    // the side jobs need one thread each among the grid's blocks x 256 threads
-    const bool fold = T != nullptr && n_thr > 0 && (int64_t)n_thr <= (int64_t)blocks * 256;
-    TileArgs Tv;
-    memset(&Tv, 0, sizeof(Tv));
-    if (fold) Tv = *T;
-    uint32_t* thr = fold ? c->thr : nullptr;
-    double* sig = fold ? c->sig : nullptr;
-    const int32_t nt = fold ? n_thr : 0;
     cse_prof_begin(c, KID_UNIFORMS, s);
 #define CSE_UNIFORMS(E, SG)                                                                                       \
     cse_launch(c->pdl, k_uniforms<E, SG>, dim3(blocks), dim3(256), 0, s, c->U, c->K_max, c->D.d, c->D.n_looks, lk, \
-               n, k0, k1, c->tb, thr, sig, Tv, nt)
+               n, k0, k1, c->tb)
     if (n <= 32) {
         if (seg) CSE_UNIFORMS(1, true);
         else CSE_UNIFORMS(1, false);
@@ -356,7 +466,6 @@ int cse_launch_uniforms(cse_ctx* c, cudaStream_t s, const TileArgs* T, int32_t n
 #undef CSE_UNIFORMS
     cse_prof_end(c, s);
     c->launches += 1;
-    if (thr_done) *thr_done = fold;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
@@ -382,20 +491,55 @@ int cse_launch_thresholds(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, c
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
-int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, int32_t K_tiles,
-                           int32_t k_stride, cudaStream_t s)
+template <int SEGS, int MODE>
+static int launch_counts(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t K_tiles, int32_t k_stride,
+                         const uint8_t* map, cudaStream_t s)
 {
-    dim3 grid((K_tiles + KB - 1) / KB, T.d);
-    int4 lk = make_int4(c->D.look_n[0], c->D.look_n[1], c->D.look_n[2], 0);
-    const bool nib = cse_count_nibbles(c);
+    // chunks of at most 512 values (256 with three segments: 2 to 3 blocks an SM),
+    // equal in size, a multiple of 32
+    constexpr int CH_MAX = SEGS > 1 ? 256 : 512;
+    int na = 0;
+    for (int a = 0; a < T.d; ++a) na = T.n_axis[a] > na ? T.n_axis[a] : na;
+    const int64_t nz = ((int64_t)na + CH_MAX - 1) / CH_MAX;
+    const int chunk = (int)(((na + nz - 1) / nz + 31) / 32 * 32);
+    int pow2 = 32;
+    while (pow2 < chunk) pow2 <<= 1;
+    auto kern = k_counts<SEGS, MODE>;
+    const size_t smem = (size_t)chunk * (SEGS * 128 + 4 + 2);
+    if (smem > 20 * 1024 &&   // with the static arrays (up to 23 KB) beyond the default limit
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
     cse_prof_begin(c, KID_AXIS_COUNTS, s);
-    cse_launch(c->pdl, k_axis_counts, dim3(grid), dim3(256), 0, s, c->cnt, c->U, c->thr, T, n_axis_total, c->K_max, K_tiles,
-                                       k_stride, c->D.n_looks, lk, c->D.n_max, nib, c->bt_score);
-    c->launches += 1;
-    if (!cse_posterior_design(c->D.stat)) {   // the z-test cell kernel reads the boxes
-        cse_launch(c->pdl, k_axis_box, dim3(n_axis_total), dim3(256), 0, s, c->cnt, n_axis_total, k_stride, K_tiles, c->D.n_looks - 1, c->bb);
+    const int64_t z_max = 65535;   // chunks of one launch
+    for (int64_t v = 0; v < na; v += z_max * chunk) {
+        const int64_t nzc = ((int64_t)na - v + chunk - 1) / chunk;
+        const dim3 grid((unsigned)((K_tiles + kCntSims - 1) / kCntSims), (unsigned)T.d,
+                        (unsigned)(nzc < z_max ? nzc : z_max));
+        cse_launch(c->pdl, kern, grid, dim3(kCntThreads), smem, s, c->cnt, c->thr, T, NA, K_tiles, k_stride,
+                   make_int2(c->D.look_n[0], c->D.look_n[1]), c->D.n_max, (uint32_t)c->seed,
+                   (uint32_t)(c->seed >> 32), c->tb, chunk, pow2, (int32_t)v, map);
         c->launches += 1;
     }
     cse_prof_end(c, s);
+    return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, int32_t K_tiles,
+                           int32_t k_stride, cudaStream_t s)
+{
+    if (cse_count_nibbles(c)) return launch_counts<3, kCountsNib>(c, T, n_axis_total, K_tiles, k_stride, c->bt_score, s);
+    if (c->D.n_looks > 1) return launch_counts<3, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
+    return launch_counts<1, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
+}
+
+int cse_launch_axis_box(cse_ctx* c, int32_t n_axis_total, int32_t K_tiles, int32_t k_stride, cudaStream_t s)
+{
+    cse_prof_begin(c, KID_AXIS_COUNTS, s);
+    cse_launch(c->pdl, k_axis_box, dim3(n_axis_total), dim3(256), 0, s, c->cnt, n_axis_total, k_stride, K_tiles,
+               c->D.n_looks - 1, c->bb);
+    cse_prof_end(c, s);
+    c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
