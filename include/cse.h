@@ -270,7 +270,8 @@ int cse_reseed(cse_ctx* ctx, uint64_t seed, cse_stream_t stream);
 
 /* Autotuner: times the fused simulation pass of `tiles` (at `lambda`, with the
  * calibration selection for level `alpha`) in each configuration of the z-test
- * cell-histogram kernel, (threads per block, tiles per block) in (128, 1),
+ * cell-histogram kernel (where a call runs it: see cse_set_option), (threads per
+ * block, tiles per block) in (128, 1),
  * (256, 1), (512, 1), (64, 1), (128, 2), (256, 2), (256, 4) -- a block of T
  * threads working on G tiles at once gives each tile T / G threads, so the sims
  * per block and step are 16 T and the tiles in flight per SM follow from the
@@ -295,6 +296,10 @@ enum { CSE_OPT_BAYES_DIRECT = 1, CSE_OPT_PLAIN = 2, CSE_OPT_SIM_THREADS = 3, CSE
  * uniforms, which the first such call of a key generates (no axis count table), the bound pass entirely in FP64 (bisection
  * over q, Newton for Clopper-Pearson, no FP32 stage), and for BAYES4 and BERRY4
  * the direct per-trial posterior.  0 (default) is the chosen path.
+ * The z-test designs simulate by byte-parallel rejection counts (calls without an
+ * order statistic, n_max <= 126), by candidate trials (two arms, lambda <= -1 and
+ * alpha <= 0.1) or by a histogram over count cells (the rest); the next three
+ * options fix a configuration of the last, which then runs every call.
  * CSE_OPT_SIM_THREADS (z-test designs): 64, 128, 256 or 512 fixes the block size
  * of the simulation kernels with one tile per block (64: the cell kernel only;
  * default 128).  CSE_OPT_SIM_TILES (z-test designs): 1, 2 or 4 tiles per block of

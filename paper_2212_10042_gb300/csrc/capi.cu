@@ -99,7 +99,10 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
 
     CSE_TRY(grow((void**)&c->thr, &c->thr_cap, sizeof(uint32_t) * (size_t)na));
     CSE_TRY(grow((void**)&c->sig, &c->sig_cap, sizeof(double) * (size_t)na));
-    const size_t cnt_bytes = (size_t)c->D.n_looks * (size_t)na * (size_t)P->k_stride;
+    // (two arms: arm 0's values have a second row in ZMODE_COUNT)
+    const size_t cnt_rows = (size_t)c->D.n_looks * (size_t)na +
+                            (c->D.stat == CSE_STAT_TWO_ARM_POOLED_Z ? (size_t)t->n_axis[0] : 0);
+    const size_t cnt_bytes = cnt_rows * (size_t)P->k_stride;
     CSE_TRY(grow((void**)&c->cnt, &c->cnt_cap, cnt_bytes));
     CSE_TRY(grow((void**)&c->bb, &c->bb_cap, sizeof(uint32_t) * 2 * (size_t)na));
     if ((size_t)t->n_tiles > c->tile_cap) {
@@ -172,9 +175,32 @@ int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = f
         if (!counts) return CSE_OK;
     }
     CSE_TRY(cse_launch_axis_counts(c, P.T, P.NA, P.K_tiles, P.k_stride, s));
-    // the z-test cell kernel reads each axis value's least and greatest count
-    if (!cse_posterior_design(c->D.stat)) CSE_TRY(cse_launch_axis_box(c, P.NA, P.K_tiles, P.k_stride, s));
+    // the z-test cell and candidate kernels read each axis value's least and greatest count
+    if (!cse_posterior_design(c->D.stat) && c->zmode != ZMODE_COUNT) CSE_TRY(cse_launch_axis_box(c, P.NA, P.K_tiles, P.k_stride, s));
     return CSE_OK;
+}
+
+// How the z-test simulation of a call runs (results do not depend on it).  Without a
+// selection, rejections by byte-parallel counts (counts and cuts up to 127 keep each
+// sum in its byte: 1,500 one-arm tiles, K <= 65,536 34 -> 14 us, 2,048 free points
+// 28 -> 14).  With one, two arms: candidates, unless alpha or lambda reach so far
+// into the statistic that a good part of the trials are candidates, at about eight
+// times the cost of a histogram increment: lambda <= -1 and alpha <= 0.1 leave at
+// most one in six (256^2 grid, lambda = -1.96, alpha = 0.025: 7 %, 323 -> 265 us).
+// The cell histogram takes the rest -- one arm among them, whose n + 1 cells are
+// read off at once (64 tiles 10.8 us against 12.4) -- and every call whose
+// configuration the caller fixed.
+void choose_zmode(cse_ctx* c, bool want_R, double lambda, bool select, double alpha)
+{
+    if (!c) return;
+    c->zmode = ZMODE_CELLS;
+    if (cse_posterior_design(c->D.stat) || c->plain || c->cells_fixed || c->cells_box) return;
+    c->z_lambda = want_R ? lambda_float_up(lambda) : -INFINITY;
+    if (!select) {
+        if (c->D.n_max <= 126) c->zmode = ZMODE_COUNT;
+    } else if (c->D.stat == CSE_STAT_TWO_ARM_POOLED_Z && alpha <= 0.1 && (!want_R || lambda <= -1.0)) {
+        c->zmode = ZMODE_TAIL;
+    }
 }
 
 int prepare(cse_ctx* c, const cse_tiles* t, cudaStream_t s, Prepared* P, bool geom = true, bool counts = false)
@@ -203,6 +229,8 @@ int sim_pass(cse_ctx* c, const Prepared& P, double lambda, const SimOut& o, cuda
 {
     c->min_folded = false;   // set by a kernel that writes o.min_out itself
     c->cp_marked = false;    // set by a kernel that fills the Clopper-Pearson memo itself
+    if (c->zmode == ZMODE_COUNT) return cse_launch_sim_count(c, P.T, P.NA, P.k_stride, P.K_tiles, o, s);
+    if (c->zmode == ZMODE_TAIL) return cse_launch_sim_tail(c, P.T, P.NA, P.k_stride, P.K_tiles, o, false, nullptr, s);
     if (c->D.stat == CSE_STAT_ONE_ARM_Z || c->D.stat == CSE_STAT_TWO_ARM_POOLED_Z)
         return cse_launch_sim_ztest(c, P.T, P.NA, P.k_stride, P.K_tiles, lambda, o, s);
     if (c->D.stat == CSE_STAT_BAYES4)
@@ -257,6 +285,7 @@ int cse_autotune(cse_ctx* c, const cse_tiles* t, double lambda, double alpha, in
         if (tiles_out) *tiles_out = 1;
         return CSE_OK;
     }
+    if (c) c->zmode = ZMODE_CELLS;   // the cell kernel is what is tuned
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, c->aprime, s));
@@ -322,6 +351,7 @@ int cse_set_option(cse_ctx* c, int option, int64_t value)
         const int cfg = cse_cells_config_index((int)value, 1);
         if (cfg < 0) return CSE_INVALID_ARG;
         c->cells_cfg = cfg;   // one tile per block
+        c->cells_fixed = true;
         if (value == 128) c->sim_topt = 0;
         else if (value == 256) c->sim_topt = 1;
         else if (value == 512) c->sim_topt = 2;
@@ -334,6 +364,7 @@ int cse_set_option(cse_ctx* c, int option, int64_t value)
         const int cfg = cse_cells_config_index(nt, (int)value);
         if (cfg < 0) return CSE_INVALID_ARG;
         c->cells_cfg = cfg;
+        c->cells_fixed = true;
         return CSE_OK;
     }
     case CSE_OPT_CELLS_BOX: {   // histogram capacity of the cell kernel (0: the allocated one)
@@ -491,7 +522,11 @@ int cse_create(cse_ctx** out, const cse_design* design, uint64_t seed, int32_t K
             if (cudaMalloc(&c->S_tab, 4 * (size_t)c->n_cells) != cudaSuccess ||
                 cudaMalloc(&c->rank_tab, 2 * (size_t)c->n_cells) != cudaSuccess ||
                 cudaMalloc(&c->val_of_rank, 4 * (size_t)c->n_cells) != cudaSuccess ||
-                cudaMalloc(&c->cell_of_pos, 8 * (size_t)c->n_cells) != cudaSuccess) { st = CSE_OOM; break; }
+                cudaMalloc(&c->cell_of_pos, 8 * (size_t)c->n_cells) != cudaSuccess ||
+                cudaMalloc(&c->zpar, 64) != cudaSuccess || cudaMalloc(&c->zcut, 256) != cudaSuccess) {
+                st = CSE_OOM;
+                break;
+            }
         }
         if (cudaMalloc(&c->counter, 64) != cudaSuccess || cudaMalloc(&c->err, 64) != cudaSuccess ||
             cudaMalloc(&c->cp_nkeys, 64) != cudaSuccess || cudaMalloc(&c->min_key, 64) != cudaSuccess ||
@@ -555,6 +590,8 @@ int cse_destroy(cse_ctx* c)
     cudaFree(c->rank_tab);
     cudaFree(c->val_of_rank);
     cudaFree(c->cell_of_pos);
+    cudaFree(c->zpar);
+    cudaFree(c->zcut);
     cudaFree(c->xs);
     cudaFree(c->tie_rm);
     cudaFree(c->thr);
@@ -607,6 +644,7 @@ int cse_simulate_tiles(cse_ctx* c, const cse_tiles* t, double lambda, int64_t* R
                        double* score_out, cse_stream_t stream)
 {
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, true, lambda, false, 0.0);
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P));
     SimOut o = {c->sig, R_out, Xrej_out, score_out, nullptr, nullptr};
@@ -661,6 +699,7 @@ int cse_type1_error(cse_ctx* c, int64_t n_points, const double* theta, const uin
     t.null_mask = null_mask;
     t.K = K;
     t.K_max = K_max;
+    choose_zmode(c, true, lambda, false, 0.0);
     Prepared P;
     CSE_TRY(prepare(c, &t, s, &P, false));
     int64_t* R = R_out ? R_out : c->R;
@@ -675,6 +714,7 @@ int cse_validate(cse_ctx* c, const cse_tiles* t, double lambda, double delta, in
 {
     if (!(delta > 0.0 && delta < 1.0)) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, true, lambda, false, 0.0);
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P));
     int64_t* R = R_out ? R_out : c->R;
@@ -689,6 +729,7 @@ int cse_validate_lower(cse_ctx* c, const cse_tiles* t, double lambda, double del
 {
     if (!(delta > 0.0 && delta < 1.0)) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, true, lambda, false, 0.0);
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P));
     int64_t* R = R_out ? R_out : c->R;
@@ -703,6 +744,7 @@ int cse_validate_band(cse_ctx* c, const cse_tiles* t, double lambda, double delt
 {
     if (!(delta > 0.0 && delta < 1.0)) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, true, lambda, false, 0.0);
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P));
     int64_t* R = R_out ? R_out : c->R;
@@ -720,11 +762,14 @@ int cse_validate_rand(cse_ctx* c, const cse_tiles* t, double lambda, uint32_t c_
     if (!(delta > 0.0 && delta < 1.0)) return CSE_INVALID_ARG;
     if (c && cse_posterior_design(c->D.stat)) return CSE_UNSUPPORTED_DESIGN;
     cudaStream_t s = (cudaStream_t)stream;
+    if (c_thr == 0u) choose_zmode(c, true, lambda, false, 0.0);   // no words: the plain rule
+    else if (c) c->zmode = ZMODE_CELLS;
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P, true, true));
     int64_t* R = R_out ? R_out : c->R;
     SimOut o = {c->sig, R, Xrej_out, score_out, nullptr, nullptr};
-    CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, lambda, c_thr, o, nullptr, s));
+    if (c->zmode == ZMODE_COUNT) CSE_TRY(cse_launch_sim_count(c, P.T, P.NA, P.k_stride, P.K_tiles, o, s));
+    else CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, lambda, c_thr, o, nullptr, s));
     return cse_launch_bounds(c, P.T, R, delta, false, u0_out, bound_out, qstar_out, s);
 }
 
@@ -736,11 +781,13 @@ int cse_calibrate_rand(cse_ctx* c, const cse_tiles* t, double alpha, double* alp
     if (!lambda_tile_out || !c_tile_out) return CSE_INVALID_ARG;
     if (c && cse_posterior_design(c->D.stat)) return CSE_UNSUPPORTED_DESIGN;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, false, INFINITY, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s, nullptr, true));
     SimOut o = {c->sig, nullptr, nullptr, nullptr, lambda_tile_out, c->ksel};
-    CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, INFINITY, 0u, o, c_tile_out, s));
+    if (c->zmode == ZMODE_TAIL) CSE_TRY(cse_launch_sim_tail(c, P.T, P.NA, P.k_stride, P.K_tiles, o, true, c_tile_out, s));
+    else CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, INFINITY, 0u, o, c_tile_out, s));
     // (lambda*, c*) through the device scalars lam_dev and lam_dev + 1 (its low 4 bytes)
     uint32_t* c_dev = reinterpret_cast<uint32_t*>(c->lam_dev + 1);
     CSE_TRY(cse_launch_min_pair(c, lambda_tile_out, c_tile_out, t->n_tiles, c->lam_dev, c_dev, s));
@@ -756,6 +803,7 @@ int cse_calibrate(cse_ctx* c, const cse_tiles* t, double alpha, double* alpha_pr
 {
     if (!(alpha > 0.0 && alpha < 1.0)) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, false, INFINITY, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
     double* lam_tile = lambda_tile_out ? lambda_tile_out : c->lam_tile;
@@ -778,6 +826,7 @@ int cse_step(cse_ctx* c, const cse_tiles* t, double lambda, double delta, double
     if (!(delta > 0.0 && delta < 1.0) || !(alpha > 0.0 && alpha < 1.0)) return CSE_INVALID_ARG;
     if (!lambda_tile_out || !lambda_dev) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    choose_zmode(c, true, lambda, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
     int64_t* R = R_out ? R_out : c->R;
@@ -808,6 +857,7 @@ int cse_statistics(cse_ctx* c, const cse_tiles* t, const int64_t* offsets, float
 {
     if (!offsets || !S_out) return CSE_INVALID_ARG;
     cudaStream_t s = (cudaStream_t)stream;
+    if (c) c->zmode = ZMODE_CELLS;
     Prepared P;
     CSE_TRY(prepare(c, t, s, &P, true, true));   // the export reads the axis count table
     if (c->D.stat == CSE_STAT_BAYES4)

@@ -245,6 +245,66 @@ __device__ int block_find_kth(const uint32_t* counts, int n, int ks, int* s_scan
 }
 
 // ---------------------------------------------------------------------------
+// Tiles by groups of threads (the kernels that evaluate candidate trials).
+// ---------------------------------------------------------------------------
+template <int TT, int G>
+__device__ __forceinline__ void tile_sync(int g)
+{
+    // the TT threads of group g: a warp, the block, or named barrier 1 + g (barrier 0
+    // is __syncthreads)
+    if (TT == 32) __syncwarp();
+    else if (G == 1) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(TT) : "memory");
+}
+
+// One warp: the bin of counts[0..256) holding the ks-th unit (from bin 0 up), -1
+// if the total is below ks, and the sum before it; ZERO clears the bins.
+template <bool ZERO>
+__device__ __forceinline__ int warp_pick256(uint32_t* counts, int ks, int lane, int* before)
+{
+    uint32_t h[8];
+    int local = 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+        h[j] = counts[lane * 8 + j];
+        local += (int)h[j];
+    }
+    if (ZERO)
+#pragma unroll
+        for (int j = 0; j < 8; ++j) counts[lane * 8 + j] = 0u;
+    int incl = local;
+#pragma unroll
+    for (int off = 1; off < 32; off <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, incl, off);
+        if (lane >= off) incl += y;
+    }
+    const unsigned who = __ballot_sync(0xffffffffu, incl >= ks);
+    if (who == 0u) return -1;
+    const int src = __ffs(who) - 1;
+    int b = 0, cum = incl - local;
+#pragma unroll
+    for (int j = 0; j < 7; ++j)
+        if (b == j && cum + (int)h[j] < ks) {
+            cum += (int)h[j];
+            b = j + 1;
+        }
+    *before = __shfl_sync(0xffffffffu, cum, src);
+    return __shfl_sync(0xffffffffu, lane * 8 + b, src);
+}
+
+// Bits 8 j + q of a candidate word for trials 4 q + j < rem (rem > 0).
+__device__ __forceinline__ uint32_t trials_below(int rem)
+{
+    uint32_t in = 0u;
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const int nb = min(max(rem - 4 * q, 0), 4);
+        in |= (nb == 4 ? 0x01010101u : (((1u << (8 * nb)) - 1u) & 0x01010101u)) << q;
+    }
+    return in;
+}
+
+// ---------------------------------------------------------------------------
 // Kernel argument bundles (passed by value).
 // ---------------------------------------------------------------------------
 struct TileArgs {
@@ -296,6 +356,10 @@ enum KernelId {
     KID_TIE,
     KID_COUNT
 };
+
+// How a z-test call simulates: the cell histogram (sim_ztest.cu), byte-parallel
+// rejection counts, or candidates for the order statistic (sim_tail.cu).
+enum ZMode { ZMODE_CELLS = 0, ZMODE_COUNT, ZMODE_TAIL };
 
 struct ProfRec {
     int kid;
@@ -367,6 +431,13 @@ struct cse_ctx {
     int32_t cells_grid[2][8];   // its persistent grid per [selection][configuration]
     bool cells_ok;          // the cell-histogram kernel fits this design's shared memory
     int32_t cells_box;      // box capacity of the cell histogram in cells (0: the allocated one)
+    bool cells_fixed;       // the caller fixed a configuration of the cell kernel (cse_set_option)
+    // the current z-test call (sim_tail.cu): which kernel simulates, the smallest
+    // float >= lambda, and its constants on the device
+    int32_t zmode;
+    float z_lambda;
+    int32_t* zpar;          // [1] number of cells with S < lambda
+    uint8_t* zcut;          // [n_max + 1] ZMODE_COUNT: least x_1 with S(x_0, x_1) < lambda (one arm: [0], least x)
     bool pdl;               // step kernels start with programmatic dependent launch
     bool min_folded;        // the last simulation launch wrote the minimum over tiles (SimOut::min_out)
     bool cp_marked;         // the last simulation launch filled the Clopper-Pearson memo (SimOut::cp_key)
@@ -508,6 +579,12 @@ int cse_launch_emit_basket(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_
 int cse_launch_bounds(cse_ctx* c, const TileArgs& T, const int64_t* R, double delta, bool lower, double* u0,
                       double* bound, double* qstar, cudaStream_t s, const double* geom = nullptr,
                       bool marked = false);
+// z-test calls without a selection (ZMODE_COUNT), with one (ZMODE_TAIL; words: the
+// randomised test's pairs, c_tile its output)
+int cse_launch_sim_count(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                         cudaStream_t s);
+int cse_launch_sim_tail(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                        bool words, uint32_t* c_tile, cudaStream_t s);
 int cse_launch_sim_rand(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, double lambda,
                         uint32_t c_thr, const SimOut& o, uint32_t* c_tile, cudaStream_t s);
 int cse_launch_min_pair(cse_ctx* c, const double* lam_tile, const uint32_t* c_tile, int64_t n, double* lam_out,

@@ -591,49 +591,6 @@ __global__ void __launch_bounds__(256) k_table_dmin(const float4* __restrict__ F
         if (m[j] != 0x7F800000u) atomicMin(&dmin[j], m[j]);
 }
 
-template <int TT, int G>
-__device__ __forceinline__ void tile_sync(int g)
-{
-    // the TT threads of group g: named barrier 1 + g (barrier 0 is __syncthreads)
-    if (G == 1) __syncthreads();
-    else asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(TT) : "memory");
-}
-
-// One warp: the bin of counts[0..256) holding the ks-th unit (from bin 0 up), -1
-// if the total is below ks, and the sum before it; ZERO clears the bins.
-template <bool ZERO>
-__device__ __forceinline__ int warp_pick256(uint32_t* counts, int ks, int lane, int* before)
-{
-    uint32_t h[8];
-    int local = 0;
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-        h[j] = counts[lane * 8 + j];
-        local += (int)h[j];
-    }
-    if (ZERO)
-#pragma unroll
-        for (int j = 0; j < 8; ++j) counts[lane * 8 + j] = 0u;
-    int incl = local;
-#pragma unroll
-    for (int off = 1; off < 32; off <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, incl, off);
-        if (lane >= off) incl += y;
-    }
-    const unsigned who = __ballot_sync(0xffffffffu, incl >= ks);
-    if (who == 0u) return -1;
-    const int src = __ffs(who) - 1;
-    int b = 0, cum = incl - local;
-#pragma unroll
-    for (int j = 0; j < 7; ++j)
-        if (b == j && cum + (int)h[j] < ks) {
-            cum += (int)h[j];
-            b = j + 1;
-        }
-    *before = __shfl_sync(0xffffffffu, cum, src);
-    return __shfl_sync(0xffffffffu, lane * 8 + b, src);
-}
-
 // Threads and blocks per SM: the packed form's shared-memory tables (57.6 KB)
 // and queues leave room for two blocks of 512; the byte form reads its tables
 // from global memory.
@@ -791,15 +748,7 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
                         m = ((t[0] >> 7) & 0x01010101u) | ((t[1] >> 6) & 0x02020202u) | ((t[2] >> 5) & 0x04040404u) |
                             ((t[3] >> 4) & 0x08080808u);
                     }
-                    if (kw + 16 > kend) {   // trials at or past K
-                        uint32_t in = 0u;
-#pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            const int nb = min(max(kend - kw - 4 * q, 0), 4);
-                            in |= (nb == 4 ? 0x01010101u : (((1u << (8 * nb)) - 1u) & 0x01010101u)) << q;
-                        }
-                        m &= in;
-                    }
+                    if (kw + 16 > kend) m &= trials_below(kend - kw);   // trials at or past K
                 }
                 const int nm = __popc(m);
                 int incl = nm;

@@ -1,0 +1,558 @@
+// sim_tail.cu -- the z-test simulation without a histogram over every trial: counts
+// of the rejections alone (k_sim_count), and the order statistic from a small tail
+// of the trials (k_sim_tail).
+//
+// The cell-histogram kernel (sim_ztest.cu) increments a shared-memory cell for
+// every trial, then reads the tile's box of ~1,700 cells off: about twelve thread
+// instructions a trial at K = 16,384, half of them the read-off.
+//
+// k_sim_count.  S(x_0, x_1) < lambda iff x_1 >= b(x_0), b(x_0) the least such x_1
+// (every row of S falls in x_1).  The count table carries b(x_0) in a row of its own
+// beside arm 0's counts (k_counts), so four trials are one word: bit 7 of byte
+// x_1 + (0x80 - b) is the rejection, no carry crossing a byte while counts and cuts
+// stay below 128.  R and the successes of the rejecting trials follow by byte dot
+// products: 2.3 thread instructions a trial, no branch, no shared memory.
+//
+// k_sim_tail (two arms).  The k_i-th smallest S of a tile lies near a known quantile: S is
+// nearly normal with mean and variance from the tile's point, and k_i / K_i is
+// given.  cap = that quantile at k_i + 3 sqrt(k_i) + 1 (and at least lambda), and
+// the trials with S < cap are among those with x_1 - x_0 >= d, where d is the least
+// cut(x_0) - x_0 over the tile's reachable x_0 (the axis box); four trials a word
+// again.  Each warp queues these candidates in shared memory and evaluates them 32
+// at a time: the cell's rank (rank = number of cells with a smaller statistic), the
+// rejections, the rank as a key in global memory (the warp's own stretch) and in
+// 256 bins.  Then the bin of the k_i-th key and its rank within the bin.  Trials
+// left out have S >= cap, so the result is exact when it is at most cap and there
+// are k_i keys; otherwise the pass is repeated with cap + 1/2, and after three
+// tries with every trial.  Randomised test: the candidates hold every trial of the
+// tying rank, so their words are gathered from the keys and the m-th smallest
+// taken; no second pass over the count rows.
+//
+// What bounds it: issue slots (54 to 60 % issue; 10 thread instructions a trial, of
+// which the test and the queueing take half, the 7 % candidates a third) and the
+// latency of the scattered count reads.
+// 256^2 grid, K = 16,384 (32,896 tiles): 323 -> 265 us; 2^18 batch: 3.34 -> 2.53 ms;
+// randomised calibration of the 128^2 grid: 95 + 67 (tie pass) -> 136 us.  Five blocks an
+// SM at 48 registers are no faster than four at 56.
+//
+// Tiles: a group of TT threads per tile, G tiles a block.  With many tiles a warp
+// per tile: no barriers and the most tiles in flight.  Fewer than 32 tiles an SM
+// take 128 threads each, fewer than 8 an SM a block of 256, for the latency of one
+// tile.
+#include <cuda_runtime.h>
+#include <math.h>
+
+#include "cse_internal.cuh"
+
+namespace {
+
+constexpr int kQueue = 288;   // a warp's candidate queue (up to 31 left over, at least 8 lanes' trials a round)
+constexpr int kList = 256;    // words of a tying rank ranked in shared memory
+constexpr int kTailThreads = 256;
+
+__device__ __forceinline__ int tail_warp_sum(int v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// A selection key: the rank, or (with the randomised test's words) rank << 17 | the
+// trial's place among its warp's.  Ranks lie below 129^2 < 2^15.
+template <bool WORDS>
+struct tail_key {
+    using type = uint16_t;
+};
+template <>
+struct tail_key<true> {
+    using type = uint32_t;
+};
+
+template <bool WORDS, int G>
+__global__ void __launch_bounds__(kTailThreads, 4)
+    k_sim_tail(TileArgs T, int32_t n_max, const uint8_t* __restrict__ cnt, int32_t NA, int32_t k_stride,
+               int32_t K_tiles, const uint16_t* __restrict__ rank_g, const float* __restrict__ S_g,
+               const float* __restrict__ vor_g, int32_t n_cells, int32_t n1p, int32_t bin_shift,
+               const uint32_t* __restrict__ bb, const int32_t* __restrict__ zpar, float lambda_up,
+               const uint32_t* __restrict__ W, SimOut o, uint32_t* __restrict__ c_tile, void* __restrict__ keys,
+               int32_t key_seg, int32_t* __restrict__ counter, int32_t* __restrict__ err)
+{
+    pdl_entry();
+    constexpr int TT = kTailThreads / G, NW = TT / 32;
+    using Key = typename tail_key<WORDS>::type;
+    __shared__ uint32_t s_hist[G][256];
+    __shared__ uint32_t s_list[WORDS ? G : 1][kList];
+    __shared__ uint16_t s_queue[kTailThreads / 32][kQueue];
+    __shared__ int s_tile[G], s_next[G], s_pick[G], s_before[G], s_nlist[G], s_nk[G][NW];
+    __shared__ uint32_t s_res[G];
+    __shared__ int s_red[G][3][NW];
+    __shared__ unsigned long long s_min[G];   // order key of the least lambda_i of the group's tiles
+    const int tid = threadIdx.x, lane = tid & 31;
+    const int g = tid / TT, lt = tid - g * TT, warp = lt >> 5;
+    uint32_t* const hist = s_hist[g];
+    uint32_t* const list = s_list[WORDS ? g : 0];
+    uint16_t* const queue = s_queue[tid >> 5];
+    // each warp appends its keys to its own stretch
+    Key* const kbuf = reinterpret_cast<Key*>(keys) + ((int64_t)(blockIdx.x * G + g) * NW + warp) * key_seg;
+    constexpr int d = 2;
+
+    for (int b = tid; b < G * 256; b += kTailThreads) (&s_hist[0][0])[b] = 0u;
+    if (tid < G) s_min[tid] = ~0ull;
+    __syncthreads();
+    const int rho = zpar[0];   // S < lambda iff rank < rho
+
+    if (lt == 0) s_next[g] = atomicAdd(counter, 1);
+    for (;;) {
+        if (lt == 0) {
+            s_tile[g] = s_next[g];
+            s_nlist[g] = 0;
+        }
+        tile_sync<TT, G>(g);
+        const int64_t i = s_tile[g];
+        if (i >= T.n_tiles) break;
+        if (lt == 0) s_next[g] = atomicAdd(counter, 1);   // the next tile, fetched while this one runs
+        const int K = T.K[i];
+        const int v0 = T.center_idx[i * d + 0];
+        const int v1 = T.center_idx[i * d + 1];
+        // device-side argument checks: K_i in [1, K_max of the set], axis indices in range
+        const bool bad = (K < 1) || (K > K_tiles) || v0 < 0 || v0 >= T.n_axis[0] || v1 < 0 ||
+                         v1 >= T.n_axis[1];
+        const int Kc = bad ? 0 : K;
+        const int a0 = T.axis_off[0] + (bad ? 0 : v0);
+        const int a1 = T.axis_off[1] + (bad ? 0 : v1);
+        const int ks = bad ? 0 : o.ksel[i];
+        const uint8_t* const c0 = cnt + (int64_t)a0 * k_stride;
+        const uint8_t* const c1 = cnt + (int64_t)a1 * k_stride;
+        int r_acc = 0, x0_acc = 0, x1_acc = 0;
+        double lam_i = -INFINITY;
+        uint32_t c_i = 0u;
+        // the tile's reachable counts, and the normal quantile that caps the selection
+        const int lo0 = (int)min(bb[a0], (uint32_t)n_max), hi0 = (int)min(bb[NA + a0], (uint32_t)n_max);
+        const int lo1 = (int)min(bb[a1], (uint32_t)n_max), hi1 = (int)min(bb[NA + a1], (uint32_t)n_max);
+        float cap = lambda_up;
+        if (ks >= 1) {
+            const float share = ((float)ks + 3.0f * sqrtf((float)ks) + 1.0f) / (float)K;
+            const float fn = (float)n_max, q0 = (float)o.sig[a0], q1 = (float)o.sig[a1];
+            const float pb = 0.5f * (q0 + q1), den = rsqrtf(pb * (1.0f - pb) * 2.0f / fn);
+            const float mean = (q0 - q1) * den;
+            const float sd = sqrtf((q0 * (1.0f - q0) + q1 * (1.0f - q1)) / fn) * den;
+            const float c = mean + normcdfinvf(fminf(share, 0.9f)) * sd + 0.05f;
+            cap = c > cap ? c : cap;
+        }
+        for (int tries = 0;; ++tries) {
+            // d: S < cap needs x_1 - x_0 >= d
+            bool all = ks >= 1 && (tries == 3 || !(cap < 30.0f));
+            int d_test = 1;
+            if (!all) {
+                int dl = 1 << 20;
+                for (int x0 = lo0 + lane; x0 <= hi0; x0 += 32) {
+                    const float* row = S_g + x0 * n1p;
+                    int lo = 0, hi = n_max + 1;   // least x_1 with S < cap
+                    while (lo < hi) {
+                        const int mid = (lo + hi) >> 1;
+                        if (row[mid] < cap) hi = mid;
+                        else lo = mid + 1;
+                    }
+                    dl = min(dl, lo - x0);
+                }
+                d_test = __reduce_min_sync(0xffffffffu, dl);
+                // every byte 0x80 - d + (x_1 - x_0) stays in 0 .. 255
+                const int dmin = lo1 - hi0, dmax = hi1 - lo0;
+                if (d_test <= dmin || dmax - dmin > 126) all = true;
+                d_test = min(d_test, dmax + 1);
+            }
+            const uint32_t zc = 0x80808080u - (uint32_t)d_test * 0x01010101u;
+            int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
+            for (int st = 0; st * (TT * 32) < Kc; ++st) {   // group-uniform
+                // thirty-two consecutive trials per thread and step; bit 8 j + q of a
+                // thread's candidate word is trial 4 q + j.  kb: first trial of the warp
+                // in the queue's block of 64 steps
+                const int kb = (st & ~63) * (TT * 32) + warp * 1024, stq = st & 63;
+                const int kw = kb + stq * (TT * 32) + lane * 32;
+                uint32_t m = 0u;
+                if (kw < Kc) {
+                    if (all) {
+                        m = 0xFFFFFFFFu;
+                    } else {
+                        const bool two = kw + 16 < Kc;   // the second sixteen lie in the row
+                        const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+                        const uint4 xa = *reinterpret_cast<const uint4*>(c1 + kw);
+                        const uint4 xb = two ? *reinterpret_cast<const uint4*>(c1 + kw + 16) : zero;
+                        uint32_t t[8] = {xa.x, xa.y, xa.z, xa.w, xb.x, xb.y, xb.z, xb.w};
+                        const uint4 ya = *reinterpret_cast<const uint4*>(c0 + kw);
+                        const uint4 yb = two ? *reinterpret_cast<const uint4*>(c0 + kw + 16) : zero;
+                        const uint32_t y[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) t[q] = t[q] - y[q] + zc;
+#pragma unroll
+                        for (int q = 0; q < 8; ++q) m |= (t[q] >> (7 - q)) & (0x01010101u << q);
+                    }
+                    if (kw + 32 > Kc) m &= trials_below(Kc - kw);
+                }
+                const int nm = __popc(m);
+                int incl = nm;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += y;
+                }
+                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                const bool flush = stq == 63 || (st + 1) * (TT * 32) >= Kc;
+                const int ent = (stq << 10) | (lane << 5);   // entry: step (6 bits), lane, bit
+                int done = 0;   // candidates of this step queued so far
+                do {
+                    // the lanes whose candidates fit the queue (a prefix of those left)
+                    const bool mine = incl - nm >= done && incl - done <= kQueue - qn;
+                    const unsigned who = __ballot_sync(0xffffffffu, mine);
+                    const int upto = __shfl_sync(0xffffffffu, incl, 31 - __clz(who));
+                    if (mine) {
+                        uint16_t* at = queue + qn + (incl - nm - done);
+                        while (m) {
+                            const int b = __ffs(m) - 1;
+                            m &= m - 1u;
+                            *at++ = (uint16_t)(ent | b);
+                        }
+                    }
+                    qn += upto - done;
+                    done = upto;
+                    __syncwarp();
+                    while (qn >= 32 || (flush && done == total && qn > 0)) {
+                        const int n = min(qn, 32);
+                        qn -= n;
+                        const int ev = queue[qn + (lane < n ? lane : 0)];
+                        const int k = kb + (ev >> 10) * (TT * 32) + (ev & 0x3E0) + ((ev & 7) << 2) + ((ev >> 3) & 3);
+                        const int x0 = (int)__ldg(c0 + k), x1 = (int)__ldg(c1 + k);
+                        int r = (int)__ldg(rank_g + min(x0 * n1p + x1, n_cells - 1));
+                        if (lane >= n) r = 0x7FFFFFFF;
+                        const int rej = r < rho ? 1 : 0;
+                        r_acc += rej;
+                        x0_acc += rej ? x0 : 0;
+                        x1_acc += rej ? x1 : 0;
+                        if (ks >= 1) {
+                            if (lane < n) {
+                                // WORDS: the trial by its place among the warp's (below 2^17)
+                                if (WORDS)
+                                    kbuf[wk + lane] =
+                                        (Key)(((uint32_t)r << 17) |
+                                              (uint32_t)(((st & ~63) + (ev >> 10)) * 1024 + ((k - kb) & 1023)));
+                                else kbuf[wk + lane] = (Key)r;
+                                atomicAdd(&hist[r >> bin_shift], 1u);
+                            }
+                            wk += n;
+                        }
+                        __syncwarp();   // the queue's entries read before the next round writes
+                    }
+                } while (done < total);
+            }
+            if (ks < 1) break;
+            if (lane == 0) s_nk[g][warp] = wk;
+            tile_sync<TT, G>(g);
+            int nk = 0;
+#pragma unroll
+            for (int w2 = 0; w2 < NW; ++w2) nk += s_nk[g][w2];
+            if (nk < ks && !all) {   // fewer candidates than k_i: again further out
+                for (int b = lt; b < 256; b += TT) hist[b] = 0u;
+                cap += 0.5f;
+                r_acc = x0_acc = x1_acc = 0;
+                tile_sync<TT, G>(g);
+                continue;
+            }
+            // the ks-th smallest rank: its bin, then the rank within the bin
+            auto key_rank = [&](int k) { return (uint32_t)kbuf[k] >> (WORDS ? 17 : 0); };
+            auto key_word = [&](int k) {
+                const int at = (int)((uint32_t)kbuf[k] & 0x1FFFFu);
+                return W[(at >> 10) * (TT * 32) + warp * 1024 + (at & 1023)];
+            };
+            if (warp == 0) {
+                int before = 0;
+                const int b = warp_pick256<true>(hist, ks, lane, &before);
+                if (lane == 0) {
+                    s_pick[g] = b;
+                    s_before[g] = before;
+                }
+            }
+            tile_sync<TT, G>(g);
+            const int B = s_pick[g], kr = ks - s_before[g];
+            for (int k = lane; k < wk; k += 32) {
+                const uint32_t r = key_rank(k);
+                if ((int)(r >> bin_shift) == B) atomicAdd(&hist[r & ((1u << bin_shift) - 1u)], 1u);
+            }
+            tile_sync<TT, G>(g);
+            if (warp == 0) {
+                int before = 0;
+                const int b = warp_pick256<true>(hist, kr, lane, &before);
+                if (lane == 0) {
+                    s_pick[g] = (B << bin_shift) + b;
+                    s_before[g] = kr - before;   // order of the ks-th trial among the rank's trials
+                }
+            }
+            tile_sync<TT, G>(g);
+            const int rstar = s_pick[g], mrem = s_before[g];
+            const float lam = vor_g[rstar];
+            lam_i = (double)lam;
+            if (!all && !(lam <= cap)) {   // a trial left out might be smaller: again further out
+                cap += 0.5f;
+                r_acc = x0_acc = x1_acc = 0;
+                tile_sync<TT, G>(g);
+                continue;
+            }
+            if (WORDS) {
+                // the mrem-th smallest word among the trials of rank rstar
+                for (int k = lane; k < wk; k += 32)
+                    if ((int)key_rank(k) == rstar) {
+                        const int at = atomicAdd(&s_nlist[g], 1);
+                        if (at < kList) list[at] = key_word(k);
+                    }
+                tile_sync<TT, G>(g);
+                const int nl = s_nlist[g];
+                if (nl <= kList) {
+                    for (int j = lt; j < nl; j += TT) {
+                        const uint32_t w = list[j];
+                        int rank = 0;
+                        for (int q = 0; q < nl; ++q) {
+                            const uint32_t u = list[q];
+                            rank += (u < w || (u == w && q < j)) ? 1 : 0;
+                        }
+                        if (rank == mrem - 1) s_res[g] = w;
+                    }
+                    tile_sync<TT, G>(g);
+                } else {   // radix select over the rank's words: four 8-bit digits
+                    uint32_t prefix = 0u, pmask = 0u;
+                    int kq = mrem;
+                    for (int sh = 24; sh >= 0; sh -= 8) {
+                        for (int k = lane; k < wk; k += 32)
+                            if ((int)key_rank(k) == rstar) {
+                                const uint32_t w = key_word(k);
+                                if ((w & pmask) == prefix) atomicAdd(&hist[(w >> sh) & 0xFFu], 1u);
+                            }
+                        tile_sync<TT, G>(g);
+                        if (warp == 0) {
+                            int before = 0;
+                            const int digit = warp_pick256<true>(hist, kq, lane, &before);
+                            if (lane == 0) {
+                                s_pick[g] = digit;
+                                s_before[g] = before;
+                            }
+                        }
+                        tile_sync<TT, G>(g);
+                        prefix |= (uint32_t)s_pick[g] << sh;
+                        pmask |= 0xFFu << sh;
+                        kq -= s_before[g];
+                    }
+                    if (lt == 0) s_res[g] = prefix;
+                    tile_sync<TT, G>(g);
+                }
+                c_i = s_res[g];
+            }
+            break;
+        }
+        r_acc = tail_warp_sum(r_acc);
+        x0_acc = tail_warp_sum(x0_acc);
+        x1_acc = tail_warp_sum(x1_acc);
+        if (lane == 0) {
+            s_red[g][0][warp] = r_acc;
+            s_red[g][1][warp] = x0_acc;
+            s_red[g][2][warp] = x1_acc;
+        }
+        tile_sync<TT, G>(g);
+        if (lt < d) {   // lane a: arm a's outputs, lane 0 the tile's
+            int64_t Rt = 0, X = 0;
+            for (int w2 = 0; w2 < NW; ++w2) {
+                Rt += s_red[g][0][w2];
+                X += s_red[g][1 + lt][w2];
+            }
+            if (o.Xrej) o.Xrej[i * d + lt] = X;
+            if (o.score) {
+                const double sg = bad ? NAN : o.sig[lt == 0 ? a0 : a1];
+                o.score[i * d + lt] = (double)X - (double)n_max * sg * (double)Rt;
+            }
+            if (lt == 0) {
+                if (bad) atomicOr(err, CSE_ERR_BAD_K);
+                if (o.R) o.R[i] = Rt;
+                if (o.cp_key)   // the tile's (K, R) in the Clopper-Pearson memo, as k_cp_mark would
+                    o.cp_slot[i] = cp_memo_insert(((unsigned long long)(uint32_t)K << 32) | (uint32_t)Rt, o.cp_key,
+                                                  o.cp_cap, o.cp_list, o.cp_nkeys);
+                o.lam_tile[i] = lam_i;
+                s_min[g] = min(s_min[g], order_key(lam_i));
+                if (WORDS && c_tile) c_tile[i] = c_i;
+            }
+        }
+        tile_sync<TT, G>(g);
+    }
+    __syncthreads();   // every group done before the queue is reset
+    unsigned long long mine = ~0ull;
+    if (tid == 0)
+        for (int q = 0; q < G; ++q) mine = min(mine, s_min[q]);
+    queue_reset_min(counter, o.min_key, mine, o.min_out);
+}
+
+template <bool WORDS, int G>
+int launch_tail(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                uint32_t* c_tile, cudaStream_t s)
+{
+    auto kern = k_sim_tail<WORDS, G>;
+    constexpr int TT = kTailThreads / G, NW = TT / 32;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTailThreads, 0) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
+    int64_t grid = (int64_t)per_sm * c->num_sms;
+    const int64_t blocks = (T.n_tiles + G - 1) / G;
+    if (grid > blocks) grid = blocks;
+    // a warp's keys: its 1,024 trials of every step
+    const int32_t key_seg = (K_tiles + TT * 32 - 1) / (TT * 32) * 1024;
+    const size_t need = sizeof(typename tail_key<WORDS>::type) * (size_t)grid * G * NW * (size_t)key_seg;
+    if (need > c->keys_cap) {
+        cudaFree(c->keys);
+        c->keys = nullptr;
+        c->keys_cap = 0;
+        if (cudaMalloc(&c->keys, need) != cudaSuccess) {
+            cudaGetLastError();
+            return CSE_OOM;
+        }
+        c->keys_cap = need;
+    }
+    int sh = 0;   // ranks per bin: at most 256 bins, at most 128 ranks a bin (n_cells <= 129^2)
+    while (((c->n_cells - 1) >> sh) > 255) ++sh;
+    if (o.min_out) c->min_folded = true;
+    if (o.cp_key) c->cp_marked = true;
+    cse_prof_begin(c, KID_SIM_ZTEST, s);
+    cse_launch(c->pdl, kern, dim3((unsigned)grid), dim3(kTailThreads), 0, s, T, c->D.n_max, c->cnt, NA, k_stride,
+               K_tiles, c->rank_tab, c->S_tab, c->val_of_rank, c->n_cells, c->n1p, sh, c->bb, c->zpar,
+               c->z_lambda, c->tb, o, c_tile, c->keys, key_seg, c->counter, c->err);
+    cse_prof_end(c, s);
+    c->launches += 1;
+    return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+template <bool WORDS>
+int launch_groups(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                  uint32_t* c_tile, cudaStream_t s)
+{
+    // (wider groups for the largest K: the keys of a launch stay below 1 GB, a trial's
+    // place within a warp below 2^17)
+    const int64_t key_bytes = (int64_t)K_tiles * (WORDS ? 4 : 2);
+    if (T.n_tiles < 8 * (int64_t)c->num_sms || K_tiles > (1 << 18))
+        return launch_tail<WORDS, 1>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    if (T.n_tiles < 32 * (int64_t)c->num_sms || key_bytes > (1 << 17))
+        return launch_tail<WORDS, 2>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    return launch_tail<WORDS, 8>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+}
+
+// Rejections alone: a group of TT threads per tile, sixteen trials a thread and step.
+template <bool TWO, int TT>
+__global__ void __launch_bounds__(256)
+    k_sim_count(TileArgs T, int32_t n_max, const uint8_t* __restrict__ cnt, int32_t NA, int32_t k_stride,
+                int32_t K_tiles, const uint8_t* __restrict__ zcut, SimOut o, int32_t* __restrict__ err)
+{
+    pdl_entry();
+    constexpr int NW = TT / 32, G = 256 / TT, d = TWO ? 2 : 1;
+    __shared__ int s_red[G][3][NW];
+    const int tid = threadIdx.x, lane = tid & 31, g = tid / TT, lt = tid - g * TT, warp = lt >> 5;
+    const uint32_t b1 = TWO ? 0u : (uint32_t)zcut[0] * 0x01010101u;
+    for (int64_t i0 = (int64_t)blockIdx.x * G; i0 < T.n_tiles; i0 += (int64_t)gridDim.x * G) {   // block-uniform
+        const int64_t i = i0 + g;
+        const bool live = i < T.n_tiles;
+        const int K = live ? T.K[i] : 0;
+        const int v0 = live ? T.center_idx[i * d] : 0, v1 = (TWO && live) ? T.center_idx[i * d + 1] : 0;
+        // device-side argument checks: K_i in [1, K_max of the set], axis indices in range
+        const bool bad = (K < 1) || (K > K_tiles) || v0 < 0 || v0 >= T.n_axis[0] ||
+                         (TWO && (v1 < 0 || v1 >= T.n_axis[1]));
+        const int Kc = bad ? 0 : K;
+        const int a0 = T.axis_off[0] + (bad ? 0 : v0), a1 = TWO ? T.axis_off[1] + (bad ? 0 : v1) : a0;
+        const uint8_t* const c0 = cnt + (int64_t)a0 * k_stride;
+        const uint8_t* const c1 = cnt + (int64_t)a1 * k_stride;   // the tested row
+        const uint8_t* const cb = c0 + (int64_t)NA * k_stride;    // b(x_0) (two arms)
+        uint32_t R = 0u, X0 = 0u, X1 = 0u;
+#pragma unroll 2
+        for (int k = lt * 16; k < Kc; k += TT * 16) {
+            const uint4 x = *reinterpret_cast<const uint4*>(c1 + k);
+            uint4 y = make_uint4(0u, 0u, 0u, 0u), b = make_uint4(b1, b1, b1, b1);
+            if (TWO) {
+                y = *reinterpret_cast<const uint4*>(c0 + k);
+                b = *reinterpret_cast<const uint4*>(cb + k);
+            }
+            const uint32_t xw[4] = {x.x, x.y, x.z, x.w}, yw[4] = {y.x, y.y, y.z, y.w}, bw[4] = {b.x, b.y, b.z, b.w};
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                uint32_t m = ((xw[q] - bw[q] + 0x80808080u) >> 7) & 0x01010101u;   // one per rejecting trial
+                const int rem = Kc - k - 4 * q;
+                if (rem < 4) m &= rem > 0 ? (1u << (8 * rem)) - 1u : 0u;
+                const uint32_t full = m * 255u;
+                R = __dp4a(m, 0x01010101u, R);
+                X1 = __dp4a(xw[q] & full, 0x01010101u, X1);
+                if (TWO) X0 = __dp4a(yw[q] & full, 0x01010101u, X0);
+            }
+        }
+        const int r = tail_warp_sum((int)R), x1 = tail_warp_sum((int)X1), x0 = TWO ? tail_warp_sum((int)X0) : x1;
+        if (lane == 0) {
+            s_red[g][0][warp] = r;
+            s_red[g][1][warp] = x0;
+            s_red[g][2][warp] = x1;
+        }
+        if (TT == 32) __syncwarp();
+        else __syncthreads();
+        if (live && lt < d) {   // lane a: arm a's outputs, lane 0 the tile's
+            int64_t Rt = 0, X = 0;
+            for (int w2 = 0; w2 < NW; ++w2) {
+                Rt += s_red[g][0][w2];
+                X += s_red[g][1 + lt][w2];
+            }
+            if (lt == 0) {
+                if (bad) atomicOr(err, CSE_ERR_BAD_K);
+                if (o.R) o.R[i] = Rt;
+            }
+            if (o.Xrej) o.Xrej[i * d + lt] = X;
+            if (o.score) {
+                const double sg = bad ? NAN : o.sig[lt == 0 ? a0 : a1];
+                o.score[i * d + lt] = (double)X - (double)n_max * sg * (double)Rt;
+            }
+        }
+        if (TT == 32) __syncwarp();
+        else __syncthreads();
+    }
+}
+
+template <bool TWO, int TT>
+int launch_count(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                 cudaStream_t s)
+{
+    auto kern = k_sim_count<TWO, TT>;
+    constexpr int G = 256 / TT;
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, 0) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
+    // blocks in turn over the tiles: several rounds each, so that ragged K evens out
+    int64_t grid = (T.n_tiles + G - 1) / G;
+    if (grid > 8 * (int64_t)per_sm * c->num_sms) grid = 8 * (int64_t)per_sm * c->num_sms;
+    cse_prof_begin(c, KID_SIM_ZTEST, s);
+    cse_launch(c->pdl, kern, dim3((unsigned)grid), dim3(256), 0, s, T, c->D.n_max, c->cnt, NA, k_stride, K_tiles,
+               c->zcut, o, c->err);
+    cse_prof_end(c, s);
+    c->launches += 1;
+    return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+}  // namespace
+
+int cse_launch_sim_count(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                         cudaStream_t s)
+{
+    // a warp per tile once every resident warp has one, else a block of 256
+    const bool many = T.n_tiles >= 32 * (int64_t)c->num_sms;
+    if (c->D.stat == CSE_STAT_TWO_ARM_POOLED_Z)
+        return many ? launch_count<true, 32>(c, T, NA, k_stride, K_tiles, o, s)
+                    : launch_count<true, 256>(c, T, NA, k_stride, K_tiles, o, s);
+    return many ? launch_count<false, 32>(c, T, NA, k_stride, K_tiles, o, s)
+                : launch_count<false, 256>(c, T, NA, k_stride, K_tiles, o, s);
+}
+
+int cse_launch_sim_tail(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
+                        bool words, uint32_t* c_tile, cudaStream_t s)
+{
+    return words ? launch_groups<true>(c, T, NA, k_stride, K_tiles, o, c_tile, s)
+                 : launch_groups<false>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+}

@@ -111,10 +111,43 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
     }
 }
 
-// Success threshold and sigmoid (for the score's grad A) of every axis value.
-__global__ void k_thresholds(uint32_t* __restrict__ thr, double* __restrict__ sig, TileArgs T, int32_t n_total)
+// Success threshold and sigmoid (for the score's grad A) of every axis value.  With
+// Z.S set (z-test calls that do not run the cell histogram) the last block finds
+// the call's constants: the number of cells with S < lambda (Z.pos) or per x_0 the least x_1 with S < lambda (n_max + 1: none; each row of S falls in x_1).
+struct TailArgs {
+    const float* S;
+    int32_t n_cells, n1p, n_max;   // row length n1p: n_max + 1, or 1 for one arm
+    float lambda_up;
+    const int32_t* pos;   // the cells sorted by S, or NULL
+    int32_t* zpar;
+    uint8_t* zcut;        // or NULL
+};
+
+__global__ void __launch_bounds__(256) k_thresholds(uint32_t* __restrict__ thr, double* __restrict__ sig, TileArgs T,
+                                                    int32_t n_total, TailArgs Z)
 {
     pdl_entry();
+    if (Z.S && blockIdx.x == gridDim.x - 1) {
+        if (Z.pos) {   // the sorted cells (pos): the block's threads search in two rounds
+            const int step = (Z.n_cells + (int)blockDim.x - 1) / (int)blockDim.x;
+            auto below = [&](int p) { return p < Z.n_cells && Z.S[Z.pos[p]] < Z.lambda_up; };
+            const int c1 = __syncthreads_count(below(threadIdx.x * step));   // positions 0, step, ... below lambda
+            const int base = c1 > 0 ? (c1 - 1) * step + 1 : 0;
+            const int c2 = __syncthreads_count(c1 > 0 && (int)threadIdx.x < step - 1 && below(base + threadIdx.x));
+            if (threadIdx.x == 0) Z.zpar[0] = base + c2;
+        }
+        if (Z.zcut && threadIdx.x < (Z.n1p > 1 ? Z.n1p : 1)) {
+            const float* row = Z.S + threadIdx.x * Z.n1p;   // one arm: the table itself is the row
+            int lo = 0, hi = Z.n_max + 1;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (row[mid] < Z.lambda_up) hi = mid;
+                else lo = mid + 1;
+            }
+            Z.zcut[threadIdx.x] = (uint8_t)lo;
+        }
+        return;
+    }
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= n_total) return;
     threshold_of(i, thr, sig, T);
@@ -484,8 +517,18 @@ int cse_launch_tables(cse_ctx* c, cudaStream_t s)
 
 int cse_launch_thresholds(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, cudaStream_t s)
 {
+    TailArgs Z = {};
+    if (c->zmode != ZMODE_CELLS)
+        Z = {c->S_tab, c->n_cells, c->n1p, c->D.n_max, c->z_lambda, nullptr, nullptr, nullptr};
+    if (c->zmode == ZMODE_TAIL) {
+        Z.pos = c->cell_of_pos;
+        Z.zpar = c->zpar;
+    } else {
+        Z.zcut = c->zcut;
+    }
     cse_prof_begin(c, KID_THRESHOLDS, s);
-    cse_launch(c->pdl, k_thresholds, dim3((n_axis_total + 255) / 256), dim3(256), 0, s, c->thr, c->sig, T, n_axis_total);
+    cse_launch(c->pdl, k_thresholds, dim3((n_axis_total + 255) / 256 + (Z.S ? 1 : 0)), dim3(256), 0, s, c->thr, c->sig,
+               T, n_axis_total, Z);
     cse_prof_end(c, s);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
@@ -531,6 +574,8 @@ int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, 
 {
     if (cse_count_nibbles(c)) return launch_counts<3, kCountsNib>(c, T, n_axis_total, K_tiles, k_stride, c->bt_score, s);
     if (c->D.n_looks > 1) return launch_counts<3, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
+    if (c->zmode == ZMODE_COUNT && T.d == 2)
+        return launch_counts<1, kCountsMapped>(c, T, n_axis_total, K_tiles, k_stride, c->zcut, s);
     return launch_counts<1, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
 }
 
