@@ -616,6 +616,7 @@ int cse_destroy(cse_ctx* c)
     cudaFree(c->bt_score);
     cudaFree(c->bt_f4);
     cudaFree(c->bk_q);
+    cudaFree(c->bk_bits);
     cudaFree(c->keys);
     cudaFree(c->counter);
     cudaFree(c->err);

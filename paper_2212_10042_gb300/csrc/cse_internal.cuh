@@ -292,6 +292,13 @@ __device__ __forceinline__ int warp_pick256(uint32_t* counts, int ks, int lane, 
     return __shfl_sync(0xffffffffu, lane * 8 + b, src);
 }
 
+// Bin of a key (S >= 0 as bits) in a 256-bin histogram: sixteen bins an
+// octave from 2^-16 up, the ends clamped.  Monotone in S.
+__device__ __forceinline__ int key_bin(uint32_t key)
+{
+    return min(max((int)(key >> 19) - (int)(0x37800000u >> 19), 0), 255);
+}
+
 // Bits 8 j + q of a candidate word for trials 4 q + j < rem (rem > 0).
 __device__ __forceinline__ uint32_t trials_below(int rem)
 {
@@ -456,6 +463,8 @@ struct cse_ctx {
     int32_t bt_top;         //   final plane holds scores (strictly rising with the count)
     uint32_t* bt_dmin;      // least final S per (counted treatment - control) score difference (float bits)
     float4* bt_f4;          // final-analysis P(theta_self > theta_0) of the three treatments per sorted code triple
+    uint2* bk_bits;         // basket design: a bit per count state and arm, Q_i below each level of S; the last
+                            // level is the call's lambda (k_basket_bits)
     float4* bk_q;           // basket design: (1 - P(theta_i > t_i | x)) per count state (see sim_basket.cu)
     uint32_t* keys;         // per-CTA statistic keys for order-statistic selection
     size_t keys_cap;

@@ -11,13 +11,11 @@
 //
 // The posterior depends on a trial only through its four success counts, so the
 // context tabulates Q_i = 1 - P_i in FP32 over all (n + 1)^4 count states once
-// (a float4 per state, 27 MB for n = 35, L2-resident).  A simulated trial then
-// costs four count-byte reads (coalesced) and one 16-byte gather.  The direct
-// mode (plain path) evaluates the same FP32 function per trial instead.
+// (a float4 per state, 27 MB for n = 35, L2-resident) and, from it, the trials
+// that cannot decide anything (k_sim_basket).  The direct mode (plain path)
+// evaluates the same FP32 function for every trial instead.
 #include <cuda_runtime.h>
 #include <math.h>
-
-#include <type_traits>
 
 #include "cse_internal.cuh"
 
@@ -25,7 +23,7 @@ namespace {
 
 constexpr int BT = 256;          // threads of the simulation kernel
 constexpr int BWARP = BT / 32;
-constexpr int SPT = 8;           // consecutive sims per thread and step (one 8-byte count load per arm)
+constexpr int SPT = 8;           // direct mode: consecutive sims per thread and step (one 8-byte count load per arm)
 
 struct Basket {
     int n;        // patients per arm
@@ -133,17 +131,510 @@ __device__ __forceinline__ int basket_warp_sum(int v)
     return v;
 }
 
-// Persistent: each CTA takes tiles from the work queue; the tile's K sims are
-// spread over the block, SPT consecutive sims per thread and step, their eight
-// gathers issued before any is used.  SELECT adds the per-tile order statistic
-// lambda_i = S_(ksel_i) by a three-digit radix select (11, 11, 10 bits of the
-// FP32 keys, which order like the non-negative S) over the keys the CTA stored.
-template <bool TABLE, bool SELECT>
-__global__ void __launch_bounds__(BT, 4) k_sim_basket(TileArgs T, Basket B, const uint8_t* __restrict__ cnt,
-                                                      int32_t k_stride, int32_t K_tiles,
-                                                      const float4* __restrict__ Qt, float lambda_up, SimOut o,
-                                                      uint32_t* __restrict__ keys, int32_t* __restrict__ counter,
-                                                      int32_t* __restrict__ err)
+// One thread: the tile's outputs from the warps' sums.
+__device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B, const SimOut& o, int64_t i, int K,
+                                             bool bad, const int* v, const int (*red)[BWARP], int warps, bool select, double lam_i,
+                                             int32_t* err)
+{
+    if (bad) atomicOr(err, CSE_ERR_BAD_K);
+    int64_t Rt = 0, X[4] = {0, 0, 0, 0};
+    for (int w = 0; w < warps; ++w) {
+        Rt += red[0][w];
+        for (int a = 0; a < 4; ++a) X[a] += red[1 + a][w];
+    }
+    if (o.R) o.R[i] = Rt;
+    if (o.cp_key)   // the tile's (K, R) in the Clopper-Pearson memo, as k_cp_mark would
+        o.cp_slot[i] = cp_memo_insert(((unsigned long long)(uint32_t)K << 32) | (uint32_t)Rt, o.cp_key, o.cp_cap,
+                                      o.cp_list, o.cp_nkeys);
+    for (int a = 0; a < 4; ++a) {
+        if (o.Xrej) o.Xrej[i * 4 + a] = X[a];
+        if (o.score) {
+            const double sg = bad ? NAN : o.sig[T.axis_off[a] + v[a]];
+            o.score[i * 4 + a] = (double)X[a] - (double)B.n * sg * (double)Rt;
+        }
+    }
+    if (select && o.lam_tile) o.lam_tile[i] = lam_i;
+}
+
+// ---------------------------------------------------------------------------
+// The tabulated simulation: counting by bits, evaluating only the trials that can
+// decide the order statistic.
+//
+// A 16-byte gather from the state table touches a line of L1 per trial, and L1
+// looks up one line a clock: one clock a trial and SM whatever else the kernel does
+// (3.1 of the 3.67 ms of the 16^4 grid at K = 2^14).  Whether a trial rejects, and
+// whether it can be among the k_i smallest S, is a bit of its count state.  Before
+// the launch k_basket_bits packs "Q_a < lambda" over all states, a bit per x_3 in a
+// word per (arm, x_0, x_1, x_2); the context keeps the same for kLevels fixed levels
+// of S.  A tile takes the states within kWindow standard deviations of its expected
+// counts (w_a counts of arm a), ORs the words of its null arms and puts them in
+// shared memory: w_0 w_1 w_2 words (~2,000), against K trials that each read one.
+// A trial's four counts are the bytes of one word P (byte transposes); two additions
+// and a mask tell whether all lie in the window, a dot product and a multiply-add
+// give its word, and the rotation by P brings its bit to the top.  The sign bits of
+// four trials become a byte mask, and one dot product per arm adds their counts.
+//
+// Evaluated from the state table, queued per warp and 32 at a time: trials outside
+// the window (4 in a hundred) and, with a selection, those below the tile's level L_c,
+// the least one above the k_i smallest S as far as the first kSample trials (all
+// evaluated) tell, with a margin of 2.5 standard deviations.  Keys below L_c go to
+// the warp's stretch of global memory and into 256 bins; the k_i-th is ranked within
+// its bin.  It is exact when it is at most L_c; otherwise the pass is repeated with
+// every trial evaluated.
+//
+// What bounds it: issue slots (65 %) and the integer pipe (64 %): per 32 trials ~17
+// warp instructions of test and count, ~10 of queue and scan, ~7 of evaluation, and
+// ~20 of the tile's own work (building the window, setup, selection).  16^4 grid,
+// K = 2^14, with a selection (59,992 tiles): 3.67 -> 1.98 ms; 6,036 tiles of 1,000 to
+// 30,000 trials without one: 152 -> 112 us, plus 10 for the bits of lambda.  Measured
+// on the way: one bit per state at a fixed level and every rejection evaluated 3.28 ms
+// (the candidates' own work), lambda's and the level's bits in separate words 2.58,
+// in one 2.34; 128 threads a tile instead of 256 1.98 (more tiles in flight to cover
+// the window's loads and the barriers).
+// ---------------------------------------------------------------------------
+constexpr int kLevels = 32;        // levels of S for selections: 2^((c + 1) / 4 - 8), the last +inf
+constexpr int kMaxM = 64;          // count states of an arm: two 32-bit words of x_3
+constexpr int NT = 128;            // threads of the tabulated kernel
+constexpr int kSample = 512;       // first trials of a tile, all evaluated to place c
+// up to this K every trial is evaluated: below it the window (a few thousand words, 50 instructions
+// a word) and the bits of lambda cost more than the evaluations they save
+constexpr int kAllK = 2048;
+constexpr int kQueue = 288;        // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
+constexpr int kList = 256;         // keys of the selected bin ranked in shared memory
+constexpr float kWindow = 2.6f;    // half-width of the window in standard deviations
+
+__host__ __device__ inline float basket_level(int c)
+{
+    return c >= kLevels - 1 ? INFINITY : exp2f(0.25f * (float)(c + 1) - 8.0f);
+}
+
+// most counts of an arm in the window (p = 1/2; of arm 3 at most 16, the bits of half a word)
+inline int basket_span(int n)
+{
+    const int w = (int)(kWindow * sqrtf((float)n)) + 2;
+    return w < n + 1 ? w : n + 1;
+}
+
+// bits[(l 4 + a) rows + row] of levels l = first .. first + count - 1: bit 31 - (x_3 & 31) of half
+// x_3 >> 5 is Q_a(row, x_3) < level (lambda_up for l = kLevels).  A warp per row: the table's row is
+// read once for all arms and levels: bound by its loads (the lambda level of n = 35: 10 us, 27 MB read).
+__global__ void __launch_bounds__(256) k_basket_bits(uint2* __restrict__ bits, const float4* __restrict__ Qt, int m,
+                                                     int rows, int first, int count, float lambda_up)
+{
+    const int row = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (row >= rows) return;
+    const int x0 = 31 - lane, x1 = 63 - lane;
+    const float4 none = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+    const float4 q0 = x0 < m ? __ldg(Qt + (int64_t)row * m + x0) : none;
+    const float4 q1 = x1 < m ? __ldg(Qt + (int64_t)row * m + x1) : none;
+    for (int l = first; l < first + count; ++l) {
+        const float lev = l == kLevels ? lambda_up : basket_level(l);
+        const uint32_t b[8] = {__ballot_sync(0xffffffffu, q0.x < lev), __ballot_sync(0xffffffffu, q1.x < lev),
+                               __ballot_sync(0xffffffffu, q0.y < lev), __ballot_sync(0xffffffffu, q1.y < lev),
+                               __ballot_sync(0xffffffffu, q0.z < lev), __ballot_sync(0xffffffffu, q1.z < lev),
+                               __ballot_sync(0xffffffffu, q0.w < lev), __ballot_sync(0xffffffffu, q1.w < lev)};
+        if (lane < 4) {
+            uint2 h = make_uint2(b[0], b[1]);
+            if (lane == 1) h = make_uint2(b[2], b[3]);
+            if (lane == 2) h = make_uint2(b[4], b[5]);
+            if (lane == 3) h = make_uint2(b[6], b[7]);
+            bits[((int64_t)l * 4 + lane) * rows + row] = h;
+        }
+    }
+}
+
+// Bits 31 .. 32 - s cleared (s in 0 .. 32).
+__device__ __forceinline__ uint32_t bits_from(int s) { return s >= 32 ? 0u : 0xFFFFFFFFu >> s; }
+
+// Bits 31 (HIGH) or 15 of f[0..3] as bytes 0xFF / 0x00 (prmt's replicated sign: selector bit 3).
+template <bool HIGH>
+__device__ __forceinline__ uint32_t sign_bytes(const uint32_t* f)
+{
+    uint32_t a, b;
+    if (HIGH) {
+        asm("prmt.b32 %0, %1, %2, 0x00FB;" : "=r"(a) : "r"(f[0]), "r"(f[1]));
+        asm("prmt.b32 %0, %1, %2, 0xFB00;" : "=r"(b) : "r"(f[2]), "r"(f[3]));
+    } else {
+        asm("prmt.b32 %0, %1, %2, 0x00D9;" : "=r"(a) : "r"(f[0]), "r"(f[1]));
+        asm("prmt.b32 %0, %1, %2, 0xD900;" : "=r"(b) : "r"(f[2]), "r"(f[3]));
+    }
+    return __byte_perm(a, b, 0x7610);
+}
+
+// The window's bits of a row, x_3 = lo .. hi - 1 (at most 16), at 15 - (x_3 & 15): m[j] selects the
+// window's part of states 16 j .. 16 j + 15.
+__device__ __forceinline__ uint32_t fold16(const uint2& h, const uint2& mk)
+{
+    const uint32_t t = (h.x & mk.x) | (h.y & mk.y);
+    return (t | (t >> 16)) & 0xFFFFu;
+}
+
+template <bool SELECT>
+__global__ void __launch_bounds__(NT, 8)
+    k_sim_basket(TileArgs T, Basket B, const uint8_t* __restrict__ cnt, int32_t k_stride, int32_t K_tiles,
+                 const float4* __restrict__ Qt, const uint2* __restrict__ planes, int32_t span, float lambda_up,
+                 bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg, int32_t* __restrict__ counter,
+                 int32_t* __restrict__ err)
+{
+    constexpr int NW = NT / 32;
+    constexpr int ALL = kLevels - 1;   // every trial evaluated
+    // word 0: a trial outside the window (evaluated, not counted); then w_0 w_1 w_2 words: lambda's bits
+    // in the upper half, those of the level in the lower
+    extern __shared__ uint32_t bits[];
+    __shared__ uint16_t s_queue[NW][kQueue];
+    __shared__ uint32_t hist[SELECT ? 256 : 1];
+    __shared__ uint32_t list[SELECT ? kList : 1];
+    __shared__ int s_tile, s_next, s_pick, s_before, s_nlist, s_nk[NW];
+    __shared__ uint32_t s_res;
+    __shared__ int s_red[5][BWARP];
+    __shared__ unsigned long long s_min;   // order key of the least lambda_i of this CTA's tiles
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    uint16_t* const queue = s_queue[warp];
+    // each warp appends its keys to its own stretch of key_seg words
+    uint32_t* const kbuf = keys + ((int64_t)blockIdx.x * NW + warp) * key_seg;
+    const unsigned below = (1u << lane) - 1u;
+    const int m = B.m;
+    if (SELECT)
+        for (int b = tid; b < 256; b += NT) hist[b] = 0u;
+    if (tid == 0) {
+        s_min = ~0ull;
+        s_next = atomicAdd(counter, 1);
+        bits[0] = 0xFFFFu;
+    }
+
+    for (;;) {
+        __syncthreads();
+        if (tid == 0) {
+            s_tile = s_next;
+            s_nlist = 0;
+        }
+        __syncthreads();
+        const int64_t i = s_tile;
+        if (i >= T.n_tiles) break;
+        if (tid == 0) s_next = atomicAdd(counter, 1);   // the next tile, fetched while this one runs
+        const int K = T.K[i];
+        // each lane one arm's index and window, then shared: counts lo .. lo + w - 1, within 0 .. n
+        const int la = lane & 3;
+        const int vl = T.center_idx[i * 4 + la];
+        int na = T.n_axis[0], ao = T.axis_off[0];
+#pragma unroll
+        for (int a = 1; a < 4; ++a)   // by selection: no runtime index into the argument
+            if (la == a) na = T.n_axis[a], ao = T.axis_off[a];
+        const bool bad = __any_sync(0xffffffffu, vl < 0 || vl >= na) || K < 1 || K > K_tiles;
+        const int atl = ao + (bad ? 0 : vl);
+        const float pl = bad ? 0.5f : (float)o.sig[atl], mu = (float)B.n * pl;
+        const int wl = min((int)(2.0f * kWindow * sqrtf(mu * (1.0f - pl))) + 2, la == 3 ? min(span, 16) : span);
+        const int ll = min(max((int)(mu + 0.5f - 0.5f * (float)(wl - 1)), 0), m - wl);
+        const uint32_t mask = T.null_mask[i] & 15u;   // null arms (none: S = +inf throughout)
+        const int Kc = (bad || mask == 0u) ? 0 : K;
+        const uint8_t* rowp[4];
+        int lo[4], w[4], v[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+            v[a] = __shfl_sync(0xffffffffu, vl, a);
+            rowp[a] = cnt + (int64_t)__shfl_sync(0xffffffffu, atl, a) * k_stride;
+            w[a] = __shfl_sync(0xffffffffu, wl, a);
+            lo[a] = __shfl_sync(0xffffffffu, ll, a);
+        }
+        const int ks = (SELECT && !bad) ? o.ksel[i] : 0;
+        const bool sel = SELECT && ks >= 1;
+        // A selection starts with a sample, every trial of it evaluated.  c: the level of the
+        // trials to come (-1: none is needed)
+        bool sample = sel && Kc > kAllK;
+        int c = (sel || Kc <= kAllK) ? ALL : -1;
+        int r_neg = 0, x_neg[4] = {0, 0, 0, 0};   // minus the rejections and their counts
+        double lam_i = -INFINITY;
+        for (;;) {
+            int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
+            const int k0 = sample ? kSample : 0;
+            bool built = false;   // the window's bits are those of c
+            // bytes of P: x_3, x_2, x_1, x_0.  C1: bit 7 of a byte set iff x >= lo; C2: iff
+            // x >= lo + w (bytes up to 127: no carry)
+            const uint32_t C1 = 0x80808080u - (uint32_t)(lo[3] | (lo[2] << 8) | (lo[1] << 16) | (lo[0] << 24));
+            const uint32_t C2 = C1 - (uint32_t)(w[3] | (w[2] << 8) | (w[1] << 16) | (w[0] << 24));
+            // byte address of a trial's word: 4 ((x_0 w_1 + x_1) w_2 + x_2) + base
+            const uint32_t W0 = 4u * (uint32_t)(w[1] * w[2]), WD = (4u << 8) | ((uint32_t)(4 * w[2]) << 16);
+            const uint32_t base = 4u - 4u * (uint32_t)((lo[0] * w[1] + lo[1]) * w[2] + lo[2]);
+            float level = c < 0 ? 0.0f : basket_level(c);
+            // one trial a lane
+            auto eval = [&](int k, bool live) {
+                int x[4];
+                bool count = c == ALL;   // a rejection inside the window is counted by its bit
+#pragma unroll
+                for (int a = 0; a < 4; ++a) {
+                    x[a] = min((int)__ldg(rowp[a] + k), B.n);
+                    count |= (uint32_t)(x[a] - lo[a]) >= (uint32_t)w[a];
+                }
+                const float4 q = __ldg(Qt + ((x[0] * m + x[1]) * m + x[2]) * m + x[3]);
+                const float S = live ? masked_min(q, mask) : INFINITY;
+                const int rej = (S < lambda_up && live && count) ? 1 : 0;
+                r_neg -= rej;
+#pragma unroll
+                for (int a = 0; a < 4; ++a) x_neg[a] -= rej ? x[a] : 0;
+                if (sel) {
+                    const bool keep = S < level;
+                    const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                    if (keep) {
+                        kbuf[wk + __popc(kept & below)] = __float_as_uint(S);
+                        atomicAdd(&hist[key_bin(__float_as_uint(S))], 1u);
+                    }
+                    wk += __popc(kept);
+                }
+            };
+            if (sample) {   // the sample, spread over the warps, and the level of the trials to come
+                for (int k = warp * (kSample / NW) + lane; k < (warp + 1) * (kSample / NW); k += 32) eval(k, true);
+                __syncthreads();
+                if (warp == 0) {
+                    // the least level with the keys below it so far, scaled to all K trials and
+                    // less 2.5 standard deviations, reaching k_i
+                    const float f = ((float)Kc - (float)kSample) / (float)kSample, d = 2.5f * sqrtf(f * (1.0f + f));
+                    const float r = (d + sqrtf(d * d + 4.0f * (1.0f + f) * (float)ks)) / (2.0f * (1.0f + f));
+                    int before = 0;
+                    const int b = warp_pick256<false>(hist, (int)ceilf(r * r) + 1, lane, &before);
+                    const bool above = b >= 0 && (lane == ALL || key_bin(__float_as_uint(basket_level(lane))) > b);
+                    const unsigned who = __ballot_sync(0xffffffffu, above);   // a lane a level
+                    if (lane == 0) s_pick = who ? __ffs(who) - 1 : ALL;
+                }
+                __syncthreads();
+                c = s_pick;
+                level = basket_level(c);
+            }
+            // sixteen consecutive trials per thread and step from k0 on
+            for (int st = 0; k0 + st * (NT * 16) < Kc; ++st) {
+                if (c != ALL && !built) {
+                    // a thread a word; its place steps by NT words
+                    const int hi3 = lo[3] + w[3], w12 = w[1] * w[2], rows = w[0] * w12, rm = m * m * m;
+                    const uint2 mk = make_uint2(bits_from(lo[3]) & ~bits_from(min(hi3, 32)),
+                                                bits_from(max(lo[3] - 32, 0)) & ~bits_from(max(hi3 - 32, 0)));
+                    const int d0 = NT / w12, e0 = NT - d0 * w12, d1 = e0 / w[2], d2 = e0 - d1 * w[2];
+                    int y1 = tid % w12, src = tid / w12;
+                    int y2 = y1 % w[2];
+                    y1 /= w[2];
+                    src = ((lo[0] + src) * m + lo[1] + y1) * m + lo[2] + y2;
+                    const int step = (d0 * m + d1) * m + d2, c2 = m - w[2], c1 = (m - w[1]) * m;
+                    const uint2* const pl = planes + (int64_t)kLevels * 4 * rm;
+                    const uint2* const pc = planes + (int64_t)max(c, 0) * 4 * rm;
+#pragma unroll 2
+                    for (int r = tid; r < rows; r += NT) {
+                        uint2 hl = make_uint2(0u, 0u), hc = make_uint2(0u, 0u);
+#pragma unroll
+                        for (int a = 0; a < 4; ++a)
+                            if ((mask >> a) & 1u) {
+                                if (want_R) {
+                                    const uint2 h = __ldg(pl + a * rm + src);
+                                    hl.x |= h.x, hl.y |= h.y;
+                                }
+                                if (SELECT && c >= 0) {
+                                    const uint2 h = __ldg(pc + a * rm + src);
+                                    hc.x |= h.x, hc.y |= h.y;
+                                }
+                            }
+                        bits[1 + r] = (fold16(hl, mk) << 16) | (SELECT ? fold16(hc, mk) : 0u);
+                        y2 += d2, y1 += d1, src += step;
+                        if (y2 >= w[2]) y2 -= w[2], y1 += 1, src += c2;
+                        if (y1 >= w[1]) y1 -= w[1], src += c1;
+                    }
+                    built = true;
+                    __syncthreads();
+                }
+                // first trial of the warp at the start of the queue's block of 64 steps
+                const int kb = k0 + (st & ~63) * (NT * 16) + warp * 512;
+                const int stq = st & 63;
+                const int kw = kb + stq * (NT * 16) + lane * 16;
+                uint32_t cm = 0u;   // bit t: trial kw + t is evaluated
+                if (kw < Kc) {
+                    cm = 0xFFFFu;
+                    if (c != ALL) {
+                        uint32_t A[4][4];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) {   // kw + 16 <= k_stride (a multiple of 16)
+                            const uint4 x = __ldg(reinterpret_cast<const uint4*>(rowp[a] + kw));
+                            A[a][0] = x.x, A[a][1] = x.y, A[a][2] = x.z, A[a][3] = x.w;
+                        }
+                        if (kw + 16 > Kc) {   // trials at or past K: outside the window (lo + w <= 64 < 127)
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                const int left = Kc - kw - 4 * q;
+                                const uint32_t past = left >= 4 ? 0u : left <= 0 ? ~0u : ~0u << (8 * left);
+#pragma unroll
+                                for (int a = 0; a < 4; ++a) A[a][q] = (A[a][q] & ~past) | (0x7F7F7F7Fu & past);
+                            }
+                        }
+                        int cneg = 0;   // minus the candidates' bits
+#pragma unroll
+                        for (int q = 3; q >= 0; --q) {
+                            const uint32_t l01 = __byte_perm(A[3][q], A[2][q], 0x5140);
+                            const uint32_t l23 = __byte_perm(A[3][q], A[2][q], 0x7362);
+                            const uint32_t h01 = __byte_perm(A[1][q], A[0][q], 0x5140);
+                            const uint32_t h23 = __byte_perm(A[1][q], A[0][q], 0x7362);
+                            const uint32_t P[4] = {__byte_perm(l01, h01, 0x5410), __byte_perm(l01, h01, 0x7632),
+                                                   __byte_perm(l23, h23, 0x5410), __byte_perm(l23, h23, 0x7632)};
+                            uint32_t f[4];
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t out = (~(P[j] + C1) | (P[j] + C2)) & 0x80808080u;
+                                uint32_t at = (P[j] >> 24) * W0 + __dp4a(P[j], WD, base);
+                                at = out ? 0u : at;
+                                f[j] = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(bits) + at)
+                                       << (P[j] & 15u);
+                            }
+                            const int M = (int)sign_bytes<true>(f), C = (int)sign_bytes<false>(f);
+                            r_neg = __dp4a(M, 0x01010101, r_neg);
+#pragma unroll
+                            for (int a = 0; a < 4; ++a) x_neg[a] = __dp4a(M, (int)A[a][q], x_neg[a]);
+                            cneg = __dp4a(C, 0x08040201, cneg * 16);
+                        }
+                        cm = (uint32_t)(-cneg);
+                    }
+                    if (kw + 16 > Kc) cm &= (1u << (Kc - kw)) - 1u;   // trials at or past K
+                }
+                const int nm = __popc(cm);
+                int incl = nm;
+#pragma unroll
+                for (int off = 1; off < 32; off <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, incl, off);
+                    if (lane >= off) incl += y;
+                }
+                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                const bool flush = (st & 63) == 63 || k0 + (st + 1) * (NT * 16) >= Kc;
+                const int ent = (stq << 9) | (lane << 4);   // entry: step (6 bits), lane, trial
+                int done = 0;   // candidates of this step queued so far
+                do {
+                    // the lanes whose candidates fit the queue (a prefix of those left)
+                    const bool mine = incl - nm >= done && incl - done <= kQueue - qn;
+                    const unsigned who = __ballot_sync(0xffffffffu, mine);
+                    const int upto = __shfl_sync(0xffffffffu, incl, 31 - __clz(who));
+                    if (mine) {
+                        uint16_t* at = queue + qn + (incl - nm - done);
+                        while (cm) {
+                            const int b = __ffs(cm) - 1;
+                            cm &= cm - 1u;
+                            *at++ = (uint16_t)(ent | b);
+                        }
+                    }
+                    qn += upto - done;
+                    done = upto;
+                    __syncwarp();
+                    while (qn >= 32 || (flush && done == total && qn > 0)) {
+                        const int n = min(qn, 32);
+                        qn -= n;
+                        const int ev = queue[qn + (lane < n ? lane : 0)];
+                        const int k = kb + (ev >> 9) * (NT * 16) + (ev & 511);
+                        eval(k, lane < n);
+                        __syncwarp();   // the queue's entries read before the next round writes
+                    }
+                } while (done < total);
+            }
+            if (!sel) break;
+            if (lane == 0) s_nk[warp] = wk;
+            __syncthreads();
+            // the ks-th smallest key: its bin, then its rank among the bin's keys
+            int nk = 0;
+#pragma unroll
+            for (int w2 = 0; w2 < NW; ++w2) nk += s_nk[w2];
+            bool found = nk >= ks;
+            if (found) {
+                if (warp == 0) {
+                    int before = 0;
+                    const int b = warp_pick256<true>(hist, ks, lane, &before);
+                    if (lane == 0) {
+                        s_pick = b;
+                        s_before = before;
+                    }
+                }
+                __syncthreads();
+                const int b = s_pick, kr = ks - s_before;
+                for (int k = lane; k < wk; k += 32) {   // each warp its own keys
+                    const uint32_t key = kbuf[k];
+                    if (key_bin(key) == b) {
+                        const int at = atomicAdd(&s_nlist, 1);
+                        if (at < kList) list[at] = key;
+                    }
+                }
+                __syncthreads();
+                const int nl = s_nlist;
+                if (nl <= kList) {
+                    for (int j = tid; j < nl; j += NT) {
+                        const uint32_t key = list[j];
+                        int rank = 0;
+                        for (int q = 0; q < nl; ++q) {
+                            const uint32_t u = list[q];
+                            rank += (u < key || (u == key && q < j)) ? 1 : 0;
+                        }
+                        if (rank == kr - 1) s_res = key;
+                    }
+                    __syncthreads();
+                } else {   // radix select over the bin's keys: digits of 8, 8, 8 and 7 bits (S >= 0)
+                    uint32_t prefix = 0u, pmask = 0u;
+                    int kq = kr;
+                    for (int pass = 0; pass < 4; ++pass) {
+                        const int sh = pass < 3 ? 23 - 8 * pass : 0;
+                        const uint32_t dm = pass < 3 ? 0xFFu : 0x7Fu;
+                        for (int k = lane; k < wk; k += 32) {
+                            const uint32_t key = kbuf[k];
+                            if (key_bin(key) == b && (key & pmask) == prefix) atomicAdd(&hist[(key >> sh) & dm], 1u);
+                        }
+                        __syncthreads();
+                        if (warp == 0) {
+                            int before = 0;
+                            const int digit = warp_pick256<true>(hist, kq, lane, &before);
+                            if (lane == 0) {
+                                s_pick = digit;
+                                s_before = before;
+                            }
+                        }
+                        __syncthreads();
+                        prefix |= (uint32_t)s_pick << sh;
+                        pmask |= dm << sh;
+                        kq -= s_before;
+                    }
+                    if (tid == 0) s_res = prefix;
+                    __syncthreads();
+                }
+                lam_i = (double)__uint_as_float(s_res);
+                // exact unless it lies above the level of the trials left out
+                found = lam_i <= (double)basket_level(c);
+            } else {
+                for (int b = tid; b < 256; b += NT) hist[b] = 0u;
+                lam_i = INFINITY;   // with every trial evaluated, the k_i-th smallest S is +inf
+            }
+            if (found || c == ALL) break;
+            // too few keys below the level: the pass again with every trial
+            c = ALL;
+            sample = false;
+            r_neg = 0;
+#pragma unroll
+            for (int a = 0; a < 4; ++a) x_neg[a] = 0;
+            __syncthreads();   // every thread has read the counts
+            if (tid == 0) s_nlist = 0;
+            __syncthreads();
+        }
+        const int Rw = -basket_warp_sum(r_neg);
+        int Xw[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) Xw[a] = -basket_warp_sum(x_neg[a]);
+        if (lane == 0) {
+            s_red[0][warp] = Rw;
+            for (int a = 0; a < 4; ++a) s_red[1 + a][warp] = Xw[a];
+        }
+        __syncthreads();
+        if (tid == 0) {
+            basket_store(T, B, o, i, K, bad, v, s_red, NW, SELECT, lam_i, err);
+            if (SELECT) s_min = min(s_min, order_key(lam_i));
+        }
+    }
+    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr);
+}
+
+// The plain path's form: every trial through the posterior function.  SELECT adds
+// the per-tile order statistic lambda_i = S_(ksel_i) by a three-digit radix select
+// (11, 11, 10 bits of the FP32 keys, which order like the non-negative S) over the
+// keys the CTA stored.
+template <bool SELECT>
+__global__ void __launch_bounds__(BT, 4) k_sim_basket_direct(TileArgs T, Basket B, const uint8_t* __restrict__ cnt,
+                                                             int32_t k_stride, int32_t K_tiles, float lambda_up,
+                                                             SimOut o, uint32_t* __restrict__ keys,
+                                                             int32_t* __restrict__ counter, int32_t* __restrict__ err)
 {
     __shared__ uint32_t hist[2048];
     __shared__ int s_tile, s_scan[BWARP], s_res[2];
@@ -151,8 +642,7 @@ __global__ void __launch_bounds__(BT, 4) k_sim_basket(TileArgs T, Basket B, cons
     __shared__ unsigned long long s_min;   // order key of the least lambda_i of this CTA's tiles
     if (threadIdx.x == 0) s_min = ~0ull;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    NodeConst C;
-    if (!TABLE) C = node_const();
+    const NodeConst C = node_const();
     uint32_t* kbuf = keys + (int64_t)blockIdx.x * k_stride;
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(counter, 1);
@@ -175,90 +665,43 @@ __global__ void __launch_bounds__(BT, 4) k_sim_basket(TileArgs T, Basket B, cons
 #pragma unroll
         for (int a = 0; a < 4; ++a) rowp[a] = cnt + (int64_t)(T.axis_off[a] + (bad ? 0 : v[a])) * k_stride;
         int r_acc = 0, xs[4] = {0, 0, 0, 0};
-        if constexpr (TABLE) {
-            // full steps without per-trial bounds checks, the tail step with them:
-            // straight-line work for the eight trials (16^4 grid: 4.08 -> 3.66 ms)
-            auto step8 = [&](int k8, auto full) {
-                // k8 + SPT <= k_stride (k_stride is a multiple of 16): the loads stay in the row
-                uint2 w[4];
+        for (int k8 = tid * SPT; k8 < Kc; k8 += BT * SPT) {
+            // k8 + SPT <= k_stride (k_stride is a multiple of 16): the loads stay in the row
+            uint2 w[4];
 #pragma unroll
-                for (int a = 0; a < 4; ++a) w[a] = __ldg(reinterpret_cast<const uint2*>(rowp[a] + k8));
-                float4 q[SPT];
+            for (int a = 0; a < 4; ++a) w[a] = __ldg(reinterpret_cast<const uint2*>(rowp[a] + k8));
+            float4 q[SPT];
 #pragma unroll
-                for (int j = 0; j < SPT; ++j) {
-                    q[j] = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-                    if (decltype(full)::value || k8 + j < Kc) {
-                        int x[4];
+            for (int j = 0; j < SPT; ++j) {
+                q[j] = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
+                if (k8 + j < Kc) {
+                    int x[4];
 #pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            x[a] = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
-                        q[j] = state_q<TABLE>(Qt, B, C, x);
+                    for (int a = 0; a < 4; ++a)
+                        x[a] = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
+                    q[j] = state_q<false>(nullptr, B, C, x);
+                }
+            }
+            uint32_t kq[SPT];
+#pragma unroll
+            for (int j = 0; j < SPT; ++j) {
+                float S = INFINITY;
+                if (k8 + j < Kc) {
+                    S = masked_min(q[j], mask);
+                    const int rej = (S < lambda_up) ? 1 : 0;
+                    r_acc += rej;
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) {
+                        const int x = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
+                        xs[a] += rej ? x : 0;
                     }
+                    if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
                 }
-                uint32_t kq[SPT];
-#pragma unroll
-                for (int j = 0; j < SPT; ++j) {
-                    float S = INFINITY;
-                    if (decltype(full)::value || k8 + j < Kc) {
-                        S = masked_min(q[j], mask);
-                        const int rej = (S < lambda_up) ? 1 : 0;
-                        r_acc += rej;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            const int x = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
-                            xs[a] += rej ? x : 0;
-                        }
-                        if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
-                    }
-                    kq[j] = __float_as_uint(S);
-                }
-                if (SELECT) {
-                    *reinterpret_cast<uint4*>(kbuf + k8) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
-                    *reinterpret_cast<uint4*>(kbuf + k8 + 4) = make_uint4(kq[4], kq[5], kq[6], kq[7]);
-                }
-            };
-            int k8 = tid * SPT;
-            for (; k8 + SPT <= Kc; k8 += BT * SPT) step8(k8, std::true_type{});
-            if (k8 < Kc) step8(k8, std::false_type{});
-        } else {
-            for (int k8 = tid * SPT; k8 < Kc; k8 += BT * SPT) {
-                // k8 + SPT <= k_stride (k_stride is a multiple of 16): the loads stay in the row
-                uint2 w[4];
-#pragma unroll
-                for (int a = 0; a < 4; ++a) w[a] = __ldg(reinterpret_cast<const uint2*>(rowp[a] + k8));
-                float4 q[SPT];
-#pragma unroll
-                for (int j = 0; j < SPT; ++j) {
-                    q[j] = make_float4(INFINITY, INFINITY, INFINITY, INFINITY);
-                    if (k8 + j < Kc) {
-                        int x[4];
-#pragma unroll
-                        for (int a = 0; a < 4; ++a)
-                            x[a] = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
-                        q[j] = state_q<TABLE>(Qt, B, C, x);
-                    }
-                }
-                uint32_t kq[SPT];
-#pragma unroll
-                for (int j = 0; j < SPT; ++j) {
-                    float S = INFINITY;
-                    if (k8 + j < Kc) {
-                        S = masked_min(q[j], mask);
-                        const int rej = (S < lambda_up) ? 1 : 0;
-                        r_acc += rej;
-#pragma unroll
-                        for (int a = 0; a < 4; ++a) {
-                            const int x = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
-                            xs[a] += rej ? x : 0;
-                        }
-                        if (SELECT) atomicAdd(&hist[__float_as_uint(S) >> 21], 1u);
-                    }
-                    kq[j] = __float_as_uint(S);
-                }
-                if (SELECT) {
-                    *reinterpret_cast<uint4*>(kbuf + k8) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
-                    *reinterpret_cast<uint4*>(kbuf + k8 + 4) = make_uint4(kq[4], kq[5], kq[6], kq[7]);
-                }
+                kq[j] = __float_as_uint(S);
+            }
+            if (SELECT) {
+                *reinterpret_cast<uint4*>(kbuf + k8) = make_uint4(kq[0], kq[1], kq[2], kq[3]);
+                *reinterpret_cast<uint4*>(kbuf + k8 + 4) = make_uint4(kq[4], kq[5], kq[6], kq[7]);
             }
         }
         r_acc = basket_warp_sum(r_acc);
@@ -294,21 +737,7 @@ __global__ void __launch_bounds__(BT, 4) k_sim_basket(TileArgs T, Basket B, cons
             }
         }
         if (tid == 0) {
-            if (bad) atomicOr(err, CSE_ERR_BAD_K);
-            int64_t Rt = 0, X[4] = {0, 0, 0, 0};
-            for (int w2 = 0; w2 < BWARP; ++w2) {
-                Rt += s_red[0][w2];
-                for (int a = 0; a < 4; ++a) X[a] += s_red[1 + a][w2];
-            }
-            if (o.R) o.R[i] = Rt;
-            for (int a = 0; a < 4; ++a) {
-                if (o.Xrej) o.Xrej[i * 4 + a] = X[a];
-                if (o.score) {
-                    const double sg = bad ? NAN : o.sig[T.axis_off[a] + v[a]];
-                    o.score[i * 4 + a] = (double)X[a] - (double)B.n * sg * (double)Rt;
-                }
-            }
-            if (SELECT && o.lam_tile) o.lam_tile[i] = lam_i;
+            basket_store(T, B, o, i, K, bad, v, s_red, BWARP, SELECT, lam_i, err);
             if (SELECT) s_min = min(s_min, order_key(lam_i));
         }
         __syncthreads();
@@ -354,35 +783,75 @@ Basket make_basket(const DesignArgs& D)
     return B;
 }
 
-template <bool TABLE, bool SEL>
-int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_tiles, double lambda, const SimOut& o,
-                  cudaStream_t s)
+// Blocks of a launch, and the key buffer for `words` words a block.
+template <typename Kern>
+int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64_t words, int64_t* grid)
 {
-    auto kern = k_sim_basket<TABLE, SEL>;
     int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, BT, 0) != cudaSuccess || per_sm < 1) {
+    if (smem > 0 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
         cudaGetLastError();
         return CSE_CUDA_ERROR;
     }
-    int64_t grid = (int64_t)per_sm * c->num_sms;
-    if (grid > T.n_tiles) grid = T.n_tiles;
-    if (SEL) {
-        const size_t need = (size_t)grid * (size_t)k_stride * sizeof(uint32_t);
-        if (need > c->keys_cap) {
-            cudaFree(c->keys);
-            c->keys = nullptr;
-            c->keys_cap = 0;
-            if (cudaMalloc(&c->keys, need) != cudaSuccess) {
-                cudaGetLastError();
-                return CSE_OOM;
-            }
-            c->keys_cap = need;
-        }
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem) != cudaSuccess || per_sm < 1) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
     }
+    *grid = (int64_t)per_sm * c->num_sms;
+    if (*grid > tiles) *grid = tiles;
+    const size_t need = (size_t)*grid * (size_t)words * sizeof(uint32_t);
+    if (need > c->keys_cap) {
+        cudaFree(c->keys);
+        c->keys = nullptr;
+        c->keys_cap = 0;
+        if (cudaMalloc(&c->keys, need) != cudaSuccess) {
+            cudaGetLastError();
+            return CSE_OOM;
+        }
+        c->keys_cap = need;
+    }
+    return CSE_OK;
+}
+
+template <bool SEL>
+int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_tiles, double lambda, const SimOut& o,
+                  cudaStream_t s)
+{
+    // a warp's keys: its share of the sample and its 512 trials of every step
+    const int32_t key_seg = kSample / (NT / 32) + (K_tiles + NT * 16 - 1) / (NT * 16) * 512;
+    int64_t grid = 0;
+    const Basket B = make_basket(c->D);
+    const int span = basket_span(B.n), rows = B.m * B.m * B.m;
+    const size_t smem = ((size_t)span * span * span + 1) * sizeof(uint32_t);
+    const float lam = lambda_float_up(lambda);
+    const bool want_R = o.R || o.Xrej || o.score || o.cp_key;
+    const int st = basket_grid(c, k_sim_basket<SEL>, NT, smem, T.n_tiles, SEL ? (int64_t)(NT / 32) * key_seg : 0, &grid);
+    if (st != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
+    if (o.cp_key) c->cp_marked = true;
     cse_prof_begin(c, KID_SIM_BASKET, s);
-    kern<<<(unsigned)grid, BT, 0, s>>>(T, make_basket(c->D), c->cnt, k_stride, K_tiles, c->bk_q,
-                                      lambda_float_up(lambda), o, c->keys, c->counter, c->err);
+    if (want_R && K_tiles > kAllK) {   // the bits of this call's lambda
+        k_basket_bits<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(c->bk_bits, c->bk_q, B.m, rows, kLevels, 1, lam);
+        c->launches += 1;
+    }
+    k_sim_basket<SEL><<<(unsigned)grid, NT, smem, s>>>(T, B, c->cnt, k_stride, K_tiles, c->bk_q, c->bk_bits, span, lam,
+                                                      want_R, o, c->keys, key_seg, c->counter, c->err);
+    cse_prof_end(c, s);
+    c->launches += 1;
+    return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+template <bool SEL>
+int launch_basket_direct(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_tiles, double lambda,
+                         const SimOut& o, cudaStream_t s)
+{
+    int64_t grid = 0;
+    const int st = basket_grid(c, k_sim_basket_direct<SEL>, BT, 0, T.n_tiles, SEL ? k_stride : 0, &grid);
+    if (st != CSE_OK) return st;
+    if (SEL && o.min_out) c->min_folded = true;
+    if (o.cp_key) c->cp_marked = true;
+    cse_prof_begin(c, KID_SIM_BASKET, s);
+    k_sim_basket_direct<SEL><<<(unsigned)grid, BT, 0, s>>>(T, make_basket(c->D), c->cnt, k_stride, K_tiles,
+                                                          lambda_float_up(lambda), o, c->keys, c->counter, c->err);
     cse_prof_end(c, s);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
@@ -394,16 +863,21 @@ int cse_basket_setup(cse_ctx* c, cudaStream_t s)
 {
     const Basket B = make_basket(c->D);
     const int64_t states = (int64_t)B.m * B.m * B.m * B.m;
-    c->bt_tables = states <= CSE_BAYES_TABLE_MAX;
+    c->bt_tables = states <= CSE_BAYES_TABLE_MAX && B.m <= kMaxM;
     if (!c->bt_tables) return CSE_OK;   // direct evaluation per simulation
-    if (cudaMalloc(&c->bk_q, (size_t)states * sizeof(float4)) != cudaSuccess) {
+    const int rows = B.m * B.m * B.m;
+    const size_t bits_bytes = (size_t)(kLevels + 1) * 4 * (size_t)rows * sizeof(uint2);
+    if (cudaMalloc(&c->bk_q, (size_t)states * sizeof(float4)) != cudaSuccess ||
+        cudaMalloc(&c->bk_bits, bits_bytes) != cudaSuccess) {
         cudaGetLastError();
         return CSE_OOM;
     }
     cse_prof_begin(c, KID_BASKET_TABLE, s);
     k_table_basket<<<(unsigned)((states + 255) / 256), 256, 0, s>>>(c->bk_q, B);
     cse_prof_end(c, s);
-    c->launches += 1;
+    // level +inf (kLevels - 1) is never read
+    k_basket_bits<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(c->bk_bits, c->bk_q, B.m, rows, 0, kLevels - 1, 0.0f);
+    c->launches += 2;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
@@ -429,8 +903,8 @@ int cse_launch_sim_basket(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_s
     (void)NA;
     const bool sel = (o.lam_tile != nullptr && o.ksel != nullptr);
     if (c->bt_tables && !c->bt_direct)
-        return sel ? launch_basket<true, true>(c, T, k_stride, K_tiles, lambda, o, s)
-                   : launch_basket<true, false>(c, T, k_stride, K_tiles, lambda, o, s);
-    return sel ? launch_basket<false, true>(c, T, k_stride, K_tiles, lambda, o, s)
-               : launch_basket<false, false>(c, T, k_stride, K_tiles, lambda, o, s);
+        return sel ? launch_basket<true>(c, T, k_stride, K_tiles, lambda, o, s)
+                   : launch_basket<false>(c, T, k_stride, K_tiles, lambda, o, s);
+    return sel ? launch_basket_direct<true>(c, T, k_stride, K_tiles, lambda, o, s)
+               : launch_basket_direct<false>(c, T, k_stride, K_tiles, lambda, o, s);
 }

@@ -556,13 +556,6 @@ constexpr int kAllK = 1024;      // up to this K every trial is evaluated
 constexpr int kQueue = 288;      // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
 constexpr int kList = 256;       // keys of the selected bin ranked in shared memory
 
-// Bin of a key (S >= 0 as bits) in a group's 256-bin histogram: sixteen bins an
-// octave from 2^-16 up, the ends clamped.  Monotone in S.
-__device__ __forceinline__ int key_bin(uint32_t key)
-{
-    return min(max((int)(key >> 19) - (int)(0x37800000u >> 19), 0), 255);
-}
-
 // dmin[D + u(n3)] (float bits, preset to +inf) = the least S an active treatment
 // with final score difference D to the control can give, over every state of the
 // final table.
