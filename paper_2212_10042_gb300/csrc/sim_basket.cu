@@ -95,8 +95,9 @@ __global__ void k_table_basket(float4* __restrict__ Qt, Basket B)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int m = B.m;
+    __shared__ NodeConst C;
+    node_const_block(C);
     if (s >= m * m * m * m) return;
-    const NodeConst C = node_const();
     const int x[4] = {s / (m * m * m), (s / (m * m)) % m, (s / m) % m, s % m};
     float Q[4];
     basket_q_f32(x, B, C, Q);

@@ -131,8 +131,9 @@ __global__ void k_table_d1(uint8_t* __restrict__ D1, Looks L, float drop)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int m = L.n1 + 1;
+    __shared__ NodeConst C;
+    node_const_block(C);
     if (s >= m * m * m * m) return;
-    const NodeConst C = node_const();
     int x[4] = {s / (m * m * m), (s / (m * m)) % m, (s / m) % m, s % m};
     int n[4] = {L.n1, L.n1, L.n1, L.n1};
     float P[3];
@@ -183,8 +184,9 @@ __global__ void k_table_d2(uint8_t* __restrict__ D2, Looks L, float drop)
 {
     const int s = blockIdx.x * blockDim.x + threadIdx.x;
     const int S2 = L.S2;
+    __shared__ NodeConst C;
+    node_const_block(C);
     if (s >= (L.n2 + 1) * S2 * S2 * S2) return;
-    const NodeConst C = node_const();
     const int c = s / (S2 * S2 * S2);
     const int t[3] = {(s / (S2 * S2)) % S2, (s / S2) % S2, s % S2};
     D2[s] = (uint8_t)d2_bits(L, C, drop, c, t);
@@ -235,8 +237,9 @@ __global__ void k_table_f4(float4* __restrict__ F4, Looks L)
 {
     const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t tot = (int64_t)(L.n3 + 1) * L.NT;
+    __shared__ NodeConst C;
+    node_const_block(C);
     if (s >= tot) return;
-    const NodeConst C = node_const();
     const int c = (int)(s / L.NT);
     int a, b, z;
     decode_triple((int)(s % L.NT), &a, &b, &z);

@@ -451,19 +451,26 @@ __global__ void k_stat_table(float* __restrict__ S, DesignArgs D, int32_t n_cell
 // With pos and ntie (may be NULL): pos[rank[c] + #{c' < c : S[c'] = S[c]}] = c,
 // the cells sorted by (S, index), so the cells of rank r sit at positions r,
 // r + 1, ..., r + ntie[r] - 1, ntie[r] = #{c' : S[c'] = S[c]}.
-__global__ void k_rank_table(const float* __restrict__ S, uint16_t* __restrict__ rank,
-                             float* __restrict__ vor, int32_t* __restrict__ pos, int32_t* __restrict__ ntie,
-                             int32_t n_cells)
+// A warp a cell: bound by the n_cells^2 comparisons (a thread a cell left most of the
+// SMs without a block: 10,201 cells 306 us, so 41).
+__global__ void __launch_bounds__(256) k_rank_table(const float* __restrict__ S, uint16_t* __restrict__ rank,
+                                                    float* __restrict__ vor, int32_t* __restrict__ pos,
+                                                    int32_t* __restrict__ ntie, int32_t n_cells)
 {
-    const int c = blockIdx.x * blockDim.x + threadIdx.x;
+    const int c = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (c >= n_cells) return;
     const float s = S[c];
     int r = 0, e = 0, t = 0;
-    for (int j = 0; j < n_cells; ++j) {
-        r += (S[j] < s);
-        e += (j < c && S[j] == s);
-        t += (S[j] == s);
+    for (int j = lane; j < n_cells; j += 32) {
+        const float v = S[j];
+        r += (v < s);
+        e += (j < c && v == s);
+        t += (v == s);
     }
+    r = __reduce_add_sync(0xffffffffu, r);
+    e = __reduce_add_sync(0xffffffffu, e);
+    t = __reduce_add_sync(0xffffffffu, t);
+    if (lane != 0) return;
     rank[c] = (uint16_t)r;
     vor[r] = s;
     if (pos) {
@@ -508,7 +515,7 @@ int cse_launch_tables(cse_ctx* c, cudaStream_t s)
     const int n = c->n_cells;
     cse_prof_begin(c, KID_TABLES, s);
     k_stat_table<<<(n + 255) / 256, 256, 0, s>>>(c->S_tab, c->D, n, c->n1p);
-    k_rank_table<<<(n + 255) / 256, 256, 0, s>>>(c->S_tab, c->rank_tab, c->val_of_rank, c->cell_of_pos,
+    k_rank_table<<<(n + 7) / 8, 256, 0, s>>>(c->S_tab, c->rank_tab, c->val_of_rank, c->cell_of_pos,
                                                 c->cell_of_pos ? c->cell_of_pos + n : nullptr, n);
     cse_prof_end(c, s);
     c->launches += 2;
