@@ -202,6 +202,7 @@ constexpr int kSample = 512;       // first trials of a tile, all evaluated to p
 constexpr int kAllK = 2048;
 constexpr int kQueue = 288;        // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
 constexpr int kList = 256;         // keys of the selected bin ranked in shared memory
+constexpr int kSpan3 = 16;         // most counts of arm 3 in the window: the bits of half a word
 constexpr float kWindow = 2.6f;    // half-width of the window in standard deviations
 
 __host__ __device__ inline float basket_level(int c)
@@ -209,7 +210,7 @@ __host__ __device__ inline float basket_level(int c)
     return c >= kLevels - 1 ? INFINITY : exp2f(0.25f * (float)(c + 1) - 8.0f);
 }
 
-// most counts of an arm in the window (p = 1/2; of arm 3 at most 16, the bits of half a word)
+// most counts of an arm in the window (p = 1/2; of arm 3 at most kSpan3)
 inline int basket_span(int n)
 {
     const int w = (int)(kWindow * sqrtf((float)n)) + 2;
@@ -324,7 +325,7 @@ __global__ void __launch_bounds__(NT, 8)
         const bool bad = __any_sync(0xffffffffu, vl < 0 || vl >= na) || K < 1 || K > K_tiles;
         const int atl = ao + (bad ? 0 : vl);
         const float pl = bad ? 0.5f : (float)o.sig[atl], mu = (float)B.n * pl;
-        const int wl = min((int)(2.0f * kWindow * sqrtf(mu * (1.0f - pl))) + 2, la == 3 ? min(span, 16) : span);
+        const int wl = min((int)(2.0f * kWindow * sqrtf(mu * (1.0f - pl))) + 2, la == 3 ? min(span, kSpan3) : span);
         const int ll = min(max((int)(mu + 0.5f - 0.5f * (float)(wl - 1)), 0), m - wl);
         const uint32_t mask = T.null_mask[i] & 15u;   // null arms (none: S = +inf throughout)
         const int Kc = (bad || mask == 0u) ? 0 : K;
@@ -789,10 +790,6 @@ template <typename Kern>
 int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64_t words, int64_t* grid)
 {
     int per_sm = 0;
-    if (smem > 0 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
-        cudaGetLastError();
-        return CSE_CUDA_ERROR;
-    }
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem) != cudaSuccess || per_sm < 1) {
         cudaGetLastError();
         return CSE_CUDA_ERROR;
@@ -822,6 +819,8 @@ int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_til
     int64_t grid = 0;
     const Basket B = make_basket(c->D);
     const int span = basket_span(B.n), rows = B.m * B.m * B.m;
+    // the words of the widest window, w_0 w_1 w_2 <= span^3, and word 0: at most 42,596 bytes (n = 63:
+    // span 22), with the static arrays below the default limit of 48 KB
     const size_t smem = ((size_t)span * span * span + 1) * sizeof(uint32_t);
     const float lam = lambda_float_up(lambda);
     const bool want_R = o.R || o.Xrej || o.score || o.cp_key;

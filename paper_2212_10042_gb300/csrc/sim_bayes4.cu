@@ -1216,10 +1216,15 @@ int b4_grow_keys(cse_ctx* c, int64_t rows, int64_t words)
     return CSE_OK;
 }
 
+constexpr int kSmemLimit = 96 * 1024;
+
 template <typename Kern>
 int b4_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t blocks, int64_t* grid)
 {
-    if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    // one limit for every design (the tables take at most 70 KB): it belongs to the kernel, and
+    // another thread may be launching a design with larger tables
+    if (smem > 0 &&
+        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemLimit) != cudaSuccess) {
         cudaGetLastError();
         return CSE_UNSUPPORTED_DESIGN;
     }

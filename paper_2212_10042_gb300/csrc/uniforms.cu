@@ -556,8 +556,10 @@ static int launch_counts(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t K_ti
     while (pow2 < chunk) pow2 <<= 1;
     auto kern = k_counts<SEGS, MODE>;
     const size_t smem = (size_t)chunk * (SEGS * 128 + 4 + 2);
-    if (smem > 20 * 1024 &&   // with the static arrays (up to 23 KB) beyond the default limit
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess) {
+    // the limit of the largest chunk, whatever this call's: it belongs to the kernel, and another
+    // thread may be launching with a larger chunk (with the static arrays, up to 23 KB, it passes 48 KB)
+    if (smem > 20 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 CH_MAX * (SEGS * 128 + 4 + 2)) != cudaSuccess) {
         cudaGetLastError();
         return CSE_CUDA_ERROR;
     }
