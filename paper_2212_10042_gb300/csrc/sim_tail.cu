@@ -35,10 +35,10 @@
 // randomised calibration of the 128^2 grid: 95 + 67 (tie pass) -> 136 us.  Five blocks an
 // SM at 48 registers are no faster than four at 56.
 //
-// Tiles: a group of TT threads per tile, G tiles a block.  With many tiles a warp
-// per tile: no barriers and the most tiles in flight.  Fewer than 32 tiles an SM
-// take 128 threads each, fewer than 8 an SM a block of 256, for the latency of one
-// tile.
+// Tiles: a group of TT threads per tile, G tiles a block: 64 threads with many
+// tiles (a warp per tile: 32,896 tiles 20 us a step slower, 8,256 randomised tiles
+// 33, 2^18 level, and twice the keys in memory), 128 below 32 tiles an SM, a block
+// of 256 below 8 an SM, for the latency of one tile.
 #include <cuda_runtime.h>
 #include <math.h>
 
@@ -437,7 +437,7 @@ int launch_groups(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, i
         return launch_tail<WORDS, 1>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
     if (T.n_tiles < 32 * (int64_t)c->num_sms || key_bytes > (1 << 17))
         return launch_tail<WORDS, 2>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
-    return launch_tail<WORDS, 8>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    return launch_tail<WORDS, 4>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
 }
 
 // Rejections alone: a group of TT threads per tile, sixteen trials a thread and step.
