@@ -69,7 +69,8 @@ WORKLOADS = {
                                 "double K (up to 2^16) for up to 6 rounds"),
 }
 # Algorithmic lane operations per (sim, tile) of each design's simulation pass,
-# the method's own work in the form this library computes it:
+# the method's own work when every trial is evaluated (the kernels evaluate only
+# the trials that can decide an output):
 #   one arm: 1 count read, 1 compare, 2 predicated accumulates (R, X), 1
 #     selection insert;
 #   two arms (axis count tables, rejection monotone in both counts): 2 count
@@ -83,22 +84,25 @@ WORKLOADS = {
 OPS_PER_SIM_TILE = {"one_arm_z": 5, "two_arm_pooled_z": 6, "bayes4": 22, "berry4": 12}
 # What bounds each simulation kernel, from its ncu profile (profiles/)
 LIMITER = {
-    "sim_ztest": "issue and latency: the histogram loop (byte extracts, index, one shared-memory increment per "
-                 "sim) and each tile's loads, barriers and read-off",
-    "sim_bayes4": "L1 throughput (83 %: the final-table gathers, count reads, key stores and the radix passes' "
-                  "key reads) and the integer ALU pipe (71 %: byte transposes, table indexing, code sorts)",
-    "sim_basket": "L1 tag throughput of the scattered 16-byte table gathers",
+    "sim_ztest": "two arms with a selection: issue slots (60 %: byte tests, queueing, 7 % of the sims evaluated) and "
+                 "the latency of the candidates' reads; one arm: latency",
+    "sim_bayes4": "issue slots (63 to 65 %; four fifths of the instructions evaluate the 13 to 19 % candidate trials) "
+                  "at the latency of their scattered reads",
+    "sim_basket": "issue slots (66 %) and the integer ALU pipe (64 %: byte transposes, window tests, word indexing)",
 }
 # DRAM bytes (read + write) per launch of the dominant kernel from one ncu
 # capture of the same kernel build, scaled to the workload where the capture
 # ran on a smaller case; None until captured for the current kernel
 MEASURED_TRAFFIC = {
-    # profiles/k_sim_bayes4_four_arm_refined_sample_65536x65536.md: 26.73 GB on the
-    # 65,536-tile sample, scaled by the sim-tiles to the full platten (x 16.0)
-    ("c5", "sim_bayes4"): 427.70e9,
-    ("c5_sample", "sim_bayes4"): 26.73e9,
-    # profiles/k_sim_cells_two_arm_256x256_K16384.md: one capture at the full size
-    ("c2", "sim_ztest"): 9.09e6,
+    # profiles/k_sim_bayes4_four_arm_refined_sample_65536x65536.md: 24.4 GB on 2^18 tiles of the
+    # platten, scaled by the sim-tiles (x 4.0); 6.34 GB on the 65,536-tile sample
+    ("c5", "sim_bayes4"): 97.6e9,
+    ("c5_sample", "sim_bayes4"): 6.34e9,
+    # profiles/k_sim_tail_two_arm_256x256_K16384.md: one capture at the full size, and the 2^18 batch
+    ("c2", "sim_ztest"): 9.69e6,
+    ("c3", "sim_ztest"): 709e6,
+    # profiles/k_sim_basket_basket_8x8x8x8_K16384.md
+    ("berry", "sim_basket"): 52.4e6,
 }
 # designs whose statistic is an FP32 posterior (decisions may flip against the FP64 oracle)
 POSTERIOR = ("bayes4", "berry4")
@@ -594,7 +598,7 @@ def run_chosen(args):
                                "SM clock of %s MHz" % peaks["clocks"].get("sm_mhz"),
                 "ops_per_unit": ops, "units_per_launch": units, "ms_per_launch": ms_l,
                 "limiter": LIMITER.get(kname)}
-        if design.stat in ("one_arm_z", "two_arm_pooled_z"):
+        if design.stat == "one_arm_z":
             # the cell histogram: one shared-memory atomic increment per (sim, tile)
             a_peak = peaks["smem_atomic"]["lane_ops_per_s"] / 1e12
             roof["smem_atomic"] = {"achieved": units / (ms_l * 1e-3) / 1e12, "peak": a_peak, "unit": "Tatomic/s",

@@ -271,17 +271,16 @@ int cse_reseed(cse_ctx* ctx, uint64_t seed, cse_stream_t stream);
 /* Autotuner: times the fused simulation pass of `tiles` (at `lambda`, with the
  * calibration selection for level `alpha`) in each configuration of the z-test
  * cell-histogram kernel (where a call runs it: see cse_set_option), (threads per
- * block, tiles per block) in (128, 1),
- * (256, 1), (512, 1), (64, 1), (128, 2), (256, 2), (256, 4) -- a block of T
- * threads working on G tiles at once gives each tile T / G threads, so the sims
- * per block and step are 16 T and the tiles in flight per SM follow from the
- * blocks that fit -- and keeps the fastest for this context's later calls (the
- * plain path: its per-sim kernel at 128, 256, 512 threads).  *threads_out and
- * *tiles_out (host, may be NULL) receive the choice.  The four-arm designs have
- * one configuration each: (512, 1) for the selection design's tabulated form
- * when its codes fit the packed per-trial form, else (256, 1).  Synchronises
- * `stream`.  Results never depend on
- * the choice.  Errors: INVALID_ARG, as cse_simulate_tiles. */
+ * block, tiles per block) in (128, 1), (256, 1), (512, 1), (64, 1), (128, 2),
+ * (256, 2), (256, 4) -- a block of T threads working on G tiles at once gives
+ * each tile T / G threads, so the sims per block and step are 16 T and the tiles
+ * in flight per SM follow from the blocks that fit -- and keeps the fastest for
+ * this context's later calls (the plain path: its per-sim kernel at 128, 256, 512
+ * threads).  *threads_out and *tiles_out (host, may be NULL) receive the choice.
+ * The posterior designs have nothing to choose and report (512, 1) for the
+ * selection design's tabulated form when its codes fit the packed per-trial form,
+ * else (256, 1).  Synchronises `stream`.  Results never depend on the choice.
+ * Errors: INVALID_ARG, as cse_simulate_tiles. */
 int cse_autotune(cse_ctx* ctx, const cse_tiles* tiles, double lambda, double alpha, int32_t* threads_out,
                  int32_t* tiles_out, cse_stream_t stream);
 

@@ -502,7 +502,7 @@ struct cse_ctx {
     int64_t prof_n[KID_COUNT];
 };
 
-// The packed four-arm form keeps its count table in two planes (see k_axis_counts):
+// The packed four-arm form keeps its count table in two planes (see k_counts):
 // both interim segments' counts in one byte, and the final count's score.
 inline bool cse_count_nibbles(const cse_ctx* c)
 {

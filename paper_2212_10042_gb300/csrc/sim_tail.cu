@@ -31,8 +31,8 @@
 // What bounds it: issue slots (54 to 60 % issue; 10 thread instructions a trial, of
 // which the test and the queueing take half, the 7 % candidates a third) and the
 // latency of the scattered count reads.
-// 256^2 grid, K = 16,384 (32,896 tiles): 323 -> 265 us; 2^18 batch: 3.34 -> 2.53 ms;
-// randomised calibration of the 128^2 grid: 95 + 67 (tie pass) -> 136 us.  Five blocks an
+// 256^2 grid, K = 16,384 (32,896 tiles): 323 -> 263 us; 2^18 batch: 3.34 -> 2.55 ms;
+// randomised calibration of the 128^2 grid, the whole call: 275 -> 210 us.  Five blocks an
 // SM at 48 registers are no faster than four at 56.
 //
 // Tiles: a group of TT threads per tile, G tiles a block: 64 threads with many
