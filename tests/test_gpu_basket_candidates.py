@@ -60,3 +60,17 @@ def test_candidates_match_every_trial(B, n, n_tiles):
     b = _outputs(ctx, dt, lams, (0.025, 0.6))
     for j, (x, y) in enumerate(zip(a, b)):
         assert torch.equal(x, y), j
+
+
+def test_candidates_beyond_a_block_of_steps(B):
+    """K past the 64 steps of 2,048 trials that a queue entry can address."""
+    K = np.array([131072 + 511, 131072 + 512, 131072 + 513, 133120 + 512, 262144 + 513, 300001])
+    tiles = W.from_centers(np.linspace(-2.5, 0.8, 24).reshape(6, 4), 0.02, np.array([15, 1, 6, 9, 3, 12], np.uint32),
+                           K.astype(np.int32))
+    ctx = B.Context(W.BERRY4, seed=9, K_max=int(K.max()))
+    dt = B.DeviceTiles(tiles)
+    a = _outputs(ctx, dt, (0.0, 0.15), (0.025,))
+    ctx.set_option(B.OPT_BAYES_DIRECT, 1)
+    b = _outputs(ctx, dt, (0.0, 0.15), (0.025,))
+    for j, (x, y) in enumerate(zip(a, b)):
+        assert torch.equal(x, y), j
