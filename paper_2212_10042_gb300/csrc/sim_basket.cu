@@ -191,14 +191,15 @@ __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B,
 // on the way: one bit per state at a fixed level and every rejection evaluated 3.28 ms
 // (the candidates' own work), lambda's and the level's bits in separate words 2.58,
 // in one 2.34; 128 threads a tile instead of 256 1.98 (more tiles in flight to cover
-// the window's loads and the barriers).
+// the window's loads and the barriers); the sample and the tiles without a test a trial a
+// lane, unqueued: another 40 us off the step.
 // ---------------------------------------------------------------------------
 constexpr int kLevels = 32;        // levels of S for selections: 2^((c + 1) / 4 - 8), the last +inf
 constexpr int kMaxM = 64;          // count states of an arm: two 32-bit words of x_3
 constexpr int NT = 128;            // threads of the tabulated kernel
 constexpr int kSample = 512;       // first trials of a tile, all evaluated to place c
-// up to this K every trial is evaluated: below it the window (a few thousand words, 50 instructions
-// a word) and the bits of lambda cost more than the evaluations they save
+// up to this K every trial is evaluated, a trial a lane: 19,056 tiles, a step at K = 1,500 509 us
+// against 580 by bits, at 2,000 587 against 593
 constexpr int kAllK = 2048;
 constexpr int kQueue = 288;        // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
 constexpr int kList = 256;         // keys of the selected bin ranked in shared memory
@@ -349,7 +350,6 @@ __global__ void __launch_bounds__(NT, 8)
         for (;;) {
             int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
             const int k0 = sample ? kSample : 0;
-            bool built = false;   // the window's bits are those of c
             // bytes of P: x_3, x_2, x_1, x_0.  C1: bit 7 of a byte set iff x >= lo; C2: iff
             // x >= lo + w (bytes up to 127: no carry)
             const uint32_t C1 = 0x80808080u - (uint32_t)(lo[3] | (lo[2] << 8) | (lo[1] << 16) | (lo[0] << 24));
@@ -401,9 +401,11 @@ __global__ void __launch_bounds__(NT, 8)
                 c = s_pick;
                 level = basket_level(c);
             }
+            if (c == ALL)   // no test: a trial a lane (k - lane is the warp's)
+                for (int k = k0 + tid; k - lane < Kc; k += NT) eval(min(k, Kc - 1), k < Kc);
             // sixteen consecutive trials per thread and step from k0 on
-            for (int st = 0; k0 + st * (NT * 16) < Kc; ++st) {
-                if (c != ALL && !built) {
+            for (int st = 0; c != ALL && k0 + st * (NT * 16) < Kc; ++st) {
+                if (st == 0) {
                     // a thread a word; its place steps by NT words
                     const int hi3 = lo[3] + w[3], w12 = w[1] * w[2], rows = w[0] * w12, rm = m * m * m;
                     const uint2 mk = make_uint2(bits_from(lo[3]) & ~bits_from(min(hi3, 32)),
@@ -436,7 +438,6 @@ __global__ void __launch_bounds__(NT, 8)
                         if (y2 >= w[2]) y2 -= w[2], y1 += 1, src += c2;
                         if (y1 >= w[1]) y1 -= w[1], src += c1;
                     }
-                    built = true;
                     __syncthreads();
                 }
                 // first trial of the warp at the start of the queue's block of 64 steps
@@ -445,49 +446,46 @@ __global__ void __launch_bounds__(NT, 8)
                 const int kw = kb + stq * (NT * 16) + lane * 16;
                 uint32_t cm = 0u;   // bit t: trial kw + t is evaluated
                 if (kw < Kc) {
-                    cm = 0xFFFFu;
-                    if (c != ALL) {
-                        uint32_t A[4][4];
+                    uint32_t A[4][4];
 #pragma unroll
-                        for (int a = 0; a < 4; ++a) {   // kw + 16 <= k_stride (a multiple of 16)
-                            const uint4 x = __ldg(reinterpret_cast<const uint4*>(rowp[a] + kw));
-                            A[a][0] = x.x, A[a][1] = x.y, A[a][2] = x.z, A[a][3] = x.w;
-                        }
-                        if (kw + 16 > Kc) {   // trials at or past K: outside the window (lo + w <= 64 < 127)
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                const int left = Kc - kw - 4 * q;
-                                const uint32_t past = left >= 4 ? 0u : left <= 0 ? ~0u : ~0u << (8 * left);
-#pragma unroll
-                                for (int a = 0; a < 4; ++a) A[a][q] = (A[a][q] & ~past) | (0x7F7F7F7Fu & past);
-                            }
-                        }
-                        int cneg = 0;   // minus the candidates' bits
-#pragma unroll
-                        for (int q = 3; q >= 0; --q) {
-                            const uint32_t l01 = __byte_perm(A[3][q], A[2][q], 0x5140);
-                            const uint32_t l23 = __byte_perm(A[3][q], A[2][q], 0x7362);
-                            const uint32_t h01 = __byte_perm(A[1][q], A[0][q], 0x5140);
-                            const uint32_t h23 = __byte_perm(A[1][q], A[0][q], 0x7362);
-                            const uint32_t P[4] = {__byte_perm(l01, h01, 0x5410), __byte_perm(l01, h01, 0x7632),
-                                                   __byte_perm(l23, h23, 0x5410), __byte_perm(l23, h23, 0x7632)};
-                            uint32_t f[4];
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) {
-                                const uint32_t out = (~(P[j] + C1) | (P[j] + C2)) & 0x80808080u;
-                                uint32_t at = (P[j] >> 24) * W0 + __dp4a(P[j], WD, base);
-                                at = out ? 0u : at;
-                                f[j] = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(bits) + at)
-                                       << (P[j] & 15u);
-                            }
-                            const int M = (int)sign_bytes<true>(f), C = (int)sign_bytes<false>(f);
-                            r_neg = __dp4a(M, 0x01010101, r_neg);
-#pragma unroll
-                            for (int a = 0; a < 4; ++a) x_neg[a] = __dp4a(M, (int)A[a][q], x_neg[a]);
-                            cneg = __dp4a(C, 0x08040201, cneg * 16);
-                        }
-                        cm = (uint32_t)(-cneg);
+                    for (int a = 0; a < 4; ++a) {   // kw + 16 <= k_stride (a multiple of 16)
+                        const uint4 x = __ldg(reinterpret_cast<const uint4*>(rowp[a] + kw));
+                        A[a][0] = x.x, A[a][1] = x.y, A[a][2] = x.z, A[a][3] = x.w;
                     }
+                    if (kw + 16 > Kc) {   // trials at or past K: outside the window (lo + w <= 64 < 127)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int left = Kc - kw - 4 * q;
+                            const uint32_t past = left >= 4 ? 0u : left <= 0 ? ~0u : ~0u << (8 * left);
+#pragma unroll
+                            for (int a = 0; a < 4; ++a) A[a][q] = (A[a][q] & ~past) | (0x7F7F7F7Fu & past);
+                        }
+                    }
+                    int cneg = 0;   // minus the candidates' bits
+#pragma unroll
+                    for (int q = 3; q >= 0; --q) {
+                        const uint32_t l01 = __byte_perm(A[3][q], A[2][q], 0x5140);
+                        const uint32_t l23 = __byte_perm(A[3][q], A[2][q], 0x7362);
+                        const uint32_t h01 = __byte_perm(A[1][q], A[0][q], 0x5140);
+                        const uint32_t h23 = __byte_perm(A[1][q], A[0][q], 0x7362);
+                        const uint32_t P[4] = {__byte_perm(l01, h01, 0x5410), __byte_perm(l01, h01, 0x7632),
+                                               __byte_perm(l23, h23, 0x5410), __byte_perm(l23, h23, 0x7632)};
+                        uint32_t f[4];
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) {
+                            const uint32_t out = (~(P[j] + C1) | (P[j] + C2)) & 0x80808080u;
+                            uint32_t at = (P[j] >> 24) * W0 + __dp4a(P[j], WD, base);
+                            at = out ? 0u : at;
+                            f[j] = *reinterpret_cast<const uint32_t*>(reinterpret_cast<const char*>(bits) + at)
+                                   << (P[j] & 15u);
+                        }
+                        const int M = (int)sign_bytes<true>(f), C = (int)sign_bytes<false>(f);
+                        r_neg = __dp4a(M, 0x01010101, r_neg);
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) x_neg[a] = __dp4a(M, (int)A[a][q], x_neg[a]);
+                        cneg = __dp4a(C, 0x08040201, cneg * 16);
+                    }
+                    cm = (uint32_t)(-cneg);
                     if (kw + 16 > Kc) cm &= (1u << (Kc - kw)) - 1u;   // trials at or past K
                 }
                 const int nm = __popc(cm);
