@@ -186,13 +186,13 @@ __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B,
 // What bounds it: issue slots (65 %) and the integer pipe (64 %): per 32 trials ~17
 // warp instructions of test and count, ~10 of queue and scan, ~7 of evaluation, and
 // ~20 of the tile's own work (building the window, setup, selection).  16^4 grid,
-// K = 2^14, with a selection (59,992 tiles): 3.67 -> 1.98 ms; 6,036 tiles of 1,000 to
+// K = 2^14, with a selection (59,992 tiles): 3.67 -> 1.95 ms; 6,036 tiles of 1,000 to
 // 30,000 trials without one: 152 -> 112 us, plus 10 for the bits of lambda.  Measured
 // on the way: one bit per state at a fixed level and every rejection evaluated 3.28 ms
 // (the candidates' own work), lambda's and the level's bits in separate words 2.58,
 // in one 2.34; 128 threads a tile instead of 256 1.98 (more tiles in flight to cover
 // the window's loads and the barriers); the sample and the tiles without a test a trial a
-// lane, unqueued: another 40 us off the step.
+// lane, unqueued: 1.95.
 // ---------------------------------------------------------------------------
 constexpr int kLevels = 32;        // levels of S for selections: 2^((c + 1) / 4 - 8), the last +inf
 constexpr int kMaxM = 64;          // count states of an arm: two 32-bit words of x_3
