@@ -24,9 +24,10 @@
 // 256 bins.  Then the bin of the k_i-th key and its rank within the bin.  Trials
 // left out have S >= cap, so the result is exact when it is at most cap and there
 // are k_i keys; otherwise the pass is repeated with cap + 1/2, and after three
-// tries with every trial.  Randomised test: the candidates hold every trial of the
-// tying rank, so their words are gathered from the keys and the m-th smallest
-// taken; no second pass over the count rows.
+// tries with every trial.  Randomised test: when the result lies below cap the
+// candidates hold every trial of the tying rank (at cap itself they need not: cells
+// of one statistic differ in x_1 - x_0), so their words are gathered from the keys
+// and the m-th smallest taken; no second pass over the count rows.
 //
 // What bounds it: issue slots (54 to 60 % issue; 10 thread instructions a trial, of
 // which the test and the queueing take half, the 7 % candidates a third) and the
@@ -290,7 +291,8 @@ __global__ void __launch_bounds__(kTailThreads, 4)
             const int rstar = s_pick[g], mrem = s_before[g];
             const float lam = vor_g[rstar];
             lam_i = (double)lam;
-            if (!all && !(lam <= cap)) {   // a trial left out might be smaller: again further out
+            // a trial left out might be smaller, or (words) of the same rank: again further out
+            if (!all && !(WORDS ? lam < cap : lam <= cap)) {
                 cap += 0.5f;
                 r_acc = x0_acc = x1_acc = 0;
                 tile_sync<TT, G>(g);
