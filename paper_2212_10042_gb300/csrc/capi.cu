@@ -183,10 +183,10 @@ int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = f
 // How the z-test simulation of a call runs (results do not depend on it).  Without a
 // selection, rejections by byte-parallel counts (counts and cuts up to 127 keep each
 // sum in its byte: 1,500 one-arm tiles, K <= 65,536 34 -> 14 us, 2,048 free points
-// 28 -> 14).  With one, two arms: candidates, unless alpha or lambda reach so far
-// into the statistic that a good part of the trials are candidates, at about eight
-// times the cost of a histogram increment: lambda <= -1 and alpha <= 0.1 leave at
-// most one in six (256^2 grid, lambda = -1.96, alpha = 0.025: 7 %, 323 -> 263 us).
+// 28 -> 14).  With one, two arms: candidates, unless alpha or lambda reach so far into
+// the statistic that a good part of the trials are candidates, at about ten times the
+// cost of a histogram increment (256^2 grid, lambda = -1.96, alpha = 0.025: 7 %, 323 ->
+// 267 us; 128^2 grid, lambda = -1, alpha = 0.1: the whole call 395 -> 239).
 // The cell histogram takes the rest -- one arm among them, whose n + 1 cells are
 // read off at once (64 tiles 10.8 us against 12.4) -- and every call whose
 // configuration the caller fixed.

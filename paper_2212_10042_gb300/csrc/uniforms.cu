@@ -530,9 +530,8 @@ int cse_launch_thresholds(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, c
     if (c->zmode == ZMODE_TAIL) {
         Z.pos = c->cell_of_pos;
         Z.zpar = c->zpar;
-    } else {
-        Z.zcut = c->zcut;
     }
+    Z.zcut = c->zcut;
     cse_prof_begin(c, KID_THRESHOLDS, s);
     cse_launch(c->pdl, k_thresholds, dim3((n_axis_total + 255) / 256 + (Z.S ? 1 : 0)), dim3(256), 0, s, c->thr, c->sig,
                T, n_axis_total, Z);
@@ -583,7 +582,9 @@ int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, 
 {
     if (cse_count_nibbles(c)) return launch_counts<3, kCountsNib>(c, T, n_axis_total, K_tiles, k_stride, c->bt_score, s);
     if (c->D.n_looks > 1) return launch_counts<3, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
-    if (c->zmode == ZMODE_COUNT && T.d == 2)
+    // (b(x_0) beside arm 0's counts: where the kernel counts rejections by bytes)
+    const bool map = c->zmode == ZMODE_COUNT || (c->zmode == ZMODE_TAIL && c->D.n_max <= 126 && c->z_lambda > -INFINITY);
+    if (map && T.d == 2)
         return launch_counts<1, kCountsMapped>(c, T, n_axis_total, K_tiles, k_stride, c->zcut, s);
     return launch_counts<1, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
 }
