@@ -77,6 +77,40 @@ __device__ __forceinline__ int tail_warp_sum(int v)
     return v;
 }
 
+// Rejections x >= b among trials k = k0, k0 + 1, .. k0 + 15, then step on, below K: adds
+// their number, the sum of their x and (TWO) of their y.  x: the tested counts, y: the
+// other arm's, b: each trial's cut (one arm: b1 in every byte).
+template <bool TWO = true>
+__device__ __forceinline__ void count_rejections(const uint8_t* __restrict__ x, const uint8_t* __restrict__ y,
+                                                 const uint8_t* __restrict__ b, int K, int k0, int step, int* R,
+                                                 int* X, int* Y, uint32_t b1 = 0u)
+{
+    uint32_t r = 0u, sx = 0u, sy = 0u;
+#pragma unroll 2
+    for (int k = k0; k < K; k += step) {   // k + 16 <= k_stride
+        const uint4 u = *reinterpret_cast<const uint4*>(x + k);
+        uint4 v = make_uint4(0u, 0u, 0u, 0u), c = make_uint4(b1, b1, b1, b1);
+        if (TWO) {
+            v = *reinterpret_cast<const uint4*>(y + k);
+            c = *reinterpret_cast<const uint4*>(b + k);
+        }
+        const uint32_t xw[4] = {u.x, u.y, u.z, u.w}, yw[4] = {v.x, v.y, v.z, v.w}, bw[4] = {c.x, c.y, c.z, c.w};
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            uint32_t m = ((xw[q] - bw[q] + 0x80808080u) >> 7) & 0x01010101u;   // one per rejecting trial
+            const int rem = K - k - 4 * q;
+            if (rem < 4) m &= rem > 0 ? (1u << (8 * rem)) - 1u : 0u;
+            const uint32_t full = m * 255u;
+            r = __dp4a(m, 0x01010101u, r);
+            sx = __dp4a(xw[q] & full, 0x01010101u, sx);
+            if (TWO) sy = __dp4a(yw[q] & full, 0x01010101u, sy);
+        }
+    }
+    *R += (int)r;
+    *X += (int)sx;
+    *Y += (int)sy;
+}
+
 // A selection key: the rank, or (with the randomised test's words) rank << 17 | the
 // trial's place among its warp's.  Ranks lie below 129^2 < 2^15.
 template <bool WORDS>
@@ -305,8 +339,9 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                 const float share = ((float)ks + 3.0f * sqrtf((float)ks) + 1.0f) / (float)K;
                 const float fn = (float)n_max, q0 = (float)o.sig[a0], q1 = (float)o.sig[a1];
                 // S = (p_0 - p_1) / sqrt(2 pb (1 - pb) / n) to first order in the counts' shares
+                // (below the diagonal the spread at a fixed pb does, and leaves fewer candidates)
                 const float pb = 0.5f * (q0 + q1), v = pb * (1.0f - pb), den = rsqrtf(v * 2.0f / fn);
-                const float e = (q1 - q0) * (1.0f - 2.0f * pb) / (4.0f * v);
+                const float e = q1 > q0 ? (q1 - q0) * (1.0f - 2.0f * pb) / (4.0f * v) : 0.0f;
                 const float sd = den * sqrtf(((1.0f + e) * (1.0f + e) * q0 * (1.0f - q0) +
                                               (1.0f - e) * (1.0f - e) * q1 * (1.0f - q1)) / fn);
                 cap = (q0 - q1) * den + normcdfinvf(fminf(share, 0.9f)) * sd + 0.05f;
@@ -324,10 +359,13 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                 d_rej = __reduce_min_sync(0xffffffffu, d_rej);
                 if (n_max > 126) d_test = min(d_test, max(d_rej, dmin));
             }
+            const bool bytes = d_rej < d_test;
+            const int rho_c = bytes ? 0 : rho;   // ranks of the rejections among the candidates
+            if (bytes)
+                count_rejections(c1, c0, c0 + (int64_t)NA * k_stride, Kc, lt * 16, TT * 16, &r_acc, &x1_acc, &x0_acc);
             const bool wide = dmax - dmin > 126;
             for (int tries = 0;; ++tries) {
                 const bool all = wide || d_test <= dmin;   // every trial, without the test
-                const bool by_bytes = !all && d_rej < d_test;
                 const uint32_t zc = 0x80808080u - (uint32_t)d_test * 0x01010101u;
                 int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
                 for (int st = 0; st * (TT * 32) < Kc; ++st) {   // group-uniform
@@ -338,8 +376,7 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                     const int kw = kb + stq * (TT * 32) + lane * 32;
                     uint32_t m = 0u;
                     if (kw < Kc) {
-                        const uint32_t in = kw + 32 > Kc ? trials_below(Kc - kw) : 0xFFFFFFFFu;
-                        if (all) {
+                            if (all) {
                             m = 0xFFFFFFFFu;
                         } else {
                             const bool two = kw + 16 < Kc;   // the second sixteen lie in the row
@@ -350,25 +387,12 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                             const uint4 ya = *reinterpret_cast<const uint4*>(c0 + kw);
                             const uint4 yb = two ? *reinterpret_cast<const uint4*>(c0 + kw + 16) : zero;
                             const uint32_t y[8] = {ya.x, ya.y, ya.z, ya.w, yb.x, yb.y, yb.z, yb.w};
-                            if (by_bytes) {   // as k_sim_count
-                                const uint8_t* const cb = c0 + (int64_t)NA * k_stride;
-                                const uint4 za = *reinterpret_cast<const uint4*>(cb + kw);
-                                const uint4 zb = two ? *reinterpret_cast<const uint4*>(cb + kw + 16) : zero;
-                                const uint32_t z[8] = {za.x, za.y, za.z, za.w, zb.x, zb.y, zb.z, zb.w};
-#pragma unroll
-                                for (int q = 0; q < 8; ++q) {
-                                    const uint32_t one = ((t[q] - z[q] + 0x80808080u) >> 7) & (in >> q) & 0x01010101u;
-                                    r_acc = (int)__dp4a(one, 0x01010101u, (uint32_t)r_acc);
-                                    x0_acc = (int)__dp4a(one * 255u & y[q], 0x01010101u, (uint32_t)x0_acc);
-                                    x1_acc = (int)__dp4a(one * 255u & t[q], 0x01010101u, (uint32_t)x1_acc);
-                                }
-                            }
 #pragma unroll
                             for (int q = 0; q < 8; ++q) t[q] = t[q] - y[q] + zc;
 #pragma unroll
                             for (int q = 0; q < 8; ++q) m |= (t[q] >> (7 - q)) & (0x01010101u << q);
                         }
-                        m &= in;
+                        if (kw + 32 > Kc) m &= trials_below(Kc - kw);
                     }
                     const int nm = __popc(m);
                     int incl = nm;
@@ -406,7 +430,7 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                             const int x0 = (int)__ldg(c0 + k), x1 = (int)__ldg(c1 + k);
                             int r = (int)__ldg(rank_g + min(x0 * n1p + x1, n_cells - 1));
                             if (lane >= n) r = 0x7FFFFFFF;
-                            const int rej = r < rho && !by_bytes ? 1 : 0;
+                            const int rej = r < rho_c ? 1 : 0;
                             r_acc += rej;
                             x0_acc += rej ? x0 : 0;
                             x1_acc += rej ? x1 : 0;
@@ -435,7 +459,7 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                 if (nk < ks && !all) {   // fewer candidates than k_i: again from a lower difference
                     for (int b = lt; b < 256; b += TT) hist[b] = 0u;
                     d_test = tries < 3 ? max(d_test - 1 - tries, dmin) : dmin;
-                    r_acc = x0_acc = x1_acc = 0;
+                    if (!bytes) r_acc = x0_acc = x1_acc = 0;
                     tile_sync<TT, G>(g);
                     continue;
                 }
@@ -484,7 +508,7 @@ __global__ void __launch_bounds__(kTailThreads, 4)
                     for (int o2 = 16; o2 > 0; o2 >>= 1) sigma = fminf(sigma, __shfl_xor_sync(0xffffffffu, sigma, o2));
                     if (!(WORDS ? lam < sigma : lam <= sigma)) {
                         d_test = max(least_diff(WORDS ? nextafterf(lam, INFINITY) : lam, lo0, hi0, lo1, hi1), dmin);
-                        r_acc = x0_acc = x1_acc = 0;
+                        if (!bytes) r_acc = x0_acc = x1_acc = 0;
                         tile_sync<TT, G>(g);
                         continue;
                     }
@@ -624,28 +648,9 @@ __global__ void __launch_bounds__(256)
         const uint8_t* const c0 = cnt + (int64_t)a0 * k_stride;
         const uint8_t* const c1 = cnt + (int64_t)a1 * k_stride;   // the tested row
         const uint8_t* const cb = c0 + (int64_t)NA * k_stride;    // b(x_0) (two arms)
-        uint32_t R = 0u, X0 = 0u, X1 = 0u;
-#pragma unroll 2
-        for (int k = lt * 16; k < Kc; k += TT * 16) {
-            const uint4 x = *reinterpret_cast<const uint4*>(c1 + k);
-            uint4 y = make_uint4(0u, 0u, 0u, 0u), b = make_uint4(b1, b1, b1, b1);
-            if (TWO) {
-                y = *reinterpret_cast<const uint4*>(c0 + k);
-                b = *reinterpret_cast<const uint4*>(cb + k);
-            }
-            const uint32_t xw[4] = {x.x, x.y, x.z, x.w}, yw[4] = {y.x, y.y, y.z, y.w}, bw[4] = {b.x, b.y, b.z, b.w};
-#pragma unroll
-            for (int q = 0; q < 4; ++q) {
-                uint32_t m = ((xw[q] - bw[q] + 0x80808080u) >> 7) & 0x01010101u;   // one per rejecting trial
-                const int rem = Kc - k - 4 * q;
-                if (rem < 4) m &= rem > 0 ? (1u << (8 * rem)) - 1u : 0u;
-                const uint32_t full = m * 255u;
-                R = __dp4a(m, 0x01010101u, R);
-                X1 = __dp4a(xw[q] & full, 0x01010101u, X1);
-                if (TWO) X0 = __dp4a(yw[q] & full, 0x01010101u, X0);
-            }
-        }
-        const int r = tail_warp_sum((int)R), x1 = tail_warp_sum((int)X1), x0 = TWO ? tail_warp_sum((int)X0) : x1;
+        int R = 0, X0 = 0, X1 = 0;
+        count_rejections<TWO>(c1, c0, cb, Kc, lt * 16, TT * 16, &R, &X1, &X0, b1);
+        const int r = tail_warp_sum(R), x1 = tail_warp_sum(X1), x0 = TWO ? tail_warp_sum(X0) : x1;
         if (lane == 0) {
             s_red[g][0][warp] = r;
             s_red[g][1][warp] = x0;
