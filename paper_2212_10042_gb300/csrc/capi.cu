@@ -110,16 +110,17 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
         cudaFree(c->aprime);
         cudaFree(c->lam_tile);
         cudaFree(c->R);
-        c->ksel = nullptr;
+        c->ksel = c->left = nullptr;
         c->aprime = c->lam_tile = nullptr;
         c->R = nullptr;
         c->tile_cap = 0;
         const size_t n = (size_t)t->n_tiles;
-        if (cudaMalloc(&c->ksel, n * 4) != cudaSuccess || cudaMalloc(&c->aprime, n * 8) != cudaSuccess ||
+        if (cudaMalloc(&c->ksel, n * 8) != cudaSuccess || cudaMalloc(&c->aprime, n * 8) != cudaSuccess ||
             cudaMalloc(&c->lam_tile, n * 8) != cudaSuccess || cudaMalloc(&c->R, n * 8) != cudaSuccess) {
             cudaGetLastError();
             return CSE_OOM;
         }
+        c->left = c->ksel + n;
         c->tile_cap = n;
     }
     if (c->cp_cap < 2 * (uint64_t)t->n_tiles) {

@@ -96,6 +96,18 @@ __device__ __forceinline__ void queue_reset(int32_t* counter)
     }
 }
 
+// Tiles of a launch: all of the set, or those of a list (the kernel before wrote
+// counter[2] of them; the one over the list sets the count back to zero).  *blocks:
+// those that take part (the others return at once, so an empty list costs one block's
+// arrival).
+__device__ __forceinline__ int64_t queue_tiles(const int32_t* list, const int32_t* counter, int64_t n_tiles,
+                                               int* blocks)
+{
+    const int64_t n = list ? (int64_t)counter[2] : n_tiles;
+    *blocks = list && n < (int64_t)gridDim.x ? max((int)n, 1) : (int)gridDim.x;
+    return n;
+}
+
 // Order-preserving map of a double to uint64 (x < y iff key(x) < key(y); a NaN
 // with the sign bit clear orders above +inf).
 __device__ __forceinline__ unsigned long long order_key(double x)
@@ -111,17 +123,19 @@ __device__ __forceinline__ double order_unkey(unsigned long long k)
 
 // queue_reset with the minimum over tiles of the per-tile thresholds folded in
 // (Eq. calibrated-threshold-final): every CTA's thread 0 adds its own minimum
-// `mine` (an order key) to *min_key before taking its ticket, and the last CTA
-// writes the decoded minimum to *min_out and sets *min_key back to all ones.
-// Without min_out it is queue_reset.
+// `mine` (an order key) to *min_key before taking its ticket, and the last of `blocks`
+// CTAs writes the decoded minimum to *min_out and sets *min_key back to all ones.
+// Without min_out it is queue_reset.  more: a kernel over the list of tiles left out
+// follows, which decodes; list: this is that kernel.
 __device__ __forceinline__ void queue_reset_min(int32_t* counter, unsigned long long* min_key,
-                                                unsigned long long mine, double* min_out)
+                                                unsigned long long mine, double* min_out, int blocks,
+                                                bool more = false, bool list = false)
 {
     if (threadIdx.x == 0) {
         if (min_out) atomicMin(min_key, mine);
         __threadfence();
-        if (atomicAdd(counter + 1, 1) == (int)gridDim.x - 1) {
-            if (min_out) {
+        if (atomicAdd(counter + 1, 1) == blocks - 1) {
+            if (min_out && !more) {
                 __threadfence();
                 const unsigned long long k = atomicAdd(min_key, 0ull);
                 *min_out = (k == ~0ull) ? INFINITY : order_unkey(k);
@@ -129,6 +143,7 @@ __device__ __forceinline__ void queue_reset_min(int32_t* counter, unsigned long 
             }
             counter[0] = 0;
             counter[1] = 0;
+            if (list) counter[2] = 0;
         }
     }
 }
@@ -478,6 +493,7 @@ struct cse_ctx {
     uint2* bk_bits;         // basket design: a bit per count state and arm, Q_i below each level of S; the last
                             // level is the call's lambda (k_basket_bits)
     float4* bk_q;           // basket design: (1 - P(theta_i > t_i | x)) per count state (see sim_basket.cu)
+    int32_t* left;          // [tile_cap] tiles that a candidate kernel leaves to the kernel after it (counter[2] of them)
     uint32_t* keys;         // per-CTA statistic keys for order-statistic selection
     size_t keys_cap;
 

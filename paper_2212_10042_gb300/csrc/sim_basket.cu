@@ -180,8 +180,16 @@ __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B,
 // the least one above the k_i smallest S as far as the first kSample trials (all
 // evaluated) tell, with a margin of 2.5 standard deviations.  Keys below L_c go to
 // the warp's stretch of global memory and into 256 bins; the k_i-th is ranked within
-// its bin.  It is exact when it is at most L_c; otherwise the pass is repeated with
-// every trial evaluated.
+// its bin.  It is exact when it is at most L_c.
+//
+// Otherwise, and where the sample shows a large share of the trials below L_c (rates far
+// from the null rates: every S near 0 or near 1, which the levels do not resolve), the
+// tile goes to a list for k_sim_basket_all, which evaluates every trial: there the counts
+// hardly vary and its gathers meet in few lines.  8^4 grid, K = 16,384, a step over logits
+// [1, 4] 837 -> 334 us (every trial through the queue before; 366 with the gathers alone),
+// [-1, 2] 1,080 -> 540 (567), [-6, -4] 612 -> 338 (409), [-3.5, 1] 358 -> 346 (812).
+// The share: a quarter against a half 536 / 612 us over [-1, 2], but n = 20 313 / 291.
+// 256 threads a tile below 4 tiles an SM: 150 tiles of 2^18 trials 1,565 -> 700 us.
 //
 // What bounds it: issue slots (65 %) and the integer pipe (64 %): per 32 trials ~17
 // warp instructions of test and count, ~10 of queue and scan, ~7 of evaluation, and
@@ -196,11 +204,13 @@ __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B,
 // ---------------------------------------------------------------------------
 constexpr int kLevels = 32;        // levels of S for selections: 2^((c + 1) / 4 - 8), the last +inf
 constexpr int kMaxM = 64;          // count states of an arm: two 32-bit words of x_3
-constexpr int NT = 128;            // threads of the tabulated kernel
 constexpr int kSample = 512;       // first trials of a tile, all evaluated to place c
 // up to this K every trial is evaluated, a trial a lane: 19,056 tiles, a step at K = 1,500 509 us
 // against 580 by bits, at 2,000 587 against 593
 constexpr int kAllK = 2048;
+// up to this K a tile that turns out dense is finished here, every trial evaluated, instead of
+// starting again in the kernel over the list (8^4 grid, a step at K = 4,096: 231 us against 241)
+constexpr int kHereK = 8192;
 constexpr int kQueue = 288;        // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
 constexpr int kList = 256;         // keys of the selected bin ranked in shared memory
 constexpr int kSpan3 = 16;         // most counts of arm 3 in the window: the bits of half a word
@@ -272,12 +282,12 @@ __device__ __forceinline__ uint32_t fold16(const uint2& h, const uint2& mk)
     return (t | (t >> 16)) & 0xFFFFu;
 }
 
-template <bool SELECT>
-__global__ void __launch_bounds__(NT, 8)
+template <bool SELECT, int NT>
+__global__ void __launch_bounds__(NT, 1024 / NT)
     k_sim_basket(TileArgs T, Basket B, const uint8_t* __restrict__ cnt, int32_t k_stride, int32_t K_tiles,
                  const float4* __restrict__ Qt, const uint2* __restrict__ planes, int32_t span, float lambda_up,
-                 bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg, int32_t* __restrict__ counter,
-                 int32_t* __restrict__ err)
+                 bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg, int32_t* __restrict__ left,
+                 int32_t* __restrict__ counter, int32_t* __restrict__ err)
 {
     constexpr int NW = NT / 32;
     constexpr int ALL = kLevels - 1;   // every trial evaluated
@@ -297,6 +307,7 @@ __global__ void __launch_bounds__(NT, 8)
     uint32_t* const kbuf = keys + ((int64_t)blockIdx.x * NW + warp) * key_seg;
     const unsigned below = (1u << lane) - 1u;
     const int m = B.m;
+    const int dense = B.n > 24 ? kSample / 4 : kSample / 2;   // (few patients: few values of S, so large steps)
     if (SELECT)
         for (int b = tid; b < 256; b += NT) hist[b] = 0u;
     if (tid == 0) {
@@ -347,7 +358,8 @@ __global__ void __launch_bounds__(NT, 8)
         int c = (sel || Kc <= kAllK) ? ALL : -1;
         int r_neg = 0, x_neg[4] = {0, 0, 0, 0};   // minus the rejections and their counts
         double lam_i = -INFINITY;
-        for (;;) {
+        bool found = false, leave = false;   // leave: to the kernel that evaluates every trial
+        do {
             int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
             const int k0 = sample ? kSample : 0;
             // bytes of P: x_3, x_2, x_1, x_0.  C1: bit 7 of a byte set iff x >= lo; C2: iff
@@ -395,10 +407,20 @@ __global__ void __launch_bounds__(NT, 8)
                     const int b = warp_pick256<false>(hist, (int)ceilf(r * r) + 1, lane, &before);
                     const bool above = b >= 0 && (lane == ALL || key_bin(__float_as_uint(basket_level(lane))) > b);
                     const unsigned who = __ballot_sync(0xffffffffu, above);   // a lane a level
-                    if (lane == 0) s_pick = who ? __ffs(who) - 1 : ALL;
+                    const int cl = who ? __ffs(who) - 1 : ALL;
+                    // the sample's keys below it: with more than dense of the trials among them the
+                    // test saves nothing
+                    const int kb = key_bin(__float_as_uint(basket_level(cl)));
+                    int nb = 0;
+#pragma unroll
+                    for (int j = 0; j < 8; ++j) nb += lane * 8 + j < kb ? (int)hist[lane * 8 + j] : 0;
+                    nb = basket_warp_sum(nb);
+                    if (lane == 0) s_pick = cl == ALL || nb > dense ? ALL : cl;
                 }
                 __syncthreads();
                 c = s_pick;
+                leave = c == ALL && Kc > kHereK;
+                if (leave) break;
                 level = basket_level(c);
             }
             if (c == ALL)   // no test: a trial a lane (k - lane is the warp's)
@@ -532,7 +554,7 @@ __global__ void __launch_bounds__(NT, 8)
             int nk = 0;
 #pragma unroll
             for (int w2 = 0; w2 < NW; ++w2) nk += s_nk[w2];
-            bool found = nk >= ks;
+            found = nk >= ks;
             if (found) {
                 if (warp == 0) {
                     int before = 0;
@@ -593,21 +615,19 @@ __global__ void __launch_bounds__(NT, 8)
                 }
                 lam_i = (double)__uint_as_float(s_res);
                 // exact unless it lies above the level of the trials left out
-                found = lam_i <= (double)basket_level(c);
+                leave = !(lam_i <= (double)basket_level(c));
             } else {
-                for (int b = tid; b < 256; b += NT) hist[b] = 0u;
                 lam_i = INFINITY;   // with every trial evaluated, the k_i-th smallest S is +inf
+                leave = c != ALL;   // too few keys below the level
             }
-            if (found || c == ALL) break;
-            // too few keys below the level: the pass again with every trial
-            c = ALL;
-            sample = false;
-            r_neg = 0;
-#pragma unroll
-            for (int a = 0; a < 4; ++a) x_neg[a] = 0;
+        } while (false);
+        if (SELECT && sel && !found) {   // (the selection clears the bins)
             __syncthreads();   // every thread has read the counts
-            if (tid == 0) s_nlist = 0;
-            __syncthreads();
+            for (int b = tid; b < 256; b += NT) hist[b] = 0u;
+        }
+        if (leave) {
+            if (tid == 0) left[atomicAdd(counter + 2, 1)] = (int32_t)i;
+            continue;
         }
         const int Rw = -basket_warp_sum(r_neg);
         int Xw[4];
@@ -623,34 +643,42 @@ __global__ void __launch_bounds__(NT, 8)
             if (SELECT) s_min = min(s_min, order_key(lam_i));
         }
     }
-    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr);
+    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr, (int)gridDim.x, left != nullptr);
 }
 
-// The plain path's form: every trial through the posterior function.  SELECT adds
+// Every trial evaluated, from the state table (the tiles that k_sim_basket leaves: one
+// 16-byte gather a trial, which costs little where the counts hardly vary) or, the
+// plain path's form, through the posterior function.  SELECT adds
 // the per-tile order statistic lambda_i = S_(ksel_i) by a three-digit radix select
 // (11, 11, 10 bits of the FP32 keys, which order like the non-negative S) over the
 // keys the CTA stored.
-template <bool SELECT>
-__global__ void __launch_bounds__(BT, 4) k_sim_basket_direct(TileArgs T, Basket B, const uint8_t* __restrict__ cnt,
-                                                             int32_t k_stride, int32_t K_tiles, float lambda_up,
-                                                             SimOut o, uint32_t* __restrict__ keys,
-                                                             int32_t* __restrict__ counter, int32_t* __restrict__ err)
+template <bool TABLE, bool SELECT>
+__global__ void __launch_bounds__(BT, 4)
+    k_sim_basket_all(TileArgs T, Basket B, const uint8_t* __restrict__ cnt, int32_t k_stride, int32_t K_tiles,
+                     const float4* __restrict__ Qt, float lambda_up, SimOut o, uint32_t* __restrict__ keys,
+                     const int32_t* __restrict__ list, int32_t* __restrict__ counter, int32_t* __restrict__ err)
 {
+    pdl_entry();
+    int blocks;
+    const int64_t n_todo = queue_tiles(list, counter, T.n_tiles, &blocks);
+    if ((int)blockIdx.x >= blocks) return;
     __shared__ uint32_t hist[2048];
     __shared__ int s_tile, s_scan[BWARP], s_res[2];
     __shared__ int s_red[5][BWARP];
     __shared__ unsigned long long s_min;   // order key of the least lambda_i of this CTA's tiles
     if (threadIdx.x == 0) s_min = ~0ull;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const NodeConst C = node_const();
+    NodeConst C;
+    if (!TABLE) C = node_const();
     uint32_t* kbuf = keys + (int64_t)blockIdx.x * k_stride;
     for (;;) {
         if (tid == 0) s_tile = atomicAdd(counter, 1);
         if (SELECT)
             for (int b = tid; b < 2048; b += BT) hist[b] = 0u;
         __syncthreads();
-        const int64_t i = s_tile;
-        if (i >= T.n_tiles) break;
+        const int64_t turn = s_tile;
+        if (turn >= n_todo) break;
+        const int64_t i = list ? (int64_t)list[turn] : turn;
         const int K = T.K[i];
         bool bad = (K < 1) || (K > K_tiles);
         int v[4];
@@ -679,7 +707,7 @@ __global__ void __launch_bounds__(BT, 4) k_sim_basket_direct(TileArgs T, Basket 
 #pragma unroll
                     for (int a = 0; a < 4; ++a)
                         x[a] = min((int)(((j < 4 ? w[a].x : w[a].y) >> (8 * (j & 3))) & 0xFFu), B.n);
-                    q[j] = state_q<false>(nullptr, B, C, x);
+                    q[j] = state_q<TABLE>(Qt, B, C, x);
                 }
             }
             uint32_t kq[SPT];
@@ -742,7 +770,7 @@ __global__ void __launch_bounds__(BT, 4) k_sim_basket_direct(TileArgs T, Basket 
         }
         __syncthreads();
     }
-    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr);
+    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr, blocks, false, list != nullptr);
 }
 
 template <bool TABLE>
@@ -808,7 +836,7 @@ int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64
     return CSE_OK;
 }
 
-template <bool SEL>
+template <bool SEL, int NT>
 int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_tiles, double lambda, const SimOut& o,
                   cudaStream_t s)
 {
@@ -818,11 +846,17 @@ int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_til
     const Basket B = make_basket(c->D);
     const int span = basket_span(B.n), rows = B.m * B.m * B.m;
     // the words of the widest window, w_0 w_1 w_2 <= span^3, and word 0: at most 42,596 bytes (n = 63:
-    // span 22), with the static arrays below the default limit of 48 KB
+    // span 22), with the static arrays of 128 threads below the default limit of 48 KB, of 256 above
     const size_t smem = ((size_t)span * span * span + 1) * sizeof(uint32_t);
+    if (NT > 128 && smem > 40 * 1024 &&   // one limit for every design: it belongs to the kernel
+        cudaFuncSetAttribute(k_sim_basket<SEL, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 42 * 1024) !=
+            cudaSuccess) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
     const float lam = lambda_float_up(lambda);
     const bool want_R = o.R || o.Xrej || o.score || o.cp_key;
-    const int st = basket_grid(c, k_sim_basket<SEL>, NT, smem, T.n_tiles, SEL ? (int64_t)(NT / 32) * key_seg : 0, &grid);
+    const int st = basket_grid(c, k_sim_basket<SEL, NT>, NT, smem, T.n_tiles, SEL ? (int64_t)(NT / 32) * key_seg : 0, &grid);
     if (st != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
@@ -831,10 +865,24 @@ int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_til
         k_basket_bits<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(c->bk_bits, c->bk_q, B.m, rows, kLevels, 1, lam);
         c->launches += 1;
     }
-    k_sim_basket<SEL><<<(unsigned)grid, NT, smem, s>>>(T, B, c->cnt, k_stride, K_tiles, c->bk_q, c->bk_bits, span, lam,
-                                                      want_R, o, c->keys, key_seg, c->counter, c->err);
-    cse_prof_end(c, s);
+    // selections over more than kAllK trials leave the tiles without use for a test
+    int32_t* left = SEL && K_tiles > kAllK ? c->left : nullptr;
+    k_sim_basket<SEL, NT><<<(unsigned)grid, NT, smem, s>>>(T, B, c->cnt, k_stride, K_tiles, c->bk_q, c->bk_bits, span,
+                                                          lam, want_R, o, c->keys, key_seg, left, c->counter, c->err);
     c->launches += 1;
+    if (left) {   // a block's keys hold at least k_stride words
+        int per_sm = 0;
+        auto all = k_sim_basket_all<true, SEL>;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, all, BT, 0) != cudaSuccess || per_sm < 1) {
+            cudaGetLastError();
+            return CSE_CUDA_ERROR;
+        }
+        if (grid > (int64_t)per_sm * c->num_sms) grid = (int64_t)per_sm * c->num_sms;
+        cse_launch(true, all, dim3((unsigned)grid), dim3(BT), 0, s, T, B, c->cnt, k_stride, K_tiles, c->bk_q, lam, o,
+                   c->keys, left, c->counter, c->err);
+        c->launches += 1;
+    }
+    cse_prof_end(c, s);
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
 }
 
@@ -843,13 +891,14 @@ int launch_basket_direct(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_
                          const SimOut& o, cudaStream_t s)
 {
     int64_t grid = 0;
-    const int st = basket_grid(c, k_sim_basket_direct<SEL>, BT, 0, T.n_tiles, SEL ? k_stride : 0, &grid);
+    const int st = basket_grid(c, k_sim_basket_all<false, SEL>, BT, 0, T.n_tiles, SEL ? k_stride : 0, &grid);
     if (st != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
     cse_prof_begin(c, KID_SIM_BASKET, s);
-    k_sim_basket_direct<SEL><<<(unsigned)grid, BT, 0, s>>>(T, make_basket(c->D), c->cnt, k_stride, K_tiles,
-                                                          lambda_float_up(lambda), o, c->keys, c->counter, c->err);
+    k_sim_basket_all<false, SEL><<<(unsigned)grid, BT, 0, s>>>(T, make_basket(c->D), c->cnt, k_stride, K_tiles, nullptr,
+                                                              lambda_float_up(lambda), o, c->keys, nullptr, c->counter,
+                                                              c->err);
     cse_prof_end(c, s);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
@@ -900,9 +949,14 @@ int cse_launch_sim_basket(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_s
 {
     (void)NA;
     const bool sel = (o.lam_tile != nullptr && o.ksel != nullptr);
-    if (c->bt_tables && !c->bt_direct)
-        return sel ? launch_basket<true>(c, T, k_stride, K_tiles, lambda, o, s)
-                   : launch_basket<false>(c, T, k_stride, K_tiles, lambda, o, s);
+    if (c->bt_tables && !c->bt_direct) {
+        // 256 threads a tile while there are too few tiles to fill the SMs with blocks of 128
+        if (T.n_tiles <= 4 * (int64_t)c->num_sms)
+            return sel ? launch_basket<true, 256>(c, T, k_stride, K_tiles, lambda, o, s)
+                       : launch_basket<false, 256>(c, T, k_stride, K_tiles, lambda, o, s);
+        return sel ? launch_basket<true, 128>(c, T, k_stride, K_tiles, lambda, o, s)
+                   : launch_basket<false, 128>(c, T, k_stride, K_tiles, lambda, o, s);
+    }
     return sel ? launch_basket_direct<true>(c, T, k_stride, K_tiles, lambda, o, s)
                : launch_basket_direct<false>(c, T, k_stride, K_tiles, lambda, o, s);
 }

@@ -982,7 +982,7 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
     unsigned long long mine = ~0ull;
     if (tid == 0)
         for (int q = 0; q < G; ++q) mine = min(mine, s_min[q]);
-    queue_reset_min(counter, o.min_key, mine, SELECT ? o.min_out : nullptr);
+    queue_reset_min(counter, o.min_key, mine, SELECT ? o.min_out : nullptr, (int)gridDim.x);
 }
 
 // The direct form (plain path, CSE_OPT_BAYES_DIRECT, and designs whose tables
@@ -1116,7 +1116,7 @@ __global__ void __launch_bounds__(BT, 5)
         }
         __syncthreads();
     }
-    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr);
+    queue_reset_min(counter, o.min_key, s_min, SELECT ? o.min_out : nullptr, (int)gridDim.x);
 }
 
 template <bool TABLES>

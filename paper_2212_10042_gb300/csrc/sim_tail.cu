@@ -567,7 +567,7 @@ __global__ void __launch_bounds__(kTailThreads, 4)
     unsigned long long mine = ~0ull;
     if (tid == 0)
         for (int q = 0; q < G; ++q) mine = min(mine, s_min[q]);
-    queue_reset_min(counter, o.min_key, mine, o.min_out);
+    queue_reset_min(counter, o.min_key, mine, o.min_out, (int)gridDim.x);
 }
 
 template <bool WORDS, int G>

@@ -571,7 +571,7 @@ __global__ void __launch_bounds__(NT, cells_min_blocks<NT>(G)) k_sim_cells(
     unsigned long long mine = ~0ull;
     if (tid == 0)
         for (int q = 0; q < G; ++q) mine = min(mine, s_min[q]);
-    queue_reset_min(counter, o.min_key, mine, SELECT ? o.min_out : nullptr);
+    queue_reset_min(counter, o.min_key, mine, SELECT ? o.min_out : nullptr, (int)gridDim.x);
 }
 
 // Statistic of every (tile, sim): S_out[off[i] + k] (testing and export).
