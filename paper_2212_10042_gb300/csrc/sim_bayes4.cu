@@ -433,6 +433,17 @@ __device__ __forceinline__ float design_stat_packed(const Looks& L, const Packed
     return use == 0u ? INFINITY : 1.0f - pm;
 }
 
+// Four words of four trials each, an arm a word, to a word a trial, an arm a byte.
+__device__ __forceinline__ void transpose4(const uint32_t in[4], uint32_t out[4])
+{
+    const uint32_t t0 = __byte_perm(in[0], in[1], 0x5140u), t1 = __byte_perm(in[2], in[3], 0x5140u);
+    const uint32_t t2 = __byte_perm(in[0], in[1], 0x7362u), t3 = __byte_perm(in[2], in[3], 0x7362u);
+    out[0] = __byte_perm(t0, t1, 0x5410u);
+    out[1] = __byte_perm(t0, t1, 0x7632u);
+    out[2] = __byte_perm(t2, t3, 0x5410u);
+    out[3] = __byte_perm(t2, t3, 0x7632u);
+}
+
 __device__ __forceinline__ int warp_sum_i(int v)
 {
 #pragma unroll
@@ -542,13 +553,19 @@ __device__ __forceinline__ void packed_tables(int tid, int nth, int* tri, uint32
 // Keys go to the CTA's own stretch of global memory (4 % of the trials) and into
 // 256 bins of 1/16 octave; the order statistic is ranked within its bin.
 //
-// What bounds it: issue slots at the latency of the candidates' scattered reads
-// (47 % issue, 52 % ALU pipe, 62 warp instructions per 32 trials of which the
-// candidates take four fifths).  262,144 refined tiles x 65,536 trials:
-// 103 -> 40 ms; the 16^4 grid at K = 2^14: 5.6 -> 2.2 ms.  Measured on the way:
-// evaluating every candidate by raw counts with a margin fixed by the sample 65
-// ms, with d raised along the pass 51 ms; final-table loads that skip L1 lost
-// 10 %.
+// A warp of whose 512 trials of a step more than kDense are candidates evaluates all of
+// them, a lane four consecutive trials from whole count words: no queue, no scattered
+// bytes (a candidate costs about twice a trial read that way).
+//
+// What bounds it: issue slots at the latency of the candidates' scattered reads (65 %
+// issue, 61 % ALU pipe, 69 warp instructions per 32 trials of which the candidates,
+// ~290 each, take four fifths).  262,144 refined tiles x 65,536 trials: 103 -> 38 ms; the
+// 16^4 grid at K = 2^14: 5.6 -> 1.9 ms.  Measured on the way: evaluating every candidate
+// by raw counts with a margin fixed by the sample 65 ms, with d raised along the pass
+// 51 ms; final-table loads that skip L1 lost 10 %.  Levels that make most trials
+// candidates, 8^4 grid at K = 2^14, the whole call (every trial in a straight line / all
+// through the queue / now): validation at lambda = 1 570 / 616 / 475 us, calibration at
+// alpha = 0.3 530 / 568 / 471, at 0.5 534 / 635 / 540.
 //
 // Tiles: a group of NT / G threads per tile (named barriers), G tiles a block;
 // G = 1 only when there are too few tiles to give every group one.
@@ -558,6 +575,7 @@ constexpr int kSample = 512;     // first trials of a tile, all evaluated to pla
 constexpr int kAllK = 1024;      // up to this K every trial is evaluated
 constexpr int kQueue = 288;      // a warp's candidate queue (up to 31 left over, at least 16 lanes' trials a round)
 constexpr int kList = 256;       // keys of the selected bin ranked in shared memory
+constexpr int kDense = 320;      // candidates among a warp's 512 trials of a step from which all are evaluated
 
 // dmin[D + u(n3)] (float bits, preset to +inf) = the least S an active treatment
 // with final score difference D to the control can give, over every state of the
@@ -607,8 +625,8 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
     k_sim_bayes4(TileArgs T, Looks L, const uint8_t* __restrict__ cnt, int32_t NA, int32_t k_stride, int32_t K_tiles,
                  const uint8_t* __restrict__ D1g, const uint8_t* __restrict__ D2, const float4* __restrict__ F4,
                  const uint8_t* __restrict__ score, const uint32_t* __restrict__ dmin, int32_t top, int32_t dlo,
-                 int32_t nd, float lambda_up, bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg, int32_t* __restrict__ counter, int32_t* __restrict__ err,
-                 const PackedConst Q, const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
+                 int32_t nd, float lambda_up, bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg,
+                 int32_t* __restrict__ counter, int32_t* __restrict__ err, const PackedConst Q, const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
 {
     constexpr int NT = b4_threads<PACKED>();
     constexpr int TT = b4_group<PACKED, G>();
@@ -633,7 +651,8 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
     uint32_t* const hists = reinterpret_cast<uint32_t*>(smem + d1_bytes + d2s_bytes);
     uint32_t* const hist = hists + g * 256;
     uint32_t* const list = hists + G * 256 + (SELECT ? g * kList : 0);
-    uint16_t* const queue = reinterpret_cast<uint16_t*>(hists + G * 256 + (SELECT ? G * kList : 0)) + (tid >> 5) * kQueue;
+    uint16_t* const queue =
+        reinterpret_cast<uint16_t*>(hists + G * 256 + (SELECT ? G * kList : 0)) + (tid >> 5) * kQueue;
     // each warp appends its keys to its own stretch of key_seg words
     uint32_t* const kgrp = keys + (int64_t)(blockIdx.x * G + g) * NW * key_seg;
     uint32_t* const kbuf = kgrp + (int64_t)warp * key_seg;
@@ -710,6 +729,37 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
             float sigma = s_sig[e];
             int qn = 0, wk = 0;   // queued candidates, kept keys of this warp
             uint32_t a02 = 0u, a13 = 0u, waves = 0u;
+            // a trial's S, its final counts (bytes P2, or xf) and whether the lane has one
+            auto account = [&](float S, uint32_t P2, const int* xf, bool live) {
+                if (!live) S = INFINITY;
+                const uint32_t rej = (S < lambda_up) ? 1u : 0u;
+                r_acc += (int)rej;
+                if (PACKED) {
+                    a02 += (P2 & 0x00FF00FFu) * rej;
+                    a13 += __byte_perm(P2, 0u, 0x4341u) * rej;
+                    if ((++waves & 127u) == 0u) {   // 16-bit halves: 128 x 255 < 2^16
+                        xs[0] += (int)(a02 & 0xFFFFu);
+                        xs[2] += (int)(a02 >> 16);
+                        xs[1] += (int)(a13 & 0xFFFFu);
+                        xs[3] += (int)(a13 >> 16);
+                        a02 = a13 = 0u;
+                    }
+                } else {
+#pragma unroll
+                    for (int a = 0; a < 4; ++a) xs[a] += (int)rej * xf[a];
+                }
+                if (SELECT) {
+                    const bool keep = S < sigma;
+                    const unsigned kept = __ballot_sync(0xffffffffu, keep);
+                    if (ks >= 1) {
+                        if (keep) {
+                            kbuf[wk + __popc(kept & below)] = __float_as_uint(S);
+                            atomicAdd(&hist[key_bin(__float_as_uint(S))], 1u);
+                        }
+                        wk += __popc(kept);
+                    }
+                }
+            };
             // step -1 of a first pass: the sample, spread over the warps; then sixteen
             // consecutive trials per thread and step from k0 on.  Bit 8 j + q of a
             // thread's candidate word is trial 4 q + j.
@@ -746,14 +796,59 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
                     }
                     if (kw + 16 > kend) m &= trials_below(kend - kw);   // trials at or past K
                 }
-                const int nm = __popc(m);
-                int incl = nm;
+                int nm = __popc(m), incl = nm;
 #pragma unroll
                 for (int off = 1; off < 32; off <<= 1) {
                     const int y = __shfl_up_sync(0xffffffffu, incl, off);
                     if (lane >= off) incl += y;
                 }
-                const int total = __shfl_sync(0xffffffffu, incl, 31);
+                int total = __shfl_sync(0xffffffffu, incl, 31);
+                if (total > kDense) {   // most of the warp's trials: all of them, from whole count words
+                    const int k0w = kw - lane * 16;
+#pragma unroll 1
+                    for (int k4 = k0w + lane * 4; k4 - lane * 4 < min(k0w + 512, kend); k4 += 128) {
+                        const Off at = (Off)min(k4, (Kc - 1) & ~3);   // (its four lie in the row)
+                        uint32_t wf[4], wi[PACKED ? 4 : 8];
+#pragma unroll
+                        for (int a = 0; a < 4; ++a) {
+                            wf[a] = __ldg(reinterpret_cast<const uint32_t*>(cnt + (Off)(row[a] + at)));
+                            wi[a] = __ldg(reinterpret_cast<const uint32_t*>(cnt + (Off)(row[a] + at - plane)));
+                            if constexpr (!PACKED)
+                                wi[4 + a] =
+                                    __ldg(reinterpret_cast<const uint32_t*>(cnt + (Off)(row[a] + at - 2 * plane)));
+                        }
+                        if constexpr (PACKED) {
+                            uint32_t E[4], F[4];
+                            transpose4(wi, E);
+                            transpose4(wf, F);
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) {
+                                const uint32_t P0 = (E[j] >> 4) & 0x0F0F0F0Fu, P1 = P0 + (E[j] & 0x0F0F0F0Fu);
+                                const uint32_t P2 = (uint32_t)s_inv[F[j] & 0x7Fu] |
+                                                    (uint32_t)s_inv[(F[j] >> 8) & 0x7Fu] << 8 |
+                                                    (uint32_t)s_inv[(F[j] >> 16) & 0x7Fu] << 16 |
+                                                    (uint32_t)s_inv[(F[j] >> 24) & 0x7Fu] << 24;
+                                account(design_stat_packed(L, Q, smem, D2s, F4, s_tri, s_perm, P0, P1, P2, mask), P2,
+                                        nullptr, k4 + j < kend);
+                            }
+                        } else {
+#pragma unroll 1
+                            for (int j = 0; j < 4; ++j) {
+                                int xl[3][4];
+#pragma unroll
+                                for (int a = 0; a < 4; ++a) {
+                                    xl[0][a] = (int)((wi[4 + a] >> (8 * j)) & 0xFFu);
+                                    xl[1][a] = (int)((wi[a] >> (8 * j)) & 0xFFu);
+                                    xl[2][a] = (int)((wf[a] >> (8 * j)) & 0xFFu);
+                                }
+                                const NodeConst C{};   // not read by the tabulated form
+                                account(design_stat<true>(L, D1g, D2, F4, C, 0.0f, xl, mask), 0u, xl[2], k4 + j < kend);
+                            }
+                        }
+                    }
+                    m = 0u;
+                    nm = incl = total = 0;
+                }
                 const bool flush = (st & 63) == 63 || k0 + (st + 1) * (TT * 16) >= Kc;
                 const int ent = (stq << 10) | (lane << 5);   // entry: step (6 bits), lane, bit
                 int done = 0;   // candidates of this step queued so far
@@ -796,40 +891,14 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
 #pragma unroll
                             for (int l = 0; l < 3; ++l)
 #pragma unroll
-                                for (int a = 0; a < 4; ++a) xl[l][a] = (int)__ldg(cnt + (Off)(row[a] + k - (Off)(2 - l) * plane));
+                                for (int a = 0; a < 4; ++a)
+                                    xl[l][a] = (int)__ldg(cnt + (Off)(row[a] + k - (Off)(2 - l) * plane));
 #pragma unroll
                             for (int a = 0; a < 4; ++a) xf[a] = xl[2][a];
                             const NodeConst C{};   // not read by the tabulated form
                             S = design_stat<true>(L, D1g, D2, F4, C, 0.0f, xl, mask);
                         }
-                        if (lane >= n) S = INFINITY;
-                        const uint32_t rej = (S < lambda_up) ? 1u : 0u;
-                        r_acc += (int)rej;
-                        if (PACKED) {
-                            a02 += (P2 & 0x00FF00FFu) * rej;
-                            a13 += __byte_perm(P2, 0u, 0x4341u) * rej;
-                            if ((++waves & 127u) == 0u) {   // 16-bit halves: 128 x 255 < 2^16
-                                xs[0] += (int)(a02 & 0xFFFFu);
-                                xs[2] += (int)(a02 >> 16);
-                                xs[1] += (int)(a13 & 0xFFFFu);
-                                xs[3] += (int)(a13 >> 16);
-                                a02 = a13 = 0u;
-                            }
-                        } else {
-#pragma unroll
-                            for (int a = 0; a < 4; ++a) xs[a] += (int)rej * xf[a];
-                        }
-                        if (SELECT) {
-                            const bool keep = S < sigma;
-                            const unsigned kept = __ballot_sync(0xffffffffu, keep);
-                            if (ks >= 1) {
-                                if (keep) {
-                                    kbuf[wk + __popc(kept & below)] = __float_as_uint(S);
-                                    atomicAdd(&hist[key_bin(__float_as_uint(S))], 1u);
-                                }
-                                wk += __popc(kept);
-                            }
-                        }
+                        account(S, P2, xf, lane < n);
                         __syncwarp();   // the queue's entries read before the next round writes
                     }
                 } while (done < total);
@@ -882,6 +951,7 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
                 }
                 tile_sync<TT, G>(g);
                 const int B = s_pick[g], kr = ks - s_before[g];
+#pragma unroll 4
                 for (int k = lane; k < wk; k += 32) {   // each warp its own keys
                     const uint32_t key = kbuf[k];
                     if (key_bin(key) == B) {
@@ -908,6 +978,7 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
                     for (int pass = 0; pass < 4; ++pass) {
                         const int sh = pass < 3 ? 23 - 8 * pass : 0;
                         const uint32_t dm = pass < 3 ? 0xFFu : 0x7Fu;
+#pragma unroll 4
                         for (int k = lane; k < wk; k += 32) {
                             const uint32_t key = kbuf[k];
                             if (key_bin(key) == B && (key & pmask) == prefix) atomicAdd(&hist[(key >> sh) & dm], 1u);
