@@ -991,10 +991,15 @@ __device__ __forceinline__ Mat2<T> mat2_first(const Mat2<T>& A, unsigned mask)
 // the composition of the maps applied to t = 0: with Q the product of their
 // matrices, Q01 / Q11.  In FP64 a step is multiplied through by (a+2n-1)^2
 // (a+2n+1) instead of divided (a common factor does not change the map); in FP32
-// it is scaled by a + 2n, which keeps the entries in range.  The convergents close
-// in geometrically, so a half-depth difference of 1e-9 (FP32: 1e-3) leaves the
-// full depth at rounding; one pass does at the usual delta, more are needed as u
-// nears the mean.
+// it is scaled by a + 2n, which keeps the entries in range.  The even contraction of a
+// continued fraction: Jones and Thron, Continued Fractions (1980), ch. 2.
+// The convergents close in geometrically, so in the first pass a difference of 1e-9
+// (FP32: 1e-3) between half and full depth leaves the full depth at rounding (5e-16
+// at most, in extended precision, over N = 100 .. 2^20 and delta = 1e-6 .. 0.999); one pass
+// does at the usual delta.  As u nears the mean more are needed, and from the second
+// pass on the two depths compared are 24 steps apart in 72 and more, so the
+// difference has to be at rounding itself (1e-14 there leaves 4e-16; 1e-9 left 7e-11 at
+// N = 2^20, delta = 0.5).
 template <typename T, int L>
 __device__ T beta_cf_group(T a, T b, T x, T lam, int l, unsigned mask)
 {
@@ -1043,7 +1048,7 @@ __device__ T beta_cf_group(T a, T b, T x, T lam, int l, unsigned mask)
         P = mat2_first<T, L>(P, mask);
         const T f_mid = __shfl_sync(mask, Ph.m01 / Ph.m11, 0, L);
         f = P.m01 / P.m11;
-        if (!(fabs(f - f_mid) > (T)(F64 ? 1e-9 : 1e-3) * fabs(f))) break;
+        if (!(fabs(f - f_mid) > (T)(F64 ? (pass == 0 ? 1e-9 : 1e-14) : 1e-3) * fabs(f))) break;
     }
     return f;
 }
@@ -1135,18 +1140,17 @@ __device__ T log_tail_sum(int R, T N, T u, bool upper, T* r, int l, unsigned mas
 
 // One Halley step on phi(u) = log tail - target from f = phi(u): phi' = -r (upper)
 // or r, phi'' = phi' ((a-1)/u - (b-1)/(1-u)) - r^2; kept inside the bracket (lo,
-// hi), which the sign of f narrows.  The second-order term in FP32: it enters
-// times f.
+// hi), which the sign of f narrows.
 template <typename T>
 __device__ __forceinline__ T cp_halley(T u, T f, T r, T a, T b, bool upper, T* lo, T* hi)
 {
     const T p1 = upper ? -r : r;
-    const float uf = (float)u, pf = (float)p1;
-    const float p2 = pf * (((float)a - 1.0f) / uf - ((float)b - 1.0f) / (1.0f - uf)) - pf * pf;
-    const T den = (T)2 * p1 * p1 - f * (T)p2;
+    // (numerator and denominator times u (1 - u): one division)
+    const T v = u * ((T)1 - u), p2v = p1 * ((a - (T)1) - (a + b - (T)2) * u) - p1 * p1 * v;
+    const T den = (T)2 * p1 * p1 * v - f * p2v;
     if ((f > (T)0) == upper) *lo = u;
     else *hi = u;
-    const T un = u - (T)2 * f * p1 / den;
+    const T un = u - (T)2 * f * p1 * v / den;
     return (un >= *lo && un <= *hi) ? un : (T)0.5 * (*lo + *hi);
 }
 
@@ -1195,7 +1199,8 @@ __device__ double cp_upper_group(int64_t R, int64_t N, double delta, double comp
         ud = __shfl_sync(mask, un, 0, L);
         // far on the wrong side of the mean the fraction loses its sign: the serial solve
         if (!(__shfl_sync(mask, r, 0, L) > 0.0)) return cp_upper_serial(R, N, delta);
-        if (!(step > 2e-5 * fmin((double)sd, fmin(ud, 1.0 - ud))) || hi - lo <= 4e-16 * hi) break;
+        // Halley's error is at most 0.12 step^3 / sd^2 (largest at delta = 1/2): below 1e-16 of u
+        if (!(step > fmin(2e-5 * (double)sd, 3e-6 * fmin(ud, 1.0 - ud))) || hi - lo <= 4e-16 * hi) break;
     }
     return ud;
 }
