@@ -44,11 +44,11 @@ cudaEvent_t prof_event(cse_ctx* c)
     return e;
 }
 
-int grow(void** p, size_t* cap, size_t bytes)
+int grow(cse_ctx* c, void** p, size_t* cap, size_t bytes)
 {
     if (bytes <= *cap && *p) return CSE_OK;
     if (*p) {
-        cudaFree(*p);
+        cse_release(c, *p);
         *p = nullptr;
         *cap = 0;
     }
@@ -97,19 +97,19 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
     P->K_tiles = t->K_max;
     P->k_stride = (t->K_max + 15) / 16 * 16;
 
-    CSE_TRY(grow((void**)&c->thr, &c->thr_cap, sizeof(uint32_t) * (size_t)na));
-    CSE_TRY(grow((void**)&c->sig, &c->sig_cap, sizeof(double) * (size_t)na));
+    CSE_TRY(grow(c, (void**)&c->thr, &c->thr_cap, sizeof(uint32_t) * (size_t)na));
+    CSE_TRY(grow(c, (void**)&c->sig, &c->sig_cap, sizeof(double) * (size_t)na));
     // (two arms: arm 0's values have a second row in ZMODE_COUNT)
     const size_t cnt_rows = (size_t)c->D.n_looks * (size_t)na +
                             (c->D.stat == CSE_STAT_TWO_ARM_POOLED_Z ? (size_t)t->n_axis[0] : 0);
     const size_t cnt_bytes = cnt_rows * (size_t)P->k_stride;
-    CSE_TRY(grow((void**)&c->cnt, &c->cnt_cap, cnt_bytes));
-    CSE_TRY(grow((void**)&c->bb, &c->bb_cap, sizeof(uint32_t) * 2 * (size_t)na));
+    CSE_TRY(grow(c, (void**)&c->cnt, &c->cnt_cap, cnt_bytes));
+    CSE_TRY(grow(c, (void**)&c->bb, &c->bb_cap, sizeof(uint32_t) * 2 * (size_t)na));
     if ((size_t)t->n_tiles > c->tile_cap) {
-        cudaFree(c->ksel);
-        cudaFree(c->aprime);
-        cudaFree(c->lam_tile);
-        cudaFree(c->R);
+        cse_release(c, c->ksel);
+        cse_release(c, c->aprime);
+        cse_release(c, c->lam_tile);
+        cse_release(c, c->R);
         c->ksel = c->left = nullptr;
         c->aprime = c->lam_tile = nullptr;
         c->R = nullptr;
@@ -126,10 +126,10 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
     if (c->cp_cap < 2 * (uint64_t)t->n_tiles) {
         uint64_t cap = 1024;
         while (cap < 2 * (uint64_t)t->n_tiles) cap <<= 1;
-        cudaFree(c->cp_key);
-        cudaFree(c->cp_val);
-        cudaFree(c->cp_slot);
-        cudaFree(c->cp_list);
+        cse_release(c, c->cp_key);
+        cse_release(c, c->cp_val);
+        cse_release(c, c->cp_slot);
+        cse_release(c, c->cp_list);
         c->cp_key = nullptr;
         c->cp_val = nullptr;
         c->cp_slot = nullptr;
@@ -159,6 +159,7 @@ int prepare_args(cse_ctx* c, const cse_tiles* t, Prepared* P, bool geom = true)
 // after a new key; what else it runs may ask for the counts as well.
 int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = false)
 {
+    cse_capturing(c, s);
     CSE_TRY(cse_launch_thresholds(c, P.T, P.NA, s));
     if (c->plain && !cse_posterior_design(c->D.stat)) {
         if (!c->U) {
@@ -204,6 +205,13 @@ void choose_zmode(cse_ctx* c, bool want_R, double lambda, bool select, double al
     }
 }
 
+// Candidates need key scratch; the cell histogram none: it takes the call when that
+// cannot be had (memory short, or a capture with too little reserved before).
+void tail_or_cells(cse_ctx* c, const Prepared& P, bool words, cudaStream_t s)
+{
+    if (c->zmode == ZMODE_TAIL && cse_tail_reserve(c, P.T, P.K_tiles, words, s) != CSE_OK) c->zmode = ZMODE_CELLS;
+}
+
 int prepare(cse_ctx* c, const cse_tiles* t, cudaStream_t s, Prepared* P, bool geom = true, bool counts = false)
 {
     CSE_TRY(prepare_args(c, t, P, geom));
@@ -242,6 +250,47 @@ int sim_pass(cse_ctx* c, const Prepared& P, double lambda, const SimOut& o, cuda
 }
 
 }  // namespace
+
+// A captured graph holds the addresses of the scratch it was captured with, so what grows
+// later keeps the old buffer: a call after it (other tiles, another form) may need more.
+void cse_release(cse_ctx* c, void* p)
+{
+    if (!p) return;
+    Retired* r = c->captured ? new (std::nothrow) Retired{p, c->retired} : nullptr;
+    if (r) c->retired = r;
+    else if (!c->captured) cudaFree(p);   // (no memory for the record: the buffer stays)
+}
+
+bool cse_capturing(cse_ctx* c, cudaStream_t s)
+{
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &st) != cudaSuccess) cudaGetLastError();
+    if (st == cudaStreamCaptureStatusNone) return false;
+    c->captured = true;
+    return true;
+}
+
+int cse_reserve_keys(cse_ctx* c, size_t bytes, int64_t* grid, cudaStream_t s)
+{
+    const int64_t most = std::max<int64_t>(1, (int64_t)(kKeyBytesMax / bytes));
+    *grid = std::min(*grid, most);
+    if (bytes * (size_t)*grid <= c->keys_cap) return CSE_OK;
+    if (cse_capturing(c, s)) {
+        *grid = (int64_t)(c->keys_cap / bytes);
+        return *grid >= 1 ? CSE_OK : CSE_OOM;
+    }
+    cse_release(c, c->keys);
+    c->keys = nullptr;
+    c->keys_cap = 0;
+    for (;; *grid = (*grid + 1) / 2) {   // memory short: fewer blocks
+        if (cudaMalloc(&c->keys, bytes * (size_t)*grid) == cudaSuccess) break;
+        cudaGetLastError();
+        c->keys = nullptr;
+        if (*grid == 1) return CSE_OOM;
+    }
+    c->keys_cap = bytes * (size_t)*grid;
+    return CSE_OK;
+}
 
 void cse_prof_begin(cse_ctx* c, int kid, cudaStream_t s)
 {
@@ -619,6 +668,12 @@ int cse_destroy(cse_ctx* c)
     cudaFree(c->bk_q);
     cudaFree(c->bk_bits);
     cudaFree(c->keys);
+    while (c->retired) {
+        Retired* r = c->retired;
+        c->retired = r->next;
+        cudaFree(r->p);
+        delete r;
+    }
     cudaFree(c->counter);
     cudaFree(c->err);
     cudaFree(c->lam_dev);
@@ -786,6 +841,7 @@ int cse_calibrate_rand(cse_ctx* c, const cse_tiles* t, double alpha, double* alp
     choose_zmode(c, false, INFINITY, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
+    tail_or_cells(c, P, true, s);
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s, nullptr, true));
     SimOut o = {c->sig, nullptr, nullptr, nullptr, lambda_tile_out, c->ksel};
     if (c->zmode == ZMODE_TAIL) CSE_TRY(cse_launch_sim_tail(c, P.T, P.NA, P.k_stride, P.K_tiles, o, true, c_tile_out, s));
@@ -808,6 +864,7 @@ int cse_calibrate(cse_ctx* c, const cse_tiles* t, double alpha, double* alpha_pr
     choose_zmode(c, false, INFINITY, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
+    tail_or_cells(c, P, false, s);
     double* lam_tile = lambda_tile_out ? lambda_tile_out : c->lam_tile;
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s));
     SimOut o = {c->sig, nullptr, nullptr, nullptr, lam_tile, c->ksel};
@@ -831,11 +888,12 @@ int cse_step(cse_ctx* c, const cse_tiles* t, double lambda, double delta, double
     choose_zmode(c, true, lambda, true, alpha);
     Prepared P;
     CSE_TRY(prepare_args(c, t, &P));
+    tail_or_cells(c, P, false, s);
     int64_t* R = R_out ? R_out : c->R;
     // alpha' leaves each tile's per-arm softplus terms for the bound pass
     double* geom = nullptr;
     if (!c->plain) {
-        CSE_TRY(grow((void**)&c->geom, &c->geom_cap, sizeof(double) * 3 * (size_t)P.T.d * (size_t)t->n_tiles));
+        CSE_TRY(grow(c, (void**)&c->geom, &c->geom_cap, sizeof(double) * 3 * (size_t)P.T.d * (size_t)t->n_tiles));
         geom = c->geom;
     }
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s, geom));

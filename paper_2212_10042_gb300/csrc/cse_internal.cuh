@@ -395,6 +395,12 @@ enum KernelId {
 // rejection counts, or candidates for the order statistic (sim_tail.cu).
 enum ZMode { ZMODE_CELLS = 0, ZMODE_COUNT, ZMODE_TAIL };
 
+// A scratch buffer that a captured graph may read, kept until the context is destroyed.
+struct Retired {
+    void* p;
+    Retired* next;
+};
+
 struct ProfRec {
     int kid;
     cudaEvent_t a, b;
@@ -494,8 +500,11 @@ struct cse_ctx {
                             // level is the call's lambda (k_basket_bits)
     float4* bk_q;           // basket design: (1 - P(theta_i > t_i | x)) per count state (see sim_basket.cu)
     int32_t* left;          // [tile_cap] tiles that a candidate kernel leaves to the kernel after it (counter[2] of them)
-    uint32_t* keys;         // per-CTA statistic keys for order-statistic selection
+    uint32_t* keys;         // per-CTA statistic keys for order-statistic selection (cse_reserve_keys)
     size_t keys_cap;
+    int64_t tail_grid;      // blocks of the current call's k_sim_tail (cse_tail_reserve)
+    bool captured;          // a call was captured: scratch that grows is retired, not freed
+    Retired* retired;
 
     // simulation at arbitrary points (cse_type1_error): the axis-indexed form
     // built on the device (see points.cu)
@@ -537,6 +546,14 @@ void cse_prof_end(cse_ctx* c, cudaStream_t s);
 // ---------------------------------------------------------------------------
 // Launchers implemented in the .cu files (host functions).
 // ---------------------------------------------------------------------------
+void cse_release(cse_ctx* c, void* p);   // frees a scratch buffer, or retires it
+bool cse_capturing(cse_ctx* c, cudaStream_t s);
+// The key buffer for *grid blocks of `bytes` each.  *grid falls to what kKeyBytesMax, the
+// memory left, or under capture the present buffer allows (the kernels are persistent);
+// CSE_OOM when that is not one block.
+constexpr size_t kKeyBytesMax = (size_t)5 << 29;   // 2.5 GiB: every K up to 2^20 at full occupancy but the basket's
+int cse_reserve_keys(cse_ctx* c, size_t bytes, int64_t* grid, cudaStream_t s);
+int cse_tail_reserve(cse_ctx* c, const TileArgs& T, int32_t K_tiles, bool words, cudaStream_t s);
 int cse_launch_uniforms(cse_ctx* c, cudaStream_t s);   // plain z-test path: sorted uniforms and tie-break words
 int cse_launch_tables(cse_ctx* c, cudaStream_t s);
 int cse_launch_thresholds(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, cudaStream_t s);

@@ -813,7 +813,8 @@ Basket make_basket(const DesignArgs& D)
 
 // Blocks of a launch, and the key buffer for `words` words a block.
 template <typename Kern>
-int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64_t words, int64_t* grid)
+int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64_t words, int64_t* grid,
+                cudaStream_t s)
 {
     int per_sm = 0;
     if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, nt, smem) != cudaSuccess || per_sm < 1) {
@@ -822,18 +823,7 @@ int basket_grid(cse_ctx* c, Kern kern, int nt, size_t smem, int64_t tiles, int64
     }
     *grid = (int64_t)per_sm * c->num_sms;
     if (*grid > tiles) *grid = tiles;
-    const size_t need = (size_t)*grid * (size_t)words * sizeof(uint32_t);
-    if (need > c->keys_cap) {
-        cudaFree(c->keys);
-        c->keys = nullptr;
-        c->keys_cap = 0;
-        if (cudaMalloc(&c->keys, need) != cudaSuccess) {
-            cudaGetLastError();
-            return CSE_OOM;
-        }
-        c->keys_cap = need;
-    }
-    return CSE_OK;
+    return words ? cse_reserve_keys(c, sizeof(uint32_t) * (size_t)words, grid, s) : CSE_OK;
 }
 
 template <bool SEL, int NT>
@@ -856,7 +846,8 @@ int launch_basket(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_t K_til
     }
     const float lam = lambda_float_up(lambda);
     const bool want_R = o.R || o.Xrej || o.score || o.cp_key;
-    const int st = basket_grid(c, k_sim_basket<SEL, NT>, NT, smem, T.n_tiles, SEL ? (int64_t)(NT / 32) * key_seg : 0, &grid);
+    const int st = basket_grid(c, k_sim_basket<SEL, NT>, NT, smem, T.n_tiles, SEL ? (int64_t)(NT / 32) * key_seg : 0,
+                               &grid, s);
     if (st != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
@@ -891,7 +882,7 @@ int launch_basket_direct(cse_ctx* c, const TileArgs& T, int32_t k_stride, int32_
                          const SimOut& o, cudaStream_t s)
 {
     int64_t grid = 0;
-    const int st = basket_grid(c, k_sim_basket_all<false, SEL>, BT, 0, T.n_tiles, SEL ? k_stride : 0, &grid);
+    const int st = basket_grid(c, k_sim_basket_all<false, SEL>, BT, 0, T.n_tiles, SEL ? k_stride : 0, &grid, s);
     if (st != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;

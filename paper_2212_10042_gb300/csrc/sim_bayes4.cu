@@ -626,7 +626,8 @@ __global__ void __launch_bounds__(b4_threads<PACKED>(), PACKED ? 2 : 4)
                  const uint8_t* __restrict__ D1g, const uint8_t* __restrict__ D2, const float4* __restrict__ F4,
                  const uint8_t* __restrict__ score, const uint32_t* __restrict__ dmin, int32_t top, int32_t dlo,
                  int32_t nd, float lambda_up, bool want_R, SimOut o, uint32_t* __restrict__ keys, int32_t key_seg,
-                 int32_t* __restrict__ counter, int32_t* __restrict__ err, const PackedConst Q, const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
+                 int32_t* __restrict__ counter, int32_t* __restrict__ err, const PackedConst Q,
+                 const uint32_t* __restrict__ D2sg, int32_t d1_bytes, int32_t d2s_bytes)
 {
     constexpr int NT = b4_threads<PACKED>();
     constexpr int TT = b4_group<PACKED, G>();
@@ -1271,22 +1272,6 @@ int64_t b4_d1_bytes(const Looks& L)
     return b4_round16((n + 1) / 2);
 }
 
-// Selection keys: `rows` rows of `words` words.
-int b4_grow_keys(cse_ctx* c, int64_t rows, int64_t words)
-{
-    const size_t need = (size_t)rows * (size_t)words * sizeof(uint32_t);
-    if (need <= c->keys_cap) return CSE_OK;
-    cudaFree(c->keys);
-    c->keys = nullptr;
-    c->keys_cap = 0;
-    if (cudaMalloc(&c->keys, need) != cudaSuccess) {
-        cudaGetLastError();
-        return CSE_OOM;
-    }
-    c->keys_cap = need;
-    return CSE_OK;
-}
-
 constexpr int kSmemLimit = 96 * 1024;
 
 template <typename Kern>
@@ -1347,7 +1332,7 @@ int launch_b4(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32
     // a warp's keys: its share of the sample and its 512 trials of every step
     constexpr int TT = b4_group<PACKED, G>(), NW = TT / 32;
     const int32_t key_seg = kSample / NW + (K_tiles + TT * 16 - 1) / (TT * 16) * 512;
-    if (SEL && (st = b4_grow_keys(c, grid * G, (int64_t)NW * key_seg)) != CSE_OK) return st;
+    if (SEL && (st = cse_reserve_keys(c, sizeof(uint32_t) * G * NW * (size_t)key_seg, &grid, s)) != CSE_OK) return st;
     int32_t dlo = 0, nd = 1;
     b4_diff_range(c->bt_top, &dlo, &nd);
     if (SEL && o.min_out) c->min_folded = true;
@@ -1370,7 +1355,7 @@ int launch_b4_direct(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride
     int64_t grid = 0;
     int st = b4_grid(c, kern, BT, 0, T.n_tiles, &grid);
     if (st != CSE_OK) return st;
-    if (SEL && (st = b4_grow_keys(c, grid, k_stride)) != CSE_OK) return st;
+    if (SEL && (st = cse_reserve_keys(c, sizeof(uint32_t) * (size_t)k_stride, &grid, s)) != CSE_OK) return st;
     if (SEL && o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
     cse_prof_begin(c, KID_SIM_BAYES4, s);
@@ -1391,8 +1376,8 @@ int launch_b4_tables(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride
     // 32-bit offsets into the count table while it is smaller than 4 GB
     if ((uint64_t)(PACKED ? 2 : 3) * (uint64_t)NA * (uint64_t)k_stride > 0xFFFFFFFFull)
         return launch_b4<SEL, PACKED, 1, uint64_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);
-    // (the groups' key rows are K words each: no more than one tile a block for
-    // the largest K, which keeps the keys of a launch below 1.3 GB)
+    // (a group's keys are K words: one tile a block for the largest K keeps the keys of a
+    // launch at 1.3 GB, in the byte form 2.6 GB)
     if (T.n_tiles >= (int64_t)c->num_sms * 2 * G && K_tiles <= (1 << 17))
         return launch_b4<SEL, PACKED, G, uint32_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);
     return launch_b4<SEL, PACKED, 1, uint32_t>(c, T, NA, k_stride, K_tiles, lambda, o, s);

@@ -54,6 +54,8 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include <algorithm>
+
 #include "cse_internal.cuh"
 
 namespace {
@@ -570,58 +572,78 @@ __global__ void __launch_bounds__(kTailThreads, 4)
     queue_reset_min(counter, o.min_key, mine, o.min_out, (int)gridDim.x);
 }
 
+// A warp's keys: its 1,024 trials of every step.
+template <int G>
+int32_t tail_key_seg(int32_t K_tiles)
+{
+    constexpr int TT = kTailThreads / G;
+    return (K_tiles + TT * 32 - 1) / (TT * 32) * 1024;
+}
+
+template <bool WORDS, int G>
+int reserve_tail(cse_ctx* c, const TileArgs& T, int32_t K_tiles, cudaStream_t s)
+{
+    int per_sm = 0;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_sim_tail<WORDS, G>, kTailThreads, 0) != cudaSuccess ||
+        per_sm < 1) {
+        cudaGetLastError();
+        return CSE_CUDA_ERROR;
+    }
+    c->tail_grid = std::min<int64_t>((int64_t)per_sm * c->num_sms, (T.n_tiles + G - 1) / G);
+    const size_t bytes =
+        sizeof(typename tail_key<WORDS>::type) * (kTailThreads / 32) * (size_t)tail_key_seg<G>(K_tiles);
+    return cse_reserve_keys(c, bytes, &c->tail_grid, s);
+}
+
 template <bool WORDS, int G>
 int launch_tail(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
                 uint32_t* c_tile, cudaStream_t s)
 {
     auto kern = k_sim_tail<WORDS, G>;
-    constexpr int TT = kTailThreads / G, NW = TT / 32;
-    int per_sm = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kTailThreads, 0) != cudaSuccess || per_sm < 1) {
-        cudaGetLastError();
-        return CSE_CUDA_ERROR;
-    }
-    int64_t grid = (int64_t)per_sm * c->num_sms;
-    const int64_t blocks = (T.n_tiles + G - 1) / G;
-    if (grid > blocks) grid = blocks;
-    // a warp's keys: its 1,024 trials of every step
-    const int32_t key_seg = (K_tiles + TT * 32 - 1) / (TT * 32) * 1024;
-    const size_t need = sizeof(typename tail_key<WORDS>::type) * (size_t)grid * G * NW * (size_t)key_seg;
-    if (need > c->keys_cap) {
-        cudaFree(c->keys);
-        c->keys = nullptr;
-        c->keys_cap = 0;
-        if (cudaMalloc(&c->keys, need) != cudaSuccess) {
-            cudaGetLastError();
-            return CSE_OOM;
-        }
-        c->keys_cap = need;
-    }
+    const int32_t key_seg = tail_key_seg<G>(K_tiles);
     int sh = 0;   // ranks per bin: at most 256 bins, at most 128 ranks a bin (n_cells <= 129^2)
     while (((c->n_cells - 1) >> sh) > 255) ++sh;
     if (o.min_out) c->min_folded = true;
     if (o.cp_key) c->cp_marked = true;
     cse_prof_begin(c, KID_SIM_ZTEST, s);
-    cse_launch(c->pdl, kern, dim3((unsigned)grid), dim3(kTailThreads), 0, s, T, c->D.n_max, c->cnt, NA, k_stride,
-               K_tiles, c->rank_tab, c->S_tab, c->val_of_rank, c->cell_of_pos, c->n_cells, c->n1p, sh, c->bb, c->zpar,
-               c->zcut, c->z_lambda, c->tb, o, c_tile, c->keys, key_seg, c->counter, c->err);
+    cse_launch(c->pdl, kern, dim3((unsigned)c->tail_grid), dim3(kTailThreads), 0, s, T, c->D.n_max, c->cnt, NA,
+               k_stride, K_tiles, c->rank_tab, c->S_tab, c->val_of_rank, c->cell_of_pos, c->n_cells, c->n1p, sh, c->bb,
+               c->zpar, c->zcut, c->z_lambda, c->tb, o, c_tile, c->keys, key_seg, c->counter, c->err);
     cse_prof_end(c, s);
     c->launches += 1;
     return cudaGetLastError() == cudaSuccess ? CSE_OK : CSE_CUDA_ERROR;
+}
+
+// Tiles a block (wider groups for the largest K: fewer keys, and a trial's place within a
+// warp below 2^17).
+template <bool WORDS>
+int tail_groups(const cse_ctx* c, const TileArgs& T, int32_t K_tiles)
+{
+    const int64_t key_bytes = (int64_t)K_tiles * (WORDS ? 4 : 2);
+    if (T.n_tiles < 8 * (int64_t)c->num_sms || K_tiles > (1 << 18)) return 1;
+    if (T.n_tiles < 32 * (int64_t)c->num_sms || key_bytes > (1 << 17)) return 2;
+    return 4;
 }
 
 template <bool WORDS>
 int launch_groups(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_stride, int32_t K_tiles, const SimOut& o,
                   uint32_t* c_tile, cudaStream_t s)
 {
-    // (wider groups for the largest K: the keys of a launch stay below 1 GB, a trial's
-    // place within a warp below 2^17)
-    const int64_t key_bytes = (int64_t)K_tiles * (WORDS ? 4 : 2);
-    if (T.n_tiles < 8 * (int64_t)c->num_sms || K_tiles > (1 << 18))
-        return launch_tail<WORDS, 1>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
-    if (T.n_tiles < 32 * (int64_t)c->num_sms || key_bytes > (1 << 17))
-        return launch_tail<WORDS, 2>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
-    return launch_tail<WORDS, 4>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    switch (tail_groups<WORDS>(c, T, K_tiles)) {
+    case 1: return launch_tail<WORDS, 1>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    case 2: return launch_tail<WORDS, 2>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    default: return launch_tail<WORDS, 4>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+    }
+}
+
+template <bool WORDS>
+int reserve_groups(cse_ctx* c, const TileArgs& T, int32_t K_tiles, cudaStream_t s)
+{
+    switch (tail_groups<WORDS>(c, T, K_tiles)) {
+    case 1: return reserve_tail<WORDS, 1>(c, T, K_tiles, s);
+    case 2: return reserve_tail<WORDS, 2>(c, T, K_tiles, s);
+    default: return reserve_tail<WORDS, 4>(c, T, K_tiles, s);
+    }
 }
 
 // Rejections alone: a group of TT threads per tile, sixteen trials a thread and step.
@@ -720,4 +742,9 @@ int cse_launch_sim_tail(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t k_str
 {
     return words ? launch_groups<true>(c, T, NA, k_stride, K_tiles, o, c_tile, s)
                  : launch_groups<false>(c, T, NA, k_stride, K_tiles, o, c_tile, s);
+}
+
+int cse_tail_reserve(cse_ctx* c, const TileArgs& T, int32_t K_tiles, bool words, cudaStream_t s)
+{
+    return words ? reserve_groups<true>(c, T, K_tiles, s) : reserve_groups<false>(c, T, K_tiles, s);
 }
