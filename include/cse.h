@@ -292,8 +292,9 @@ enum { CSE_OPT_BAYES_DIRECT = 1, CSE_OPT_PLAIN = 2, CSE_OPT_SIM_THREADS = 3, CSE
        CSE_OPT_PDL = 5, CSE_OPT_SIM_TILES = 7 };
 /* CSE_OPT_PLAIN: 1 selects the plain comparison path with the same results:
  * success counts by one binary search per (tile, sim, arm) in sorted
- * uniforms, which the first such call of a key generates (no axis count table), the bound pass entirely in FP64 (bisection
- * over q, Newton for Clopper-Pearson, no FP32 stage), and for BAYES4 and BERRY4
+ * uniforms (z-test designs: allocated here, CSE_OOM if that fails; the first such call
+ * of a key generates them) instead of the axis count table, the bound pass entirely in
+ * FP64 (bisection over q, Newton for Clopper-Pearson, no FP32 stage), and for BAYES4 and BERRY4
  * the direct per-trial posterior.  0 (default) is the chosen path.
  * The z-test designs simulate by byte-parallel rejection counts (calls without an
  * order statistic, n_max <= 126), by candidate trials (two arms, lambda <= -1 and

@@ -162,14 +162,6 @@ int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = f
     cse_capturing(c, s);
     CSE_TRY(cse_launch_thresholds(c, P.T, P.NA, s));
     if (c->plain && !cse_posterior_design(c->D.stat)) {
-        if (!c->U) {
-            const size_t ub = sizeof(uint32_t) * (size_t)c->D.d * (size_t)c->K_max * (size_t)c->D.n_max;
-            if (cudaMalloc(&c->U, ub) != cudaSuccess) {
-                cudaGetLastError();
-                c->U = nullptr;
-                return CSE_OOM;
-            }
-        }
         if (c->u_stale) {
             CSE_TRY(cse_launch_uniforms(c, s));
             c->u_stale = false;
@@ -393,6 +385,15 @@ int cse_set_option(cse_ctx* c, int option, int64_t value)
     if (!c) return CSE_INVALID_ARG;
     switch (option) {
     case CSE_OPT_PLAIN:
+        // the plain z-test path's uniforms: here, so that its first call can be captured
+        if (value != 0 && !c->U && !cse_posterior_design(c->D.stat)) {
+            const size_t ub = sizeof(uint32_t) * (size_t)c->D.d * (size_t)c->K_max * (size_t)c->D.n_max;
+            if (cudaMalloc(&c->U, ub) != cudaSuccess) {
+                cudaGetLastError();
+                c->U = nullptr;
+                return CSE_OOM;
+            }
+        }
         c->plain = value != 0;
         if (cse_posterior_design(c->D.stat) && c->bt_tables) c->bt_direct = c->plain;
         return CSE_OK;

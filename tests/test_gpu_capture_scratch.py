@@ -1,7 +1,8 @@
 """Selection keys and CUDA graphs: a step that needs more key scratch than the calls
 before it reserved is captured all the same (fewer blocks, or the cell histogram, which
-needs none), as nothing may be allocated during a capture; and a captured step keeps its
-scratch when a later call of the same context needs more."""
+needs none), as nothing may be allocated during a capture; so is the first call of the
+plain path; and a captured step keeps its scratch when a later call of the same context
+needs more."""
 import pytest
 import torch
 
@@ -51,6 +52,18 @@ def test_step_that_needs_more_keys_is_captured(B, design, tiles, K_before, alpha
     ref = B.Context(design, seed=9, K_max=K_before).step(dt, lam, 0.01, 0.025)
     torch.cuda.synchronize()
     for k in KEYS:
+        assert torch.equal(got[k], ref[k]), k
+
+
+def test_plain_call_is_captured(B):
+    """The sorted uniforms of the plain path are there before its first call."""
+    dt = B.DeviceTiles(W.two_arm_grid(12, 700))
+    ctx = B.Context(W.TWO_ARM, seed=9, K_max=700)
+    out = ctx.step_buffers(dt)
+    ref = {k: v.clone() for k, v in ctx.step(dt, -1.96, 0.01, 0.025, out).items() if k in KEYS}
+    ctx.set_option(B.OPT_PLAIN, 1)
+    got = _replayed(_capture(ctx, dt, -1.96, 0.025, out), out)
+    for k in ("R", "Xrej", "lambda_tile", "lam"):
         assert torch.equal(got[k], ref[k]), k
 
 
