@@ -380,12 +380,18 @@ def run_chosen(args):
         step(i)
     torch.cuda.synchronize()
     ctx.sync()
-    if args.sim_threads:   # fixed configuration (e.g. to match a live run's choice under a profiler)
+    # the cell-histogram kernel's (threads, tiles) per block, where the step runs that kernel:
+    # the one-arm design, and two arms when a configuration is fixed (the step's own choice
+    # there is the candidate kernel)
+    tuned = None
+    if args.sim_threads and design.stat not in POSTERIOR:
         ctx.set_option(B.OPT_SIM_THREADS, args.sim_threads)
         ctx.set_option(B.OPT_SIM_TILES, args.sim_tiles)
         tuned = (args.sim_threads, args.sim_tiles)
-    else:
-        tuned = ctx.autotune(dt, LAMBDA, ALPHA)   # (threads, tiles) per block of the simulation kernel
+    elif design.stat == "one_arm_z":
+        tuned = ctx.autotune(dt, LAMBDA, ALPHA)
+    form = {"bayes4": "k_sim_bayes4", "berry4": "k_sim_basket"}.get(design.stat,
+                                                                    "k_sim_cells" if tuned else "k_sim_tail")
 
     clocks = ClockSampler(local)
     clocks.start()
@@ -659,8 +665,9 @@ def run_chosen(args):
                 "cuda_graph": None if graph_ms is None else {
                     "ms_per_step": graph_ms, "value": units * world / (graph_ms * 1e-3),
                     "note": "same step replayed from one captured CUDA graph (CRN key fixed in the graph)"},
-                "autotune": {"sim_threads_per_block": tuned[0], "tiles_per_block": tuned[1],
-                             "sims_per_block_step": 16 * tuned[0] if design.stat not in POSTERIOR else 4 * tuned[0]},
+                "simulation_kernel": form,
+                "autotune": None if not tuned else {"sim_threads_per_block": tuned[0], "tiles_per_block": tuned[1],
+                                                    "sims_per_block_step": 16 * tuned[0]},
                 "peaks_measured": peaks,
                 "context_setup": {"ms": setup_ms, "what": "cse_create, once per context (host clock): the first CRN "
                                   "uniforms and the design's statistic tables (the four-arm and basket designs' "
@@ -689,7 +696,8 @@ def main():
     ap.add_argument("--no-plain", action="store_true", help="skip the plain-path comparison")
     ap.add_argument("--no-band", action="store_true", help="skip the validation-band timing")
     ap.add_argument("--sim-threads", type=int, default=0, choices=[0, 64, 128, 256, 512],
-                    help="fix the simulation kernel's block size instead of autotuning (z-tests)")
+                    help="run the z-test cell-histogram kernel in this block size (two arms: instead of the "
+                         "candidate kernel that the step runs otherwise)")
     ap.add_argument("--sim-tiles", type=int, default=1, choices=[1, 2, 4],
                     help="with --sim-threads: tiles per block of the z-test cell kernel")
     ap.add_argument("--no-graph", action="store_true", help="skip the CUDA-graph replay timing")

@@ -1541,7 +1541,7 @@ __global__ void k_backward(int64_t n, int32_t d, const double* __restrict__ g, c
 }  // namespace
 
 // z with Phi(z) = p (0 < p < 1), to ~1e-7: the start of the Clopper-Pearson solves.
-double normal_quantile(double p)
+static double normal_quantile(double p)
 {
     double lo = -40.0, hi = 40.0;
     for (int it = 0; it < 60; ++it) {

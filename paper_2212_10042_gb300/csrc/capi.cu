@@ -170,7 +170,8 @@ int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = f
     }
     CSE_TRY(cse_launch_axis_counts(c, P.T, P.NA, P.K_tiles, P.k_stride, s));
     // the z-test cell and candidate kernels read each axis value's least and greatest count
-    if (!cse_posterior_design(c->D.stat) && c->zmode != ZMODE_COUNT) CSE_TRY(cse_launch_axis_box(c, P.NA, P.K_tiles, P.k_stride, s));
+    if (!cse_posterior_design(c->D.stat) && c->zmode != ZMODE_COUNT)
+        CSE_TRY(cse_launch_axis_box(c, P.NA, P.K_tiles, P.k_stride, s));
     return CSE_OK;
 }
 
@@ -599,7 +600,8 @@ int cse_create(cse_ctx** out, const cse_design* design, uint64_t seed, int32_t K
         // ticket 0, key count 0, running-minimum key all ones and its ticket 0
         if (cudaMemsetAsync(c->err, 0, 64, s) != cudaSuccess || cudaMemsetAsync(c->min_key, 0, 64, s) != cudaSuccess ||
             cudaMemsetAsync(c->min_key, 0xFF, sizeof(unsigned long long), s) != cudaSuccess ||
-            cudaMemsetAsync(c->counter, 0, 64, s) != cudaSuccess || cudaMemsetAsync(c->cp_nkeys, 0, 64, s) != cudaSuccess) {
+            cudaMemsetAsync(c->counter, 0, 64, s) != cudaSuccess ||
+            cudaMemsetAsync(c->cp_nkeys, 0, 64, s) != cudaSuccess) {
             st = CSE_CUDA_ERROR;
             break;
         }
@@ -845,7 +847,8 @@ int cse_calibrate_rand(cse_ctx* c, const cse_tiles* t, double alpha, double* alp
     tail_or_cells(c, P, true, s);
     CSE_TRY(tables_and_alpha_prime(c, P, alpha, alpha_prime_out, s, nullptr, true));
     SimOut o = {c->sig, nullptr, nullptr, nullptr, lambda_tile_out, c->ksel};
-    if (c->zmode == ZMODE_TAIL) CSE_TRY(cse_launch_sim_tail(c, P.T, P.NA, P.k_stride, P.K_tiles, o, true, c_tile_out, s));
+    if (c->zmode == ZMODE_TAIL)
+        CSE_TRY(cse_launch_sim_tail(c, P.T, P.NA, P.k_stride, P.K_tiles, o, true, c_tile_out, s));
     else CSE_TRY(cse_launch_sim_rand(c, P.T, P.NA, P.k_stride, P.K_tiles, INFINITY, 0u, o, c_tile_out, s));
     // (lambda*, c*) through the device scalars lam_dev and lam_dev + 1 (its low 4 bytes)
     uint32_t* c_dev = reinterpret_cast<uint32_t*>(c->lam_dev + 1);

@@ -499,7 +499,7 @@ struct cse_ctx {
     uint2* bk_bits;         // basket design: a bit per count state and arm, Q_i below each level of S; the last
                             // level is the call's lambda (k_basket_bits)
     float4* bk_q;           // basket design: (1 - P(theta_i > t_i | x)) per count state (see sim_basket.cu)
-    int32_t* left;          // [tile_cap] tiles that a candidate kernel leaves to the kernel after it (counter[2] of them)
+    int32_t* left;          // [tile_cap] tiles that k_sim_basket leaves to the kernel after it (counter[2] of them)
     uint32_t* keys;         // per-CTA statistic keys for order-statistic selection (cse_reserve_keys)
     size_t keys_cap;
     int64_t tail_grid;      // blocks of the current call's k_sim_tail (cse_tail_reserve)

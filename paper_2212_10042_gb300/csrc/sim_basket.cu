@@ -134,8 +134,8 @@ __device__ __forceinline__ int basket_warp_sum(int v)
 
 // One thread: the tile's outputs from the warps' sums.
 __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B, const SimOut& o, int64_t i, int K,
-                                             bool bad, const int* v, const int (*red)[BWARP], int warps, bool select, double lam_i,
-                                             int32_t* err)
+                                             bool bad, const int* v, const int (*red)[BWARP], int warps,
+                                             bool select, double lam_i, int32_t* err)
 {
     if (bad) atomicOr(err, CSE_ERR_BAD_K);
     int64_t Rt = 0, X[4] = {0, 0, 0, 0};

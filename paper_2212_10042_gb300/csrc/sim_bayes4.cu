@@ -1425,7 +1425,7 @@ int cse_bayes4_setup(cse_ctx* c, cudaStream_t s)
     // constant variance, so one difference cuts at about the same S for every
     // control count) scaled to 0 .. kScoreTop where that keeps them distinct; the
     // counts themselves otherwise
-    std::vector<uint8_t> score((size_t)L.n3 + 1);
+    uint8_t score[CSE_MAX_NMAX + 1];
     const double lo = asin(sqrt(1.0 / (L.n3 + 2.0))), hi = asin(sqrt((L.n3 + 1.0) / (L.n3 + 2.0)));
     bool distinct = c->bt_packed;
     for (int x = 0; x <= L.n3; ++x) {
@@ -1435,13 +1435,15 @@ int cse_bayes4_setup(cse_ctx* c, cudaStream_t s)
     if (!distinct)
         for (int x = 0; x <= L.n3; ++x) score[x] = (uint8_t)x;
     c->bt_top = score[L.n3];
-    std::vector<uint32_t> none((size_t)(2 * c->bt_top + 1), 0x7F800000u);
-    if (cudaMalloc(&c->bt_dmin, none.size() * 4) != cudaSuccess || cudaMalloc(&c->bt_score, score.size()) != cudaSuccess) {
+    uint32_t none[2 * CSE_MAX_NMAX + 1];
+    for (uint32_t& x : none) x = 0x7F800000u;
+    if (cudaMalloc(&c->bt_dmin, sizeof(none)) != cudaSuccess ||
+        cudaMalloc(&c->bt_score, sizeof(score)) != cudaSuccess) {
         cudaGetLastError();
         return CSE_OOM;
     }
-    if (cudaMemcpyAsync(c->bt_dmin, none.data(), none.size() * 4, cudaMemcpyHostToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(c->bt_score, score.data(), score.size(), cudaMemcpyHostToDevice, s) != cudaSuccess) {
+    if (cudaMemcpyAsync(c->bt_dmin, none, sizeof(none), cudaMemcpyHostToDevice, s) != cudaSuccess ||
+        cudaMemcpyAsync(c->bt_score, score, (size_t)L.n3 + 1, cudaMemcpyHostToDevice, s) != cudaSuccess) {
         cudaGetLastError();
         return CSE_CUDA_ERROR;
     }

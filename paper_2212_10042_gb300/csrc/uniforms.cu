@@ -10,7 +10,6 @@
 #include <cuda_runtime.h>
 
 #include <cstring>
-#include <type_traits>
 
 #include "cse_internal.cuh"
 
@@ -19,12 +18,6 @@ namespace {
 // what a count table holds (see k_counts)
 constexpr int kCountsRaw = 0, kCountsNib = 1, kCountsMapped = 2;
 
-// One warp per (arm, sim) row: lane L generates and holds elements L*E .. L*E+E-1
-// (E = 32-padded power of two / 32), and a bitonic network over the 32*E keys
-// (in-register pairs when the partner distance is below E, warp shuffles above)
-// sorts the row.  With several analysis segments the key carries the segment
-// index above the word, so the row comes out sorted within each segment and
-// segments in order; pad keys (all ones) sort last and are not written.
 // Success threshold and sigmoid of axis value i of a tile set (flattened over
 // the arms' axes).
 __device__ __forceinline__ void threshold_of(int i, uint32_t* __restrict__ thr, double* __restrict__ sig,
@@ -37,14 +30,18 @@ __device__ __forceinline__ void threshold_of(int i, uint32_t* __restrict__ thr, 
     if (sig) sig[i] = 1.0 / (1.0 + exp(-th));
 }
 
+// One warp per (arm, sim) row: lane L generates and holds elements L*E .. L*E+E-1
+// (E = 32-padded power of two / 32), and a bitonic network over the 32*E keys
+// (in-register pairs when the partner distance is below E, warp shuffles above)
+// sorts the row; pad keys (all ones) sort last and are not written.
 //
 // The randomised test's tie-break word of every sim rides on the first blocks, one
 // thread each (tb; word 0 of Philox4x32-10(counter (k, 0, 0, 1), key = seed), the
 // patients' draws using counter word 3 = 0).
-template <int E, bool SEG>
+template <int E>
 __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int32_t K_max, int32_t d,
-                                                  int32_t n_looks, int4 looks, int32_t n_max,
-                                                  uint32_t key0, uint32_t key1, uint32_t* __restrict__ tb)
+                                                  int32_t n_max, uint32_t key0, uint32_t key1,
+                                                  uint32_t* __restrict__ tb)
 {
     pdl_entry();
     const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -52,13 +49,12 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
         u32x4 c = {(uint32_t)g, 0u, 0u, 1u};
         tb[g] = philox4x32_10(c, key0, key1).x;
     }
-    using Key = typename std::conditional<SEG, unsigned long long, uint32_t>::type;
     constexpr int NP = 32 * E;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int64_t row = (int64_t)blockIdx.x * 8 + warp;   // row = a * K_max + k
     if (row >= (int64_t)d * K_max) return;                  // the whole warp leaves together
     const uint32_t a = (uint32_t)(row / K_max), k = (uint32_t)(row % K_max);
-    Key v[E];
+    uint32_t v[E];
     u32x4 w = {0u, 0u, 0u, 0u};
 #pragma unroll
     for (int i = 0; i < E; ++i) {
@@ -68,13 +64,7 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
             w = philox4x32_10(c, key0, key1);
         }
         const uint32_t u = ((e & 3) == 0) ? w.x : ((e & 3) == 1) ? w.y : ((e & 3) == 2) ? w.z : w.w;
-        if (SEG) {
-            const unsigned long long seg = (unsigned long long)((n_looks > 1 && e >= looks.x) ? 1 : 0) +
-                                           ((n_looks > 2 && e >= looks.y) ? 1 : 0);
-            v[i] = (e < n_max) ? (Key)((seg << 32) | u) : (Key)~0ull;
-        } else {
-            v[i] = (e < n_max) ? (Key)u : (Key)0xFFFFFFFFu;
-        }
+        v[i] = (e < n_max) ? u : 0xFFFFFFFFu;
     }
 #pragma unroll
     for (int kk = 2; kk <= NP; kk <<= 1) {
@@ -84,7 +74,7 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
 #pragma unroll
                 for (int i = 0; i < E; ++i) {
                     const int e = lane * E + i;
-                    const Key p = __shfl_xor_sync(0xffffffffu, v[i], j / E);
+                    const uint32_t p = __shfl_xor_sync(0xffffffffu, v[i], j / E);
                     const bool keep_min = ((e & kk) == 0) == ((e & j) == 0);
                     v[i] = keep_min ? (p < v[i] ? p : v[i]) : (p > v[i] ? p : v[i]);
                 }
@@ -94,8 +84,8 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
                     if ((i & j) == 0) {
                         const int i2 = i | j;
                         const bool up = ((lane * E + i) & kk) == 0;
-                        const Key x = v[i], y = v[i2];
-                        const Key lo = x < y ? x : y, hi = x < y ? y : x;
+                        const uint32_t x = v[i], y = v[i2];
+                        const uint32_t lo = x < y ? x : y, hi = x < y ? y : x;
                         v[i] = up ? lo : hi;
                         v[i2] = up ? hi : lo;
                     }
@@ -107,13 +97,14 @@ __global__ void __launch_bounds__(256) k_uniforms(uint32_t* __restrict__ U, int3
 #pragma unroll
     for (int i = 0; i < E; ++i) {
         const int e = lane * E + i;
-        if (e < n_max) out[e] = (uint32_t)v[i];
+        if (e < n_max) out[e] = v[i];
     }
 }
 
 // Success threshold and sigmoid (for the score's grad A) of every axis value.  With
 // Z.S set (z-test calls that do not run the cell histogram) the last block finds
-// the call's constants: the number of cells with S < lambda (Z.pos) or per x_0 the least x_1 with S < lambda (n_max + 1: none; each row of S falls in x_1).
+// the call's constants: the number of cells with S < lambda (Z.pos), and per x_0 the least
+// x_1 with S < lambda (n_max + 1: none; each row of S falls in x_1).
 struct TailArgs {
     const float* S;
     int32_t n_cells, n1p, n_max;   // row length n1p: n_max + 1, or 1 for one arm
@@ -485,24 +476,14 @@ int cse_launch_uniforms(cse_ctx* c, cudaStream_t s)
 {
     const int64_t rows = (int64_t)c->D.d * c->K_max;
     const int blocks = (int)((rows + 7) / 8);
-    int4 lk = make_int4(c->D.look_n[0], c->D.look_n[1], c->D.look_n[2], 0);
     const int n = c->D.n_max;
-    const bool seg = c->D.n_looks > 1;
     const uint32_t k0 = (uint32_t)c->seed, k1 = (uint32_t)(c->seed >> 32);
     cse_prof_begin(c, KID_UNIFORMS, s);
-#define CSE_UNIFORMS(E, SG)                                                                                       \
-    cse_launch(c->pdl, k_uniforms<E, SG>, dim3(blocks), dim3(256), 0, s, c->U, c->K_max, c->D.d, c->D.n_looks, lk, \
-               n, k0, k1, c->tb)
-    if (n <= 32) {
-        if (seg) CSE_UNIFORMS(1, true);
-        else CSE_UNIFORMS(1, false);
-    } else if (n <= 64) {
-        if (seg) CSE_UNIFORMS(2, true);
-        else CSE_UNIFORMS(2, false);
-    } else {
-        if (seg) CSE_UNIFORMS(4, true);
-        else CSE_UNIFORMS(4, false);
-    }
+#define CSE_UNIFORMS(E) \
+    cse_launch(c->pdl, k_uniforms<E>, dim3(blocks), dim3(256), 0, s, c->U, c->K_max, c->D.d, n, k0, k1, c->tb)
+    if (n <= 32) CSE_UNIFORMS(1);
+    else if (n <= 64) CSE_UNIFORMS(2);
+    else CSE_UNIFORMS(4);
 #undef CSE_UNIFORMS
     cse_prof_end(c, s);
     c->launches += 1;
@@ -580,10 +561,12 @@ static int launch_counts(cse_ctx* c, const TileArgs& T, int32_t NA, int32_t K_ti
 int cse_launch_axis_counts(cse_ctx* c, const TileArgs& T, int32_t n_axis_total, int32_t K_tiles,
                            int32_t k_stride, cudaStream_t s)
 {
-    if (cse_count_nibbles(c)) return launch_counts<3, kCountsNib>(c, T, n_axis_total, K_tiles, k_stride, c->bt_score, s);
+    if (cse_count_nibbles(c))
+        return launch_counts<3, kCountsNib>(c, T, n_axis_total, K_tiles, k_stride, c->bt_score, s);
     if (c->D.n_looks > 1) return launch_counts<3, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
     // (b(x_0) beside arm 0's counts: where the kernel counts rejections by bytes)
-    const bool map = c->zmode == ZMODE_COUNT || (c->zmode == ZMODE_TAIL && c->D.n_max <= 126 && c->z_lambda > -INFINITY);
+    const bool map = c->zmode == ZMODE_COUNT ||
+                     (c->zmode == ZMODE_TAIL && c->D.n_max <= 126 && c->z_lambda > -INFINITY);
     if (map && T.d == 2)
         return launch_counts<1, kCountsMapped>(c, T, n_axis_total, K_tiles, k_stride, c->zcut, s);
     return launch_counts<1, kCountsRaw>(c, T, n_axis_total, K_tiles, k_stride, nullptr, s);
