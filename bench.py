@@ -84,23 +84,23 @@ WORKLOADS = {
 OPS_PER_SIM_TILE = {"one_arm_z": 5, "two_arm_pooled_z": 6, "bayes4": 22, "berry4": 12}
 # What bounds each simulation kernel, from its ncu profile (profiles/)
 LIMITER = {
-    "sim_ztest": "two arms with a selection: issue slots (60 %: byte tests, queueing, 7 % of the sims evaluated) and "
+    "sim_ztest": "two arms with a selection: issue slots (67 %: byte tests, queueing, 7 % of the sims evaluated) and "
                  "the latency of the candidates' reads; one arm: latency",
-    "sim_bayes4": "issue slots (63 to 65 %; four fifths of the instructions evaluate the 13 to 19 % candidate trials) "
+    "sim_bayes4": "issue slots (71 %; four fifths of the instructions evaluate the 13 to 19 % candidate trials) "
                   "at the latency of their scattered reads",
-    "sim_basket": "issue slots (66 %) and the integer ALU pipe (64 %: byte transposes, window tests, word indexing)",
+    "sim_basket": "issue slots (71 %) and the integer ALU pipe (65 %: byte transposes, window tests, word indexing)",
 }
 # DRAM bytes (read + write) per launch of the dominant kernel from one ncu
 # capture of the same kernel build, scaled to the workload where the capture
 # ran on a smaller case; None until captured for the current kernel
 MEASURED_TRAFFIC = {
-    # profiles/k_sim_bayes4_four_arm_refined_sample_65536x65536.md: 24.4 GB on 2^18 tiles of the
-    # platten, scaled by the sim-tiles (x 4.0); 6.34 GB on the 65,536-tile sample
-    ("c5", "sim_bayes4"): 97.6e9,
-    ("c5_sample", "sim_bayes4"): 6.34e9,
+    # profiles/k_sim_bayes4_four_arm_refined_sample_65536x65536.md: 27.6 GB on 2^18 tiles of the
+    # platten, scaled by the sim-tiles (x 4.0); 7.53 GB on the 65,536-tile sample
+    ("c5", "sim_bayes4"): 110e9,
+    ("c5_sample", "sim_bayes4"): 7.53e9,
     # profiles/k_sim_tail_two_arm_256x256_K16384.md: one capture at the full size, and the 2^18 batch
-    ("c2", "sim_ztest"): 9.69e6,
-    ("c3", "sim_ztest"): 709e6,
+    ("c2", "sim_ztest"): 9.57e6,
+    ("c3", "sim_ztest"): 365e6,
     # profiles/k_sim_basket_basket_8x8x8x8_K16384.md
     ("berry", "sim_basket"): 52.4e6,
 }

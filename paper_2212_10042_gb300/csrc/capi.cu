@@ -181,7 +181,7 @@ int launch_tables(cse_ctx* c, const Prepared& P, cudaStream_t s, bool counts = f
 // 28 -> 14).  With one, two arms: candidates, unless alpha or lambda reach so far into
 // the statistic that a good part of the trials are candidates, at about ten times the
 // cost of a histogram increment (256^2 grid, lambda = -1.96, alpha = 0.025: 7 %, 323 ->
-// 267 us; 128^2 grid, lambda = -1, alpha = 0.1: the whole call 395 -> 239).
+// 261 us; 128^2 grid, lambda = -1, alpha = 0.1: the whole call 395 -> 239).
 // The cell histogram takes the rest -- one arm among them, whose n + 1 cells are
 // read off at once (64 tiles 10.8 us against 12.4) -- and every call whose
 // configuration the caller fixed.

@@ -191,10 +191,10 @@ __device__ __forceinline__ void basket_store(const TileArgs& T, const Basket& B,
 // The share: a quarter against a half 536 / 612 us over [-1, 2], but n = 20 313 / 291.
 // 256 threads a tile below 4 tiles an SM: 150 tiles of 2^18 trials 1,565 -> 700 us.
 //
-// What bounds it: issue slots (65 %) and the integer pipe (64 %): per 32 trials ~17
+// What bounds it: issue slots (71 %) and the integer pipe (65 %): per 32 trials ~17
 // warp instructions of test and count, ~10 of queue and scan, ~7 of evaluation, and
 // ~20 of the tile's own work (building the window, setup, selection).  16^4 grid,
-// K = 2^14, with a selection (59,992 tiles): 3.67 -> 1.95 ms; 6,036 tiles of 1,000 to
+// K = 2^14, with a selection (59,992 tiles): 3.67 -> 1.90 ms; 6,036 tiles of 1,000 to
 // 30,000 trials without one: 152 -> 112 us, plus 10 for the bits of lambda.  Measured
 // on the way: one bit per state at a fixed level and every rejection evaluated 3.28 ms
 // (the candidates' own work), lambda's and the level's bits in separate words 2.58,

@@ -557,9 +557,9 @@ __device__ __forceinline__ void packed_tables(int tid, int nth, int* tri, uint32
 // them, a lane four consecutive trials from whole count words: no queue, no scattered
 // bytes (a candidate costs about twice a trial read that way).
 //
-// What bounds it: issue slots at the latency of the candidates' scattered reads (65 %
-// issue, 61 % ALU pipe, 69 warp instructions per 32 trials of which the candidates,
-// ~290 each, take four fifths).  262,144 refined tiles x 65,536 trials: 103 -> 38 ms; the
+// What bounds it: issue slots at the latency of the candidates' scattered reads (71 %
+// issue, 64 % ALU pipe, 62 to 68 warp instructions per 32 trials of which the candidates,
+// ~290 each, take four fifths).  262,144 refined tiles x 65,536 trials: 103 -> 36.8 ms; the
 // 16^4 grid at K = 2^14: 5.6 -> 1.9 ms.  Measured on the way: evaluating every candidate
 // by raw counts with a margin fixed by the sample 65 ms, with d raised along the pass
 // 51 ms; final-table loads that skip L1 lost 10 %.  Levels that make most trials

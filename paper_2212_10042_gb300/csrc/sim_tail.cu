@@ -40,11 +40,11 @@
 // theta = -2 and 2 1.5 (one trial in five is a candidate), 3 and beyond 1.2 to 1.3 (by
 // candidates 3.5 to 7); theta_1 = theta_0 + 2 1.5 (rejections as candidates 6).
 //
-// What bounds it: issue slots (54 to 60 % issue; 10 thread instructions a trial, of
+// What bounds it: issue slots (67 % issue; 10 to 12 thread instructions a trial, of
 // which the test and the queueing take half, the 7 % candidates a third) and the
 // latency of the scattered count reads.
-// 256^2 grid, K = 16,384 (32,896 tiles): 323 -> 267 us; 2^18 batch: 3.34 -> 2.55 ms;
-// randomised calibration of the 128^2 grid, the whole call: 275 -> 190 us.  Five blocks an
+// 256^2 grid, K = 16,384 (32,896 tiles): 323 -> 261 us; 2^18 batch: 3.34 -> 2.56 ms;
+// randomised calibration of the 128^2 grid, the whole call: 276 -> 187 us.  Five blocks an
 // SM at 48 registers were no faster than four at 56.
 //
 // Tiles: a group of TT threads per tile, G tiles a block: 64 threads with many
